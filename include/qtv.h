@@ -22,7 +22,7 @@
  *   psi      device pointer, complex64 interleaved (re, im) as two float32,
  *            nx*ny*nz elements, x fastest: node (i,j,k) is element
  *            (k*ny + j)*nx + i.  At least 8-byte aligned (16-byte alignment
- *            and even nx enable 16-byte vector loads).
+ *            and even nx are fastest).
  *   faces    named by the minimum corner (i,j,k) and orientation o:
  *            o = 0: xy plaquette, normal +z, loop (i,j)->(i+1,j)->(i+1,j+1)->(i,j+1)
  *            o = 1: yz plaquette, normal +x, loop (j,k)->(j+1,k)->(j+1,k+1)->(j,k+1)
@@ -81,9 +81,10 @@ typedef struct qtv_handle_s* qtv_handle;
 /* Grid geometry.  h and origin only scale and shift output positions:
  * node (i,j,k) sits at origin + h*(i,j,k).  periodic must be 0.  Sizes: nx up
  * to 2048, any ny and nz (node indices are 64-bit, so grids beyond 2^32
- * nodes such as 2048^3 work).  Even nx with a 16-byte aligned field takes the
- * staged sweeps (the bit-sliced default up to 2048 columns, the nibble sweep
- * up to 1024); odd nx or an 8-byte aligned field takes the register sweep. */
+ * nodes such as 2048^3 work).  The default is the bit-sliced staged sweep (odd
+ * nx or an 8-byte aligned field takes its instantiation for unaligned rows);
+ * a handle set to the nibble sweep takes that for even nx up to 1024 with a
+ * 16-byte aligned field, else the register sweep. */
 typedef struct {
   int32_t nx, ny, nz;
   float h;
@@ -330,8 +331,8 @@ QTV_API int qtv_locator_load(qtv_handle h, const char* path);
  * calls.  variant 0: nibble sweep (7-row bands, 64 columns per warp, warps
  * per tile 1..16, 0 = one tile per row); variant 1: bit-sliced sweep (16-row
  * bands, 31 columns per warp, warps per tile 2, 4 or 8, 0 = 4; stages 2 or 3
- * shared-memory ring slots, 0 = 3; rows wider than 32 warps of tiles fall back
- * to variant 0); -1: the library default.  ctas_per_sm caps resident CTAs per
+ * shared-memory ring slots, 0 = 3; rows of more warps of tiles than the expand
+ * pass takes fall back to variant 0); -1: the library default.  ctas_per_sm caps resident CTAs per
  * SM (0 = as many as fit).  Both variants give identical results.
  */
 QTV_API int qtv_configure_sweep(qtv_handle h, int variant, int warps_per_tile, int stages,

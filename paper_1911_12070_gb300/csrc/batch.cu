@@ -276,7 +276,7 @@ int autotune(qtv_handle h, BatchPlan* b, uint64_t faces, cudaStream_t st, TileCo
     for (int stages : {2, 3}) {
       int bps = 0;
       size_t smem = 0;
-      if (bits_variant_occupancy(nwt, stages, &bps, &smem)) continue;
+      if (bits_variant_occupancy(nwt, stages, false, &bps, &smem)) continue;
       std::vector<int> occ = {bps, std::max(1, bps / 2)};
       occ.erase(std::unique(occ.begin(), occ.end()), occ.end());
       for (int c : occ)

@@ -13,5 +13,7 @@ constexpr int BR = 16;            // owned rows per band
 constexpr int BRH = BR + 1;       // plus the halo row
 constexpr int BL = 31;            // owned columns per warp
 constexpr uint32_t kRows16 = 0xFFFFu;
+// set beside the lane in a record whose faces with code (0, 1) may be W = -2
+constexpr uint32_t kRecordTwos = 32u;
 }  // namespace bits
 }  // namespace qtv

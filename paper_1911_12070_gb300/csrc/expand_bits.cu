@@ -28,9 +28,25 @@ __device__ __forceinline__ uint32_t spread4(uint32_t m, int q) {
   return (((m >> (4 * q)) & 0xFu) * 0x00204081u) & 0x01010101u;
 }
 
+// W of a face from its corners, by the exact edge test (a record marked
+// kRecordTwos: only for determinants that underflow or overflow)
+__device__ __noinline__ int exact_winding(const float2* __restrict__ psi, unsigned long long nx,
+                                          unsigned long long ny, unsigned long long lin, int o) {
+  const unsigned long long d[3] = {1ull, nx, nx * ny};
+  const unsigned long long du = d[o], dv = d[o == 2 ? 0 : o + 1];
+  const float2 p0 = psi[lin], p1 = psi[lin + du], p2 = psi[lin + du + dv], p3 = psi[lin + dv];
+  // each grid edge is taken in its forward direction
+  auto r = [](float2 a, float2 b) {
+    const uint32_t e = exact_edge(a, b);
+    return (int)(e & 1u) - (int)(e >> 1);
+  };
+  return r(p0, p1) + r(p1, p2) - r(p3, p2) - r(p0, p3);
+}
+
 // MAXE: table entries a lane may hold (1 when every band row has at most 32
 // (tile, warp) steps, the common case, compiled without the wider selection)
-template <int MAXE>
+// TWOS: records may carry kRecordTwos (sweeps of unaligned rows)
+template <int MAXE, bool TWOS>
 __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expand_bits_kernel(
     const __grid_constant__ BulkParams a, const unsigned long long* __restrict__ seg_off,
     uint64_t* __restrict__ face_ids, int8_t* __restrict__ winding, unsigned long long capacity,
@@ -215,7 +231,9 @@ __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expan
             if (L | H) {
               if (pos < capacity) {
                 face_ids[pos] = (lin << 2) | (unsigned)o;
-                winding[pos] = (int8_t)(L ? (H ? -1 : 1) : 2);
+                int wv = L ? (H ? -1 : 1) : 2;
+                if (TWOS && !L && (rec.w & kRecordTwos)) wv = exact_winding(sd.psi, nx, ny, lin, o);
+                winding[pos] = (int8_t)wv;
               }
               ++pos;
             }
@@ -291,14 +309,13 @@ __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expan
 
 cudaError_t bits_expand_launch(const BulkParams& p, int blocks, const unsigned long long* seg_off,
                                uint64_t* face_ids, int8_t* winding, unsigned long long capacity,
-                               uint64_t* offsets, cudaStream_t st) {
+                               uint64_t* offsets, bool unal, cudaStream_t st) {
   bool wide = false;
   for (int i = 0; i < p.nsnap; ++i) wide |= p.s[i].ntx * p.s[i].nwt > 32;
-  if (wide)
-    return launch_dependent(expand_bits_kernel<kMaxE>, dim3(blocks), dim3(32 * kExpandWarps), 0,
-                            st, p, seg_off, face_ids, winding, capacity, offsets);
-  return launch_dependent(expand_bits_kernel<1>, dim3(blocks), dim3(32 * kExpandWarps), 0, st, p,
-                          seg_off, face_ids, winding, capacity, offsets);
+  auto* kern = wide ? (unal ? expand_bits_kernel<kMaxE, true> : expand_bits_kernel<kMaxE, false>)
+                    : (unal ? expand_bits_kernel<1, true> : expand_bits_kernel<1, false>);
+  return launch_dependent(kern, dim3(blocks), dim3(32 * kExpandWarps), 0, st, p, seg_off, face_ids,
+                          winding, capacity, offsets);
 }
 
 }  // namespace qtv

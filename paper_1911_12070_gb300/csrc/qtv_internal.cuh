@@ -197,8 +197,9 @@ int identify_launch(qtv_handle h, const qtv_grid& g, const float2* psi, uint64_t
                     cudaStream_t st, const IdentScratch& sc, uint64_t max_warps,
                     float* xyz = nullptr, float* resid = nullptr, uint8_t* flags = nullptr);
 
-// Bulk-copy staged sweeps (sweep_bulk.cu, sweep_bits.cu): even nx and a
-// 16-byte aligned psi; nx <= 1024 for the nibble sweep, <= 2048 for the
+// Bulk-copy staged sweeps (sweep_bulk.cu, sweep_bits.cu): nx <= 1024 for the
+// nibble sweep, <= 2048 for the bit-sliced one; even nx and a 16-byte aligned
+// psi in batches and for the nibble sweep, any in single-snapshot calls of the
 // bit-sliced one.
 struct BulkNeeds {
   uint64_t recs = 0, table = 0, seg_off = 0, tiles = 0, segf = 0;
@@ -249,6 +250,7 @@ struct TileConfig {
   int concurrent = 0;
   int variant = 0;
   int stages = 3;
+  bool unal = false;  // bit-sliced sweep: take odd nx and 8-byte aligned fields too
 };
 
 // One sweep launch: the snapshots of one group (same warps per tile), units
@@ -266,6 +268,7 @@ struct BatchLayout {
   std::vector<int> group_of;
   BulkParams fin;
   int variant = 0, stages = 3;
+  bool unal = false;  // the sweep's instantiation for unaligned rows
   int rec_words = 6;  // 32-bit words per staged record
   bool concurrent = false;
   int expand_blocks = 1;
@@ -341,8 +344,8 @@ __device__ __forceinline__ int geo_snapshot(const FaceGeo& G, unsigned long long
 
 int bulk_variant_occupancy(int nw, int* ctas_per_sm, size_t* smem);
 // bit-sliced sweep (sweep_bits.cu)
-int bits_variant_occupancy(int nw, int stages, int* ctas_per_sm, size_t* smem);
-void bits_sweep_launch(const BulkParams& p, int grid, int nw, int stages, size_t smem,
+int bits_variant_occupancy(int nw, int stages, bool unal, int* ctas_per_sm, size_t* smem);
+void bits_sweep_launch(const BulkParams& p, int grid, int nw, int stages, bool unal, size_t smem,
                        cudaStream_t st);
 // resident CTAs per SM of the bit-sliced expand kernel (its launch bound)
 constexpr int kBitsExpandCtasPerSm = 3;
@@ -352,7 +355,7 @@ constexpr int kBitsBandWarps = 96;
 constexpr int kNibbleBandWarps = 32;
 cudaError_t bits_expand_launch(const BulkParams& p, int blocks, const unsigned long long* seg_off,
                                uint64_t* face_ids, int8_t* winding, unsigned long long capacity,
-                               uint64_t* offsets, cudaStream_t st);
+                               uint64_t* offsets, bool unal, cudaStream_t st);
 int batch_layout(int num_sms, int nsnap, const qtv_grid* grids, const float2* const* psis,
                  const TileConfig& tc, uint64_t capacity, uint64_t max_warps, BatchLayout* B);
 int batch_launch(qtv_handle h, BatchLayout& B, const IdentScratch& sc, uint64_t* face_ids,
@@ -361,8 +364,9 @@ int batch_launch(qtv_handle h, BatchLayout& B, const IdentScratch& sc, uint64_t*
                  const SweepBranches* br);
 int batch_sweep_only(qtv_handle h, BatchLayout& B, const IdentScratch& sc, cudaStream_t st,
                      const SweepBranches* br);
-// whether a staged sweep (variant 1: bit-sliced, 0: nibble) can take a grid
-bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi);
+// whether a staged sweep (variant 1: bit-sliced, 0: nibble) can take a grid;
+// unal: with the bit-sliced sweep's instantiation for unaligned rows
+bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi, bool unal = false);
 // the staged sweep a single-snapshot call of handle h takes for a grid: the
 // handle's variant when it can, else the nibble sweep when that can, else -1
 // (the register sweep of identify.cu)

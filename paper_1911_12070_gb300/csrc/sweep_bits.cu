@@ -48,6 +48,21 @@
 // so each warp fills its own strip with 16-byte cp.async copies, one commit
 // group per plane, and the warps of a stacked unit run independently.
 //
+// Unaligned rows (UNAL).  With odd nx, or a field on an 8-byte boundary, a row
+// starts 8 bytes off a 16-byte boundary in some or all rows.  Its bulk copy is
+// widened to the boundaries (the neighbours in the field come along), which
+// shifts the row by one element in its slot row; a lane reads the even and the
+// odd rows of a plane at two column offsets.  Such fields took the register
+// sweep (identify.cu), whose edge test is exact, so this instantiation decides
+// the same windings: per edge it keeps the margin by which |cross| clears its
+// rounding errors, and a plane in which an edge is within reach of them (or a
+// component is zero or not finite) is redone with exact_edge.  Bound by issue:
+// five more instructions a row than the aligned instantiation.  512 x 512 x
+// 511: 0.284 ms against 0.785 for the register sweep (0.222 aligned at 512^3);
+// 275 x 301 x 253: 0.067 against 0.116; 256 x 256 x 255: 0.054 against 0.094.
+// Holding the smallest |cross| against a per-plane bound from the largest
+// component instead took 0.413 ms: near-parallel neighbours tripped it.
+//
 // Output and finalize.  Each lane with faces in a plane writes one 16-byte
 // record (L and H words of the three orientations, 16 rows each, and the lane)
 // into the fixed slot block of its (plane, band, tile, warp) step (32 records,
@@ -123,6 +138,46 @@ __device__ __forceinline__ void mod4(uint32_t a, uint32_t a1, uint32_t b, uint32
   H = a1 ^ b1 ^ c1 ^ d1 ^ e2;
 }
 
+// ---- exact edge test of the unaligned instantiation (see "Unaligned rows")
+// The FP32 cross value of a -> b has the sign of the exact determinant unless
+// |cross| <= 2^-21 |Im a Re b| (eight times its rounding errors) or its
+// products underflow (kTieMin is far above what that costs).  cross_m gives
+// the value and the margin by which it clears the first bound.
+constexpr float kTieMin = 1e-37f;
+constexpr float kTieFar = 3.402823466e38f;
+__device__ __forceinline__ float cross_m(float2 a, float2 b, float& m) {
+  const float p = a.y * b.x;
+  const float c = fmaf(a.x, b.y, -p);
+  m = fmaf(-4.76837158203125e-7f, fabsf(p), fabsf(c));
+  return c;
+}
+// Padding of rows past the grid: vectors whose x-, y- and z-neighbours differ,
+// so that no edge between them is a tie.
+__device__ __forceinline__ float2 pad_value(int row, int col, int slot) {
+  return make_float2(1.f, (float)(1 + (col & 1) + 2 * (row & 1) + 4 * slot));
+}
+// minima that keep a NaN
+__device__ __forceinline__ float min_nan(float a, float b) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2;" : "=f"(d) : "f"(a), "f"(b));
+  return d;
+}
+__device__ __forceinline__ float min_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ Edge edge_pn(uint32_t P, uint32_t N) {
+  Edge e;
+  e.P = P;
+  e.N = N;
+  e.Z = P | N;
+  return e;
+}
+__device__ __forceinline__ Edge edge_dn(const Edge& e) {
+  return edge_pn(__shfl_down_sync(0xffffffffu, e.P, 1), __shfl_down_sync(0xffffffffu, e.N, 1));
+}
+
 __device__ __forceinline__ uint32_t zero_bit(float2 v) {
   return ((__float_as_uint(v.x) | __float_as_uint(v.y)) << 1) == 0u ? 1u : 0u;
 }
@@ -130,14 +185,14 @@ __device__ __forceinline__ uint32_t bad_bit(float2 v) {
   return (finite_f(v.x) && finite_f(v.y)) ? 0u : 1u;
 }
 
-template <int NW, int MINB, int STAGES>
+template <int NW, int MINB, int STAGES, bool UNAL>
 __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_constant__ BulkParams a) {
   extern __shared__ __align__(128) unsigned char dsm[];
   pdl_trigger();  // the segment scan may queue behind this grid's blocks
   const int tid = threadIdx.x;
   const int lane = tid & 31;
   const int w = tid >> 5;
-  constexpr int W2 = BL * NW + 2;  // row pitch of a slot, in elements
+  constexpr int W2 = BL * NW + (UNAL ? 4 : 2);  // row pitch of a slot, in elements
   float2* ring = reinterpret_cast<float2*>(dsm);
   uint64_t* full =
       reinterpret_cast<uint64_t*>(dsm + ((size_t)STAGES * BRH * W2 + kTail) * sizeof(float2));
@@ -196,7 +251,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
     const int nsteps = ke - kb;
     const int xt0 = tile * sd.st;
     const bool last_tile = tile == ntx - 1;
-    const int tw = last_tile ? nx - xt0 : sd.st + 2;
+    // (an odd row may leave its last tile one column, which the tile before
+    // stages as its halo)
+    const int tw = last_tile ? nx - xt0 : (UNAL ? min(sd.st + 2, nx - xt0) : sd.st + 2);
     const int own_end = last_tile ? tw : sd.st;
     const uint32_t row_bytes = (uint32_t)tw * 8u;
     // first node of this warp's band (stacked) or the CTA's band in the tile,
@@ -212,7 +269,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
     if (stk) {
       if (!stk_padded) {
         for (int idx = tid; idx < STAGES * BRH * W2; idx += blockDim.x)
-          ring[idx] = make_float2(1.f, 1.f);
+          ring[idx] = UNAL ? pad_value(idx / W2 % BRH, idx % W2, idx / (BRH * W2))
+                           : make_float2(1.f, 1.f);
         fence_proxy_async();
         __syncthreads();
         stk_padded = true;
@@ -221,33 +279,99 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       valid_r = BRH;
     } else {
       stk_padded = false;
-      if (tw < valid_w || nrows < valid_r) {
-        const int cw = valid_w - tw;
+      // unaligned rows shift within their slot rows from plane to plane, so no
+      // column padding holds; lanes past the tile are left out of the test for
+      // special values instead (colv)
+      const int vw = UNAL ? W2 : tw;
+      if (vw < valid_w || nrows < valid_r) {
+        const int cw = valid_w - vw;
         if (cw > 0)
           for (int idx = tid; idx < STAGES * BRH * cw; idx += blockDim.x)
-            ring[(size_t)(idx / cw) * W2 + tw + idx % cw] = make_float2(1.f, 1.f);
+            ring[(size_t)(idx / cw) * W2 + vw + idx % cw] = make_float2(1.f, 1.f);
         const int rr = valid_r - nrows;
         if (rr > 0) {
           const int per = rr * W2;
           for (int idx = tid; idx < STAGES * per; idx += blockDim.x) {
             const int sl = idx / per, rem = idx % per;
-            ring[((size_t)sl * BRH + nrows + rem / W2) * W2 + rem % W2] = make_float2(1.f, 1.f);
+            ring[((size_t)sl * BRH + nrows + rem / W2) * W2 + rem % W2] =
+                UNAL ? pad_value(nrows + rem / W2, rem % W2, sl) : make_float2(1.f, 1.f);
           }
         }
         fence_proxy_async();
         __syncthreads();
       }
-      valid_w = tw;
+      valid_w = vw;
       valid_r = nrows;
     }
     for (int i = tid; i < nsteps; i += blockDim.x) s_faces[i] = 0u;
     __syncthreads();
+
+    // unaligned rows: shift of the even rows of the band in their slot rows
+    // in plane m (the odd rows' is the other one where nx is odd)
+    const uint32_t sh0 = UNAL && !stk
+                             ? (uint32_t)(reinterpret_cast<uintptr_t>(sd.psi) >> 3) ^
+                                   (uint32_t)((j0 & nx) ^ xt0)
+                             : 0u;
+    const uint32_t shm = UNAL && !stk ? (uint32_t)(nx & ny & 1) : 0u;
+    const uint32_t shr = UNAL && !stk ? (uint32_t)(nx & 1) : 0u;
+    auto shift = [&](int m) -> uint32_t { return (sh0 ^ ((uint32_t)m & shm)) & 1u; };
+    const bool colv = !UNAL || (wok && xs < tw);  // this lane's column is in the tile
 
     // warp 0: plane m into the next slot once every warp has released it
     auto produce = [&](int m) {
       const uint32_t q = fill;
       const int sl = (int)(q % STAGES);
       if (q >= (uint32_t)STAGES && !mbar_wait(&empty[sl], ((q / STAGES) - 1u) & 1u)) timeout = true;
+      if constexpr (UNAL) {
+        // Row `lane`, elements [lo, hi): widened to 16-byte boundaries, which
+        // adds neighbours in the field.
+        const float2* src = s_src[0] + (size_t)m * ((size_t)nx * ny) + (size_t)lane * nx;
+        const uint32_t she = shift(m), sho = she ^ shr;
+        const int sh = (int)(lane & 1 ? sho : she);
+        float2* dst = ring + ((size_t)sl * BRH + lane) * W2 + sh;  // element 0 of the row
+        if (m != 0 && m != nz - 1) {
+          const uint32_t be = (((uint32_t)tw + she + 1u) & ~1u) * 8u;
+          const uint32_t bo = (((uint32_t)tw + sho + 1u) & ~1u) * 8u;
+          if (lane == 0) {
+            fence_proxy_async();
+            mbar_arrive_expect_tx(&full[sl], be * (uint32_t)((nrows + 1) >> 1) +
+                                                 bo * (uint32_t)(nrows >> 1));
+          }
+          __syncwarp();
+          if (lane < nrows) bulk_g2s(dst - sh, src - sh, lane & 1 ? bo : be, &full[sl]);
+          ++fill;
+          return;
+        }
+        // The first and the last plane: nothing lies before the field's first
+        // element and after its last one; there one element is left to a plain
+        // copy.
+        int lo = -sh, hi = tw + ((tw + sh) & 1);
+        if (lane < nrows) {
+          if (sh && src == sd.psi) {
+            lo = 1;
+            dst[0] = src[0];
+            fence_proxy_async();
+          }
+          if (hi > tw && src + tw == sd.psi + (size_t)nx * ny * nz) {
+            hi = tw - 1;
+            dst[hi] = src[hi];
+            fence_proxy_async();
+          }
+        } else {
+          lo = hi = 0;
+        }
+        const uint32_t bytes = hi > lo ? (uint32_t)(hi - lo) * 8u : 0u;
+        const uint32_t total = __reduce_add_sync(0xffffffffu, bytes);
+        __syncwarp();  // the plain copies come before the arrival
+        if (lane == 0) {
+          fence_proxy_async();
+          mbar_arrive_expect_tx(&full[sl], total);
+        }
+        __syncwarp();
+        if (bytes) bulk_g2s(dst + lo, src + lo, bytes, &full[sl]);
+        ++fill;
+        return;
+      }
       if (lane == 0) {
         fence_proxy_async();
         mbar_arrive_expect_tx(&full[sl], row_bytes * (uint32_t)nrows);
@@ -265,13 +389,16 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
     // (plane m of a run sits in slot (m - kb) % STAGES)
     auto sfill = [&](int m) {
       if (m <= klast && wok) {
-        const int nch = (int)(row_bytes >> 4);  // 16-byte chunks of a strip row (tw is even)
+        // 16-byte chunks of a strip row (tw is even), 8-byte ones unaligned
+        constexpr int CE = UNAL ? 1 : 2;
+        const int nch = UNAL ? tw : (int)(row_bytes >> 4);
         const float2* src = s_src[w] + (size_t)m * ((size_t)nx * ny);
         float2* dst = ring + (size_t)((m - kb) % STAGES) * BRH * W2 + 32 * w;
         const int dr = 32 / nch, dc = 32 - dr * nch;
         int r = lane / nch, c = lane - (lane / nch) * nch;
         while (r < nrows) {
-          cp_async16(dst + r * W2 + 2 * c, src + (size_t)r * nx + 2 * c);
+          if constexpr (UNAL) cp_async8(dst + r * W2 + c, src + (size_t)r * nx + c);
+          else cp_async16(dst + r * W2 + CE * c, src + (size_t)r * nx + CE * c);
           r += dr;
           c += dc;
           if (c >= nch) {
@@ -328,6 +455,37 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       for (int i = 0; i < min(STAGES, nplanes); ++i) produce(kb + i);
     }
 
+    // warp-uniform test of a plane and of its edges; exact half-planes and edges
+    // of a plane (unaligned rows)
+    auto special = [&](unsigned long long prod, float mx, float myz) -> bool {
+      return colv && (prod_special(prod) || !(myz > kTieMin) ||
+                      (lane < BL && xs + 1 < tw && !(mx > kTieMin)));
+    };
+    auto half_planes = [&](const float2(&V)[BRH]) -> uint32_t {
+      uint32_t b = 0;
+#pragma unroll
+      for (int r = 0; r < BRH; ++r) b |= (V[r].y < 0.f ? 1u : 0u) << r;
+      return b;
+    };
+    auto exact_xy = [&](const float2(&V)[BRH], Edge& X, Edge& Y) {
+      uint32_t xp = 0, xn = 0, yp = 0, yn = 0;
+#pragma unroll
+      for (int r = 0; r < BRH; ++r) {
+        const float2 nb = make_float2(__shfl_down_sync(0xffffffffu, V[r].x, 1),
+                                      __shfl_down_sync(0xffffffffu, V[r].y, 1));
+        const uint32_t ex = exact_edge(V[r], nb);
+        xp |= (ex & 1u) << r;
+        xn |= (ex >> 1) << r;
+        if (r < BR) {
+          const uint32_t ey = exact_edge(V[r], V[r + 1]);
+          yp |= (ey & 1u) << r;
+          yn |= (ey >> 1) << r;
+        }
+      }
+      X = edge_pn(xp, xn);
+      Y = edge_pn(yp, yn);
+    };
+
     // ---- prologue: plane kb (values into vA)
     float2 vA[BRH], vB[BRH];
     uint32_t S0, S0n, ZB0 = 0, ZB0n = 0, BB0 = 0, BB0n = 0;
@@ -335,29 +493,42 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
     bool bad0;
     {
       const float2* sp = acquire(kb);
+      const int xe = xc + (UNAL ? (int)shift(kb) : 0), xo = UNAL ? xc + (int)(shift(kb) ^ shr) : xe;
       uint32_t SX = 0, SY = 0;
       unsigned long long prod = kProdOne;
+      float mx = kTieFar, myz = kTieFar;
       S0 = 0;
 #pragma unroll
       for (int r = BRH - 1; r >= 0; --r) {
-        const float2 v = sp[r * W2 + xc];
-        const float2 nb = sp[r * W2 + xc + 1];
+        const float2 v = sp[r * W2 + (r & 1 ? xo : xe)];
+        const float2 nb = sp[r * W2 + (r & 1 ? xo : xe) + 1];
         S0 = push1(S0, v.y);
-        SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
-        if (r < BR) SY = push1(SY, cross_f(v.x, v.y, vA[r + 1].x, vA[r + 1].y));
+        if constexpr (UNAL) {
+          float m1, m2;
+          SX = push1(SX, cross_m(v, nb, m1));
+          mx = min_nan(mx, m1);
+          if (r < BR) {
+            SY = push1(SY, cross_m(v, vA[r + 1], m2));
+            myz = min_nan(myz, m2);
+          }
+        } else {
+          SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
+          if (r < BR) SY = push1(SY, cross_f(v.x, v.y, vA[r + 1].x, vA[r + 1].y));
+        }
         prod = prod_step(prod, v);
         vA[r] = v;
       }
       release(kb);
       if (w == 0 && !stk && kb + STAGES <= klast) produce(kb + STAGES);
-      bad0 = __any_sync(0xffffffffu, prod_special(prod));
+      bad0 = __any_sync(0xffffffffu, UNAL ? special(prod, mx, myz) : prod_special(prod));
       if (bad0) {
 #pragma unroll
         for (int r = 0; r < BRH; ++r) {
-          ZB0 |= zero_bit(vA[r]) << r;
+          if constexpr (!UNAL) ZB0 |= zero_bit(vA[r]) << r;
           BB0 |= bad_bit(vA[r]) << r;
         }
       }
+      if constexpr (UNAL) if (bad0) S0 = half_planes(vA);
       S0n = __shfl_down_sync(0xffffffffu, S0, 1);
       const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
       ZB0n = __shfl_down_sync(0xffffffffu, ZB0, 1);
@@ -365,6 +536,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       X0 = edge_words(S0, S0n, SX, ZB0 | ZB0n);
       Y0 = edge_words(S0, S0 >> 1, SY, ZB0 | (ZB0 >> 1));
       Y0n = edge_words(S0n, S0n >> 1, SYn, ZB0n | (ZB0n >> 1));
+      if constexpr (UNAL) if (bad0) {
+        exact_xy(vA, X0, Y0);
+        Y0n = edge_dn(Y0);
+      }
     }
 
     // one z step: plane k = kb + t in V0 (values) and the plane-k words,
@@ -381,22 +556,39 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       bool bad1 = false;
       if (has_up) {
         const float2* sp = acquire(k + 1);
+        const int xe = xc + (UNAL ? (int)shift(k + 1) : 0);
+        const int xo = UNAL ? xc + (int)(shift(k + 1) ^ shr) : xe;
         uint32_t SX = 0, SY = 0, SZ = 0;
         unsigned long long prod = kProdOne;
+        float mx = kTieFar, myz = kTieFar;
 #pragma unroll
         for (int r = BRH - 1; r >= 0; --r) {
-          const float2 v = sp[r * W2 + xc];
-          const float2 nb = sp[r * W2 + xc + 1];
+          const float2 v = sp[r * W2 + (r & 1 ? xo : xe)];
+          const float2 nb = sp[r * W2 + (r & 1 ? xo : xe) + 1];
           S1 = push1(S1, v.y);
-          SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
-          SZ = push1(SZ, cross_f(V0[r].x, V0[r].y, v.x, v.y));
-          if (r < BR) SY = push1(SY, cross_f(v.x, v.y, V1[r + 1].x, V1[r + 1].y));
+          if constexpr (UNAL) {
+            float m1, m2, m3;
+            SX = push1(SX, cross_m(v, nb, m1));
+            SZ = push1(SZ, cross_m(V0[r], v, m2));
+            mx = min_nan(mx, m1);
+            if (r < BR) {
+              SY = push1(SY, cross_m(v, V1[r + 1], m3));
+              myz = min_nan(myz, m2, m3);
+            } else {
+              myz = min_nan(myz, m2);
+            }
+          } else {
+            SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
+            SZ = push1(SZ, cross_f(V0[r].x, V0[r].y, v.x, v.y));
+            if (r < BR) SY = push1(SY, cross_f(v.x, v.y, V1[r + 1].x, V1[r + 1].y));
+          }
           prod = prod_step(prod, v);
           V1[r] = v;
         }
         release(k + 1);
         if (w == 0 && !stk && k + 1 + STAGES <= klast) produce(k + 1 + STAGES);
-        bad1 = __any_sync(0xffffffffu, prod_special(prod));
+        bad1 = __any_sync(0xffffffffu, UNAL ? special(prod, mx, myz) : prod_special(prod));
+        if constexpr (UNAL) if (bad1) S1 = half_planes(V1);
         S1n = __shfl_down_sync(0xffffffffu, S1, 1);
         const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
         const uint32_t SZn = __shfl_down_sync(0xffffffffu, SZ, 1);
@@ -405,7 +597,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
           if (bad1) {
 #pragma unroll
             for (int r = 0; r < BRH; ++r) {
-              ZB1 |= zero_bit(V1[r]) << r;
+              if constexpr (!UNAL) ZB1 |= zero_bit(V1[r]) << r;
               BB1 |= bad_bit(V1[r]) << r;
             }
           }
@@ -416,6 +608,19 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
           Y1n = edge_words(S1n, S1n >> 1, SYn, ZB1n | (ZB1n >> 1));
           Zk = edge_words(S0, S1, SZ, ZB0 | ZB1);
           Zkn = edge_words(S0n, S1n, SZn, ZB0n | ZB1n);
+          if constexpr (UNAL) {
+            exact_xy(V1, X1, Y1);
+            uint32_t zp = 0, zn = 0;
+#pragma unroll
+            for (int r = 0; r < BRH; ++r) {
+              const uint32_t ez = exact_edge(V0[r], V1[r]);
+              zp |= (ez & 1u) << r;
+              zn |= (ez >> 1) << r;
+            }
+            Zk = edge_pn(zp, zn);
+            Zkn = edge_dn(Zk);
+            Y1n = edge_dn(Y1);
+          }
         } else {
           X1 = edge_words(S1, S1n, SX);
           Y1 = edge_words(S1, S1 >> 1, SY);
@@ -435,6 +640,12 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
         Myz &= ~(BB0 | (BB0 >> 1) | BB1 | (BB1 >> 1));
         Mzx &= ~(BB0 | BB0n | BB1 | BB1n);
       }
+      // W = -2 shares the code of 2; a sum of -2 needs determinants that
+      // underflow or overflow, so the expand pass takes it from psi
+      uint32_t mark = 0;
+      if constexpr (UNAL)
+        if (bad0 || bad1)
+          mark = ((~Lxy & Hxy & Mxy) | (~Lyz & Hyz & Myz) | (~Lzx & Hzx & Mzx)) ? kRecordTwos : 0u;
       Lxy &= Mxy;
       Hxy &= Mxy;
       Lyz &= Myz;
@@ -452,7 +663,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       const unsigned long long e = ebase + (unsigned long long)k;
       if (anyf && e * 32ull + lane < a.recs_cap)
         recs[e * 32ull + lane] =
-            make_uint4(Lxy | (Hxy << 16), Lyz | (Hyz << 16), Lzx | (Hzx << 16), (uint32_t)lane);
+            make_uint4(Lxy | (Hxy << 16), Lyz | (Hyz << 16), Lzx | (Hzx << 16), (uint32_t)lane | mark);
       if (lane == (t & 31)) tent = make_uint2(bal, faces_w);
       if (((t & 31) == 31 || t == nsteps - 1) && wok) {
         if (lane <= (t & 31)) {
@@ -495,42 +706,43 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
 
 using BitsFn = void (*)(BulkParams);
 
-template <int STAGES>
+template <int STAGES, bool UNAL>
 BitsFn bits_fn_stages(int nw) {
-  if (nw <= 2) return sweep_bits_kernel<2, 8, STAGES>;
-  if (nw <= 4) return sweep_bits_kernel<4, 4, STAGES>;
-  return sweep_bits_kernel<8, 2, STAGES>;
+  if (nw <= 2) return sweep_bits_kernel<2, 8, STAGES, UNAL>;
+  if (nw <= 4) return sweep_bits_kernel<4, 4, STAGES, UNAL>;
+  return sweep_bits_kernel<8, 2, STAGES, UNAL>;
 }
 
-BitsFn bits_fn(int nw, int stages) {
-  return stages <= 2 ? bits_fn_stages<2>(nw) : bits_fn_stages<3>(nw);
+BitsFn bits_fn(int nw, int stages, bool unal) {
+  if (unal) return stages <= 2 ? bits_fn_stages<2, true>(nw) : bits_fn_stages<3, true>(nw);
+  return stages <= 2 ? bits_fn_stages<2, false>(nw) : bits_fn_stages<3, false>(nw);
 }
 
-int bits_fn_index(int nw, int stages) {
-  return (nw <= 2 ? 0 : (nw <= 4 ? 1 : 2)) + (stages <= 2 ? 0 : 3);
+int bits_fn_index(int nw, int stages, bool unal) {
+  return (nw <= 2 ? 0 : (nw <= 4 ? 1 : 2)) + (stages <= 2 ? 0 : 3) + (unal ? 6 : 0);
 }
 
 }  // namespace
 
-size_t bits_smem_bytes(int nw, int stages) {
-  return ((size_t)stages * BRH * (BL * nw + 2) + kTail) * sizeof(float2) +
+size_t bits_smem_bytes(int nw, int stages, bool unal) {
+  return ((size_t)stages * BRH * (BL * nw + (unal ? 4 : 2)) + kTail) * sizeof(float2) +
          2 * stages * sizeof(uint64_t) + kMaxRun * sizeof(unsigned int) +
          (size_t)nw * sizeof(const float2*);
 }
 
-int bits_variant_occupancy(int nw, int stages, int* ctas_per_sm, size_t* smem) {
-  static bool attr_set[6] = {false, false, false, false, false, false};
+int bits_variant_occupancy(int nw, int stages, bool unal, int* ctas_per_sm, size_t* smem) {
+  static bool attr_set[12] = {};
   if (nw != 2 && nw != 4 && nw != 8)
     return set_error(QTV_ERR_ARG, "bit-sliced sweep: %d warps per tile (2, 4 or 8)", nw);
-  const int which = bits_fn_index(nw, stages);
-  BitsFn fn = bits_fn(nw, stages);
+  const int which = bits_fn_index(nw, stages, unal);
+  BitsFn fn = bits_fn(nw, stages, unal);
   if (!attr_set[which]) {
     cudaError_t e =
         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return check_cuda(e, "cudaFuncSetAttribute(sweep_bits)");
     attr_set[which] = true;
   }
-  *smem = bits_smem_bytes(nw, stages);
+  *smem = bits_smem_bytes(nw, stages, unal);
   int bps = 0;
   cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, fn, nw * 32, *smem);
   if (e != cudaSuccess) return check_cuda(e, "occupancy(sweep_bits)");
@@ -539,9 +751,9 @@ int bits_variant_occupancy(int nw, int stages, int* ctas_per_sm, size_t* smem) {
   return QTV_OK;
 }
 
-void bits_sweep_launch(const BulkParams& p, int grid, int nw, int stages, size_t smem,
+void bits_sweep_launch(const BulkParams& p, int grid, int nw, int stages, bool unal, size_t smem,
                        cudaStream_t st) {
-  bits_fn(nw, stages)<<<grid, nw * 32, smem, st>>>(p);
+  bits_fn(nw, stages, unal)<<<grid, nw * 32, smem, st>>>(p);
 }
 
 

@@ -909,9 +909,19 @@ int bulk_variant_occupancy(int nw, int* ctas_per_sm, size_t* smem) {
   return QTV_OK;
 }
 
-bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi) {
-  if (nx < 2 || ny < 1 || nz < 1 || (nx & 1)) return false;
-  if (reinterpret_cast<uintptr_t>(psi) & 15u) return false;
+namespace {
+// rows on 16-byte boundaries
+bool rows_aligned(int nx, const void* psi) {
+  return (nx & 1) == 0 && (reinterpret_cast<uintptr_t>(psi) & 15u) == 0;
+}
+}  // namespace
+
+bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi, bool unal) {
+  if (nx < 2 || ny < 1 || nz < 1) return false;
+  // unaligned rows no wider than a warp stay with the register sweep: the
+  // record slots of a tile (2 KB per 16-row band and plane) would outgrow the
+  // field several times, where that sweep's staging follows the faces
+  if (!rows_aligned(nx, psi) && !(unal && variant == 1 && nx > 32)) return false;
   // bit-sliced: tiles of 31 nwt columns for any nwt, at most kBitsBandWarps
   // (tile, warp) steps per band row at nwt = 4 (tiles of 124 columns)
   if (variant == 1) return (nx + 123) / 124 * 4 <= kBitsBandWarps;
@@ -933,6 +943,7 @@ int batch_layout(int num_sms, int nsnap, const qtv_grid* grids, const float2* co
   const int stages = tc.stages <= 2 ? 2 : 3;
   B->variant = tc.variant;
   B->stages = stages;
+  B->unal = false;
   B->rec_words = bits ? 4 : kRecWords;
   BulkParams& fin = B->fin;
   fin = BulkParams();
@@ -942,7 +953,8 @@ int batch_layout(int num_sms, int nsnap, const qtv_grid* grids, const float2* co
   long long nseg = 0, tab = 0;
   for (int i = 0; i < nsnap; ++i) {
     const qtv_grid& g = grids[i];
-    if (!sweep_bulk_supported(tc.variant, g.nx, g.ny, g.nz, psis[i]))
+    if (bits && tc.unal && !rows_aligned(g.nx, psis[i])) B->unal = true;
+    if (!sweep_bulk_supported(tc.variant, g.nx, g.ny, g.nz, psis[i], tc.unal))
       return set_error(QTV_ERR_ARG, "snapshot %d (%d x %d x %d): the staged sweep needs even nx "
                        "(<= 1024 for the nibble sweep) and a 16-byte aligned field", i, g.nx,
                        g.ny, g.nz);
@@ -1013,7 +1025,7 @@ int batch_layout(int num_sms, int nsnap, const qtv_grid* grids, const float2* co
     p.nseg = nseg;
     int bps = 0;
     size_t smem = 0;
-    int rc = bits ? bits_variant_occupancy(p.nwt, stages, &bps, &smem)
+    int rc = bits ? bits_variant_occupancy(p.nwt, stages, B->unal, &bps, &smem)
                   : bulk_variant_occupancy(p.nwt, &bps, &smem);
     if (rc) return rc;
     if (tc.ctas_per_sm > 0 && tc.ctas_per_sm < bps) bps = tc.ctas_per_sm;
@@ -1093,7 +1105,7 @@ int launch_sweeps(qtv_handle h, BatchLayout& B, const IdentScratch& sc, cudaStre
     }
     {
       TraceScope ts(h, K_SWEEP, s);
-      if (B.variant == 1) bits_sweep_launch(p, L.grid, p.nwt, B.stages, L.smem, s);
+      if (B.variant == 1) bits_sweep_launch(p, L.grid, p.nwt, B.stages, B.unal, L.smem, s);
       else bulk_fn(p.nwt)<<<L.grid, L.threads, L.smem, s>>>(p);
     }
     e = cudaGetLastError();
@@ -1145,7 +1157,7 @@ int batch_launch(qtv_handle h, BatchLayout& B, const IdentScratch& sc, uint64_t*
     TraceScope ts(h, K_SCATTER, st);
     if (B.variant == 1)
       e = bits_expand_launch(p, B.expand_blocks, sc.seg_off, face_ids, winding, capacity, offsets,
-                             st);
+                             B.unal, st);
     else
       e = launch_dependent(v3_expand_kernel, dim3((unsigned)B.expand_blocks),
                            dim3(32 * kExpandWarps), 0, st, p, sc.seg_off, face_ids, winding,
@@ -1177,6 +1189,7 @@ TileConfig handle_sweep_config(const qtv_handle_s* h) {
   // the bit-sliced sweep runs its CTAs over z blocks twice as tall as the
   // even split (fewer run changes, measured slightly faster)
   if (tc.variant == 1) tc.zscale = 2.f;
+  tc.unal = tc.variant == 1;
   if (h) {
     tc.nwt = h->sweep_nwt;
     tc.ctas_per_sm = h->sweep_ctas;
@@ -1187,7 +1200,7 @@ TileConfig handle_sweep_config(const qtv_handle_s* h) {
 
 int staged_variant(const qtv_handle_s* h, int nx, int ny, int nz, const void* psi) {
   const int v = handle_sweep_config(h).variant;
-  if (sweep_bulk_supported(v, nx, ny, nz, psi)) return v;
+  if (sweep_bulk_supported(v, nx, ny, nz, psi, v == 1)) return v;
   if (v != 0 && sweep_bulk_supported(0, nx, ny, nz, psi)) return 0;
   return -1;
 }

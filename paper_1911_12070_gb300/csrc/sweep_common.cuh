@@ -74,6 +74,17 @@ __device__ __forceinline__ float cross_f(float ar, float ai, float br, float bi)
   return fmaf(ar, bi, -(ai * br));
 }
 
+// Branch crossing of a -> b as the register sweep (identify.cu) decides it:
+// half-planes by Im < 0, the determinant's sign by an error-free product split;
+// exactly antiparallel or zero nodes cross nothing.  Bit 0: +1, bit 1: -1.
+__device__ __forceinline__ uint32_t exact_edge(float2 a, float2 b) {
+  const float p = __fmul_rn(a.y, b.x);
+  const float e = fmaf(a.y, b.x, -p);
+  const float c = fmaf(a.x, b.y, -p);
+  const bool sa = a.y < 0.f, sb = b.y < 0.f;
+  return (!sa && sb && c > e ? 1u : 0u) | (sa && !sb && c < e ? 2u : 0u);
+}
+
 // unit u of one snapshot's (z block, band, tile, plane) order -> column
 // (band * ntx + tile), plane, end of its z block
 __device__ __forceinline__ void unit_pos(long long u, long long cols, int nz, int H, long long& col,
@@ -108,6 +119,10 @@ __device__ __forceinline__ unsigned long long mul_f32x2(unsigned long long a, un
 // commit group
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src)
                : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() {
