@@ -497,63 +497,153 @@ __global__ void scatter_kernel(const uint2* __restrict__ seg, const unsigned lon
   }
 }
 
-// Statistics pass (only when requested): one thread per node, FP32.
-__global__ void stats_kernel(const float2* __restrict__ psi, int nx, int ny, int nz,
-                             qtv_stats* stats) {
-  unsigned long long amb = 0, zer = 0, bad = 0;
-  const long long nn = (long long)nx * ny * nz;
-  for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < nn;
-       q += (long long)gridDim.x * blockDim.x) {
-    const int i = (int)(q % nx);
-    const int j = (int)((q / nx) % ny);
-    const int k = (int)(q / ((long long)nx * ny));
+// ---------------------------------------------------------------------------
+// Statistics pass (only when requested), FP32.
+//
+// A warp owns 31 columns (lane 31 holds the next one) of kStatRows rows (plus
+// one) and marches z over a chunk of planes, so psi is read about once, in
+// coalesced rows, one plane ahead.  Ambiguous edges, zero and non-finite nodes
+// are rare: each plane is screened with one test per edge, wider than the
+// ambiguity bound by 1%, and one product per node, and only a (plane, warp)
+// with a hit counts its faces one by one (count_faces).  A thread per node
+// that loaded the corners of its three faces took 269 us at 256^3 (64-bit index
+// divisions, 12 loads and 12 edge tests a node); this takes 45 us, of 20 for the
+// bytes (272 us at 512^3, of 158): it is bound by issue, about 40 instructions a
+// node in the screen.
+// ---------------------------------------------------------------------------
+constexpr int kStatRows = 4;
+constexpr int kStatWarps = 8;   // warps of a CTA: consecutive row bands
+constexpr int kStatPlanes = 16; // planes per chunk
+
+struct StatCounts {
+  uint32_t amb = 0, zer = 0, bad = 0;
+};
+
+// |d| of the edge p -> n within 1e-4 rad of pi (zero nodes have phase 0)
+__device__ __forceinline__ bool ambiguous_edge(float2 p, float2 n) {
+  if (p.x == 0.f && p.y == 0.f) p = make_float2(1.f, 0.f);
+  if (n.x == 0.f && n.y == 0.f) n = make_float2(1.f, 0.f);
+  const float zr = fmaf(n.x, p.x, n.y * p.y);
+  const float zi = fmaf(n.y, p.x, -n.x * p.y);
+  return zr < 0.f && fabsf(zi) < 1.0e-4f * -zr;
+}
+
+__device__ __forceinline__ void count_face(float2 a, float2 b, float2 c, float2 d, StatCounts& n) {
+  const float2 v[4] = {a, b, c, d};
+  bool z = false, nf = false, am = false;
 #pragma unroll
-    for (int o = 0; o < 3; ++o) {
-      int di[4], dj[4], dk[4];
-      if (o == 0) {
-        if (i + 1 >= nx || j + 1 >= ny) continue;
-        const int a0[4] = {0, 1, 1, 0}, b0[4] = {0, 0, 1, 1};
-        for (int c = 0; c < 4; ++c) { di[c] = a0[c]; dj[c] = b0[c]; dk[c] = 0; }
-      } else if (o == 1) {
-        if (j + 1 >= ny || k + 1 >= nz) continue;
-        const int a0[4] = {0, 1, 1, 0}, b0[4] = {0, 0, 1, 1};
-        for (int c = 0; c < 4; ++c) { di[c] = 0; dj[c] = a0[c]; dk[c] = b0[c]; }
-      } else {
-        if (k + 1 >= nz || i + 1 >= nx) continue;
-        const int a0[4] = {0, 1, 1, 0}, b0[4] = {0, 0, 1, 1};
-        for (int c = 0; c < 4; ++c) { dk[c] = a0[c]; di[c] = b0[c]; dj[c] = 0; }
+  for (int q = 0; q < 4; ++q) {
+    z |= v[q].x == 0.f && v[q].y == 0.f;
+    nf |= !(finite_f(v[q].x) && finite_f(v[q].y));
+    am |= ambiguous_edge(v[q], v[(q + 1) & 3]);
+  }
+  n.bad += nf ? 1u : 0u;
+  n.zer += z && !nf ? 1u : 0u;
+  n.amb += am && !nf ? 1u : 0u;
+}
+
+// smallest of |zi| + 1.01e-4 zr over the edges seen: above kScreen when none
+// of them can be ambiguous (NaN edges have a non-finite node)
+constexpr float kScreen = 1e-37f;
+__device__ __forceinline__ float screen_edge(float m, float2 p, float2 n) {
+  const float zr = fmaf(n.x, p.x, n.y * p.y);
+  const float zi = fmaf(n.y, p.x, -n.x * p.y);
+  return fminf(m, fmaf(1.01e-4f, zr, fabsf(zi)));
+}
+
+__device__ __forceinline__ float2 lane_right(float2 v) {
+  return make_float2(__shfl_down_sync(0xffffffffu, v.x, 1), __shfl_down_sync(0xffffffffu, v.y, 1));
+}
+
+__global__ void __launch_bounds__(32 * kStatWarps) stats_kernel(const float2* __restrict__ psi, int nx,
+                                                                int ny, int nz, int nxs, int nyb,
+                                                                long long nitems, qtv_stats* stats) {
+  constexpr int R1 = kStatRows + 1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  StatCounts n;
+  for (long long item = blockIdx.x; item < nitems; item += gridDim.x) {
+    const int xs = (int)(item % nxs);
+    const long long rest = item / nxs;
+    const int j0 = ((int)(rest % nyb) * kStatWarps + w) * kStatRows;
+    const int k0 = (int)(rest / nyb) * kStatPlanes;
+    if (j0 >= ny) continue;
+    const int k1 = min(nz, k0 + kStatPlanes);
+    const int x = xs * 31 + lane;
+    const bool own = lane < 31;
+    const long long plane = (long long)nx * ny;
+    const float2* src = psi + ((long long)k0 * ny + j0) * nx + x;
+    const int rows = x < nx ? min(R1, ny - j0) : 0;
+    // plane k (nodes outside the grid hold (1, 1), which no screen rejects)
+    auto load = [&](float2(&v)[R1], int k) {
+#pragma unroll
+      for (int r = 0; r < R1; ++r)
+        v[r] = r < rows && k < nz ? __ldg(src + (k - k0) * plane + (long long)r * nx)
+                                  : make_float2(1.f, 1.f);
+    };
+    // warp-uniform: a node or an in-plane edge to look at
+    auto screen = [&](const float2(&v)[R1]) -> bool {
+      float m = 1.f, px = 1.f, py = 1.f;
+#pragma unroll
+      for (int r = 0; r < R1; ++r) {
+        m = screen_edge(m, v[r], lane_right(v[r]));
+        if (r + 1 < R1) m = screen_edge(m, v[r], v[r + 1]);
+        px *= v[r].x;
+        py *= v[r].y;
       }
-      float2 v[4];
-      bool z = false, nf = false;
-      for (int c = 0; c < 4; ++c) {
-        v[c] = psi[((long long)(k + dk[c]) * ny + (j + dj[c])) * nx + (i + di[c])];
-        z |= (v[c].x == 0.f && v[c].y == 0.f);
-        nf |= !(finite_f(v[c].x) && finite_f(v[c].y));
+      // a zero component, a non-finite node, or under- or overflow
+      const bool odd = !(fabsf(px) > 0.f && finite_f(px) && fabsf(py) > 0.f && finite_f(py));
+      return __any_sync(0xffffffffu, odd || !(m > kScreen));
+    };
+    float2 cur[R1], nxt[R1], ahead[R1];
+    load(cur, k0);
+    load(nxt, k0 + 1);
+    bool hit = screen(cur);
+    for (int k = k0; k < k1; ++k) {
+      load(ahead, k + 2);
+      const bool up = k + 1 < nz;
+      const bool hit1 = screen(nxt);
+      float m = 1.f;
+#pragma unroll
+      for (int r = 0; r < R1; ++r) m = screen_edge(m, cur[r], nxt[r]);
+      if (hit || hit1 || __any_sync(0xffffffffu, !(m > kScreen))) {
+#pragma unroll
+        for (int r = 0; r < kStatRows; ++r) {
+          const float2 c10 = lane_right(cur[r]), c11 = lane_right(cur[r + 1]);
+          const float2 n10 = lane_right(nxt[r]);
+          const bool ix = own && x + 1 < nx, jy = j0 + r + 1 < ny, in = own && r < rows;
+          if (in && ix && jy) count_face(cur[r], c10, c11, cur[r + 1], n);
+          if (in && jy && up) count_face(cur[r], cur[r + 1], nxt[r + 1], nxt[r], n);
+          if (in && up && ix) count_face(cur[r], nxt[r], n10, c10, n);
+        }
       }
-      if (nf) { ++bad; continue; }
-      if (z) ++zer;
-      bool am = false;
-      for (int c = 0; c < 4; ++c) {
-        float2 p = v[c], n = v[(c + 1) & 3];
-        if (p.x == 0.f && p.y == 0.f) p = make_float2(1.f, 0.f);
-        if (n.x == 0.f && n.y == 0.f) n = make_float2(1.f, 0.f);
-        const float zr = fmaf(n.x, p.x, n.y * p.y);
-        const float zi = fmaf(n.y, p.x, -n.x * p.y);
-        am |= (zr < 0.f) && (fabsf(zi) < 1.0e-4f * -zr);
+      hit = hit1;
+#pragma unroll
+      for (int r = 0; r < R1; ++r) {
+        cur[r] = nxt[r];
+        nxt[r] = ahead[r];
       }
-      if (am) ++amb;
     }
   }
-  for (int d = 16; d; d >>= 1) {
-    amb += __shfl_down_sync(0xffffffffu, amb, d);
-    zer += __shfl_down_sync(0xffffffffu, zer, d);
-    bad += __shfl_down_sync(0xffffffffu, bad, d);
+  n.amb = __reduce_add_sync(0xffffffffu, n.amb);
+  n.zer = __reduce_add_sync(0xffffffffu, n.zer);
+  n.bad = __reduce_add_sync(0xffffffffu, n.bad);
+  if (lane == 0) {
+    if (n.amb) atomicAdd((unsigned long long*)&stats->ambiguous, (unsigned long long)n.amb);
+    if (n.zer) atomicAdd((unsigned long long*)&stats->zero_node_faces, (unsigned long long)n.zer);
+    if (n.bad) atomicAdd((unsigned long long*)&stats->nonfinite_faces, (unsigned long long)n.bad);
   }
-  if ((threadIdx.x & 31) == 0) {
-    if (amb) atomicAdd((unsigned long long*)&stats->ambiguous, amb);
-    if (zer) atomicAdd((unsigned long long*)&stats->zero_node_faces, zer);
-    if (bad) atomicAdd((unsigned long long*)&stats->nonfinite_faces, bad);
-  }
+}
+
+cudaError_t stats_launch(qtv_handle h, const qtv_grid& g, const float2* psi, qtv_stats* stats,
+                         cudaStream_t st) {
+  const int nxs = (g.nx + 30) / 31;
+  const int nyb = (g.ny + kStatRows * kStatWarps - 1) / (kStatRows * kStatWarps);
+  const long long nitems =
+      (long long)nxs * nyb * ((g.nz + kStatPlanes - 1) / kStatPlanes);
+  TraceScope ts(h, K_STATS, st);
+  stats_kernel<<<(unsigned)(nitems < (1 << 20) ? nitems : 1 << 20), 32 * kStatWarps, 0, st>>>(
+      psi, g.nx, g.ny, g.nz, nxs, nyb, nitems, stats);
+  return cudaGetLastError();
 }
 
 struct LaunchShape {
@@ -614,9 +704,7 @@ int identify_launch(qtv_handle h, const qtv_grid& g, const float2* psi, uint64_t
                                  max_warps, xyz, resid, flags);
     if (rc) return rc;
     if (stats) {
-      TraceScope ts(h, K_STATS, st);
-      stats_kernel<<<h->num_sms * 8, 256, 0, st>>>(psi, g.nx, g.ny, g.nz, stats);
-      const cudaError_t e = cudaGetLastError();
+      const cudaError_t e = stats_launch(h, g, psi, stats, st);
       if (e != cudaSuccess) return check_cuda(e, "stats_kernel launch");
     }
     return QTV_OK;
@@ -699,9 +787,7 @@ int identify_launch(qtv_handle h, const qtv_grid& g, const float2* psi, uint64_t
     if (rc) return rc;
   }
   if (stats) {
-    TraceScope ts(h, K_STATS, st);
-    stats_kernel<<<h->num_sms * 8, 256, 0, st>>>(psi, nx, ny, nz, stats);
-    e = cudaGetLastError();
+    e = stats_launch(h, g, psi, stats, st);
     if (e != cudaSuccess) return check_cuda(e, "stats_kernel launch");
   }
   return QTV_OK;
