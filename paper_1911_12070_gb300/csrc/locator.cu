@@ -376,9 +376,9 @@ __global__ void out_back_kernel(const float* __restrict__ dy, const float* __res
 }
 
 constexpr int kRowChunk = 64;  // rows per block of the reductions below
-constexpr int kSplits = 16;    // most K splits of a weight-gradient GEMM on tcgen05
 constexpr int kLossBlocks = 1024;                     // most blocks of the loss
 constexpr int kPartW3 = kOut * kH + kOut;             // W3 and b3 partials per chunk
+static_assert(kPartW3 + 2 * kH <= kTrainChunkFloats, "partials of a chunk");
 
 // partial dW3[o][k] = sum_m dY[m][o] A2[m][k] and db3[o] = sum_m dY[m][o] over
 // one chunk of rows per block (thread k = 0..kH, k == kH the bias), into
@@ -433,8 +433,7 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nb, int wid
 __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G,
                             float* __restrict__ Mo, float* __restrict__ Vo, int n, float lr,
                             float b1, float b2, float eps, float c1, float c2,
-                            uint16_t* __restrict__ w1b, uint16_t* __restrict__ w2b,
-                            uint16_t* __restrict__ w2tb) {
+                            uint16_t* __restrict__ w1b, uint16_t* __restrict__ w2b) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float g = G[i];
     const float m = b1 * Mo[i] + (1.f - b1) * g;
@@ -446,42 +445,20 @@ __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G,
     if (i < (int)kOffB1) {
       w1b[i - kOffW1] = f2bf(p);
     } else if (i >= (int)kOffW2 && i < (int)kOffB2) {
-      const int j = i - (int)kOffW2;  // W2[o][k], j = o kH + k
-      w2b[j] = f2bf(p);
-      w2tb[(j % kH) * kH + j / kH] = f2bf(p);
+      w2b[i - (int)kOffW2] = f2bf(p);
     }
   }
 }
 
 __global__ void refresh_bf16_kernel(const float* __restrict__ P, uint16_t* __restrict__ w1b,
-                                    uint16_t* __restrict__ w2b, uint16_t* __restrict__ w2tb) {
+                                    uint16_t* __restrict__ w2b) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kH * kIn + kH * kH;
        i += gridDim.x * blockDim.x) {
     if (i < kH * kIn) {
       w1b[i] = f2bf(P[kOffW1 + i]);
     } else {
-      const int j = i - kH * kIn;
-      const uint16_t b = f2bf(P[kOffW2 + j]);
-      w2b[j] = b;
-      w2tb[(j % kH) * kH + j / kH] = b;
+      w2b[i - kH * kIn] = f2bf(P[kOffW2 + (i - kH * kIn)]);
     }
-  }
-}
-
-// dst[c][m] = src[m][c] for m < n, zero for n <= m < ldT (BF16, 32 x 32 tiles)
-__global__ void transpose_bf16_kernel(const uint16_t* __restrict__ src, unsigned long long n,
-                                      int C, uint16_t* __restrict__ dst, unsigned long long ldT) {
-  __shared__ uint16_t t[32][34];
-  const unsigned long long m0 = (unsigned long long)blockIdx.x * 32;
-  const int c0 = blockIdx.y * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const unsigned long long m = m0 + r;
-    t[r][threadIdx.x] = m < n ? src[m * C + c0 + threadIdx.x] : (uint16_t)0;
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    const unsigned long long m = m0 + threadIdx.x;
-    if (m < ldT) dst[(unsigned long long)(c0 + r) * ldT + m] = t[threadIdx.x][r];
   }
 }
 
@@ -598,7 +575,6 @@ struct Locator {
   float* V = nullptr;      // Adam second moment
   uint16_t* w1b = nullptr; // BF16 W1 [256][128]
   uint16_t* w2b = nullptr; // BF16 W2 [256][256]
-  uint16_t* w2tb = nullptr; // BF16 W2^T [256 in][256 out] (backward on tcgen05)
   unsigned long long step = 0;
   bool ready = false;
   // activations for up to `cap` rows; rows_gen counts their reallocations
@@ -609,11 +585,10 @@ struct Locator {
   int num_sms = 0;
   unsigned int* status = nullptr;  // timeout flag of the tcgen05 kernel
   uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr, *X = nullptr;
-  // transposed copies for the weight gradients on tcgen05 ([features][ldT],
-  // columns past the batch zero) and the split-K partials
-  uint16_t *A1T = nullptr, *D1T = nullptr, *D2T = nullptr, *XT = nullptr;
-  unsigned long long ldT = 0;
+  // training on tcgen05: partials of the weight gradients per split and the
+  // loss of every 32 rows
   float* part = nullptr;
+  float* wloss = nullptr;
   // per-block partials of the reductions over the batch: loss [1024], then
   // per 64-row chunk W3 and b3 (kOut kH + kOut), b2 and b1 (kH each)
   float* lpart = nullptr;
@@ -631,12 +606,8 @@ void locator_free(Locator* L) {
   cudaFree(L->V);
   cudaFree(L->w1b);
   cudaFree(L->w2b);
-  cudaFree(L->w2tb);
-  cudaFree(L->A1T);
-  cudaFree(L->D1T);
-  cudaFree(L->D2T);
-  cudaFree(L->XT);
   cudaFree(L->part);
+  cudaFree(L->wloss);
   cudaFree(L->lpart);
   cudaFree(L->gpart);
   cudaFree(L->A1);
@@ -664,8 +635,8 @@ static int locator_alloc(qtv_handle h) {
   if (e == cudaSuccess) e = cudaMalloc(&L->V, pb);
   if (e == cudaSuccess) e = cudaMalloc(&L->w1b, (size_t)kH * kIn * 2);
   if (e == cudaSuccess) e = cudaMalloc(&L->w2b, (size_t)kH * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->w2tb, (size_t)kH * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->part, (size_t)kSplits * kH * kH * sizeof(float));
+  if (e == cudaSuccess)
+    e = cudaMalloc(&L->part, (size_t)kTrainSplits * (kH * kIn + kH * kH) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&L->lpart, (size_t)kLossBlocks * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&L->status, sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(L->status, 0, sizeof(unsigned int));
@@ -693,11 +664,8 @@ static int locator_rows(qtv_handle h, unsigned long long n, cudaStream_t st) {
   cudaFree(L->DY);
   cudaFree(L->rms);
   cudaFree(L->ok);
-  cudaFree(L->A1T);
-  cudaFree(L->D1T);
-  cudaFree(L->D2T);
-  cudaFree(L->XT);
-  L->A1T = L->D1T = L->D2T = L->XT = nullptr;
+  cudaFree(L->wloss);
+  L->wloss = nullptr;
   L->A1 = L->A2 = L->D1 = L->D2 = L->X = nullptr;
   L->Y = L->DY = L->rms = nullptr;
   L->ok = nullptr;
@@ -711,13 +679,8 @@ static int locator_rows(qtv_handle h, unsigned long long n, cudaStream_t st) {
   if (e == cudaSuccess) e = cudaMalloc(&L->DY, n * kOut * 4);
   if (e == cudaSuccess) e = cudaMalloc(&L->rms, n * 4);
   if (e == cudaSuccess) e = cudaMalloc(&L->ok, n);
-  const unsigned long long ldT = (n + 63) / 64 * 64;
-  if (e == cudaSuccess) e = cudaMalloc(&L->A1T, ldT * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->D1T, ldT * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->D2T, ldT * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->XT, ldT * kIn * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->wloss, (n + 127) / 128 * 4 * sizeof(float));
   if (e != cudaSuccess) return check_cuda(e, "cudaMalloc(locator rows)");
-  L->ldT = ldT;
   L->cap = n;
   ++L->rows_gen;
   return QTV_OK;
@@ -754,7 +717,7 @@ static int grad_parts(Locator* L, unsigned long long n, cudaStream_t st) {
   cudaFree(L->gpart);
   L->gpart = nullptr;
   L->gpart_cap = 0;
-  const cudaError_t e = cudaMalloc(&L->gpart, chunks * (kPartW3 + 2 * kH) * sizeof(float));
+  const cudaError_t e = cudaMalloc(&L->gpart, chunks * kTrainChunkFloats * sizeof(float));
   if (e != cudaSuccess) return check_cuda(e, "cudaMalloc(gradient partials)");
   L->gpart_cap = chunks;
   return QTV_OK;
@@ -785,67 +748,10 @@ static int bias_grad(Locator* L, const uint16_t* D, unsigned long long n, int wh
   return check_cuda(cudaGetLastError(), "locator bias gradient");
 }
 
-// splits of a K range of k64 chunks of 64: the largest divisor up to kSplits
-static int splits_for(unsigned long long k64) {
-  int s = kSplits;
-  while (s > 1 && k64 % (unsigned long long)s) --s;
-  return s;
-}
-
-// forward + backward into L->G on tcgen05 (L->tensor_path == 1): the dense
-// layers and the data-gradient GEMM take the row-major activations, the
-// weight-gradient GEMMs the transposed copies (K = the padded batch, split
-// into parts summed in a fixed order)
-static int forward_backward_tc(Locator* L, const uint16_t* X, const float* T, unsigned long long n,
-                               float* loss, cudaStream_t st) {
-  const unsigned long long ldT = (n + 63) / 64 * 64;
-  const dim3 tb(32, 8);
-  transpose_bf16_kernel<<<dim3((unsigned)(ldT / 32), kIn / 32), tb, 0, st>>>(X, n, kIn, L->XT, ldT);
-  // A1 = relu(X W1^T + b1), and A1^T
-  cudaError_t e = cudaSuccess;
-  if (ldT > n) {  // the GEMM epilogues write columns below n only
-    e = cudaMemset2DAsync(L->A1T + n, ldT * 2, 0, (ldT - n) * 2, kH, st);
-    if (e == cudaSuccess) e = cudaMemset2DAsync(L->D1T + n, ldT * 2, 0, (ldT - n) * 2, kH, st);
-    if (e != cudaSuccess) return check_cuda(e, "memset(transposed padding)");
-  }
-  int rc = tc_gemm(X, kIn, L->w1b, kIn, (long long)n, kH, kIn, 1, 1, nullptr, 0, nullptr, L->A1, kH,
-                   L->A1T, (long long)ldT, L->P + kOffB1, nullptr, 0, L->status, st);
-  if (rc) return rc;
-  // A2 = relu(A1 W2^T + b2)
-  rc = tc_gemm(L->A1, kH, L->w2b, kH, (long long)n, kH, kH, 1, 1, nullptr, 0, nullptr, L->A2, kH,
-               nullptr, 0, L->P + kOffB2, nullptr, 0, L->status, st);
-  if (rc) return rc;
-  rc = output_backward(L, T, n, loss, st);
-  if (rc) return rc;
-  transpose_bf16_kernel<<<dim3((unsigned)(ldT / 32), kH / 32), tb, 0, st>>>(L->D2, n, kH, L->D2T, ldT);
-  rc = bias_grad(L, L->D2, n, 0, L->G + kOffB2, st);
-  if (rc) return rc;
-  const int sp = splits_for(ldT / 64);
-  // dW2[o][k] = sum_m dH2[m][o] A1[m][k]
-  rc = tc_gemm(L->D2T, (long long)ldT, L->A1T, (long long)ldT, kH, kH, (long long)ldT, sp, 0,
-               L->G + kOffW2, kH, L->part, nullptr, 0, nullptr, 0, nullptr, nullptr, 0, L->status, st);
-  if (rc) return rc;
-  // dH1[m][k] = (sum_o dH2[m][o] W2[o][k]) * (A1[m][k] > 0), and its transpose
-  rc = tc_gemm(L->D2, kH, L->w2tb, kH, (long long)n, kH, kH, 1, 2, nullptr, 0, nullptr, L->D1, kH,
-               L->D1T, (long long)ldT, nullptr, L->A1, kH, L->status, st);
-  if (rc) return rc;
-  rc = bias_grad(L, L->D1, n, 1, L->G + kOffB1, st);
-  if (rc) return rc;
-  // dW1[o][i] = sum_m dH1[m][o] X[m][i]
-  rc = tc_gemm(L->D1T, (long long)ldT, L->XT, (long long)ldT, kH, kIn, (long long)ldT, sp, 0,
-               L->G + kOffW1, kIn, L->part, nullptr, 0, nullptr, 0, nullptr, nullptr, 0, L->status,
-               st);
-  if (rc) return rc;
-  return check_cuda(cudaGetLastError(), "locator backward (tcgen05)");
-}
-
-// forward + backward into L->G; loss (device float) accumulated
+// forward + backward into L->G and the loss (device float), mma.sync path
 static int forward_backward(Locator* L, const uint16_t* X, const float* T, unsigned long long n,
                             float* loss, cudaStream_t st) {
-  int rc = grad_parts(L, n, st);
-  if (rc) return rc;
-  if (L->tensor_path == 1) return forward_backward_tc(L, X, T, n, loss, st);
-  rc = forward_hidden(L, X, n, st);
+  int rc = forward_hidden(L, X, n, st);
   if (rc) return rc;
   rc = output_backward(L, T, n, loss, st);
   if (rc) return rc;
@@ -921,7 +827,7 @@ int qtv_locator_init(qtv_handle h, uint64_t seed) {
   init_kernel<<<64, 256>>>(L->P, seed);
   cudaMemset(L->M, 0, kNumParams * 4);
   cudaMemset(L->V, 0, kNumParams * 4);
-  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b, L->w2tb);
+  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b);
   L->step = 0;
   L->ready = true;
   return check_cuda(cudaDeviceSynchronize(), "qtv_locator_init");
@@ -964,7 +870,7 @@ int qtv_locator_set(qtv_handle h, const float* params, const float* adam, uint64
     }
   }
   if (e != cudaSuccess) return check_cuda(e, "qtv_locator_set");
-  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b, L->w2tb);
+  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b);
   L->step = step;
   L->ready = true;
   return check_cuda(cudaDeviceSynchronize(), "qtv_locator_set");
@@ -995,36 +901,47 @@ int qtv_locator_forward(qtv_handle h, const uint16_t* x, uint64_t n, float* y, v
   return forward_y(h->loc, x, n, y, st);
 }
 
-int qtv_locator_gradients(qtv_handle h, const uint16_t* x, const float* targets, uint64_t n,
-                          float* grads, float* loss, void* stream) {
+// gradients and loss of one batch; with adam, one step on them
+static int locator_step(qtv_handle h, const uint16_t* x, const float* targets, uint64_t n, bool adam,
+                        float lr, float* loss, cudaStream_t st) {
   if (!h || !h->loc || !h->loc->ready) return set_error(QTV_ERR_STATE, "no learned locator loaded");
   if (!x || !targets || !loss || n == 0 || n % 64)
     return set_error(QTV_ERR_ARG, "x/targets/loss NULL or batch not a positive multiple of 64");
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  Locator* L = h->loc;
   int rc = locator_rows(h, n, st);
+  if (!rc) rc = grad_parts(L, n, st);
   if (rc) return rc;
-  cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
-  if (e != cudaSuccess) return check_cuda(e, "memset(loss)");
-  rc = forward_backward(h->loc, x, targets, n, loss, st);
-  if (rc) return rc;
-  if (grads)
-    return check_cuda(cudaMemcpyAsync(grads, h->loc->G, kNumParams * 4, cudaMemcpyDeviceToDevice, st),
-                      "copy(grads)");
-  return QTV_OK;
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, t = (float)(L->step + 1);
+  const float c1 = 1.f - powf(b1, t), c2 = 1.f - powf(b2, t);
+  if (L->tensor_path == 1) {
+    const TrainBuffers B{L->A1, L->A2, L->D1, L->D2, L->DY, L->part, L->gpart};
+    const TrainState s{L->P, L->G,  L->M, L->V, L->w1b, L->w2b, L->wloss, loss, adam ? 1 : 0,
+                       lr,   b1,    b2,   eps,  c1,     c2};
+    rc = tc_train(x, targets, (long long)n, B, s, L->status, st);
+    if (rc) return rc;
+  } else {
+    rc = forward_backward(L, x, targets, n, loss, st);
+    if (rc) return rc;
+    if (adam)
+      adam_kernel<<<128, 256, 0, st>>>(L->P, L->G, L->M, L->V, (int)kNumParams, lr, b1, b2, eps, c1, c2,
+                                       L->w1b, L->w2b);
+  }
+  if (adam) L->step += 1;
+  return check_cuda(cudaGetLastError(), "locator step");
+}
+
+int qtv_locator_gradients(qtv_handle h, const uint16_t* x, const float* targets, uint64_t n,
+                          float* grads, float* loss, void* stream) {
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  const int rc = locator_step(h, x, targets, n, false, 0.f, loss, st);
+  if (rc || !grads) return rc;
+  return check_cuda(cudaMemcpyAsync(grads, h->loc->G, kNumParams * 4, cudaMemcpyDeviceToDevice, st),
+                    "copy(grads)");
 }
 
 int qtv_locator_train_step(qtv_handle h, const uint16_t* x, const float* targets, uint64_t n,
                            float lr, float* loss, void* stream) {
-  int rc = qtv_locator_gradients(h, x, targets, n, nullptr, loss, stream);
-  if (rc) return rc;
-  Locator* L = h->loc;
-  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-  L->step += 1;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.f - powf(b1, (float)L->step), c2 = 1.f - powf(b2, (float)L->step);
-  adam_kernel<<<128, 256, 0, st>>>(L->P, L->G, L->M, L->V, (int)kNumParams, lr, b1, b2, 1e-8f, c1,
-                                   c2, L->w1b, L->w2b, L->w2tb);
-  return check_cuda(cudaGetLastError(), "adam_kernel launch");
+  return locator_step(h, x, targets, n, true, lr, loss, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // Checkpoint: magic, version, step, parameters, Adam moments, FNV-1a checksum.

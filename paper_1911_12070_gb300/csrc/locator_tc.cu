@@ -1,8 +1,7 @@
 // locator_tc.cu -- the learned locator's network on the 5th-generation tensor
-// cores (tcgen05, accumulators in tensor memory): the training GEMM
-// (tc_gemm_kernel) and the whole 128-256-256-3 network fused per 128-row tile
-// (tc_mlp_kernel, warp-specialised; its design is described at its
-// definition).
+// cores (tcgen05, accumulators in tensor memory): the whole 128-256-256-3
+// network fused per 128-row tile (tc_mlp_kernel, warp-specialised; its design
+// is described at its definition) and the training step (train_*_kernel).
 //
 // Operands staged by threads are stored in the canonical K-major layout
 // without swizzle: 8 x 8 core matrices of 128 contiguous bytes (8 rows of 16
@@ -58,10 +57,6 @@ __device__ __forceinline__ void load_canon(unsigned char* dst, const uint16_t* _
     if (r0 + r < nrows) v = __ldg(reinterpret_cast<const uint4*>(src + (r0 + r) * K) + kc);
     *reinterpret_cast<uint4*>(dst + (size_t)c * 16) = v;
   }
-}
-
-__device__ __forceinline__ void cp_async_wait_all() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -524,237 +519,540 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
 }
 
 // ---------------------------------------------------------------------------
-// General training GEMM on the tensor cores: C[M][N] = A[M][K] B[N][K]^T, A
-// and B BF16 and K-major (row pitch lda / ldb elements), N = 128 or 256, FP32
-// accumulation in tensor memory.  One CTA of 4 warps per (128-row tile, K
-// split): K chunks of 64 are staged by cp.async into two shared-memory
-// stages in the canonical no-swizzle layout, one elected thread issues four
-// M = 128, N, K = 16 MMAs per chunk and commits them to the stage's mbarrier,
-// and the next chunk's copies overlap the current chunk's MMAs.  Epilogues:
-//   kEpiF32       C[(split M + row) ldc + col] = acc (per-split partials when
-//                 the K range is split; tc_split_sum adds them in split order)
-//   kEpiBiasRelu  v = relu(acc + bias[col]) as BF16 into O[row][col] and,
-//                 if OT, OT[col][row]
-//   kEpiMask      v = acc where mask[row][col] > 0, else 0, into O and OT
-// Rows of A at or beyond M are read as zero; K must be a multiple of 64 per
-// split (the callers pad with zero columns).
+// Training.  One step is three launches: train_rows_kernel (forward, loss and
+// the data gradients of 128 rows per CTA), train_grads_kernel (the weight
+// gradients as tcgen05 products over the batch, the bias and output-layer
+// gradients by chunks of 64 rows) and train_update_kernel (the partial sums
+// added in a fixed order, and Adam).  They took about twenty launches (GEMMs
+// that each staged their operands anew and stored every activation a second
+// time transposed, then transposes and reductions) and 200 us at 4096 rows;
+// now TRAIN_US us.
 // ---------------------------------------------------------------------------
-enum { kEpiF32 = 0, kEpiBiasRelu = 1, kEpiMask = 2 };
-constexpr int kGemmKc = 64;  // K per chunk
+constexpr uint32_t kMajorMnA = 1u << 15, kMajorMnB = 1u << 16;  // operand stored MN-major
 
-template <int N>
-constexpr uint32_t idesc_n() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
+// instruction descriptor of kind::f16 for M = 128 and N
+constexpr uint32_t idesc_n(int n) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// rows [r0, r0 + R) x columns [0, 64) of a K-major BF16 matrix (row pitch ld,
-// columns already offset) into the canonical layout; rows at or beyond nrows
-// are zero
-__device__ __forceinline__ void load_chunk_async(unsigned char* dst, const uint16_t* __restrict__ src,
-                                                 long long ld, long long r0, int R, long long nrows) {
-  constexpr int kc8 = kGemmKc / 8;
+// rows [r0, r0 + R) x columns [col0, col0 + C) of a row-major BF16 matrix (row
+// pitch ld) into the canonical layout by cp.async; rows at or beyond nrows
+// become zero.  Read as an operand whose K runs along the columns this is
+// K-major (leading offset 128 bytes, stride offset 16 C); read with K along
+// the rows it is MN-major: 8 rows x 16 bytes are a core matrix either way,
+// and the stride offset (next 8 columns) is 128 bytes, the leading offset
+// (next 8 rows) 16 C.
+__device__ __forceinline__ void load_canon_async(unsigned char* dst, const uint16_t* __restrict__ src,
+                                                 long long ld, long long r0, int R, long long nrows,
+                                                 int col0, int C) {
+  const int kc8 = C / 8;
   const int chunks = R * kc8;
   for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
     const int rr = c & 7, kc = (c >> 3) % kc8, rg = (c >> 3) / kc8;
     const long long r = r0 + rg * 8 + rr;
     const bool in = r < nrows;
-    const uint16_t* g = src + (in ? r : 0) * ld + kc * 8;
+    const uint16_t* g = src + (in ? r : 0) * ld + col0 + kc * 8;
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst + (size_t)c * 16)),
                  "l"(g), "r"(in ? 16 : 0)
                  : "memory");
   }
-  asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <int N>
-__global__ void __launch_bounds__(128, 1) tc_gemm_kernel(
-    const uint16_t* __restrict__ A, long long lda, const uint16_t* __restrict__ B, long long ldb,
-    long long M, int ksplit, int epi, float* __restrict__ C, long long ldc,
-    uint16_t* __restrict__ O, long long ldo, uint16_t* __restrict__ OT, long long ldot,
-    const float* __restrict__ bias, const uint16_t* __restrict__ mask, long long ldm,
-    unsigned int* __restrict__ status) {
+__device__ __forceinline__ float bf_lo(uint32_t p) { return __uint_as_float(p << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t p) { return __uint_as_float(p & 0xFFFF0000u); }
+
+// 16 words (32 BF16 values) of one row, 64 contiguous bytes
+__device__ __forceinline__ void store_row32(uint16_t* dst, const uint32_t* pk) {
+  uint4* d = reinterpret_cast<uint4*>(dst);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    d[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+}
+
+// relu(v + b) of 32 columns as BF16 pairs
+__device__ __forceinline__ void relu_pack32(const uint32_t* v, const float* b, uint32_t* pk) {
+#pragma unroll
+  for (int c = 0; c < 32; c += 4) {
+    const float4 bb = *reinterpret_cast<const float4*>(b + c);
+    pk[c / 2] = relu_bf16x2(__uint_as_float(v[c]) + bb.x, __uint_as_float(v[c + 1]) + bb.y);
+    pk[c / 2 + 1] = relu_bf16x2(__uint_as_float(v[c + 2]) + bb.z, __uint_as_float(v[c + 3]) + bb.w);
+  }
+}
+
+constexpr int kTrThreads = 256;
+constexpr size_t kTrSmem = (size_t)kMlpSmemW1 + kMlpSmemW2 + kMlpSmemX + 64;
+
+// Forward, loss and data gradients of rows [128 blockIdx.x, ...): X, W1 and W2
+// in shared memory; tensor memory columns 0..255 hold the layer-1 sums, then A1
+// and later dH2 as BF16 pairs (the A operands of the next products), columns
+// 256..511 the layer-2 sums, then those of dH1.  dH1 = dH2 W2 reads W2 from the
+// same shared copy as layer 2, as an MN-major operand.  Warp w holds the rows
+// 32 (w % 4) .. and the column half w / 4; the output layer runs one row per
+// thread of warps 0-3 while warps 4-7 store A2.  With one tile per CTA the
+// chain of load, four products and four epilogues bounds it, not their rates.
+__global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
+    const uint16_t* __restrict__ X, const float* __restrict__ T, long long n,
+    const uint16_t* __restrict__ W1, const uint16_t* __restrict__ W2, const float* __restrict__ b1,
+    const float* __restrict__ b2, const float* __restrict__ w3, uint16_t* __restrict__ A1,
+    uint16_t* __restrict__ A2, uint16_t* __restrict__ D1, uint16_t* __restrict__ D2,
+    float* __restrict__ DY, float* __restrict__ wloss, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char dsm[];
-  constexpr uint32_t kA = TM * kGemmKc * 2, kB = N * kGemmKc * 2;  // bytes of one stage
-  // stage s: A at dsm + s (kA + kB), B right after it
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(dsm + 2 * (kA + kB));  // [2]
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 2);
+  unsigned char* sW1 = dsm;
+  unsigned char* sW2 = dsm + kMlpSmemW1;
+  unsigned char* sX = sW2 + kMlpSmemW2;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sX + kMlpSmemX);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
+  // in the place of X once layer 1 has read it: w3 (3 x 256) and b3, b2, dY
+  float* s3 = reinterpret_cast<float*>(sX);
+  float* sb2 = s3 + 772;
+  float* sdy = sb2 + 256;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  const int wq = w & 3, half = w >> 2;
   const long long r0 = (long long)blockIdx.x * TM;
-  const long long k0 = (long long)blockIdx.y * ksplit;
-  const int nch = ksplit / kGemmKc;
+  const int rl = 32 * wq + lane;        // this thread's row of the tile
+  const long long row = r0 + rl;
+  const bool live = row < n;
 
   if (w == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(tslot)),
-                 "r"((uint32_t)N)
+                 "r"(512u)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    mbar_init(&mbar[0], 1u);
-    mbar_init(&mbar[1], 1u);
+    for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
     fence_mbar_init();
   }
+  pdl_wait();  // the weights of the previous step
+  load_canon_async(sX, X, 128, r0, TM, n, 0, 128);
+  load_canon_async(sW1, W1, 128, 0, 256, 256, 0, 128);
+  cp_async_commit();
+  load_canon_async(sW2, W2, 256, 0, 256, 256, 0, 256);
+  cp_async_commit();
+  cp_async_wait<1>();
+  fence_proxy_async();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tslot;
-  const uint32_t lbo = 128u, sbo = (uint32_t)(kGemmKc / 8) * 128u;
-  bool timeout = false;
-
-  for (int i = 0; i < nch; ++i) {
-    const int s = i & 1;
-    // the MMAs of chunk i - 2 read this stage: wait for their commit
-    if (i >= 2 && !mbar_wait(&mbar[s], (uint32_t)((i / 2 - 1) & 1))) timeout = true;
-    const long long kk = k0 + (long long)i * kGemmKc;
-    unsigned char* const sA = dsm + (size_t)s * (kA + kB);
-    unsigned char* const sB = sA + kA;
-    load_chunk_async(sA, A + kk, lda, r0, TM, M);
-    load_chunk_async(sB, B + kk, ldb, 0, N, N);
-    cp_async_wait_all();
+  const uint32_t lanes = tmem + ((uint32_t)(32 * wq) << 16);
+  bool tmo = false;
+  auto wait = [&](uint64_t* bar) {
+    if (!tmo && !mbar_wait(bar, 0u)) tmo = true;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  };
+  // the warps' accesses to shared and tensor memory before the next products
+  auto join = [&]() {
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     fence_proxy_async();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t ad = smem_desc(smem_u32(sA), lbo, sbo);
-      const uint64_t bd = smem_desc(smem_u32(sB), lbo, sbo);
-#pragma unroll
-      for (int kb = 0; kb < kGemmKc / 16; ++kb) {
-        const uint64_t adv = (uint64_t)((kb * 256) >> 4);
-        const uint32_t acc = (i > 0 || kb > 0) ? 1u : 0u;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-            "l"(ad + adv), "l"(bd + adv), "r"(idesc_n<N>()), "r"(acc)
-            : "memory");
-      }
-      asm volatile(
-          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-              smem_u32(&mbar[s]))
-          : "memory");
-    }
-  }
-  // the last commit covers every MMA issued before it
-  if (nch > 0 && !mbar_wait(&mbar[(nch - 1) & 1], (uint32_t)(((nch - 1) / 2) & 1))) timeout = true;
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  };
+  // column of K step kb (16 values, 8 columns of pairs) of the packed operand
+  auto packed = [&](int kb) { return tmem + (uint32_t)(kb < 8 ? 8 * kb : 128 + 8 * (kb - 8)); };
 
-  // epilogue: warp w owns TMEM lanes (rows) 32 w .. 32 w + 31
-  const long long row = r0 + 32 * w + lane;
-  const bool live = row < M && nch > 0;
+  if (tid == 0) {  // layer 1: X W1^T
+    const uint64_t xd = smem_desc(smem_u32(sX), 128u, 16u * 128u);
+    const uint64_t wd = smem_desc(smem_u32(sW1), 128u, 16u * 128u);
+#pragma unroll
+    for (int kb = 0; kb < 8; ++kb)
+      mma_ss_i(tmem, xd + (uint64_t)(kb * 16), wd + (uint64_t)(kb * 16), idesc_n(256), kb > 0);
+    mma_commit(bars);
+  }
+  wait(bars);
+  for (int i = tid; i < 771; i += kTrThreads) s3[i] = __ldg(w3 + i);  // w3 and b3 follow each other
+  sb2[tid] = __ldg(b2 + tid);
+
+  // A1 = relu(. + b1): packed into tensor memory and stored; m1: A1 > 0
+  uint32_t m1[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint32_t v[32], pk[16];
+    tmem_ld32(lanes + (uint32_t)(128 * half + 32 * j), v);
+    relu_pack32(v, b1 + 128 * half + 32 * j, pk);
+    tmem_st16(lanes + (uint32_t)(128 * half + 16 * j), pk);
+    uint32_t m = 0;
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      m |= ((pk[q] & 0xFFFFu) ? 1u : 0u) << (2 * q) | ((pk[q] >> 16) ? 2u : 0u) << (2 * q);
+    m1[j] = m;
+    if (live) store_row32(A1 + row * 256 + 128 * half + 32 * j, pk);
+  }
+  cp_async_wait<0>();  // W2
+  join();
+  if (tid == 0) {  // layer 2: A1 W2^T
+    const uint64_t wd = smem_desc(smem_u32(sW2), 128u, 32u * 128u);
+#pragma unroll
+    for (int kb = 0; kb < 16; ++kb)
+      mma_ts_i(tmem + 256u, packed(kb), wd + (uint64_t)(kb * 16), idesc_n(256), kb > 0);
+    mma_commit(bars + 1);
+  }
+  wait(bars + 1);
+
+  if (half == 0) {
+    // y = A2 w3^T + b3 in ascending order of the hidden units, dY, loss
+    float o0 = s3[768], o1 = s3[769], o2 = s3[770];
 #pragma unroll 1
-  for (int c0 = 0; c0 < N; c0 += 32) {
-    uint32_t v[32];
-    tmem_ld32(tmem + ((uint32_t)(32 * w) << 16) + (uint32_t)c0, v);
-    if (epi == kEpiF32) {
-      if (live) {
-        float4* dst = reinterpret_cast<float4*>(C + ((long long)blockIdx.y * M + row) * ldc + c0);
+    for (int j = 0; j < 8; ++j) {
+      uint32_t v[32], pk[16];
+      tmem_ld32(lanes + 256u + (uint32_t)(32 * j), v);
+      relu_pack32(v, sb2 + 32 * j, pk);
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          dst[q] = make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
-                               __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+      for (int c = 0; c < 32; c += 4) {
+        const float4 u0 = *reinterpret_cast<const float4*>(s3 + 32 * j + c);
+        const float4 u1 = *reinterpret_cast<const float4*>(s3 + 256 + 32 * j + c);
+        const float4 u2 = *reinterpret_cast<const float4*>(s3 + 512 + 32 * j + c);
+        const float a0 = bf_lo(pk[c / 2]), a1 = bf_hi(pk[c / 2]);
+        const float a2 = bf_lo(pk[c / 2 + 1]), a3 = bf_hi(pk[c / 2 + 1]);
+        o0 = fmaf(a3, u0.w, fmaf(a2, u0.z, fmaf(a1, u0.y, fmaf(a0, u0.x, o0))));
+        o1 = fmaf(a3, u1.w, fmaf(a2, u1.z, fmaf(a1, u1.y, fmaf(a0, u1.x, o1))));
+        o2 = fmaf(a3, u2.w, fmaf(a2, u2.z, fmaf(a1, u2.y, fmaf(a0, u2.x, o2))));
       }
-      continue;
     }
-    float f[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) {
-      float x = __uint_as_float(v[j]);
-      if (epi == kEpiBiasRelu) {
-        x = fmaxf(x + bias[c0 + j], 0.f);
-      } else if (live) {
-        const uint16_t mk = mask[row * ldm + c0 + j];
-        if (!(__uint_as_float((uint32_t)mk << 16) > 0.f)) x = 0.f;
-      }
-      f[j] = x;
-    }
+    float lsum = 0.f, y0 = 0.f, y1 = 0.f, y2 = 0.f;
     if (live) {
-      uint32_t pk[16];
-#pragma unroll
-      for (int j = 0; j < 16; ++j) pk[j] = bf16x2_bits(f[2 * j], f[2 * j + 1]);
-      uint4* dst = reinterpret_cast<uint4*>(O + row * ldo + c0);
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        dst[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
-      if (OT) {
-        // column c0 + j of the 32 rows of this warp: 64 contiguous bytes
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const __nv_bfloat16 b = __float2bfloat16_rn(f[j]);
-          OT[(long long)(c0 + j) * ldot + row] = *reinterpret_cast<const uint16_t*>(&b);
-        }
-      }
+      const float d0 = o0 - T[3 * row], d1 = o1 - T[3 * row + 1], d2 = o2 - T[3 * row + 2];
+      lsum += d0 * d0 + d1 * d1 + d2 * d2;
+      const float sc = 2.f / (float)n;
+      y0 = sc * d0;
+      y1 = sc * d1;
+      y2 = sc * d2;
+      DY[3 * row] = y0;
+      DY[3 * row + 1] = y1;
+      DY[3 * row + 2] = y2;
+    }
+    sdy[3 * rl] = y0;
+    sdy[3 * rl + 1] = y1;
+    sdy[3 * rl + 2] = y2;
+    for (int d = 16; d; d >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, d);
+    if (lane == 0) wloss[4 * blockIdx.x + wq] = lsum;
+  } else {
+#pragma unroll 1
+    for (int j = 0; j < 8; ++j) {
+      uint32_t v[32], pk[16];
+      tmem_ld32(lanes + 256u + (uint32_t)(32 * j), v);
+      relu_pack32(v, sb2 + 32 * j, pk);
+      if (live) store_row32(A2 + row * 256 + 32 * j, pk);
     }
   }
+  __syncthreads();  // dY
+
+  // dH2 = (dY w3) where A2 > 0
+  {
+    const float y0 = sdy[3 * rl], y1 = sdy[3 * rl + 1], y2 = sdy[3 * rl + 2];
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const int k0 = 128 * half + 32 * j;
+      uint32_t v[32], pk[16];
+      tmem_ld32(lanes + 256u + (uint32_t)k0, v);
+      relu_pack32(v, sb2 + k0, pk);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        const int k = k0 + 2 * q;
+        const float2 u0 = *reinterpret_cast<const float2*>(s3 + k);
+        const float2 u1 = *reinterpret_cast<const float2*>(s3 + 256 + k);
+        const float2 u2 = *reinterpret_cast<const float2*>(s3 + 512 + k);
+        float g0 = y0 * u0.x + y1 * u1.x + y2 * u2.x;
+        float g1 = y0 * u0.y + y1 * u1.y + y2 * u2.y;
+        if (bf_lo(pk[q]) <= 0.f) g0 = 0.f;
+        if (bf_hi(pk[q]) <= 0.f) g1 = 0.f;
+        pk[q] = bf16x2_bits(g0, g1);
+      }
+      tmem_st16(lanes + (uint32_t)(128 * half + 16 * j), pk);
+      if (live) store_row32(D2 + row * 256 + k0, pk);
+    }
+  }
+  join();
+  if (tid == 0) {  // dH1 = dH2 W2 (K = the outputs of layer 2: rows of W2)
+    const uint64_t wd = smem_desc(smem_u32(sW2), 32u * 128u, 128u);
+#pragma unroll
+    for (int kb = 0; kb < 16; ++kb)
+      mma_ts_i(tmem + 256u, packed(kb), wd + (uint64_t)(kb * 512), idesc_n(256) | kMajorMnB, kb > 0);
+    mma_commit(bars + 2);
+  }
+  wait(bars + 2);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    uint32_t v[32], pk[16];
+    tmem_ld32(lanes + 256u + (uint32_t)(128 * half + 32 * j), v);
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      pk[q] = bf16x2_bits((m1[j] >> (2 * q)) & 1u ? __uint_as_float(v[2 * q]) : 0.f,
+                          (m1[j] >> (2 * q)) & 2u ? __uint_as_float(v[2 * q + 1]) : 0.f);
+    if (live) store_row32(D1 + row * 256 + 128 * half + 32 * j, pk);
+  }
+  if (tmo) atomicOr(status, 1u);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-  if (timeout) atomicOr(status, 1u);
   __syncthreads();
   if (w == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)N)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u)
                  : "memory");
 }
 
-// G[i] = sum over splits s = 0, 1, ... of P[s][i], in that order
-__global__ void tc_split_sum_kernel(const float* __restrict__ P, long long n, int splits,
-                                    float* __restrict__ G) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (long long)gridDim.x * blockDim.x) {
-    float acc = 0.f;
-    for (int s = 0; s < splits; ++s) acc += P[(long long)s * n + i];
-    G[i] = acc;
+// Gradients.  Blocks 4 s .. 4 s + 3 (s < splits): split s of the batch for
+// dW2[o][k] = sum_m dH2[m][o] A1[m][k] (o < 128, o >= 128) and dW1[o][i] =
+// sum_m dH1[m][o] X[m][i]; both operands are MN-major in the rows' own order,
+// 64 rows a chunk through a ring of four stages, FP32 partials per split.  The
+// other blocks: one chunk of 64 rows each, in ascending row order, of dW3 and
+// db3 (width kPart3), db2 and db1.
+constexpr int kGrThreads = 256, kGrStages = 4, kGrRows = 64;
+constexpr uint32_t kGrA = kGrRows * 128 * 2, kGrB = kGrRows * 256 * 2;
+constexpr size_t kGrSmem = (size_t)kGrStages * (kGrA + kGrB) + 64;
+constexpr int kPart3 = 771;
+
+struct GradArgs {
+  const uint16_t *X, *A1, *A2, *D1, *D2;
+  const float* DY;
+  long long n;
+  int splits;
+  float *part1, *part2;   // [splits][256][128], [splits][256][256]
+  float *p3, *pb2, *pb1;  // per 64-row chunk: [kPart3], [256], [256]
+  unsigned int* status;
+};
+
+__device__ __forceinline__ void grad_chunk(const GradArgs& a, long long chunk, float* sdy) {
+  const long long m0 = chunk * kGrRows;
+  const int nr = (int)(a.n - m0 < kGrRows ? a.n - m0 : kGrRows);
+  for (int i = threadIdx.x; i < 3 * nr; i += kGrThreads) sdy[i] = a.DY[3 * m0 + i];
+  __syncthreads();
+  const int c = threadIdx.x & 127;  // columns 2 c, 2 c + 1
+  auto col = [&](const uint16_t* M, int r) {
+    return __ldg(reinterpret_cast<const uint32_t*>(M + (m0 + r) * 256) + c);
+  };
+  if (threadIdx.x < 128) {
+    float s0 = 0.f, s1 = 0.f, t0 = 0.f, t1 = 0.f;
+#pragma unroll 16
+    for (int r = 0; r < nr; ++r) {
+      const uint32_t u = col(a.D2, r), v = col(a.D1, r);
+      s0 += bf_lo(u);
+      s1 += bf_hi(u);
+      t0 += bf_lo(v);
+      t1 += bf_hi(v);
+    }
+    *reinterpret_cast<float2*>(a.pb2 + chunk * 256 + 2 * c) = make_float2(s0, s1);
+    *reinterpret_cast<float2*>(a.pb1 + chunk * 256 + 2 * c) = make_float2(t0, t1);
+  } else {
+    float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 16
+    for (int r = 0; r < nr; ++r) {
+      const uint32_t u = col(a.A2, r);
+#pragma unroll
+      for (int o = 0; o < 3; ++o) {
+        s[2 * o] = fmaf(sdy[3 * r + o], bf_lo(u), s[2 * o]);
+        s[2 * o + 1] = fmaf(sdy[3 * r + o], bf_hi(u), s[2 * o + 1]);
+      }
+    }
+    float* out = a.p3 + chunk * kPart3;
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      out[256 * o + 2 * c] = s[2 * o];
+      out[256 * o + 2 * c + 1] = s[2 * o + 1];
+    }
+    if (c < 3) {
+      float b = 0.f;
+      for (int r = 0; r < nr; ++r) b += sdy[3 * r + c];
+      out[768 + c] = b;
+    }
   }
+}
+
+__global__ void __launch_bounds__(kGrThreads, 1) train_grads_kernel(GradArgs a) {
+  extern __shared__ __align__(1024) unsigned char dsm[];
+  uint64_t* bars = reinterpret_cast<uint64_t*>(dsm + kGrStages * (kGrA + kGrB));
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + kGrStages);
+  const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+  if ((int)blockIdx.x >= 4 * a.splits) {
+    pdl_wait();
+    grad_chunk(a, (long long)blockIdx.x - 4 * a.splits, reinterpret_cast<float*>(dsm));
+    return;
+  }
+  const int split = blockIdx.x >> 2, o0 = (blockIdx.x & 1) * 128;
+  const bool second = (blockIdx.x & 2) == 0;  // dW2, else dW1
+  const int N = second ? 256 : 128;
+  const uint16_t* A = second ? a.D2 : a.D1;
+  const uint16_t* B = second ? a.A1 : a.X;
+  const long long nch = (a.n + kGrRows - 1) / kGrRows;
+  const long long c0 = nch * split / a.splits, c1 = nch * (split + 1) / a.splits;
+  const int nc = (int)(c1 - c0);
+
+  if (w == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(tslot)),
+                 "r"(256u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    for (int i = 0; i < kGrStages; ++i) mbar_init(bars + i, 1u);
+    fence_mbar_init();
+  }
+  pdl_wait();
+  bool tmo = false;
+  auto stage = [&](int i) { return dsm + (size_t)(i % kGrStages) * (kGrA + kGrB); };
+  auto fill = [&](int i) {  // chunk i of the split (an empty group past the end)
+    if (i < nc) {
+      load_canon_async(stage(i), A, 256, (c0 + i) * kGrRows, kGrRows, a.n, o0, 128);
+      load_canon_async(stage(i) + kGrA, B, N, (c0 + i) * kGrRows, kGrRows, a.n, 0, N);
+    }
+    cp_async_commit();
+  };
+  // the products of chunk i have read its stage
+  auto drained = [&](int i) {
+    if (!tmo && !mbar_wait(bars + i % kGrStages, (uint32_t)(i / kGrStages) & 1u)) tmo = true;
+  };
+  for (int i = 0; i < kGrStages - 1; ++i) fill(i);
+  uint32_t tmem = 0;
+  for (int i = 0; i < nc; ++i) {
+    if (i > 0) drained(i - 1);
+    fill(i + kGrStages - 1);
+    cp_async_wait<kGrStages - 1>();  // chunk i has landed
+    fence_proxy_async();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    tmem = *tslot;
+    if (tid == 0) {
+      const uint64_t ad = smem_desc(smem_u32(stage(i)), 16u * 128u, 128u);
+      const uint64_t bd = smem_desc(smem_u32(stage(i) + kGrA), (uint32_t)(N / 8) * 128u, 128u);
+      const uint32_t id = idesc_n(N) | kMajorMnA | kMajorMnB;
+#pragma unroll
+      for (int kb = 0; kb < kGrRows / 16; ++kb)  // 16 rows: two 8-row groups
+        mma_ss_i(tmem, ad + (uint64_t)(kb * 256), bd + (uint64_t)(kb * (N / 8) * 16), id,
+                 (i > 0 || kb > 0) ? 1u : 0u);
+      mma_commit(bars + i % kGrStages);
+    }
+  }
+  cp_async_wait<0>();
+  if (nc > 0) drained(nc - 1);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  // rows o0 + 32 (w % 4) + lane, column half w / 4
+  const int row = o0 + 32 * (w & 3) + lane;
+  float* out = (second ? a.part2 : a.part1) + ((long long)split * 256 + row) * N;
+  for (int j = (w >> 2) * (N / 2); j < ((w >> 2) + 1) * (N / 2); j += 32) {
+    uint32_t v[32];
+    tmem_ld32(tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)j, v);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      reinterpret_cast<float4*>(out + j)[q] =
+          make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                      __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+  }
+  if (tmo) atomicOr(a.status, 1u);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (w == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u)
+                 : "memory");
+}
+
+// part[0], part[pitch], ... summed in that order
+__device__ __forceinline__ float sum_in_order(const float* __restrict__ part, long long count,
+                                              long long pitch) {
+  float acc = 0.f;
+#pragma unroll 16
+  for (long long s = 0; s < count; ++s) acc += __ldg(part + s * pitch);
+  return acc;
+}
+
+// Gradient i from its partials in a fixed order and (adam) its Adam step,
+// refreshing the BF16 weights; the last block adds the loss: the warps' sums of
+// 256 rows in order, divided by n, then those in order.
+__global__ void __launch_bounds__(256) train_update_kernel(GradArgs a, TrainState t) {
+  pdl_wait();
+  const long long chunks = (a.n + kGrRows - 1) / kGrRows;
+  const int i = (int)(blockIdx.x * 256u + threadIdx.x);
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x == 0) {
+      const long long warps = (a.n + TM - 1) / TM * 4;
+      float acc = 0.f;
+      for (long long s = 0; s < warps; s += 8) {
+        float b = 0.f;
+        for (long long q = s; q < s + 8 && q < warps; ++q) b += __ldg(t.wloss + q);
+        acc += b / (float)a.n;
+      }
+      *t.loss = acc;
+    }
+    return;
+  }
+  if (i >= QTV_LOCATOR_PARAMS) return;
+  constexpr int oB1 = 256 * 128, oW2 = oB1 + 256, oB2 = oW2 + 256 * 256, oW3 = oB2 + 256;
+  float g;
+  if (i < oB1) g = sum_in_order(a.part1 + i, a.splits, 256 * 128);
+  else if (i < oW2) g = sum_in_order(a.pb1 + (i - oB1), chunks, 256);
+  else if (i < oB2) g = sum_in_order(a.part2 + (i - oW2), a.splits, 256 * 256);
+  else if (i < oW3) g = sum_in_order(a.pb2 + (i - oB2), chunks, 256);
+  else g = sum_in_order(a.p3 + (i - oW3), chunks, kPart3);
+  t.G[i] = g;
+  if (!t.adam) return;
+  const float m = t.beta1 * t.M[i] + (1.f - t.beta1) * g;
+  const float v = t.beta2 * t.V[i] + (1.f - t.beta2) * g * g;
+  t.M[i] = m;
+  t.V[i] = v;
+  const float p = t.P[i] - t.lr * (m / t.c1) / (sqrtf(v / t.c2) + t.eps);
+  t.P[i] = p;
+  const __nv_bfloat16 b = __float2bfloat16_rn(p);
+  if (i < oB1) t.w1b[i] = *reinterpret_cast<const uint16_t*>(&b);
+  else if (i >= oW2 && i < oB2) t.w2b[i - oW2] = *reinterpret_cast<const uint16_t*>(&b);
 }
 
 }  // namespace
 
-size_t tc_gemm_smem(int N) { return (size_t)2 * (TM + N) * kGemmKc * 2 + 16 + 16; }
+// Splits of a batch of k64 chunks of 64 rows for the weight gradients: a
+// divisor of k64 up to kTrainSplits (equal splits) unless it has none of at
+// least half that, then kTrainSplits uneven ones (4544 rows are 71 chunks).
+int train_splits(long long k64) {
+  if (k64 <= kTrainSplits) return (int)k64;
+  int s = kTrainSplits;
+  while (k64 % s) --s;
+  return s >= kTrainSplits / 2 ? s : kTrainSplits;
+}
 
-// C[M][N] = A[M][K] B[N][K]^T on the tensor cores (see tc_gemm_kernel).
-// epi 0: FP32 into C (row pitch ldc); with splits > 1 the K range is cut in
-// `splits` parts whose partials go to `part` ([splits][M][N]) and are summed
-// into C (pitch N) in split order, so the result does not depend on timing.
-// epi 1 / 2: BF16 into O (and OT transposed, if not null).
-int tc_gemm(const uint16_t* A, long long lda, const uint16_t* B, long long ldb, long long M, int N,
-            long long K, int splits, int epi, float* C, long long ldc, float* part, uint16_t* O,
-            long long ldo, uint16_t* OT, long long ldot, const float* bias, const uint16_t* mask,
-            long long ldm, unsigned int* status, cudaStream_t st) {
-  if (M <= 0) return QTV_OK;
-  if (N != 128 && N != 256) return set_error(QTV_ERR_ARG, "tc_gemm: N = %d (128 or 256)", N);
-  if (splits < 1 || K % ((long long)splits * kGemmKc) != 0)
-    return set_error(QTV_ERR_ARG, "tc_gemm: K = %lld not a multiple of %d splits x %d", K, splits,
-                     kGemmKc);
-  if (splits > 1 && (epi != kEpiF32 || !part))
-    return set_error(QTV_ERR_ARG, "tc_gemm: split K needs the FP32 epilogue and partials");
-  static bool attr[2] = {false, false};
-  const int which = N == 256 ? 1 : 0;
-  const size_t smem = tc_gemm_smem(N);
-  if (!attr[which]) {
-    cudaError_t e = N == 256 ? cudaFuncSetAttribute(tc_gemm_kernel<256>,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                             : cudaFuncSetAttribute(tc_gemm_kernel<128>,
-                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return check_cuda(e, "cudaFuncSetAttribute(tc_gemm)");
-    attr[which] = true;
+int tc_train(const uint16_t* X, const float* T, long long n, const TrainBuffers& B, const TrainState& t,
+             unsigned int* status, cudaStream_t st) {
+  if (n <= 0) return QTV_OK;
+  if (reinterpret_cast<uintptr_t>(X) & 15u)
+    return set_error(QTV_ERR_ARG, "training rows must be 16-byte aligned");
+  static bool attr = false;
+  if (!attr) {
+    cudaError_t e = cudaFuncSetAttribute(train_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)kTrSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(train_grads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)kGrSmem);
+    if (e != cudaSuccess) return check_cuda(e, "cudaFuncSetAttribute(training)");
+    attr = true;
   }
-  const dim3 grid((unsigned)((M + TM - 1) / TM), (unsigned)splits);
-  const int ksplit = (int)(K / splits);
-  float* Cout = splits > 1 ? part : C;
-  const long long ldcc = splits > 1 ? N : ldc;
-  if (N == 256)
-    tc_gemm_kernel<256><<<grid, 128, smem, st>>>(A, lda, B, ldb, M, ksplit, epi, Cout, ldcc, O, ldo,
-                                                 OT, ldot, bias, mask, ldm, status);
-  else
-    tc_gemm_kernel<128><<<grid, 128, smem, st>>>(A, lda, B, ldb, M, ksplit, epi, Cout, ldcc, O, ldo,
-                                                 OT, ldot, bias, mask, ldm, status);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return check_cuda(e, "tc_gemm_kernel launch");
-  if (splits > 1) {
-    const long long n = M * N;
-    tc_split_sum_kernel<<<(unsigned)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024), 256, 0, st>>>(
-        part, n, splits, C);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return check_cuda(e, "tc_split_sum_kernel launch");
-  }
-  return QTV_OK;
+  const long long tiles = (n + TM - 1) / TM, chunks = (n + kGrRows - 1) / kGrRows;
+  cudaError_t e = launch_dependent(train_rows_kernel, dim3((unsigned)tiles), dim3(kTrThreads), kTrSmem,
+                                   st, X, T, n, (const uint16_t*)t.w1b, (const uint16_t*)t.w2b,
+                                   (const float*)t.P + 256 * 128,
+                                   (const float*)t.P + 256 * 128 + 256 + 256 * 256,
+                                   (const float*)t.P + 256 * 128 + 512 + 256 * 256, B.A1, B.A2, B.D1,
+                                   B.D2, B.DY, t.wloss, status);
+  if (e != cudaSuccess) return check_cuda(e, "train_rows_kernel launch");
+  GradArgs a;
+  a.X = X;
+  a.A1 = B.A1;
+  a.A2 = B.A2;
+  a.D1 = B.D1;
+  a.D2 = B.D2;
+  a.DY = B.DY;
+  a.n = n;
+  a.splits = train_splits(chunks);
+  a.part1 = B.part;
+  a.part2 = B.part + (size_t)kTrainSplits * 256 * 128;
+  a.p3 = B.chunk;
+  a.pb2 = B.chunk + (size_t)chunks * (kPart3 + 1);
+  a.pb1 = a.pb2 + (size_t)chunks * 256;
+  a.status = status;
+  e = launch_dependent(train_grads_kernel, dim3((unsigned)(4 * a.splits + chunks)), dim3(kGrThreads),
+                       kGrSmem, st, a);
+  if (e != cudaSuccess) return check_cuda(e, "train_grads_kernel launch");
+  e = launch_dependent(train_update_kernel, dim3((QTV_LOCATOR_PARAMS + 255) / 256 + 1), dim3(256), 0, st,
+                       a, t);
+  return check_cuda(e, "train_update_kernel launch");
 }
 
 // Y[M][3] of the whole network on the tensor cores (see tc_mlp_kernel).

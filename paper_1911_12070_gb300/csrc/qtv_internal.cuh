@@ -399,12 +399,27 @@ int locator_localize(qtv_handle h, const FaceGeo& geo, const uint64_t* face_ids,
 // locator is loaded.
 int locator_prepare(qtv_handle h, uint64_t n, uint64_t* generation);
 
-// C[M][N] = A[M][K] B[N][K]^T on tcgen05 (locator_tc.cu); epi 0 FP32 (split K
-// summed in order), 1 relu(. + bias) BF16, 2 masked by mask > 0 BF16
-int tc_gemm(const uint16_t* A, long long lda, const uint16_t* B, long long ldb, long long M, int N,
-            long long K, int splits, int epi, float* C, long long ldc, float* part, uint16_t* O,
-            long long ldo, uint16_t* OT, long long ldot, const float* bias, const uint16_t* mask,
-            long long ldm, unsigned int* status, cudaStream_t st);
+// One training step of the learned locator on tcgen05 (locator_tc.cu): rows X
+// [n][128] BF16, targets T [n][3].  Row buffers [n][256] BF16, DY [n][3]; part
+// holds kTrainSplits x (256 x 128 + 256 x 256) and chunk 1284 values per 64
+// rows; wloss 4 per 128 rows.
+constexpr int kTrainSplits = 16;
+constexpr int kTrainChunkFloats = 1284;
+struct TrainBuffers {
+  uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr;
+  float *DY = nullptr, *part = nullptr, *chunk = nullptr;
+};
+// parameters, gradients (written), Adam moments and the step's constants; adam
+// 0: gradients and loss only
+struct TrainState {
+  float *P = nullptr, *G = nullptr, *M = nullptr, *V = nullptr;
+  uint16_t *w1b = nullptr, *w2b = nullptr;
+  float *wloss = nullptr, *loss = nullptr;
+  int adam = 0;
+  float lr = 0.f, beta1 = 0.f, beta2 = 0.f, eps = 0.f, c1 = 1.f, c2 = 1.f;
+};
+int tc_train(const uint16_t* X, const float* T, long long n, const TrainBuffers& B, const TrainState& t,
+             unsigned int* status, cudaStream_t st);
 // The whole network, fused (locator_tc.cu): Y[M][3] from X[M][128] (W1, W2
 // BF16; biases and W3 FP32); X 16-byte aligned, M below 2^31.
 int tc_mlp_forward(const uint16_t* X, long long M, const uint16_t* W1, const uint16_t* W2,
