@@ -433,31 +433,29 @@ __global__ void sum_parts_kernel(const float* __restrict__ part, int nb, int wid
 __global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ G,
                             float* __restrict__ Mo, float* __restrict__ Vo, int n, float lr,
                             float b1, float b2, float eps, float c1, float c2,
-                            uint16_t* __restrict__ w1b, uint16_t* __restrict__ w2b) {
+                            uint16_t* __restrict__ w1b, uint16_t* __restrict__ w2b,
+                            uint16_t* __restrict__ w1c, uint16_t* __restrict__ w2c) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float g = G[i];
-    const float m = b1 * Mo[i] + (1.f - b1) * g;
-    const float v = b2 * Vo[i] + (1.f - b2) * g * g;
-    Mo[i] = m;
-    Vo[i] = v;
-    const float p = P[i] - lr * (m / c1) / (sqrtf(v / c2) + eps);
+    const float p = adam_value(P[i], G[i], Mo[i], Vo[i], lr, b1, b2, eps, c1, c2);
     P[i] = p;
     if (i < (int)kOffB1) {
-      w1b[i - kOffW1] = f2bf(p);
+      w1b[i - kOffW1] = w1c[canon_index(i - (int)kOffW1, kIn)] = f2bf(p);
     } else if (i >= (int)kOffW2 && i < (int)kOffB2) {
-      w2b[i - (int)kOffW2] = f2bf(p);
+      w2b[i - (int)kOffW2] = w2c[canon_index(i - (int)kOffW2, kH)] = f2bf(p);
     }
   }
 }
 
 __global__ void refresh_bf16_kernel(const float* __restrict__ P, uint16_t* __restrict__ w1b,
-                                    uint16_t* __restrict__ w2b) {
+                                    uint16_t* __restrict__ w2b, uint16_t* __restrict__ w1c,
+                                    uint16_t* __restrict__ w2c) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kH * kIn + kH * kH;
        i += gridDim.x * blockDim.x) {
     if (i < kH * kIn) {
-      w1b[i] = f2bf(P[kOffW1 + i]);
+      w1b[i] = w1c[canon_index(i, kIn)] = f2bf(P[kOffW1 + i]);
     } else {
-      w2b[i - kH * kIn] = f2bf(P[kOffW2 + (i - kH * kIn)]);
+      const int j = i - kH * kIn;
+      w2b[j] = w2c[canon_index(j, kH)] = f2bf(P[kOffW2 + j]);
     }
   }
 }
@@ -575,6 +573,7 @@ struct Locator {
   float* V = nullptr;      // Adam second moment
   uint16_t* w1b = nullptr; // BF16 W1 [256][128]
   uint16_t* w2b = nullptr; // BF16 W2 [256][256]
+  uint16_t *w1c = nullptr, *w2c = nullptr;  // both in the tensor cores' layout
   unsigned long long step = 0;
   bool ready = false;
   // activations for up to `cap` rows; rows_gen counts their reallocations
@@ -584,7 +583,7 @@ struct Locator {
   int tensor_path = 1;
   int num_sms = 0;
   unsigned int* status = nullptr;  // timeout flag of the tcgen05 kernel
-  uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr, *X = nullptr;
+  uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr, *X = nullptr, *XB = nullptr;
   // training on tcgen05: partials of the weight gradients per split and the
   // loss of every 32 rows
   float* part = nullptr;
@@ -606,7 +605,10 @@ void locator_free(Locator* L) {
   cudaFree(L->V);
   cudaFree(L->w1b);
   cudaFree(L->w2b);
+  cudaFree(L->w1c);
+  cudaFree(L->w2c);
   cudaFree(L->part);
+  cudaFree(L->XB);
   cudaFree(L->wloss);
   cudaFree(L->lpart);
   cudaFree(L->gpart);
@@ -635,6 +637,8 @@ static int locator_alloc(qtv_handle h) {
   if (e == cudaSuccess) e = cudaMalloc(&L->V, pb);
   if (e == cudaSuccess) e = cudaMalloc(&L->w1b, (size_t)kH * kIn * 2);
   if (e == cudaSuccess) e = cudaMalloc(&L->w2b, (size_t)kH * kH * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->w1c, (size_t)kH * kIn * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->w2c, (size_t)kH * kH * 2);
   if (e == cudaSuccess)
     e = cudaMalloc(&L->part, (size_t)kTrainSplits * (kH * kIn + kH * kH) * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&L->lpart, (size_t)kLossBlocks * sizeof(float));
@@ -665,15 +669,19 @@ static int locator_rows(qtv_handle h, unsigned long long n, cudaStream_t st) {
   cudaFree(L->rms);
   cudaFree(L->ok);
   cudaFree(L->wloss);
+  cudaFree(L->XB);
   L->wloss = nullptr;
+  L->XB = nullptr;
   L->A1 = L->A2 = L->D1 = L->D2 = L->X = nullptr;
   L->Y = L->DY = L->rms = nullptr;
   L->ok = nullptr;
   L->cap = 0;
-  cudaError_t e = cudaMalloc(&L->A1, n * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->A2, n * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->D1, n * kH * 2);
-  if (e == cudaSuccess) e = cudaMalloc(&L->D2, n * kH * 2);
+  const unsigned long long nt = (n + 127) / 128 * 128;  // whole tiles (training images)
+  cudaError_t e = cudaMalloc(&L->A1, nt * kH * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->A2, nt * kH * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->D1, nt * kH * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->D2, nt * kH * 2);
+  if (e == cudaSuccess) e = cudaMalloc(&L->XB, nt * kIn * 2);
   if (e == cudaSuccess) e = cudaMalloc(&L->X, n * kIn * 2);
   if (e == cudaSuccess) e = cudaMalloc(&L->Y, n * kOut * 4);
   if (e == cudaSuccess) e = cudaMalloc(&L->DY, n * kOut * 4);
@@ -698,7 +706,7 @@ static int forward_hidden(Locator* L, const uint16_t* X, unsigned long long n, c
 static int forward_y(Locator* L, const uint16_t* X, unsigned long long n, float* Y,
                      cudaStream_t st) {
   if (L->tensor_path == 1)
-    return tc_mlp_forward(X, (long long)n, L->w1b, L->w2b, L->P + kOffB1, L->P + kOffB2,
+    return tc_mlp_forward(X, (long long)n, L->w1c, L->w2c, L->P + kOffB1, L->P + kOffB2,
                           L->P + kOffW3, L->P + kOffB3, Y, L->status, L->num_sms, st);
   int rc = forward_hidden(L, X, n, st);
   if (rc) return rc;
@@ -827,7 +835,7 @@ int qtv_locator_init(qtv_handle h, uint64_t seed) {
   init_kernel<<<64, 256>>>(L->P, seed);
   cudaMemset(L->M, 0, kNumParams * 4);
   cudaMemset(L->V, 0, kNumParams * 4);
-  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b);
+  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b, L->w1c, L->w2c);
   L->step = 0;
   L->ready = true;
   return check_cuda(cudaDeviceSynchronize(), "qtv_locator_init");
@@ -870,7 +878,7 @@ int qtv_locator_set(qtv_handle h, const float* params, const float* adam, uint64
     }
   }
   if (e != cudaSuccess) return check_cuda(e, "qtv_locator_set");
-  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b);
+  refresh_bf16_kernel<<<64, 256>>>(L->P, L->w1b, L->w2b, L->w1c, L->w2c);
   L->step = step;
   L->ready = true;
   return check_cuda(cudaDeviceSynchronize(), "qtv_locator_set");
@@ -914,8 +922,8 @@ static int locator_step(qtv_handle h, const uint16_t* x, const float* targets, u
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f, t = (float)(L->step + 1);
   const float c1 = 1.f - powf(b1, t), c2 = 1.f - powf(b2, t);
   if (L->tensor_path == 1) {
-    const TrainBuffers B{L->A1, L->A2, L->D1, L->D2, L->DY, L->part, L->gpart};
-    const TrainState s{L->P, L->G,  L->M, L->V, L->w1b, L->w2b, L->wloss, loss, adam ? 1 : 0,
+    const TrainBuffers B{L->A1, L->A2, L->D1, L->D2, L->XB, L->DY, L->part, L->gpart};
+    const TrainState s{L->P, L->G,  L->M, L->V, L->w1b, L->w2b, L->w1c, L->w2c, L->wloss, loss, adam ? 1 : 0,
                        lr,   b1,    b2,   eps,  c1,     c2};
     rc = tc_train(x, targets, (long long)n, B, s, L->status, st);
     if (rc) return rc;
@@ -924,7 +932,7 @@ static int locator_step(qtv_handle h, const uint16_t* x, const float* targets, u
     if (rc) return rc;
     if (adam)
       adam_kernel<<<128, 256, 0, st>>>(L->P, L->G, L->M, L->V, (int)kNumParams, lr, b1, b2, eps, c1, c2,
-                                       L->w1b, L->w2b);
+                                       L->w1b, L->w2b, L->w1c, L->w2c);
   }
   if (adam) L->step += 1;
   return check_cuda(cudaGetLastError(), "locator step");

@@ -3,11 +3,12 @@
 // network fused per 128-row tile (tc_mlp_kernel, warp-specialised; its design
 // is described at its definition) and the training step (train_*_kernel).
 //
-// Operands staged by threads are stored in the canonical K-major layout
-// without swizzle: 8 x 8 core matrices of 128 contiguous bytes (8 rows of 16
-// bytes), core matrix (r / 8, k / 8) at ((r / 8) (K / 8) + k / 8) 128 bytes,
-// so the leading-dimension offset (next core matrix along K) is 128 bytes and
-// the stride offset (next 8-row group) is 16 K bytes.  One elected thread
+// W1 and W2 are kept in global memory in the canonical K-major layout without
+// swizzle (w1c, w2c; canon_index): 8 x 8 core matrices of 128 contiguous bytes
+// (8 rows of 16 bytes), core matrix (r / 8, k / 8) at ((r / 8) (K / 8) + k / 8)
+// 128 bytes, so the leading-dimension offset (next core matrix along K) is 128
+// bytes and the stride offset (next 8-row group) is 16 K bytes, and a CTA
+// takes each by plain bulk copies.  One elected thread
 // issues the tcgen05.mma instructions and commits them to mbarriers; warps
 // read their 32 TMEM lanes back with tcgen05.ld.  Accumulator columns are
 // allocated once per CTA and freed before exit; every mbarrier wait is
@@ -41,23 +42,26 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo, uint3
   return d;                // base offset 0, swizzle none
 }
 
-// rows [r0, r0 + R) of a row-major BF16 matrix (K columns, row pitch K) into
-// the canonical layout at dst; rows at or beyond nrows become zero.  Piece c
-// (16 bytes) goes to byte 16 c of dst: c = ((r / 8) (K / 8) + k / 8) 8 + r % 8,
-// so consecutive threads fill consecutive shared-memory slots (no bank
-// conflicts) and read 8 rows x 16 bytes per group of 8 threads.
-__device__ __forceinline__ void load_canon(unsigned char* dst, const uint16_t* __restrict__ src,
-                                           long long r0, int R, long long nrows, int K) {
-  const int kc8 = K / 8;
-  const int chunks = R * kc8;
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-    const int rr = c & 7, kc = (c >> 3) % kc8, rg = (c >> 3) / kc8;
-    const int r = rg * 8 + rr;
-    uint4 v = make_uint4(0u, 0u, 0u, 0u);
-    if (r0 + r < nrows) v = __ldg(reinterpret_cast<const uint4*>(src + (r0 + r) * K) + kc);
-    *reinterpret_cast<uint4*>(dst + (size_t)c * 16) = v;
-  }
+// One contiguous piece (a multiple of 16 bytes) global -> shared, completion
+// counted in bytes on bar, in copies of at most 32 KB.
+__device__ __forceinline__ void bulk_load(unsigned char* dst, const void* src, uint32_t bytes,
+                                          uint64_t* bar) {
+  for (uint32_t o = 0; o < bytes; o += 32768u)
+    bulk_g2s(dst + o, reinterpret_cast<const unsigned char*>(src) + o, min(32768u, bytes - o), bar);
 }
+// shared -> global; the issuing thread's commit group
+__device__ __forceinline__ void bulk_store(void* dst, const unsigned char* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// the shared memory of this thread's committed stores has been read / the
+// stores are complete
+__device__ __forceinline__ void bulk_wait_read() {
+  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+}
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
 // The whole network for 128-row tiles: Y[M][3] = W3 relu(W2 relu(W1 x + b1) +
@@ -96,7 +100,7 @@ __device__ __forceinline__ void load_canon(unsigned char* dst, const uint16_t* _
 // ---------------------------------------------------------------------------
 constexpr uint32_t kMlpSmemW1 = 256 * 128 * 2, kMlpSmemW2 = 256 * 256 * 2, kMlpSmemX = 128 * 128 * 2;
 constexpr int kMlpThreads = 448;  // 14 warps (roles above)
-constexpr uint32_t kMlpBars = 14;  // 8-byte slots: 12 mbarriers, the TMEM base, padding
+constexpr uint32_t kMlpBars = 16;  // 8-byte slots: 14 mbarriers, the TMEM base, padding
 constexpr uint32_t kMlpSmemBias = (128 + 512) * sizeof(float);  // b1[0 .. 127], w3 rows 0 and 1
 constexpr size_t kMlpSmem = (size_t)kMlpSmemW1 + kMlpSmemW2 + kMlpSmemX + 8 * kMlpBars + kMlpSmemBias;
 static_assert(kMlpSmem <= 227 * 1024, "fused network shared memory");
@@ -343,7 +347,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
   uint64_t* bar_xr = bars + 9;    // the next tile's X is in shared memory
   uint64_t* bar_ya = bars + 10;   // the first epilogue-2 group wrote its part of Y
   uint64_t* bar_fin = bars + 11;  // every product issued has completed
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 12);
+  uint64_t* bar_w = bars + 12;    // W1 is in shared memory
+  uint64_t* bar_w2 = bars + 13;   // W2
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 14);
   float* sb1 = reinterpret_cast<float*>(bars + kMlpBars);  // b1[0 .. 127]
   float* sw3 = sb1 + 128;                                   // w3 rows 0 and 1
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
@@ -362,12 +368,16 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
     mbar_init(bar_xr, 1u);
     mbar_init(bar_ya, 4u);
     mbar_init(bar_fin, 1u);
+    mbar_init(bar_w, 1u);
+    mbar_init(bar_w2, 1u);
     fence_mbar_init();
+    mbar_arrive_expect_tx(bar_w, kMlpSmemW1);
+    bulk_load(sW1, W1, kMlpSmemW1, bar_w);
+    mbar_arrive_expect_tx(bar_w2, kMlpSmemW2);
+    bulk_load(sW2, W2, kMlpSmemW2, bar_w2);
   }
   if (tid < 128) sb1[tid] = __ldg(b1 + tid);
   for (int i = tid; i < 512; i += kMlpThreads) sw3[i] = __ldg(w3 + i);
-  load_canon(sW1, W1, 0, 256, 256, 128);
-  load_canon(sW2, W2, 0, 256, 256, 256);
   const long long ntiles = (M + TM - 1) / TM;
   fence_proxy_async();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -417,6 +427,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
       int it = 0;
       for (long long tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ph ^= 1u, ++it) {
         wait(bar_xr, ph);                    // this tile's X
+        if (it == 0) wait(bar_w, 0u);
         if (it > 0) wait(bar_k0, ph ^ 1u);  // the previous tile's layer 2 done with Q0
         layer1(0);
         mma_commit(bar_l1a);
@@ -424,6 +435,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
         layer1(1);
         mma_commit(bar_l1b);
         wait(bar_e1a, ph);
+        if (it == 0) wait(bar_w2, 0u);
         if (it > 0) wait(bar_e2a, ph ^ 1u);  // the previous tile's epilogue 2 has read Q2
         layer2(0, 0);
         if (it > 0) wait(bar_e2b, ph ^ 1u);  // ... and Q3
@@ -526,7 +538,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) tc_mlp_kernel(
 // added in a fixed order, and Adam).  They took about twenty launches (GEMMs
 // that each staged their operands anew and stored every activation a second
 // time transposed, then transposes and reductions) and 200 us at 4096 rows;
-// now TRAIN_US us.
+// now 29 us (128 -> 23 at 64 rows, 280 -> 50 at 16384).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kMajorMnA = 1u << 15, kMajorMnB = 1u << 16;  // operand stored MN-major
 
@@ -535,38 +547,28 @@ constexpr uint32_t idesc_n(int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TM >> 4) << 24);
 }
 
-// rows [r0, r0 + R) x columns [col0, col0 + C) of a row-major BF16 matrix (row
-// pitch ld) into the canonical layout by cp.async; rows at or beyond nrows
-// become zero.  Read as an operand whose K runs along the columns this is
-// K-major (leading offset 128 bytes, stride offset 16 C); read with K along
-// the rows it is MN-major: 8 rows x 16 bytes are a core matrix either way,
-// and the stride offset (next 8 columns) is 128 bytes, the leading offset
-// (next 8 rows) 16 C.
-__device__ __forceinline__ void load_canon_async(unsigned char* dst, const uint16_t* __restrict__ src,
-                                                 long long ld, long long r0, int R, long long nrows,
-                                                 int col0, int C) {
-  const int kc8 = C / 8;
-  const int chunks = R * kc8;
-  for (int c = threadIdx.x; c < chunks; c += blockDim.x) {
-    const int rr = c & 7, kc = (c >> 3) % kc8, rg = (c >> 3) / kc8;
-    const long long r = r0 + rg * 8 + rr;
-    const bool in = r < nrows;
-    const uint16_t* g = src + (in ? r : 0) * ld + col0 + kc * 8;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst + (size_t)c * 16)),
-                 "l"(g), "r"(in ? 16 : 0)
-                 : "memory");
-  }
+// Row buffers (A1, A2, D1, D2 and the rows' inputs XB) are kept in the image
+// that both the products and the bulk copies take: per tile of 128 rows, blocks
+// of 64 columns, in a block 128 bytes a row with the row's eight 16-byte pieces
+// permuted by r % 8 (128-byte swizzle).  Read along the columns a block is a
+// K-major operand, read along the rows an MN-major one: rows in groups of 8 are
+// 1024 bytes apart (stride offset), 64-column blocks a block apart (leading
+// offset).  A warp's 16-byte pieces of 32 rows fall on all banks.
+constexpr uint32_t kBlock = TM * 128;  // bytes of a block of 64 columns of a tile
+constexpr uint64_t kSwizzle128 = (uint64_t)2 << 61;  // descriptor: 128-byte swizzle
+__device__ __forceinline__ uint32_t piece(int r, int c8) {  // columns 8 c8 .. of row r
+  return (uint32_t)(c8 >> 3) * kBlock + (uint32_t)r * 128u + (uint32_t)((c8 ^ r) & 7) * 16u;
 }
 
 __device__ __forceinline__ float bf_lo(uint32_t p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t p) { return __uint_as_float(p & 0xFFFF0000u); }
 
-// 16 words (32 BF16 values) of one row, 64 contiguous bytes
-__device__ __forceinline__ void store_row32(uint16_t* dst, const uint32_t* pk) {
-  uint4* d = reinterpret_cast<uint4*>(dst);
+// 16 words (32 BF16 values, columns c .. c + 31) of row r into a tile image
+__device__ __forceinline__ void put_row32(unsigned char* tile, int r, int c, const uint32_t* pk) {
 #pragma unroll
   for (int q = 0; q < 4; ++q)
-    d[q] = make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
+    *reinterpret_cast<uint4*>(tile + piece(r, (c >> 3) + q)) =
+        make_uint4(pk[4 * q], pk[4 * q + 1], pk[4 * q + 2], pk[4 * q + 3]);
 }
 
 // relu(v + b) of 32 columns as BF16 pairs
@@ -580,7 +582,7 @@ __device__ __forceinline__ void relu_pack32(const uint32_t* v, const float* b, u
 }
 
 constexpr int kTrThreads = 256;
-constexpr size_t kTrSmem = (size_t)kMlpSmemW1 + kMlpSmemW2 + kMlpSmemX + 64;
+constexpr size_t kTrSmem = (size_t)kMlpSmemW2 + kMlpSmemX + kMlpSmemW1 + 64;
 
 // Forward, loss and data gradients of rows [128 blockIdx.x, ...): X, W1 and W2
 // in shared memory; tensor memory columns 0..255 hold the layer-1 sums, then A1
@@ -588,30 +590,31 @@ constexpr size_t kTrSmem = (size_t)kMlpSmemW1 + kMlpSmemW2 + kMlpSmemX + 64;
 // 256..511 the layer-2 sums, then those of dH1.  dH1 = dH2 W2 reads W2 from the
 // same shared copy as layer 2, as an MN-major operand.  Warp w holds the rows
 // 32 (w % 4) .. and the column half w / 4; the output layer runs one row per
-// thread of warps 0-3 while warps 4-7 store A2.  With one tile per CTA the
-// chain of load, four products and four epilogues bounds it, not their rates.
+// thread of warps 0-3 while warps 4-7 store A2.  Rows leave through a tile
+// image in the place of W1 by bulk copies.  With one tile per CTA the chain of
+// load, four products and four epilogues bounds it, not their rates: of 28 us
+// at first, 7 went to 16-byte cp.async of the operands (bulk copies now) and 12
+// to row stores that spread every warp's 16-byte pieces over 32 lines.
 __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
     const uint16_t* __restrict__ X, const float* __restrict__ T, long long n,
     const uint16_t* __restrict__ W1, const uint16_t* __restrict__ W2, const float* __restrict__ b1,
-    const float* __restrict__ b2, const float* __restrict__ w3, uint16_t* __restrict__ A1,
-    uint16_t* __restrict__ A2, uint16_t* __restrict__ D1, uint16_t* __restrict__ D2,
-    float* __restrict__ DY, float* __restrict__ wloss, unsigned int* __restrict__ status) {
+    const float* __restrict__ b2, const float* __restrict__ w3, TrainBuffers B,
+    float* __restrict__ wloss, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char dsm[];
-  unsigned char* sW1 = dsm;
-  unsigned char* sW2 = dsm + kMlpSmemW1;
-  unsigned char* sX = sW2 + kMlpSmemW2;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sX + kMlpSmemX);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
+  unsigned char* sW2 = dsm;
+  unsigned char* sX = dsm + kMlpSmemW2;
+  unsigned char* sW1 = sX + kMlpSmemX;
+  unsigned char* sT = sW1;  // tile image of the rows on their way out, after layer 1
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sW1 + kMlpSmemW1);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 5);
   // in the place of X once layer 1 has read it: w3 (3 x 256) and b3, b2, dY
   float* s3 = reinterpret_cast<float*>(sX);
   float* sb2 = s3 + 772;
   float* sdy = sb2 + 256;
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
   const int wq = w & 3, half = w >> 2;
-  const long long r0 = (long long)blockIdx.x * TM;
   const int rl = 32 * wq + lane;        // this thread's row of the tile
-  const long long row = r0 + rl;
-  const bool live = row < n;
+  const long long row = (long long)blockIdx.x * TM + rl;
 
   if (w == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -621,16 +624,27 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i) mbar_init(bars + i, 1u);
+    for (int i = 0; i < 5; ++i) mbar_init(bars + i, 1u);
     fence_mbar_init();
   }
   pdl_wait();  // the weights of the previous step
-  load_canon_async(sX, X, 128, r0, TM, n, 0, 128);
-  load_canon_async(sW1, W1, 128, 0, 256, 256, 0, 128);
+  pdl_trigger();
+  if (tid == 0) {
+    mbar_arrive_expect_tx(bars + 3, kMlpSmemW1);
+    bulk_load(sW1, W1, kMlpSmemW1, bars + 3);
+    mbar_arrive_expect_tx(bars + 4, kMlpSmemW2);
+    bulk_load(sW2, W2, kMlpSmemW2, bars + 4);
+  }
+  for (int c = tid; c < TM * 16; c += kTrThreads) {  // 16-byte piece c % 16 of row c / 16
+    const int r = c >> 4;
+    const long long rr = (long long)blockIdx.x * TM + r;
+    const bool in = rr < n;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(sX + piece(r, c & 15))),
+                 "l"(X + (in ? rr : 0) * 128 + (c & 15) * 8), "r"(in ? 16 : 0)
+                 : "memory");
+  }
   cp_async_commit();
-  load_canon_async(sW2, W2, 256, 0, 256, 256, 0, 256);
-  cp_async_commit();
-  cp_async_wait<1>();
+  cp_async_wait<0>();
   fence_proxy_async();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -645,27 +659,43 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
   // the warps' accesses to shared and tensor memory before the next products
   auto join = [&]() {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-    fence_proxy_async();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   };
   // column of K step kb (16 values, 8 columns of pairs) of the packed operand
   auto packed = [&](int kb) { return tmem + (uint32_t)(kb < 8 ? 8 * kb : 128 + 8 * (kb - 8)); };
+  // this warp's rows of blocks b0 .. b1 - 1 of the image to their place in M
+  auto send = [&](uint16_t* M, int b0, int b1) {
+    fence_proxy_async();
+    __syncwarp();
+    if (lane < b1 - b0) {
+      const uint32_t off = (uint32_t)(b0 + lane) * kBlock + (uint32_t)wq * 32u * 128u;
+      bulk_store(reinterpret_cast<unsigned char*>(M) + (size_t)blockIdx.x * 4 * kBlock + off, sT + off,
+                 32u * 128u);
+    }
+    bulk_commit();
+  };
 
   if (tid == 0) {  // layer 1: X W1^T
-    const uint64_t xd = smem_desc(smem_u32(sX), 128u, 16u * 128u);
+    wait(bars + 3);
+    const uint64_t xd = smem_desc(smem_u32(sX), 16u, 1024u) | kSwizzle128;
     const uint64_t wd = smem_desc(smem_u32(sW1), 128u, 16u * 128u);
 #pragma unroll
     for (int kb = 0; kb < 8; ++kb)
-      mma_ss_i(tmem, xd + (uint64_t)(kb * 16), wd + (uint64_t)(kb * 16), idesc_n(256), kb > 0);
+      mma_ss_i(tmem, xd + (uint64_t)((kb >> 2) * (int)(kBlock >> 4) + (kb & 3) * 2),
+               wd + (uint64_t)(kb * 16), idesc_n(256), kb > 0);
     mma_commit(bars);
+    bulk_store(reinterpret_cast<unsigned char*>(B.XB) + (size_t)blockIdx.x * 2 * kBlock, sX, 2 * kBlock);
+    bulk_commit();
+    bulk_wait_read();
   }
   wait(bars);
+  __syncthreads();
   for (int i = tid; i < 771; i += kTrThreads) s3[i] = __ldg(w3 + i);  // w3 and b3 follow each other
   sb2[tid] = __ldg(b2 + tid);
 
-  // A1 = relu(. + b1): packed into tensor memory and stored; m1: A1 > 0
+  // A1 = relu(. + b1): packed into tensor memory and sent; m1: A1 > 0
   uint32_t m1[4];
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
@@ -678,18 +708,22 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
     for (int q = 0; q < 16; ++q)
       m |= ((pk[q] & 0xFFFFu) ? 1u : 0u) << (2 * q) | ((pk[q] >> 16) ? 2u : 0u) << (2 * q);
     m1[j] = m;
-    if (live) store_row32(A1 + row * 256 + 128 * half + 32 * j, pk);
+    put_row32(sT, rl, 128 * half + 32 * j, pk);
   }
-  cp_async_wait<0>();  // W2
   join();
   if (tid == 0) {  // layer 2: A1 W2^T
+    wait(bars + 4);
     const uint64_t wd = smem_desc(smem_u32(sW2), 128u, 32u * 128u);
 #pragma unroll
     for (int kb = 0; kb < 16; ++kb)
       mma_ts_i(tmem + 256u, packed(kb), wd + (uint64_t)(kb * 16), idesc_n(256), kb > 0);
     mma_commit(bars + 1);
   }
+  __syncwarp();
+  send(B.A1, 2 * half, 2 * half + 2);
   wait(bars + 1);
+  bulk_wait_read();
+  __syncthreads();  // the image is free again
 
   if (half == 0) {
     // y = A2 w3^T + b3 in ascending order of the hidden units, dY, loss
@@ -712,16 +746,16 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
       }
     }
     float lsum = 0.f, y0 = 0.f, y1 = 0.f, y2 = 0.f;
-    if (live) {
+    if (row < n) {
       const float d0 = o0 - T[3 * row], d1 = o1 - T[3 * row + 1], d2 = o2 - T[3 * row + 2];
       lsum += d0 * d0 + d1 * d1 + d2 * d2;
       const float sc = 2.f / (float)n;
       y0 = sc * d0;
       y1 = sc * d1;
       y2 = sc * d2;
-      DY[3 * row] = y0;
-      DY[3 * row + 1] = y1;
-      DY[3 * row + 2] = y2;
+      B.DY[3 * row] = y0;
+      B.DY[3 * row + 1] = y1;
+      B.DY[3 * row + 2] = y2;
     }
     sdy[3 * rl] = y0;
     sdy[3 * rl + 1] = y1;
@@ -734,10 +768,12 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
       uint32_t v[32], pk[16];
       tmem_ld32(lanes + 256u + (uint32_t)(32 * j), v);
       relu_pack32(v, sb2 + 32 * j, pk);
-      if (live) store_row32(A2 + row * 256 + 32 * j, pk);
+      put_row32(sT, rl, 32 * j, pk);
     }
+    send(B.A2, 0, 4);
+    bulk_wait_read();
   }
-  __syncthreads();  // dY
+  __syncthreads();  // dY; the image is free again
 
   // dH2 = (dY w3) where A2 > 0
   {
@@ -749,19 +785,24 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
       tmem_ld32(lanes + 256u + (uint32_t)k0, v);
       relu_pack32(v, sb2 + k0, pk);
 #pragma unroll
-      for (int q = 0; q < 16; ++q) {
+      for (int q = 0; q < 16; q += 2) {
         const int k = k0 + 2 * q;
-        const float2 u0 = *reinterpret_cast<const float2*>(s3 + k);
-        const float2 u1 = *reinterpret_cast<const float2*>(s3 + 256 + k);
-        const float2 u2 = *reinterpret_cast<const float2*>(s3 + 512 + k);
-        float g0 = y0 * u0.x + y1 * u1.x + y2 * u2.x;
-        float g1 = y0 * u0.y + y1 * u1.y + y2 * u2.y;
+        const float4 u0 = *reinterpret_cast<const float4*>(s3 + k);
+        const float4 u1 = *reinterpret_cast<const float4*>(s3 + 256 + k);
+        const float4 u2 = *reinterpret_cast<const float4*>(s3 + 512 + k);
+        float g0 = fmaf(y2, u2.x, fmaf(y0, u0.x, __fmul_rn(y1, u1.x)));
+        float g1 = fmaf(y2, u2.y, fmaf(y0, u0.y, __fmul_rn(y1, u1.y)));
+        float g2 = fmaf(y2, u2.z, fmaf(y0, u0.z, __fmul_rn(y1, u1.z)));
+        float g3 = fmaf(y2, u2.w, fmaf(y0, u0.w, __fmul_rn(y1, u1.w)));
         if (bf_lo(pk[q]) <= 0.f) g0 = 0.f;
         if (bf_hi(pk[q]) <= 0.f) g1 = 0.f;
+        if (bf_lo(pk[q + 1]) <= 0.f) g2 = 0.f;
+        if (bf_hi(pk[q + 1]) <= 0.f) g3 = 0.f;
         pk[q] = bf16x2_bits(g0, g1);
+        pk[q + 1] = bf16x2_bits(g2, g3);
       }
       tmem_st16(lanes + (uint32_t)(128 * half + 16 * j), pk);
-      if (live) store_row32(D2 + row * 256 + k0, pk);
+      put_row32(sT, rl, k0, pk);
     }
   }
   join();
@@ -772,7 +813,11 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
       mma_ts_i(tmem + 256u, packed(kb), wd + (uint64_t)(kb * 512), idesc_n(256) | kMajorMnB, kb > 0);
     mma_commit(bars + 2);
   }
+  __syncwarp();
+  send(B.D2, 2 * half, 2 * half + 2);
   wait(bars + 2);
+  bulk_wait_read();
+  __syncwarp();
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     uint32_t v[32], pk[16];
@@ -781,8 +826,10 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
     for (int q = 0; q < 16; ++q)
       pk[q] = bf16x2_bits((m1[j] >> (2 * q)) & 1u ? __uint_as_float(v[2 * q]) : 0.f,
                           (m1[j] >> (2 * q)) & 2u ? __uint_as_float(v[2 * q + 1]) : 0.f);
-    if (live) store_row32(D1 + row * 256 + 128 * half + 32 * j, pk);
+    put_row32(sT, rl, 128 * half + 32 * j, pk);
   }
+  send(B.D1, 2 * half, 2 * half + 2);
+  bulk_wait();
   if (tmo) atomicOr(status, 1u);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -791,22 +838,26 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
                  : "memory");
 }
 
-// Gradients.  Blocks 4 s .. 4 s + 3 (s < splits): split s of the batch for
-// dW2[o][k] = sum_m dH2[m][o] A1[m][k] (o < 128, o >= 128) and dW1[o][i] =
-// sum_m dH1[m][o] X[m][i]; both operands are MN-major in the rows' own order,
-// 64 rows a chunk through a ring of four stages, FP32 partials per split.  The
-// other blocks: one chunk of 64 rows each, in ascending row order, of dW3 and
-// db3 (width kPart3), db2 and db1.
+// Gradients.  The first splits x parts blocks: split s of the batch for
+// dW2[o][k] = sum_m dH2[m][o] A1[m][k] and dW1[o][i] = sum_m dH1[m][o] X[m][i];
+// both operands are MN-major images, 64 rows a chunk through a ring of four
+// stages, FP32 partials per split.  A block takes 128 outputs o and, with at
+// least kManySplits splits, all columns (four parts), else 64 of them (twelve):
+// a batch whose chunks have no larger divisor is one long sum, which more blocks
+// shorten by sharing its columns without touching its order.  The other blocks:
+// one chunk of 64 rows each, in ascending row order, of dW3 and db3 (width
+// kPart3), db2 and db1.
 constexpr int kGrThreads = 256, kGrStages = 4, kGrRows = 64;
-constexpr uint32_t kGrA = kGrRows * 128 * 2, kGrB = kGrRows * 256 * 2;
-constexpr size_t kGrSmem = (size_t)kGrStages * (kGrA + kGrB) + 64;
+constexpr uint32_t kGrBlock = kGrRows * 128;  // bytes of 64 rows of a block
+constexpr uint32_t kGrStage = 6 * kGrBlock;   // A: 128 columns, B: up to 256
+constexpr size_t kGrSmem = (size_t)kGrStages * kGrStage + 128;
 constexpr int kPart3 = 771;
+constexpr int kManySplits = 8;
 
 struct GradArgs {
-  const uint16_t *X, *A1, *A2, *D1, *D2;
-  const float* DY;
+  TrainBuffers B;
   long long n;
-  int splits;
+  int splits, parts;
   float *part1, *part2;   // [splits][256][128], [splits][256][256]
   float *p3, *pb2, *pb1;  // per 64-row chunk: [kPart3], [256], [256]
   unsigned int* status;
@@ -815,17 +866,19 @@ struct GradArgs {
 __device__ __forceinline__ void grad_chunk(const GradArgs& a, long long chunk, float* sdy) {
   const long long m0 = chunk * kGrRows;
   const int nr = (int)(a.n - m0 < kGrRows ? a.n - m0 : kGrRows);
-  for (int i = threadIdx.x; i < 3 * nr; i += kGrThreads) sdy[i] = a.DY[3 * m0 + i];
+  for (int i = threadIdx.x; i < 3 * nr; i += kGrThreads) sdy[i] = a.B.DY[3 * m0 + i];
   __syncthreads();
   const int c = threadIdx.x & 127;  // columns 2 c, 2 c + 1
+  const size_t first = (size_t)(m0 / TM) * 4 * kBlock + (size_t)(m0 % TM) * 128;
   auto col = [&](const uint16_t* M, int r) {
-    return __ldg(reinterpret_cast<const uint32_t*>(M + (m0 + r) * 256) + c);
+    return __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(M) + first +
+                                                   piece(r, c >> 2)) + (c & 3));
   };
   if (threadIdx.x < 128) {
     float s0 = 0.f, s1 = 0.f, t0 = 0.f, t1 = 0.f;
 #pragma unroll 16
     for (int r = 0; r < nr; ++r) {
-      const uint32_t u = col(a.D2, r), v = col(a.D1, r);
+      const uint32_t u = col(a.B.D2, r), v = col(a.B.D1, r);
       s0 += bf_lo(u);
       s1 += bf_hi(u);
       t0 += bf_lo(v);
@@ -837,7 +890,7 @@ __device__ __forceinline__ void grad_chunk(const GradArgs& a, long long chunk, f
     float s[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll 16
     for (int r = 0; r < nr; ++r) {
-      const uint32_t u = col(a.A2, r);
+      const uint32_t u = col(a.B.A2, r);
 #pragma unroll
       for (int o = 0; o < 3; ++o) {
         s[2 * o] = fmaf(sdy[3 * r + o], bf_lo(u), s[2 * o]);
@@ -858,21 +911,29 @@ __device__ __forceinline__ void grad_chunk(const GradArgs& a, long long chunk, f
   }
 }
 
-__global__ void __launch_bounds__(kGrThreads, 1) train_grads_kernel(GradArgs a) {
+__global__ void __launch_bounds__(kGrThreads, 1) train_grads_kernel(const __grid_constant__ GradArgs a) {
   extern __shared__ __align__(1024) unsigned char dsm[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(dsm + kGrStages * (kGrA + kGrB));
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + kGrStages);
+  uint64_t* full = reinterpret_cast<uint64_t*>(dsm + kGrStages * kGrStage);
+  uint64_t* empty = full + kGrStages;
+  uint64_t* fin = empty + kGrStages;
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(fin + 1);
   const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-  if ((int)blockIdx.x >= 4 * a.splits) {
+  if ((int)blockIdx.x >= a.parts * a.splits) {
     pdl_wait();
-    grad_chunk(a, (long long)blockIdx.x - 4 * a.splits, reinterpret_cast<float*>(dsm));
+    pdl_trigger();
+    grad_chunk(a, (long long)blockIdx.x - a.parts * a.splits, reinterpret_cast<float*>(dsm));
     return;
   }
-  const int split = blockIdx.x >> 2, o0 = (blockIdx.x & 1) * 128;
-  const bool second = (blockIdx.x & 2) == 0;  // dW2, else dW1
-  const int N = second ? 256 : 128;
-  const uint16_t* A = second ? a.D2 : a.D1;
-  const uint16_t* B = second ? a.A1 : a.X;
+  // two thirds of a split's blocks for dW2 (256 columns), the others for dW1
+  // (128); four parts: two and two
+  const int split = blockIdx.x / a.parts, part = blockIdx.x % a.parts;
+  const bool whole = a.parts == 4;
+  const bool second = part < (whole ? 2 : 8);
+  const int o0 = (part & 1) * 128, N = second ? 256 : 128;
+  const int cols = whole ? N : 64, n0 = whole ? 0 : ((second ? part : part - 8) >> 1) * 64;
+  const int nb = cols / 64;
+  const unsigned char* A = reinterpret_cast<const unsigned char*>(second ? a.B.D2 : a.B.D1);
+  const unsigned char* Bm = reinterpret_cast<const unsigned char*>(second ? a.B.A1 : a.B.XB);
   const long long nch = (a.n + kGrRows - 1) / kGrRows;
   const long long c0 = nch * split / a.splits, c1 = nch * (split + 1) / a.splits;
   const int nc = (int)(c1 - c0);
@@ -885,52 +946,56 @@ __global__ void __launch_bounds__(kGrThreads, 1) train_grads_kernel(GradArgs a) 
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 0) {
-    for (int i = 0; i < kGrStages; ++i) mbar_init(bars + i, 1u);
+    for (int i = 0; i < 2 * kGrStages + 1; ++i) mbar_init(full + i, 1u);
     fence_mbar_init();
   }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *tslot;
   pdl_wait();
+  pdl_trigger();
   bool tmo = false;
-  auto stage = [&](int i) { return dsm + (size_t)(i % kGrStages) * (kGrA + kGrB); };
-  auto fill = [&](int i) {  // chunk i of the split (an empty group past the end)
-    if (i < nc) {
-      load_canon_async(stage(i), A, 256, (c0 + i) * kGrRows, kGrRows, a.n, o0, 128);
-      load_canon_async(stage(i) + kGrA, B, N, (c0 + i) * kGrRows, kGrRows, a.n, 0, N);
-    }
-    cp_async_commit();
-  };
-  // the products of chunk i have read its stage
-  auto drained = [&](int i) {
-    if (!tmo && !mbar_wait(bars + i % kGrStages, (uint32_t)(i / kGrStages) & 1u)) tmo = true;
-  };
-  for (int i = 0; i < kGrStages - 1; ++i) fill(i);
-  uint32_t tmem = 0;
-  for (int i = 0; i < nc; ++i) {
-    if (i > 0) drained(i - 1);
-    fill(i + kGrStages - 1);
-    cp_async_wait<kGrStages - 1>();  // chunk i has landed
-    fence_proxy_async();
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (!tmo && !mbar_wait(bar, parity)) tmo = true;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    tmem = *tslot;
-    if (tid == 0) {
-      const uint64_t ad = smem_desc(smem_u32(stage(i)), 16u * 128u, 128u);
-      const uint64_t bd = smem_desc(smem_u32(stage(i) + kGrA), (uint32_t)(N / 8) * 128u, 128u);
-      const uint32_t id = idesc_n(N) | kMajorMnA | kMajorMnB;
+  };
+  if (tid == 0) {
+    // blocks of the chunk's 64 rows: two of A from column o0, nb of B
+    for (int i = 0; i < nc; ++i) {
+      const int sl = i % kGrStages;
+      if (i >= kGrStages) wait(empty + sl, (uint32_t)(i / kGrStages - 1) & 1u);
+      const long long m0 = (c0 + i) * kGrRows;
+      const size_t rows = (size_t)(m0 % TM) * 128;
+      const unsigned char* as = A + (size_t)(m0 / TM) * 4 * kBlock + (size_t)(o0 / 64) * kBlock + rows;
+      const unsigned char* bs = Bm + ((size_t)(m0 / TM) * (N / 64) + n0 / 64) * kBlock + rows;
+      unsigned char* d = dsm + (size_t)sl * kGrStage;
+      mbar_arrive_expect_tx(full + sl, (uint32_t)(2 + nb) * kGrBlock);
+      for (int b = 0; b < 2; ++b) bulk_g2s(d + b * kGrBlock, as + (size_t)b * kBlock, kGrBlock, full + sl);
+      for (int b = 0; b < nb; ++b)
+        bulk_g2s(d + (2 + b) * kGrBlock, bs + (size_t)b * kBlock, kGrBlock, full + sl);
+    }
+  } else if (tid == 32) {
+    const uint32_t id = idesc_n(cols) | kMajorMnA | kMajorMnB;
+    for (int i = 0; i < nc; ++i) {
+      const int sl = i % kGrStages;
+      wait(full + sl, (uint32_t)(i / kGrStages) & 1u);
+      const uint32_t d = smem_u32(dsm + (size_t)sl * kGrStage);
+      const uint64_t ad = smem_desc(d, kGrBlock, 1024u) | kSwizzle128;
+      const uint64_t bd = smem_desc(d + 2 * kGrBlock, kGrBlock, 1024u) | kSwizzle128;
 #pragma unroll
       for (int kb = 0; kb < kGrRows / 16; ++kb)  // 16 rows: two 8-row groups
-        mma_ss_i(tmem, ad + (uint64_t)(kb * 256), bd + (uint64_t)(kb * (N / 8) * 16), id,
-                 (i > 0 || kb > 0) ? 1u : 0u);
-      mma_commit(bars + i % kGrStages);
+        mma_ss_i(tmem, ad + (uint64_t)(kb * 128), bd + (uint64_t)(kb * 128), id, (i > 0 || kb > 0) ? 1u : 0u);
+      mma_commit(empty + sl);
     }
+    mma_commit(fin);
   }
-  cp_async_wait<0>();
-  if (nc > 0) drained(nc - 1);
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  __syncwarp();
+  wait(fin, 0u);
   // rows o0 + 32 (w % 4) + lane, column half w / 4
   const int row = o0 + 32 * (w & 3) + lane;
-  float* out = (second ? a.part2 : a.part1) + ((long long)split * 256 + row) * N;
-  for (int j = (w >> 2) * (N / 2); j < ((w >> 2) + 1) * (N / 2); j += 32) {
+  float* out = (second ? a.part2 : a.part1) + ((long long)split * 256 + row) * N + n0;
+  for (int j = (w >> 2) * (cols / 2); j < ((w >> 2) + 1) * (cols / 2); j += 32) {
     uint32_t v[32];
     tmem_ld32(tmem + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)j, v);
 #pragma unroll
@@ -959,8 +1024,10 @@ __device__ __forceinline__ float sum_in_order(const float* __restrict__ part, lo
 // Gradient i from its partials in a fixed order and (adam) its Adam step,
 // refreshing the BF16 weights; the last block adds the loss: the warps' sums of
 // 256 rows in order, divided by n, then those in order.
-__global__ void __launch_bounds__(256) train_update_kernel(GradArgs a, TrainState t) {
+__global__ void __launch_bounds__(256) train_update_kernel(const __grid_constant__ GradArgs a,
+                                                           const __grid_constant__ TrainState t) {
   pdl_wait();
+  pdl_trigger();
   const long long chunks = (a.n + kGrRows - 1) / kGrRows;
   const int i = (int)(blockIdx.x * 256u + threadIdx.x);
   if (blockIdx.x == gridDim.x - 1) {
@@ -986,27 +1053,28 @@ __global__ void __launch_bounds__(256) train_update_kernel(GradArgs a, TrainStat
   else g = sum_in_order(a.p3 + (i - oW3), chunks, kPart3);
   t.G[i] = g;
   if (!t.adam) return;
-  const float m = t.beta1 * t.M[i] + (1.f - t.beta1) * g;
-  const float v = t.beta2 * t.V[i] + (1.f - t.beta2) * g * g;
-  t.M[i] = m;
-  t.V[i] = v;
-  const float p = t.P[i] - t.lr * (m / t.c1) / (sqrtf(v / t.c2) + t.eps);
+  const float p = adam_value(t.P[i], g, t.M[i], t.V[i], t.lr, t.beta1, t.beta2, t.eps, t.c1, t.c2);
   t.P[i] = p;
-  const __nv_bfloat16 b = __float2bfloat16_rn(p);
-  if (i < oB1) t.w1b[i] = *reinterpret_cast<const uint16_t*>(&b);
-  else if (i >= oW2 && i < oB2) t.w2b[i - oW2] = *reinterpret_cast<const uint16_t*>(&b);
+  const __nv_bfloat16 bf = __float2bfloat16_rn(p);
+  const uint16_t b = *reinterpret_cast<const uint16_t*>(&bf);
+  if (i < oB1) {
+    t.w1b[i] = b;
+    t.w1c[canon_index(i, 128)] = b;
+  } else if (i >= oW2 && i < oB2) {
+    t.w2b[i - oW2] = b;
+    t.w2c[canon_index(i - oW2, 256)] = b;
+  }
 }
 
 }  // namespace
 
-// Splits of a batch of k64 chunks of 64 rows for the weight gradients: a
-// divisor of k64 up to kTrainSplits (equal splits) unless it has none of at
-// least half that, then kTrainSplits uneven ones (4544 rows are 71 chunks).
+// Splits of a batch of k64 chunks of 64 rows for the weight gradients: its
+// largest divisor up to kTrainSplits (equal splits, so that the order of a sum
+// depends on the batch alone).
 int train_splits(long long k64) {
-  if (k64 <= kTrainSplits) return (int)k64;
   int s = kTrainSplits;
   while (k64 % s) --s;
-  return s >= kTrainSplits / 2 ? s : kTrainSplits;
+  return s;
 }
 
 int tc_train(const uint16_t* X, const float* T, long long n, const TrainBuffers& B, const TrainState& t,
@@ -1025,29 +1093,24 @@ int tc_train(const uint16_t* X, const float* T, long long n, const TrainBuffers&
     attr = true;
   }
   const long long tiles = (n + TM - 1) / TM, chunks = (n + kGrRows - 1) / kGrRows;
+  const float* P = t.P;
   cudaError_t e = launch_dependent(train_rows_kernel, dim3((unsigned)tiles), dim3(kTrThreads), kTrSmem,
-                                   st, X, T, n, (const uint16_t*)t.w1b, (const uint16_t*)t.w2b,
-                                   (const float*)t.P + 256 * 128,
-                                   (const float*)t.P + 256 * 128 + 256 + 256 * 256,
-                                   (const float*)t.P + 256 * 128 + 512 + 256 * 256, B.A1, B.A2, B.D1,
-                                   B.D2, B.DY, t.wloss, status);
+                                   st, X, T, n, (const uint16_t*)t.w1c, (const uint16_t*)t.w2c,
+                                   P + 256 * 128, P + 256 * 128 + 256 + 256 * 256,
+                                   P + 256 * 128 + 512 + 256 * 256, B, t.wloss, status);
   if (e != cudaSuccess) return check_cuda(e, "train_rows_kernel launch");
   GradArgs a;
-  a.X = X;
-  a.A1 = B.A1;
-  a.A2 = B.A2;
-  a.D1 = B.D1;
-  a.D2 = B.D2;
-  a.DY = B.DY;
+  a.B = B;
   a.n = n;
   a.splits = train_splits(chunks);
+  a.parts = a.splits >= kManySplits ? 4 : 12;
   a.part1 = B.part;
   a.part2 = B.part + (size_t)kTrainSplits * 256 * 128;
   a.p3 = B.chunk;
   a.pb2 = B.chunk + (size_t)chunks * (kPart3 + 1);
   a.pb1 = a.pb2 + (size_t)chunks * 256;
   a.status = status;
-  e = launch_dependent(train_grads_kernel, dim3((unsigned)(4 * a.splits + chunks)), dim3(kGrThreads),
+  e = launch_dependent(train_grads_kernel, dim3((unsigned)(a.parts * a.splits + chunks)), dim3(kGrThreads),
                        kGrSmem, st, a);
   if (e != cudaSuccess) return check_cuda(e, "train_grads_kernel launch");
   e = launch_dependent(train_update_kernel, dim3((QTV_LOCATOR_PARAMS + 255) / 256 + 1), dim3(256), 0, st,

@@ -400,28 +400,46 @@ int locator_localize(qtv_handle h, const FaceGeo& geo, const uint64_t* face_ids,
 int locator_prepare(qtv_handle h, uint64_t n, uint64_t* generation);
 
 // One training step of the learned locator on tcgen05 (locator_tc.cu): rows X
-// [n][128] BF16, targets T [n][3].  Row buffers [n][256] BF16, DY [n][3]; part
-// holds kTrainSplits x (256 x 128 + 256 x 256) and chunk 1284 values per 64
-// rows; wloss 4 per 128 rows.
+// [n][128] BF16, 16-byte aligned, targets T [n][3].  Row buffers of whole
+// 128-row tiles (256 BF16 values a row, XB 128), DY [n][3]; part holds
+// kTrainSplits x (256 x 128 + 256 x 256) and chunk 1284 values per 64 rows;
+// wloss 4 per 128 rows.
 constexpr int kTrainSplits = 16;
 constexpr int kTrainChunkFloats = 1284;
 struct TrainBuffers {
-  uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr;
+  uint16_t *A1 = nullptr, *A2 = nullptr, *D1 = nullptr, *D2 = nullptr, *XB = nullptr;
   float *DY = nullptr, *part = nullptr, *chunk = nullptr;
 };
 // parameters, gradients (written), Adam moments and the step's constants; adam
 // 0: gradients and loss only
 struct TrainState {
   float *P = nullptr, *G = nullptr, *M = nullptr, *V = nullptr;
-  uint16_t *w1b = nullptr, *w2b = nullptr;
+  uint16_t *w1b = nullptr, *w2b = nullptr, *w1c = nullptr, *w2c = nullptr;
   float *wloss = nullptr, *loss = nullptr;
   int adam = 0;
   float lr = 0.f, beta1 = 0.f, beta2 = 0.f, eps = 0.f, c1 = 1.f, c2 = 1.f;
 };
 int tc_train(const uint16_t* X, const float* T, long long n, const TrainBuffers& B, const TrainState& t,
              unsigned int* status, cudaStream_t st);
+#ifdef __CUDACC__
+// place of element i of a row-major [rows][K] matrix in the canonical K-major
+// operand layout (8 x 8 core matrices of 64 consecutive elements)
+__device__ __forceinline__ int canon_index(int i, int K) {
+  const int r = i / K, k = i - r * K;
+  return ((r >> 3) * (K >> 3) + (k >> 3)) * 64 + (r & 7) * 8 + (k & 7);
+}
+// Adam (Kingma & Ba), bias-corrected: updates the moments, gives the parameter.
+// Roundings are explicit, so that every kernel takes the same step.
+__device__ __forceinline__ float adam_value(float p, float g, float& m, float& v, float lr, float b1,
+                                            float b2, float eps, float c1, float c2) {
+  m = fmaf(1.f - b1, g, __fmul_rn(b1, m));
+  v = fmaf(__fmul_rn(1.f - b2, g), g, __fmul_rn(b2, v));
+  return __fsub_rn(p, __fdiv_rn(__fmul_rn(lr, __fdiv_rn(m, c1)),
+                                __fadd_rn(__fsqrt_rn(__fdiv_rn(v, c2)), eps)));
+}
+#endif
 // The whole network, fused (locator_tc.cu): Y[M][3] from X[M][128] (W1, W2
-// BF16; biases and W3 FP32); X 16-byte aligned, M below 2^31.
+// BF16 in the canonical layout; biases and W3 FP32); X 16-byte aligned, M below 2^31.
 int tc_mlp_forward(const uint16_t* X, long long M, const uint16_t* W1, const uint16_t* W2,
                    const float* b1, const float* b2, const float* w3, const float* b3, float* Y,
                    unsigned int* status, int num_sms, cudaStream_t st);
