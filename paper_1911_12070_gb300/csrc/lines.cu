@@ -41,8 +41,8 @@
 // uniform Catmull-Rom, 'per_segment' points per segment, end points repeated
 // for open pieces and wrapped for closed ones, plus the last sample of an open
 // piece; lengths are the polyline lengths of the curves.  Curve points are
-// one thread each; orientation sums use one warp and lengths one block per
-// piece, FP64 in a fixed order, so results do not depend on timing.
+// one thread each; orientation sums and lengths go by chunks of entries, FP64 in
+// a fixed order, so results do not depend on timing.
 #include <cstdio>
 
 #include "qtv_internal.cuh"
@@ -65,6 +65,7 @@ namespace {
 constexpr int LT = 256;
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kMaxRounds = 64;  // jump rounds: log2 of 2^32 samples plus slack
+constexpr int kHops = 4;        // links an edge follows in a round
 constexpr int kSlots = 10;
 
 __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, const uint64_t* n_dev) {
@@ -105,7 +106,7 @@ struct LineArgs {
   unsigned long long* noff;    // exclusive scan of plen
   unsigned long long* edge_node_off;  // per starting edge slot: node offset of its piece
   uint32_t* tmp_nodes;   // unoriented node list
-  double* dots;          // per piece: orientation sum
+  double *left, *right;  // per chunk of node entries: orientation partials
   // outputs
   qtv_piece* pieces;
   unsigned long long piece_cap;
@@ -192,7 +193,8 @@ __global__ void edges_init_kernel(LineArgs a) {
   }
 }
 
-// Round r of pointer jumping (src = r & 1).  It is skipped once the previous
+// Round r of pointer jumping (src = r & 1): kHops links a round, so a chain of m
+// edges takes log(m) / log(kHops) rounds.  It is skipped once the previous
 // round left no edge with a successor (every chain has ended), so the rounds
 // beyond the longest chain cost a launch each; fbuf names the buffer that the
 // last round run wrote.
@@ -207,15 +209,20 @@ __global__ void jump_kernel(LineArgs a, int src, int r) {
     const unsigned long long e = e0 + threadIdx.x;
     bool more = false;
     if (e < ne) {
-      const uint4 J = a.jmp[src][e];
+      uint4 J = a.jmp[src][e];
       if (J.x == kNone) {
         // an edge whose chain ended two rounds ago already holds its final
         // values in both buffers
         if (r < 2 || a.jmp[d][e].x != kNone) a.jmp[d][e] = J;
       } else {
-        const uint4 N = a.jmp[src][J.x];
-        a.jmp[d][e] = make_uint4(N.x, J.y + N.y, N.z, 0u);
-        more = N.x != kNone;
+#pragma unroll
+        for (int hop = 1; hop < kHops; ++hop)
+          if (J.x != kNone) {
+            const uint4 N = a.jmp[src][J.x];
+            J = make_uint4(N.x, J.y + N.y, N.z, 0u);
+          }
+        a.jmp[d][e] = J;
+        more = J.x != kNone;
       }
     }
     // one flag per round, set by the first block that finds a live edge (a
@@ -365,67 +372,174 @@ __device__ __forceinline__ void face_dir(const LineArgs& a, uint32_t u, double d
   d[2] = (o == 0) ? w : 0.0;  // xy face: normal +z
 }
 
-// one warp per piece: orientation sum in a fixed order
+// ---------------------------------------------------------------------------
+// Sums over pieces.  The entries of all pieces (node list, curve points) are cut
+// into chunks of fixed length, one warp each, whatever the lengths of the
+// pieces: a warp per piece left the longest one (18231 samples of 1.39e6 at
+// 512^3) running alone.  A piece inside one chunk is summed there; one that
+// spans chunks leaves a partial per chunk (right: it starts in this one, left:
+// it started before), which are added in a fixed order.
+// ---------------------------------------------------------------------------
+constexpr unsigned long long kNodeChunk = 256, kPointChunk = 512;
+
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+  for (int d = 16; d; d >>= 1) v += __shfl_down_sync(0xffffffffu, v, d);
+  return __shfl_sync(0xffffffffu, v, 0);
+}
+
+// the last of np ascending values first(p) that is <= g
+template <typename F>
+__device__ __forceinline__ unsigned long long last_at_most(unsigned long long lo, unsigned long long hi,
+                                                           unsigned long long g, F first) {
+  while (hi - lo > 1) {
+    const unsigned long long mid = (lo + hi) >> 1;
+    if (first(mid) <= g) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// sum of a piece [first, end) that spans chunks, by the calling warp
+__device__ __forceinline__ double spanning_sum(const double* left, const double* right,
+                                               unsigned long long first, unsigned long long end,
+                                               unsigned long long chunk) {
+  const unsigned long long c0 = first / chunk, c1 = (end - 1) / chunk;
+  const int lane = threadIdx.x & 31;
+  double v = lane == 0 ? right[c0] : 0.0;
+  for (unsigned long long c = c0 + 1 + lane; c <= c1; c += 32) v += left[c];
+  return warp_sum(v);
+}
+
+// node entries of the pieces that fit, and the calling warp's chunks of them
+__device__ __forceinline__ unsigned long long node_total(const LineArgs& a, unsigned long long np) {
+  return np ? a.pieces[np - 1].first + a.pieces[np - 1].count : 0ull;
+}
+
+// orientation sums: final for pieces inside a chunk, partials for the others
 __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
   const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
+  const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
   const unsigned long long warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  for (unsigned long long p = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-       p < np; p += warps) {
-    const qtv_piece r = a.pieces[p];
-    double sum = 0.0;
-    if (a.face_ids && a.winding && r.count >= 2 && r.first + r.count <= a.node_cap) {
-      const unsigned long long nseg = r.closed ? r.count : r.count - 1;
-      for (unsigned long long i = lane; i < nseg; i += 32) {
-        const uint32_t u = a.tmp_nodes[r.first + i];
-        const uint32_t v = a.tmp_nodes[r.first + (i + 1 == r.count ? 0 : i + 1)];
-        double d[3];
-        face_dir(a, u, d);
+  const bool dirs = a.face_ids && a.winding;
+  for (unsigned long long c = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+       c * kNodeChunk < total; c += warps) {
+    const unsigned long long g0 = c * kNodeChunk, g1 = min(total, g0 + kNodeChunk);
+    unsigned long long p = last_at_most(0, np, g0, [&](unsigned long long m) { return a.pieces[m].first; });
+    for (; p < np; ++p) {
+      const qtv_piece r = a.pieces[p];
+      if (r.first >= g1) break;
+      const unsigned long long end = r.first + r.count;
+      double sum = 0.0;
+      if (dirs && r.count >= 2 && end <= a.node_cap) {
+        const unsigned long long last = r.closed ? end : end - 1;  // one segment per entry below it
+        for (unsigned long long i = max((unsigned long long)r.first, g0) + lane; i < min(last, g1); i += 32) {
+          const uint32_t u = a.tmp_nodes[i];
+          const uint32_t v = a.tmp_nodes[i + 1 == end ? r.first : i + 1];
+          double d[3];
+          face_dir(a, u, d);
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-          sum += ((double)a.xyz[3ull * v + c] - (double)a.xyz[3ull * u + c]) * d[c];
+          for (int k = 0; k < 3; ++k)
+            sum += ((double)a.xyz[3ull * v + k] - (double)a.xyz[3ull * u + k]) * d[k];
+        }
       }
-    }
-#pragma unroll
-    for (int dd = 16; dd; dd >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, dd);
-    if (lane == 0) {
-      a.dots[p] = sum;
-      if (sum < 0.0) a.pieces[p].reversed = 1;
+      sum = warp_sum(sum);
+      if (lane == 0) {
+        if (r.first < g0) a.left[c] = sum;
+        else if (end > g1) a.right[c] = sum;
+        else if (sum < 0.0) a.pieces[p].reversed = 1;
+      }
     }
   }
 }
 
-// final node list: each piece in order, or reversed (closed: first kept)
+// final node list: each piece in order, or reversed (closed: first kept); the
+// first chunk of a spanning piece sets its flag
 __global__ void place_kernel(LineArgs a, const unsigned long long* counts) {
   const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
+  const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
   const unsigned long long warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  for (unsigned long long p = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-       p < np; p += warps) {
-    const qtv_piece r = a.pieces[p];
-    for (unsigned long long k = lane; k < r.count; k += 32) {
-      unsigned long long src = k;
-      if (r.reversed) src = r.closed ? (k == 0 ? 0 : r.count - k) : r.count - 1 - k;
-      const unsigned long long dst = r.first + k;
-      if (dst < a.node_cap) a.nodes[dst] = a.tmp_nodes[r.first + src];
+  for (unsigned long long c = ((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+       c * kNodeChunk < total; c += warps) {
+    const unsigned long long g0 = c * kNodeChunk, g1 = min(total, g0 + kNodeChunk);
+    unsigned long long p = last_at_most(0, np, g0, [&](unsigned long long m) { return a.pieces[m].first; });
+    for (; p < np; ++p) {
+      const qtv_piece r = a.pieces[p];
+      if (r.first >= g1) break;
+      const unsigned long long end = r.first + r.count;
+      bool rev = r.reversed != 0;
+      if (r.first < g0 || end > g1) {
+        rev = spanning_sum(a.left, a.right, r.first, end, kNodeChunk) < 0.0;
+        if (rev && r.first >= g0 && lane == 0) a.pieces[p].reversed = 1;
+      }
+      for (unsigned long long i = max((unsigned long long)r.first, g0) + lane; i < min(end, g1); i += 32) {
+        const unsigned long long k = i - r.first;
+        unsigned long long src = k;
+        if (rev) src = r.closed ? (k == 0 ? 0 : r.count - k) : r.count - 1 - k;
+        if (i < a.node_cap) a.nodes[i] = a.tmp_nodes[r.first + src];
+      }
     }
   }
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of u32 values into u64 (three passes, deterministic)
+// Exclusive scan into u64, of one or two arrays at once: the sums of chunks of
+// SCHUNK values, then every block scans its chunk on top of the sums before it
+// (a single thread adding them took 11 us of each scan).
 // ---------------------------------------------------------------------------
 constexpr int SB = 1024;        // threads per scan block
 constexpr int SPER = 4;         // values per thread
 constexpr int SCHUNK = SB * SPER;
 
 template <typename T>
-__global__ void __launch_bounds__(SB) scan_blocks_kernel(const T* in, const uint64_t* n_dev,
-                                                         unsigned long long n,
-                                                         unsigned long long* out,
-                                                         unsigned long long* bsum) {
+struct ScanArgs {
+  const T* in[2];
+  unsigned long long* out[2];
+  unsigned long long* total;  // of each array
+  unsigned long long* bsum;   // [2][chunks]
+  unsigned long long n;
+  const uint64_t* n_dev;
+};
+
+// sum over the block (all threads get it)
+__device__ __forceinline__ unsigned long long block_total(unsigned long long v, unsigned long long* wt) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  __syncthreads();  // wt may still be read
+  if (lane == 0) wt[w] = v;
+  __syncthreads();
+  v = wt[lane];
+#pragma unroll
+  for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+  return v;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(SB) scan_sums_kernel(ScanArgs<T> a) {
   __shared__ unsigned long long wt[32];
-  const unsigned long long nn = limit_n(n, n_dev);
+  const unsigned long long nn = limit_n(a.n, a.n_dev);
+  const T* in = a.in[blockIdx.y];
+  unsigned long long loc = 0;
+  for (unsigned long long i = (unsigned long long)blockIdx.x * SCHUNK + threadIdx.x;
+       i < min(nn, ((unsigned long long)blockIdx.x + 1) * SCHUNK); i += SB)
+    loc += in[i];
+  loc = block_total(loc, wt);
+  if (threadIdx.x == 0) a.bsum[(unsigned long long)blockIdx.y * gridDim.x + blockIdx.x] = loc;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(SB) scan_apply_kernel(ScanArgs<T> a) {
+  __shared__ unsigned long long wt[32];
+  const unsigned long long nn = limit_n(a.n, a.n_dev);
+  const T* in = a.in[blockIdx.y];
+  unsigned long long* out = a.out[blockIdx.y];
+  const unsigned long long* bsum = a.bsum + (unsigned long long)blockIdx.y * gridDim.x;
+  unsigned long long before = 0;
+  for (unsigned long long b = threadIdx.x; b < blockIdx.x; b += SB) before += bsum[b];
+  before = block_total(before, wt);
   const unsigned long long base = (unsigned long long)blockIdx.x * SCHUNK + threadIdx.x * SPER;
   unsigned long long v[SPER], loc = 0;
 #pragma unroll
@@ -440,58 +554,29 @@ __global__ void __launch_bounds__(SB) scan_blocks_kernel(const T* in, const uint
     const unsigned long long t = __shfl_up_sync(0xffffffffu, inc, d);
     if (lane >= d) inc += t;
   }
+  __syncthreads();  // wt may still be read
   if (lane == 31) wt[w] = inc;
   __syncthreads();
-  if (w == 0) {
-    const unsigned long long x = wt[lane];
-    unsigned long long y = x;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const unsigned long long t = __shfl_up_sync(0xffffffffu, y, d);
-      if (lane >= d) y += t;
-    }
-    wt[lane] = y - x;
-    if (lane == 31) bsum[blockIdx.x] = y;
-  }
-  __syncthreads();
-  unsigned long long run = wt[w] + inc - loc;
+  unsigned long long run = before + inc - loc;
+  for (int q = 0; q < w; ++q) run += wt[q];
 #pragma unroll
   for (int i = 0; i < SPER; ++i) {
     if (base + i < nn) out[base + i] = run;
     run += v[i];
   }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SB - 1) a.total[blockIdx.y] = run;
 }
 
-__global__ void scan_sums_kernel(unsigned long long* bsum, int nb, unsigned long long* total) {
-  if (threadIdx.x == 0) {
-    unsigned long long run = 0;
-    for (int b = 0; b < nb; ++b) {
-      const unsigned long long x = bsum[b];
-      bsum[b] = run;
-      run += x;
-    }
-    *total = run;
-  }
-}
-
-__global__ void scan_add_kernel(const uint64_t* n_dev, unsigned long long n,
-                                unsigned long long* out, const unsigned long long* bsum) {
-  const unsigned long long nn = limit_n(n, n_dev);
-  for (unsigned long long i = (unsigned long long)blockIdx.x * LT + threadIdx.x; i < nn;
-       i += (unsigned long long)gridDim.x * LT)
-    out[i] += bsum[i / SCHUNK];
-}
-
+// bsum: one entry per chunk (at least one) and array
 template <typename T>
-void scan_u32(const T* in, const uint64_t* n_dev, unsigned long long n,
-              unsigned long long* out, unsigned long long* bsum, unsigned long long* total,
-              int num_sms, cudaStream_t st) {
-  const int nb = (int)((n + SCHUNK - 1) / SCHUNK);
-  scan_blocks_kernel<T><<<nb > 0 ? nb : 1, SB, 0, st>>>(in, n_dev, n, out, bsum);
-  scan_sums_kernel<<<1, 32, 0, st>>>(bsum, nb > 0 ? nb : 1, total);
-  long long g = ((long long)n + LT - 1) / LT;
-  if (g > (long long)num_sms * 16) g = (long long)num_sms * 16;
-  scan_add_kernel<<<(int)(g > 0 ? g : 1), LT, 0, st>>>(n_dev, n, out, bsum);
+void scan(const T* in0, const T* in1, const uint64_t* n_dev, unsigned long long n,
+          unsigned long long* out0, unsigned long long* out1, unsigned long long* bsum,
+          unsigned long long* total, cudaStream_t st) {
+  ScanArgs<T> a{{in0, in1}, {out0, out1}, total, bsum, n, n_dev};
+  const unsigned nb = (unsigned)((n + SCHUNK - 1) / SCHUNK);
+  const dim3 grid(nb > 0 ? nb : 1, in1 ? 2 : 1);
+  scan_sums_kernel<T><<<grid, SB, 0, st>>>(a);
+  scan_apply_kernel<T><<<grid, SB, 0, st>>>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -509,6 +594,7 @@ struct CurveArgs {
   float* curve;
   unsigned long long curve_cap;
   float* length;
+  double *left, *right;           // per chunk of curve points: length partials
 };
 
 __device__ __forceinline__ uint32_t curve_points(const qtv_piece& r, int per) {
@@ -531,18 +617,22 @@ __device__ __forceinline__ void sample_pos(const CurveArgs& a, const qtv_piece& 
   p[2] = a.xyz[3ull * u + 2];
 }
 
-// one thread per curve point: its piece by binary search over the first points
-__global__ void curve_kernel(CurveArgs a, const unsigned long long* total) {
+// one thread per curve point: its piece by binary search over the first points,
+// between the pieces of the block's first and last point
+__global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a, const unsigned long long* total) {
+  __shared__ unsigned long long ends[2];
   const unsigned long long np = limit_n(a.np, a.np_dev);
   const unsigned long long nt = min((unsigned long long)*total, a.curve_cap);
-  for (unsigned long long g = (unsigned long long)blockIdx.x * LT + threadIdx.x; g < nt;
-       g += (unsigned long long)gridDim.x * LT) {
-    unsigned long long lo = 0, hi = np;  // last piece with cfirst <= g
-    while (hi - lo > 1) {
-      const unsigned long long mid = (lo + hi) >> 1;
-      if (a.cfirst[mid] <= g) lo = mid;
-      else hi = mid;
-    }
+  auto first = [&](unsigned long long m) { return a.cfirst[m]; };
+  for (unsigned long long g0 = (unsigned long long)blockIdx.x * LT; g0 < nt;
+       g0 += (unsigned long long)gridDim.x * LT) {
+    __syncthreads();
+    if (threadIdx.x == 0) ends[0] = last_at_most(0, np, g0, first);
+    if (threadIdx.x == 32) ends[1] = last_at_most(0, np, min(g0 + LT, nt) - 1, first) + 1;
+    __syncthreads();
+    const unsigned long long g = g0 + threadIdx.x;
+    if (g >= nt) continue;
+    const unsigned long long lo = last_at_most(ends[0], ends[1], g, first);
     const qtv_piece r = a.pieces[lo];
     const long long k = (long long)(g - a.cfirst[lo]);
     const long long m = r.count;
@@ -591,40 +681,59 @@ __global__ void curve_kernel(CurveArgs a, const unsigned long long* total) {
   }
 }
 
-// one block per piece: polyline length of its curve (each segment's length in
-// FP32 from exact coordinate differences, summed in FP64: each thread sums a
-// fixed stride, then a fixed reduction tree)
-__global__ void __launch_bounds__(LT) length_kernel(CurveArgs a) {
-  __shared__ double part[LT / 32];
+// Polyline lengths of the curves (each segment's length in FP32 from exact
+// coordinate differences, summed in FP64 in a fixed order): final for pieces
+// inside a chunk, partials for the others.
+__global__ void __launch_bounds__(LT) length_kernel(CurveArgs a, const unsigned long long* total) {
   const unsigned long long np = limit_n(a.np, a.np_dev);
-  for (unsigned long long p = blockIdx.x; p < np; p += gridDim.x) {
-    const qtv_piece r = a.pieces[p];
-    const unsigned long long c0 = a.cfirst[p];
-    const unsigned long long n = a.npts[p];
-    double sum = 0.0;
-    if (n >= 2 && c0 + n <= a.curve_cap) {
-      const unsigned long long nseg = r.closed ? n : n - 1;
-      for (unsigned long long i = threadIdx.x; i < nseg; i += LT) {
-        const unsigned long long j = (i + 1 == n) ? 0 : i + 1;
-        float s2 = 0.f;
+  const unsigned long long nt = *total;
+  const int lane = threadIdx.x & 31;
+  const unsigned long long warps = ((unsigned long long)gridDim.x * LT) >> 5;
+  for (unsigned long long c = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5;
+       c * kPointChunk < min(nt, a.curve_cap); c += warps) {
+    const unsigned long long g0 = c * kPointChunk, g1 = min(nt, g0 + kPointChunk);
+    unsigned long long p = last_at_most(0, np, g0, [&](unsigned long long m) { return a.cfirst[m]; });
+    for (; p < np; ++p) {
+      const unsigned long long first = a.cfirst[p], end = first + a.npts[p];
+      if (first >= g1) break;
+      double sum = 0.0;
+      if (end - first >= 2 && end <= a.curve_cap) {
+        const unsigned long long last = a.pieces[p].closed ? end : end - 1;
+        for (unsigned long long i = max(first, g0) + lane; i < min(last, g1); i += 32) {
+          const unsigned long long j = i + 1 == end ? first : i + 1;
+          float s2 = 0.f;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          const float d = a.curve[3 * (c0 + j) + c] - a.curve[3 * (c0 + i) + c];
-          s2 = fmaf(d, d, s2);
+          for (int k = 0; k < 3; ++k) {
+            const float d = a.curve[3 * j + k] - a.curve[3 * i + k];
+            s2 = fmaf(d, d, s2);
+          }
+          sum += (double)sqrtf(s2);
         }
-        sum += (double)sqrtf(s2);
+      }
+      sum = warp_sum(sum);
+      if (lane == 0) {
+        if (first < g0) a.left[c] = sum;
+        else if (end > g1) a.right[c] = sum;
+        else a.length[p] = (float)sum;
       }
     }
-#pragma unroll
-    for (int d = 16; d; d >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, d);
-    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < LT / 32; ++w) t += part[w];
-      a.length[p] = (float)t;
+  }
+}
+
+// lengths of the pieces that span chunks, one warp each (0 for a piece whose
+// curve does not fit)
+__global__ void __launch_bounds__(LT) length_span_kernel(CurveArgs a) {
+  const unsigned long long np = limit_n(a.np, a.np_dev);
+  const unsigned long long warps = ((unsigned long long)gridDim.x * LT) >> 5;
+  for (unsigned long long p = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5; p < np;
+       p += warps) {
+    const unsigned long long first = a.cfirst[p], n = a.npts[p];
+    double sum = 0.0;
+    if (n && first + n <= a.curve_cap) {
+      if (first / kPointChunk == (first + n - 1) / kPointChunk) continue;
+      sum = spanning_sum(a.left, a.right, first, first + n, kPointChunk);
     }
-    __syncthreads();
+    if ((threadIdx.x & 31) == 0) a.length[p] = (float)sum;
   }
 }
 
@@ -778,7 +887,8 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   {
     // sizes must match the carve sequence below
     const unsigned long long sz[] = {n * 4, n, ne * 16, ne * 16, n * 4, n * 4, n * 8, n * 8, ne * 8,
-                                     nodes_max * 4, n * 8, nb * 8, nb * 8, 16,
+                                     nodes_max * 4, (nodes_max / kNodeChunk + 1) * 8,
+                                     (nodes_max / kNodeChunk + 1) * 8, nb * 16, 16,
                                      n * 4, n * 8, ne * 4, ne * 4, nb * 8, 8, kMaxRounds * 4 + 4};
     for (unsigned long long s : sz) bytes += ((s + 255) / 256) * 256;
   }
@@ -805,9 +915,9 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   a.noff = carve<unsigned long long>(p, n);
   a.edge_node_off = carve<unsigned long long>(p, ne);
   a.tmp_nodes = carve<uint32_t>(p, nodes_max);
-  a.dots = carve<double>(p, n);
-  unsigned long long* bs1 = carve<unsigned long long>(p, nb);
-  unsigned long long* bs2 = carve<unsigned long long>(p, nb);
+  a.left = carve<double>(p, nodes_max / kNodeChunk + 1);
+  a.right = carve<double>(p, nodes_max / kNodeChunk + 1);
+  unsigned long long* bs1 = carve<unsigned long long>(p, 2 * nb);
   unsigned long long* tot = carve<unsigned long long>(p, 2);
   a.deg32 = carve<uint32_t>(p, n);
   a.aoff = carve<unsigned long long>(p, n);
@@ -834,17 +944,17 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   stats_kernel<<<(int)g, LT, 0, st>>>(a);
   special_kernel<<<(int)g, LT, 0, st>>>(a);
   // compact directed edges: offsets by an exclusive scan of the degrees
-  scan_u32(a.deg32, n_dev, n, a.aoff, bs3, narcs, h->num_sms, st);
+  scan<uint32_t>(a.deg32, nullptr, n_dev, n, a.aoff, nullptr, bs3, narcs, st);
   arcs_kernel<<<(int)g, LT, 0, st>>>(a);
   edges_init_kernel<<<(int)ge, LT, 0, st>>>(a);
-  int rounds = 1;
-  while ((1ull << rounds) < (unsigned long long)n + 1) ++rounds;
+  int rounds = 0;
+  for (unsigned long long reach = 1; reach < (unsigned long long)n + 1; reach *= kHops) ++rounds;
+  if (rounds < 1) rounds = 1;
   cudaError_t e = cudaMemsetAsync(a.live, 0, (kMaxRounds + 1) * sizeof(uint32_t), st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(line rounds)");
   for (int r = 0; r < rounds; ++r) jump_kernel<<<(int)ge, LT, 0, st>>>(a, r & 1, r);
   count_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan_u32(a.pcount, n_dev, n, a.pfirst, bs1, tot, h->num_sms, st);
-  scan_u32(a.plen, n_dev, n, a.noff, bs2, tot + 1, h->num_sms, st);
+  scan<uint32_t>(a.pcount, a.plen, n_dev, n, a.pfirst, a.noff, bs1, tot, st);
   e = cudaMemcpyAsync(counts, tot, 2 * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemcpyAsync(line counts)");
   pieces_kernel<<<(int)g, LT, 0, st>>>(a);
@@ -860,7 +970,10 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
                         float* curve, uint64_t curve_cap, uint64_t* curve_first, float* length,
                         uint64_t* total, cudaStream_t st) {
   const unsigned long long nb = (np + SCHUNK - 1) / SCHUNK + 1;
-  size_t bytes = ((np * 4 + 255) / 256) * 256 + ((nb * 8 + 255) / 256) * 256 + 256;
+  const unsigned long long pc = curve_cap / kPointChunk + 1;
+  size_t bytes = 0;
+  const unsigned long long sz[] = {np * 4, nb * 8, pc * 8, pc * 8};
+  for (unsigned long long x : sz) bytes += (x + 255) / 256 * 256;
   void* buf = nullptr;
   int rc = ensure(h, bytes, st, &buf);
   if (rc) return rc;
@@ -874,6 +987,8 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   a.per = per;
   a.npts = carve<uint32_t>(p, np);
   unsigned long long* bs = carve<unsigned long long>(p, nb);
+  a.left = carve<double>(p, pc);
+  a.right = carve<double>(p, pc);
   a.cfirst = reinterpret_cast<unsigned long long*>(curve_first);
   a.curve = curve;
   a.curve_cap = curve_cap;
@@ -883,12 +998,11 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (g < 1) g = 1;
   TraceScope ts(h, K_CURVES, st);
   curve_count_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan_u32(a.npts, np_dev, np, a.cfirst, bs, reinterpret_cast<unsigned long long*>(total),
-           h->num_sms, st);
+  scan<uint32_t>(a.npts, nullptr, np_dev, np, a.cfirst, nullptr, bs,
+                 reinterpret_cast<unsigned long long*>(total), st);
   curve_kernel<<<h->num_sms * 16, LT, 0, st>>>(a, reinterpret_cast<unsigned long long*>(total));
-  long long gp = (long long)np;
-  if (gp > (long long)h->num_sms * 16) gp = (long long)h->num_sms * 16;
-  length_kernel<<<(int)(gp > 0 ? gp : 1), LT, 0, st>>>(a);
+  length_kernel<<<h->num_sms * 8, LT, 0, st>>>(a, reinterpret_cast<unsigned long long*>(total));
+  length_span_kernel<<<h->num_sms * 4, LT, 0, st>>>(a);
   const cudaError_t e = cudaGetLastError();
   return check_cuda(e, "piece curves launch");
 }
@@ -933,9 +1047,9 @@ int thin_pieces_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (gp < 1) gp = 1;
   TraceScope ts(h, K_THIN, st);
   thin_len_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan_u32(a.v, nullptr, ne, a.X, bs1, tots, h->num_sms, st);
+  scan<unsigned long long>(a.v, nullptr, nullptr, ne, a.X, nullptr, bs1, tots, st);
   thin_flag_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan_u32(a.flag, nullptr, ne, a.G, bs2, tots + 1, h->num_sms, st);
+  scan<uint32_t>(a.flag, nullptr, nullptr, ne, a.G, nullptr, bs2, tots + 1, st);
   thin_mean_kernel<<<(int)g, LT, 0, st>>>(a);
   thin_pieces_kernel<<<(int)gp, LT, 0, st>>>(a);
   cudaError_t e = cudaMemcpyAsync(total, tots + 1, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
