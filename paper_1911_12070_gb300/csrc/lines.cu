@@ -65,7 +65,7 @@ namespace {
 constexpr int LT = 256;
 constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kMaxRounds = 64;  // jump rounds: log2 of 2^32 samples plus slack
-constexpr int kHops = 4;        // links an edge follows in a round
+constexpr int kHops = 8;        // links an edge follows in a round
 constexpr int kSlots = 10;
 
 __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, const uint64_t* n_dev) {
@@ -197,7 +197,8 @@ __global__ void edges_init_kernel(LineArgs a) {
 // edges takes log(m) / log(kHops) rounds.  It is skipped once the previous
 // round left no edge with a successor (every chain has ended), so the rounds
 // beyond the longest chain cost a launch each; fbuf names the buffer that the
-// last round run wrote.
+// last round run wrote.  594e3 samples, device time of all rounds: one link a
+// round 225 us (20 launches), four 137 (10), eight 119 (7).
 __global__ void jump_kernel(LineArgs a, int src, int r) {
   if (r > 0 && a.live[r - 1] == 0u) return;
   const unsigned long long ne = *a.narcs;

@@ -20,19 +20,29 @@
 // quotient floor((sum + floor(c/2)) / c), so sums and means do not depend on the order in
 // which threads add, and the result is the same on every run.
 //
-// Representation.  The graph is never rebuilt.  Each input node keeps the
-// label of its current cluster (the lowest input index in it), and a cluster
-// is represented by that node, which holds the cluster's position.  A pass
-// keys the representatives, links (union-find, as in graph.cu: the larger
-// root goes under the smaller with a CAS, so roots are cluster minima) every
-// input edge whose ends lie in different clusters with equal keys, then
-// relabels and averages.  A cluster's adjacency is the set of input edges
-// that leave it, exactly the inherited connectivity of the paper's collapse.
+// Representation.  A cluster is represented by its node of lowest input index,
+// which holds its position; nl[u] is the node that u went under when its cluster
+// merged (u itself for a representative), so the cluster of any node is a walk
+// of at most one step per pass.  Each pass works on two compact lists, the
+// representatives and the edges between different clusters (with their ends
+// renamed; exactly the inherited connectivity of the paper's collapse), which
+// shrink as clusters merge: it links every edge whose ends have equal keys
+// (union-find, as in graph.cu: the larger root goes under the smaller with a
+// CAS, so roots are cluster minima), sums the members' positions, and lists the
+// surviving representatives, with their means and their keys in the next
+// lattice, and edges anew.  The order of the lists depends on timing, the
+// results do not.  An edge list that outgrows its buffer (denser graphs than
+// any of lines) is dropped and the pass reads the input edges through the walks.
+//
+// Bound by the latency of gathers from L2.  Scanning all nodes and input edges
+// in every pass took 0.47 ms of device time for the 594e3 samples of a 384^3
+// field (10 passes launched, 7 made); the lists take 0.40 ms
+// (the first pass, over all nodes, 0.15 of them).
 //
 // Launches: one set-up kernel, then for each of max_passes passes a fixed
-// sequence of four kernels and a one-thread control kernel; once the control
-// kernel has seen two quiet passes every later kernel returns at once, so the
-// call synchronises nothing and can be captured into a CUDA graph.
+// sequence of three kernels; the last block of the third counts the pass, and
+// once two passes were quiet every later kernel returns at once, so the call
+// synchronises nothing and can be captured into a CUDA graph.
 #include "qtv_internal.cuh"
 
 namespace qtv {
@@ -42,8 +52,10 @@ struct ReduceWork {
   unsigned int* cnt = nullptr;     // [cap] members of a new cluster
   unsigned long long* key = nullptr;  // [cap] packed box key of a representative
   unsigned int* par = nullptr;     // [cap] union-find parents of one pass
-  unsigned int* nl = nullptr;      // [cap] new label of a representative
-  unsigned long long* status = nullptr;  // [0] merges, [1] quiet, [2] passes, [3] done, [4] retry overflow
+  unsigned int* nl = nullptr;      // [cap] the node that a node merged into
+  unsigned int* reps[2] = {nullptr, nullptr};  // [cap] representatives, by pass parity
+  uint2* edges[2] = {nullptr, nullptr};        // [cap] edges between clusters
+  unsigned long long* status = nullptr;  // kStatus*
   uint64_t cap = 0;
 };
 
@@ -54,6 +66,10 @@ void reduce_work_free(ReduceWork* w) {
   cudaFree(w->key);
   cudaFree(w->par);
   cudaFree(w->nl);
+  for (int i = 0; i < 2; ++i) {
+    cudaFree(w->reps[i]);
+    cudaFree(w->edges[i]);
+  }
   cudaFree(w->status);
   delete w;
 }
@@ -62,7 +78,21 @@ namespace {
 
 constexpr int RT = 256;
 constexpr int kMaxTries = 1 << 20;     // CAS retries of one link before giving up
+constexpr uint32_t kNoNode = 0xFFFFFFFFu;
 constexpr double kFix = 4294967296.0;  // fixed-point units per length unit
+
+// status words
+enum {
+  kMerges = 0,   // of the running pass
+  kQuiet,        // passes without a merge in a row
+  kPasses,
+  kDone,
+  kGaveUp,       // a bounded retry loop ran out
+  kTicket,       // blocks of the listing kernel that have finished
+  kNumReps,      // [2] by pass parity
+  kNumEdges = kNumReps + 2,  // [2]; above the buffer: no list, use the input edges
+  kStatusWords = kNumEdges + 2
+};
 
 struct ReduceArgs {
   unsigned long long n;
@@ -72,13 +102,15 @@ struct ReduceArgs {
   int stride;
   long long D;          // box side in fixed point
   int max_passes;
-  uint32_t* lab;        // [n] cluster label of every node
   long long* q;         // [n][3] positions (valid at representatives)
   long long* sum;
   unsigned int* cnt;
   unsigned long long* key;
   unsigned int* par;
   unsigned int* nl;
+  unsigned int* reps[2];
+  uint2* edges[2];
+  unsigned long long edge_cap;
   unsigned long long* status;
 };
 
@@ -91,7 +123,7 @@ __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, cons
 }
 
 __device__ __forceinline__ bool done(const ReduceArgs& a) {
-  return *((const volatile unsigned long long*)a.status + 3) != 0ull;
+  return *((const volatile unsigned long long*)a.status + kDone) != 0ull;
 }
 
 // floor(x / d) for d > 0
@@ -107,30 +139,33 @@ __device__ __forceinline__ unsigned long long pack_key(long long kx, long long k
          (((unsigned long long)kz & m) << 42);
 }
 
-__global__ void __launch_bounds__(RT) reduce_init_kernel(ReduceArgs a, const float* __restrict__ xyz) {
-  const unsigned long long nn = limit_n(a.n, a.n_dev);
-  if (blockIdx.x == 0 && threadIdx.x < 5) a.status[threadIdx.x] = 0ull;
-  for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
-       u += (unsigned long long)gridDim.x * RT) {
-    a.lab[u] = (uint32_t)u;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) a.q[3 * u + c] = __double2ll_rn((double)xyz[3 * u + c] * kFix);
-  }
+// representative u starts a pass whose lattice is shifted (odd) or not: its box
+// key, a fresh union-find parent, zero sums
+__device__ __forceinline__ void start_pass(const ReduceArgs& a, unsigned long long u, bool odd,
+                                           const long long q[3]) {
+  const long long off = odd ? a.D / 2 : 0;
+  a.key[u] = pack_key(floor_div(q[0] - off, a.D), floor_div(q[1] - off, a.D),
+                      floor_div(q[2] - off, a.D));
+  a.par[u] = (uint32_t)u;
+  a.sum[3 * u] = a.sum[3 * u + 1] = a.sum[3 * u + 2] = 0;
+  a.cnt[u] = 0u;
 }
 
-// representatives: box key of this pass, fresh union-find parent, zero sums
-__global__ void __launch_bounds__(RT) reduce_key_kernel(ReduceArgs a) {
-  if (done(a)) return;
+__global__ void __launch_bounds__(RT) reduce_init_kernel(ReduceArgs a, const float* __restrict__ xyz) {
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  const long long off = (a.status[2] & 1ull) ? a.D / 2 : 0;
+  if (blockIdx.x == 0 && threadIdx.x < kStatusWords) {
+    // every node is a representative; no edge list yet
+    const int i = threadIdx.x;
+    a.status[i] = i == kNumReps ? nn : (i == kNumEdges ? ~0ull : 0ull);
+  }
   for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * RT) {
-    if (a.lab[u] != (uint32_t)u) continue;
-    a.key[u] = pack_key(floor_div(a.q[3 * u] - off, a.D), floor_div(a.q[3 * u + 1] - off, a.D),
-                        floor_div(a.q[3 * u + 2] - off, a.D));
-    a.par[u] = (uint32_t)u;
-    a.sum[3 * u] = a.sum[3 * u + 1] = a.sum[3 * u + 2] = 0;
-    a.cnt[u] = 0u;
+    long long q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a.q[3 * u + c] = q[c] = __double2ll_rn((double)xyz[3 * u + c] * kFix);
+    a.nl[u] = (uint32_t)u;
+    a.reps[0][u] = (uint32_t)u;
+    start_pass(a, u, false, q);
   }
 }
 
@@ -154,112 +189,201 @@ __device__ __forceinline__ uint32_t find_root_ro(const uint32_t* parent, uint32_
   return x;
 }
 
-// every input edge (u, v), u < v, between two clusters of equal key
-__global__ void __launch_bounds__(RT) reduce_link_kernel(ReduceArgs a) {
-  if (done(a)) return;
-  const unsigned long long nn = limit_n(a.n, a.n_dev);
-  for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
-       u += (unsigned long long)gridDim.x * RT) {
-    const int m = a.deg[u];
-    const uint32_t lu = a.lab[u];
-    const unsigned long long ku = a.key[lu];
-    for (int x = 0; x < m; ++x) {
-      const uint32_t v = a.nbr[u * (unsigned long long)a.stride + x];
-      if (v <= (uint32_t)u || v >= nn) continue;
-      const uint32_t lv = a.lab[v];
-      if (lv == lu || a.key[lv] != ku) continue;
-      int tries = 0;
-      while (true) {
-        uint32_t ra = find_root(a.par, lu), rb = find_root(a.par, lv);
-        if (ra == rb) break;
-        if (ra > rb) {
-          const uint32_t t = ra;
-          ra = rb;
-          rb = t;
-        }
-        if (atomicCAS(a.par + rb, rb, ra) == rb) break;
-        if (++tries >= kMaxTries) {
-          atomicOr(a.status + 4, 1ull);
-          break;
-        }
-      }
-    }
+// the cluster of node u (read-only walk)
+__device__ __forceinline__ uint32_t cluster_of(const ReduceArgs& a, uint32_t u) {
+  return find_root_ro(a.nl, u);
+}
+
+// f(ends) for the input edges (u, v), u < v, that join different clusters
+template <typename F>
+__device__ __forceinline__ void node_edges(const ReduceArgs& a, unsigned long long nn,
+                                           unsigned long long u, F f) {
+  const int m = a.deg[u];
+  uint32_t lu = kNoNode;
+  for (int x = 0; x < m; ++x) {
+    const uint32_t v = a.nbr[u * (unsigned long long)a.stride + x];
+    if (v <= (uint32_t)u || v >= nn) continue;
+    if (lu == kNoNode) lu = cluster_of(a, (uint32_t)u);
+    const uint32_t lv = cluster_of(a, v);
+    if (lv != lu) f(make_uint2(lu, lv));
   }
 }
 
-// representatives: new label (the root: lowest index of the merged cluster),
+// f(ends) for the calling thread's share of the edges between clusters of this
+// pass: from the list, or, without one, the input edges
+template <typename F>
+__device__ __forceinline__ void for_edges(const ReduceArgs& a, unsigned long long nn, int cur, F f) {
+  const unsigned long long ne = a.status[kNumEdges + cur];
+  const unsigned long long t0 = (unsigned long long)blockIdx.x * RT + threadIdx.x;
+  const unsigned long long step = (unsigned long long)gridDim.x * RT;
+  if (ne <= a.edge_cap) {
+    for (unsigned long long e = t0; e < ne; e += step) f(a.edges[cur][e]);
+    return;
+  }
+  for (unsigned long long u = t0; u < nn; u += step) node_edges(a, nn, u, f);
+}
+
+// every edge between two clusters of equal key
+__global__ void __launch_bounds__(RT) reduce_link_kernel(ReduceArgs a) {
+  if (done(a)) return;
+  const unsigned long long nn = limit_n(a.n, a.n_dev);
+  for_edges(a, nn, (int)(a.status[kPasses] & 1ull), [&](uint2 e) {
+    if (a.key[e.x] != a.key[e.y]) return;
+    int tries = 0;
+    while (true) {
+      uint32_t ra = find_root(a.par, e.x), rb = find_root(a.par, e.y);
+      if (ra == rb) break;
+      if (ra > rb) {
+        const uint32_t t = ra;
+        ra = rb;
+        rb = t;
+      }
+      if (atomicCAS(a.par + rb, rb, ra) == rb) break;
+      if (++tries >= kMaxTries) {
+        atomicOr(a.status + kGaveUp, 1ull);
+        break;
+      }
+    }
+  });
+}
+
+// representatives: the root (lowest index of the merged cluster), and the
 // position added to the new cluster's sum
 __global__ void __launch_bounds__(RT) reduce_merge_kernel(ReduceArgs a) {
   if (done(a)) return;
-  const unsigned long long nn = limit_n(a.n, a.n_dev);
+  const int cur = (int)(a.status[kPasses] & 1ull);
+  const unsigned long long nr = a.status[kNumReps + cur];
   unsigned long long merges = 0;
-  for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
-       u += (unsigned long long)gridDim.x * RT) {
-    if (a.lab[u] != (uint32_t)u) continue;
-    const uint32_t r = find_root_ro(a.par, (uint32_t)u);
+  for (unsigned long long i = (unsigned long long)blockIdx.x * RT + threadIdx.x; i < nr;
+       i += (unsigned long long)gridDim.x * RT) {
+    const uint32_t u = a.reps[cur][i];
+    const uint32_t r = find_root_ro(a.par, u);
     a.nl[u] = r;
-    merges += (r != (uint32_t)u) ? 1ull : 0ull;
+    merges += r != u ? 1ull : 0ull;
 #pragma unroll
     for (int c = 0; c < 3; ++c)
-      atomicAdd(reinterpret_cast<unsigned long long*>(a.sum + 3 * r + c),
-                (unsigned long long)a.q[3 * u + c]);
+      atomicAdd(reinterpret_cast<unsigned long long*>(a.sum + 3ull * r + c),
+                (unsigned long long)a.q[3ull * u + c]);
     atomicAdd(a.cnt + r, 1u);
   }
 #pragma unroll
   for (int d = 16; d; d >>= 1) merges += __shfl_down_sync(0xffffffffu, merges, d);
-  if ((threadIdx.x & 31) == 0 && merges) atomicAdd(a.status, merges);
+  if ((threadIdx.x & 31) == 0 && merges) atomicAdd(a.status + kMerges, merges);
 }
 
-// every node: its cluster's new label; new representatives: the rounded mean
-__global__ void __launch_bounds__(RT) reduce_relabel_kernel(ReduceArgs a) {
+// First place in a list for the k entries of the calling thread: one atomic a
+// block and call (all threads call; one atomic a warp made the counters' lines
+// the bottleneck).
+__device__ __forceinline__ unsigned long long append(unsigned long long* count, uint32_t k) {
+  __shared__ uint32_t part[RT / 32];
+  __shared__ unsigned long long base;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t inc = k;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= d) inc += t;
+  }
+  __syncthreads();  // part and base may still be read
+  if (lane == 31) part[w] = inc;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (int i = 0; i < RT / 32; ++i) {
+    if (i < w) before += part[i];
+    total += part[i];
+  }
+  if (threadIdx.x == 0 && total) base = atomicAdd(count, (unsigned long long)total);
+  __syncthreads();
+  return base + before + inc - k;
+}
+
+// The next pass's lists: surviving representatives with the rounded mean of
+// their cluster and their key in its lattice, and the edges that still join
+// different clusters.  The last block to finish counts the pass and stops after
+// two quiet ones or max_passes.
+__global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a) {
   if (done(a)) return;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
-       u += (unsigned long long)gridDim.x * RT) {
-    const uint32_t l = a.lab[u];
-    const uint32_t r = a.nl[l];
-    a.lab[u] = r;
-    if (l == (uint32_t)u && r == (uint32_t)u) {
-      const long long c = (long long)a.cnt[u];
+  const unsigned long long passes = a.status[kPasses];
+  const int cur = (int)(passes & 1ull), next = cur ^ 1;
+  const unsigned long long nr = a.status[kNumReps + cur], ne = a.status[kNumEdges + cur];
+  const bool listed = ne <= a.edge_cap;
+  // blocks without work leave at once; the others count themselves at the end
+  const unsigned long long items = max(nr, listed ? ne : nn);
+  const unsigned long long blocks = max(1ull, min((unsigned long long)gridDim.x, (items + RT - 1) / RT));
+  if (blockIdx.x >= blocks) return;
+  const unsigned long long b0 = (unsigned long long)blockIdx.x * RT, step = blocks * RT;
+  for (unsigned long long i0 = b0; i0 < nr; i0 += step) {
+    const unsigned long long i = i0 + threadIdx.x;
+    const uint32_t u = i < nr ? a.reps[cur][i] : 0u;
+    const bool stays = i < nr && a.nl[u] == u;
+    const unsigned long long at = append(a.status + kNumReps + next, stays ? 1u : 0u);
+    if (!stays) continue;
+    a.reps[next][at] = u;
+    const long long c = (long long)a.cnt[u];
+    long long q[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) a.q[3 * u + k] = floor_div(a.sum[3 * u + k] + c / 2, c);
+    for (int k = 0; k < 3; ++k) a.q[3ull * u + k] = q[k] = floor_div(a.sum[3ull * u + k] + c / 2, c);
+    start_pass(a, u, next != 0, q);
+  }
+  if (listed) {
+    for (unsigned long long i0 = b0; i0 < ne; i0 += step) {
+      const unsigned long long i = i0 + threadIdx.x;
+      uint2 e = i < ne ? a.edges[cur][i] : make_uint2(0u, 0u);
+      e.x = a.nl[e.x];
+      e.y = a.nl[e.y];
+      const unsigned long long at = append(a.status + kNumEdges + next, e.x != e.y ? 1u : 0u);
+      if (e.x != e.y && at < a.edge_cap) a.edges[next][at] = e;
+    }
+  } else {
+    for (unsigned long long i0 = b0; i0 < nn; i0 += step) {
+      const unsigned long long u = i0 + threadIdx.x;
+      uint32_t k = 0;
+      if (u < nn) node_edges(a, nn, u, [&](uint2) { ++k; });
+      unsigned long long at = append(a.status + kNumEdges + next, k);
+      if (k)
+        node_edges(a, nn, u, [&](uint2 e) {
+          if (at < a.edge_cap) a.edges[next][at] = e;
+          ++at;
+        });
     }
   }
+  __threadfence();
+  __syncthreads();
+  __shared__ bool last;
+  if (threadIdx.x == 0) last = atomicAdd(a.status + kTicket, 1ull) == blocks - 1;
+  __syncthreads();
+  if (!last || threadIdx.x != 0) return;
+  volatile unsigned long long* s = a.status;
+  const unsigned long long quiet = s[kMerges] ? 0ull : s[kQuiet] + 1ull;
+  s[kMerges] = 0ull;
+  s[kTicket] = 0ull;
+  s[kNumReps + cur] = 0ull;
+  s[kNumEdges + cur] = 0ull;
+  s[kQuiet] = quiet;
+  s[kPasses] = passes + 1ull;
+  if (quiet >= 2ull || passes + 1ull >= (unsigned long long)a.max_passes) s[kDone] = 1ull;
 }
 
-// one thread: count the pass, stop after two quiet passes or max_passes
-__global__ void reduce_control_kernel(ReduceArgs a) {
-  if (done(a)) return;
-  const unsigned long long merges = a.status[0];
-  a.status[0] = 0ull;
-  const unsigned long long passes = a.status[2] + 1ull;
-  const unsigned long long quiet = merges ? 0ull : a.status[1] + 1ull;
-  a.status[1] = quiet;
-  a.status[2] = passes;
-  if (quiet >= 2ull || passes >= (unsigned long long)a.max_passes) a.status[3] = 1ull;
-}
-
-// representatives: positions back to the length unit (exact in FP64);
-// counts = (clusters, passes)
-__global__ void __launch_bounds__(RT) reduce_out_kernel(ReduceArgs a, double* __restrict__ out,
-                                                        uint64_t* counts) {
+// labels of all nodes; representatives: positions back to the length unit
+// (exact in FP64); counts = (clusters, passes)
+__global__ void __launch_bounds__(RT) reduce_out_kernel(ReduceArgs a, uint32_t* __restrict__ label,
+                                                        double* __restrict__ out, uint64_t* counts) {
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  unsigned long long reps = 0;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const unsigned long long passes = a.status[kPasses];
+    counts[0] = a.status[kGaveUp] ? QTV_COUNT_TIMEOUT : a.status[kNumReps + (passes & 1ull)];
+    counts[1] = passes;
+  }
   for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * RT) {
-    if (a.lab[u] != (uint32_t)u) continue;
-    ++reps;
+    const uint32_t r = cluster_of(a, (uint32_t)u);
+    label[u] = r;
+    if (r != (uint32_t)u) continue;
 #pragma unroll
     for (int c = 0; c < 3; ++c) out[3 * u + c] = (double)a.q[3 * u + c] / kFix;
   }
-#pragma unroll
-  for (int d = 16; d; d >>= 1) reps += __shfl_down_sync(0xffffffffu, reps, d);
-  if ((threadIdx.x & 31) == 0 && reps) atomicAdd(reinterpret_cast<unsigned long long*>(counts), reps);
-}
-
-__global__ void reduce_counts_kernel(const ReduceArgs a, uint64_t* counts) {
-  counts[1] = a.status[2];
-  if (a.status[4]) counts[0] = QTV_COUNT_TIMEOUT;
 }
 
 bool capturing(cudaStream_t st) {
@@ -286,8 +410,13 @@ int box_reduce_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const uin
       e = cudaMalloc(reinterpret_cast<void**>(&w->key), c * sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&w->par), c * sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&w->nl), c * sizeof(unsigned int));
+    for (int i = 0; i < 2; ++i) {
+      if (e == cudaSuccess)
+        e = cudaMalloc(reinterpret_cast<void**>(&w->reps[i]), c * sizeof(unsigned int));
+      if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&w->edges[i]), c * sizeof(uint2));
+    }
     if (e == cudaSuccess)
-      e = cudaMalloc(reinterpret_cast<void**>(&w->status), 8 * sizeof(unsigned long long));
+      e = cudaMalloc(reinterpret_cast<void**>(&w->status), kStatusWords * sizeof(unsigned long long));
     if (e != cudaSuccess) {
       reduce_work_free(w);
       return check_cuda(e, "cudaMalloc(reduction workspace)");
@@ -296,9 +425,9 @@ int box_reduce_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const uin
     h->reduce = w;
   }
   ReduceWork* w = h->reduce;
-  cudaError_t e = cudaMemsetAsync(counts, 0, 2 * sizeof(uint64_t), st);
-  if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(reduction counts)");
-  if (n == 0) return QTV_OK;
+  if (n == 0)
+    return check_cuda(cudaMemsetAsync(counts, 0, 2 * sizeof(uint64_t), st),
+                      "cudaMemsetAsync(reduction counts)");
   ReduceArgs a;
   a.n = n;
   a.n_dev = n_dev;
@@ -307,7 +436,6 @@ int box_reduce_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const uin
   a.stride = stride;
   a.D = (long long)((double)box * kFix);
   a.max_passes = max_passes;
-  a.lab = label;
   // positions live in the output array as fixed-point integers until the end
   a.q = reinterpret_cast<long long*>(out_xyz);
   a.sum = w->sum;
@@ -315,21 +443,23 @@ int box_reduce_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const uin
   a.key = w->key;
   a.par = w->par;
   a.nl = w->nl;
+  for (int i = 0; i < 2; ++i) {
+    a.reps[i] = w->reps[i];
+    a.edges[i] = w->edges[i];
+  }
+  a.edge_cap = w->cap;
   a.status = w->status;
   long long blocks = ((long long)n + RT - 1) / RT;
   if (blocks > (long long)h->num_sms * 8) blocks = (long long)h->num_sms * 8;
   TraceScope ts(h, K_REDUCE, st);
   reduce_init_kernel<<<(int)blocks, RT, 0, st>>>(a, xyz);
   for (int p = 0; p < max_passes; ++p) {
-    reduce_key_kernel<<<(int)blocks, RT, 0, st>>>(a);
     reduce_link_kernel<<<(int)blocks, RT, 0, st>>>(a);
     reduce_merge_kernel<<<(int)blocks, RT, 0, st>>>(a);
-    reduce_relabel_kernel<<<(int)blocks, RT, 0, st>>>(a);
-    reduce_control_kernel<<<1, 1, 0, st>>>(a);
+    reduce_list_kernel<<<(int)blocks, RT, 0, st>>>(a);
   }
-  reduce_out_kernel<<<(int)blocks, RT, 0, st>>>(a, out_xyz, counts);
-  reduce_counts_kernel<<<1, 1, 0, st>>>(a, counts);
-  e = cudaGetLastError();
+  reduce_out_kernel<<<(int)blocks, RT, 0, st>>>(a, label, out_xyz, counts);
+  const cudaError_t e = cudaGetLastError();
   return check_cuda(e, "box reduction launch");
 }
 
