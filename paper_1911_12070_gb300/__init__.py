@@ -270,13 +270,14 @@ class Qtv:
         nz, ny, nx = psi.shape
         if capacity is None:
             capacity = max(1024, int(0.02 * nx * ny * nz))
-        count = torch.zeros(1, dtype=torch.int64, device=dev)
-        st = torch.zeros(8, dtype=torch.int64, device=dev) if stats else None
+        both = torch.zeros(9 if stats else 1, dtype=torch.int64, device=dev)  # read back at once
+        count, st = both[:1], both[1:] if stats else None
         for _ in range(2):
             ids = torch.empty(capacity, dtype=torch.int64, device=dev)
             w = torch.empty(capacity, dtype=torch.int8, device=dev)
             self.identify_into(psi, ids, w, count, st, stream=stream)
-            n = int(count.item())
+            host = both.cpu().numpy()
+            n = int(host[0])
             if n < 0:  # QTV_COUNT_TIMEOUT read as int64
                 raise QtvError(ERR_TIMEOUT, "a bounded device wait gave up")
             if n <= capacity:
@@ -284,7 +285,7 @@ class Qtv:
             capacity = n
         sd = None
         if stats:
-            vals = st.cpu().numpy().astype(np.uint64)
+            vals = host[1:].astype(np.uint64)
             sd = {f[0]: int(v) for f, v in zip(Stats._fields_, vals)}
         return ids[:n], w[:n], sd
 
@@ -700,13 +701,19 @@ class Qtv:
         dev = deg.device
         counts = torch.zeros(2, dtype=torch.int64, device=dev)
         args = (_ptr(nbr), _ptr(deg), _ptr(comp), _ptr(xyz), _ptr(face_ids), _ptr(winding))
-        _check(lib().qtv_line_pieces(self.h, n, None, *args, None, 0, None, 0, _ptr(counts),
-                                     _stream_ptr(stream)))
-        npc, nnd = (int(v) for v in counts.cpu().tolist())
-        pieces = torch.empty((max(npc, 1), 24), dtype=torch.uint8, device=dev)
-        nodes = torch.empty(max(nnd, 1), dtype=torch.int32, device=dev)
-        _check(lib().qtv_line_pieces(self.h, n, None, *args, _ptr(pieces), npc, _ptr(nodes), nnd,
-                                     _ptr(counts), _stream_ptr(stream)))
+        # room for lines of a few samples with some branches: one pass; a graph
+        # with more pieces takes a second one (a counting pass before every call
+        # cost as much as the call)
+        cap_p, cap_n = n // 8 + 64, n + n // 4 + 64
+        for _ in range(2):
+            pieces = torch.empty((cap_p, 24), dtype=torch.uint8, device=dev)
+            nodes = torch.empty(cap_n, dtype=torch.int32, device=dev)
+            _check(lib().qtv_line_pieces(self.h, n, None, *args, _ptr(pieces), cap_p, _ptr(nodes),
+                                         cap_n, _ptr(counts), _stream_ptr(stream)))
+            npc, nnd = (int(v) for v in counts.cpu().tolist())
+            if npc <= cap_p and nnd <= cap_n:
+                break
+            cap_p, cap_n = max(npc, 1), max(nnd, 1)
         return pieces[:npc], nodes[:nnd]
 
     def piece_curves(self, xyz, nodes, pieces, per_segment: int = 8, stream=None):
@@ -720,13 +727,21 @@ class Qtv:
         length = torch.empty(max(npc, 1), dtype=torch.float32, device=dev)
         total = torch.zeros(1, dtype=torch.int64, device=dev)
         args = (_ptr(xyz), _ptr(nodes), _ptr(pieces), npc, None, int(per_segment))
-        _check(lib().qtv_piece_curves(self.h, *args, None, 0, _ptr(first), _ptr(length),
-                                      _ptr(total), _stream_ptr(stream)))
-        m = int(total.item())
-        curve = torch.empty((max(m, 1), 3), dtype=torch.float32, device=dev)
-        _check(lib().qtv_piece_curves(self.h, *args, _ptr(curve), m, _ptr(first), _ptr(length),
-                                      _ptr(total), _stream_ptr(stream)))
-        return curve[:m], first[:npc], length[:npc]
+        # pieces of disjoint node ranges have at most per_segment points an entry:
+        # one pass up to 1 GB of points, else a counting pass first
+        cap = (0 if nodes is None else nodes.numel()) * max(int(per_segment), 0)
+        cap = max(cap, 1) if cap <= 2 ** 30 // 12 else 0
+        for _ in range(2):
+            curve = torch.empty((cap, 3), dtype=torch.float32, device=dev)
+            _check(lib().qtv_piece_curves(self.h, *args, _ptr(curve) if cap else None, cap,
+                                          _ptr(first), _ptr(length), _ptr(total),
+                                          _stream_ptr(stream)))
+            m = int(total.item())
+            if m <= cap:
+                break
+            cap = m
+        curve = curve[:m] if 2 * m >= cap else curve[:m].clone()  # keeps no large buffer alive
+        return curve, first[:npc], length[:npc]
 
     def thin_pieces(self, xyz, nodes, pieces, box: float, stream=None):
         """Arc-length thinning of line pieces (qtv_thin_pieces): (means float32 [m, 3],
