@@ -63,9 +63,9 @@ void line_work_free(LineWork* w) {
 namespace {
 
 constexpr int LT = 256;
-constexpr uint32_t kNone = 0xFFFFFFFFu;
 constexpr int kMaxRounds = 64;  // jump rounds: log2 of 2^32 samples plus slack
 constexpr int kHops = 8;        // links an edge follows in a round
+constexpr uint32_t kEnded = 0x80000000u;
 constexpr int kSlots = 10;
 
 __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, const uint64_t* n_dev) {
@@ -94,10 +94,10 @@ struct LineArgs {
   const unsigned long long* narcs;  // device: number of directed edges
   uint32_t* atail;   // per directed edge: tail sample
   uint32_t* ahead;   // per directed edge: head sample
-  // per directed edge, double-buffered: x = successor edge, y = distance
-  // (edges) to the end of the chain, z = last edge of the chain (one 16-byte
-  // gather per jump)
-  uint4* jmp[2];
+  // per directed edge, double-buffered: x = successor edge, y = edges from this
+  // one to it; once the chain has ended (kEnded in y) x = its last edge, y =
+  // edges to its end (one 8-byte gather per link)
+  uint2* jmp[2];
   uint32_t* live;    // per round: 1 if an edge's chain has not ended yet
   uint32_t* fbuf;    // buffer of the final jump results
   uint32_t* pcount;  // per sample: pieces started there
@@ -184,11 +184,11 @@ __global__ void edges_init_kernel(LineArgs a) {
        e += (unsigned long long)gridDim.x * LT) {
     const uint32_t u = a.atail[e], w = a.ahead[e];
     if (a.special[w]) {
-      a.jmp[0][e] = make_uint4(kNone, 1u, (uint32_t)e, 0u);
+      a.jmp[0][e] = make_uint2((uint32_t)e, 1u | kEnded);
     } else {
       // w has degree 2: continue to its other neighbour
       const int sx = (a.nbr[(unsigned long long)w * kSlots] == u) ? 1 : 0;
-      a.jmp[0][e] = make_uint4((uint32_t)(a.aoff[w] + sx), 1u, kNone, 0u);
+      a.jmp[0][e] = make_uint2((uint32_t)(a.aoff[w] + sx), 1u);
     }
   }
 }
@@ -198,7 +198,8 @@ __global__ void edges_init_kernel(LineArgs a) {
 // round left no edge with a successor (every chain has ended), so the rounds
 // beyond the longest chain cost a launch each; fbuf names the buffer that the
 // last round run wrote.  594e3 samples, device time of all rounds: one link a
-// round 225 us (20 launches), four 137 (10), eight 119 (7).
+// round 225 us (20 launches), four 137 (10), eight 119 (7); with records of 8
+// bytes instead of 16, 105.
 __global__ void jump_kernel(LineArgs a, int src, int r) {
   if (r > 0 && a.live[r - 1] == 0u) return;
   const unsigned long long ne = *a.narcs;
@@ -210,20 +211,20 @@ __global__ void jump_kernel(LineArgs a, int src, int r) {
     const unsigned long long e = e0 + threadIdx.x;
     bool more = false;
     if (e < ne) {
-      uint4 J = a.jmp[src][e];
-      if (J.x == kNone) {
+      uint2 J = a.jmp[src][e];
+      if (J.y & kEnded) {
         // an edge whose chain ended two rounds ago already holds its final
         // values in both buffers
-        if (r < 2 || a.jmp[d][e].x != kNone) a.jmp[d][e] = J;
+        if (r < 2 || !(a.jmp[d][e].y & kEnded)) a.jmp[d][e] = J;
       } else {
 #pragma unroll
         for (int hop = 1; hop < kHops; ++hop)
-          if (J.x != kNone) {
-            const uint4 N = a.jmp[src][J.x];
-            J = make_uint4(N.x, J.y + N.y, N.z, 0u);
+          if (!(J.y & kEnded)) {
+            const uint2 N = a.jmp[src][J.x];
+            J = make_uint2(N.x, J.y + N.y);
           }
         a.jmp[d][e] = J;
-        more = J.x != kNone;
+        more = !(J.y & kEnded);
       }
     }
     // one flag per round, set by the first block that finds a live edge (a
@@ -236,10 +237,15 @@ __global__ void jump_kernel(LineArgs a, int src, int r) {
   }
 }
 
+// edges of the chain that edge e starts
+__device__ __forceinline__ uint32_t chain_len(const LineArgs& a, int buf, unsigned long long e) {
+  return a.jmp[buf][e].y & ~kEnded;
+}
+
 // end sample and the sample before it, of the chain that edge e starts
 __device__ __forceinline__ void chain_end(const LineArgs& a, int buf, uint32_t e, uint32_t& end,
                                           uint32_t& before) {
-  const uint32_t l = a.jmp[buf][e].z;
+  const uint32_t l = a.jmp[buf][e].x;
   before = a.atail[l];
   end = a.ahead[l];
 }
@@ -277,7 +283,7 @@ __global__ void count_kernel(LineArgs a) {
         uint32_t end, before;
         chain_end(a, buf, (uint32_t)e, end, before);
         ++pc;
-        nl += (end == (uint32_t)u) ? a.jmp[buf][e].y : a.jmp[buf][e].y + 1;
+        nl += chain_len(a, buf, e) + (end == (uint32_t)u ? 0u : 1u);
       }
     }
     a.pcount[u] = pc;
@@ -315,7 +321,7 @@ __global__ void pieces_kernel(LineArgs a) {
       uint32_t end, before;
       chain_end(a, buf, (uint32_t)e, end, before);
       const bool closed = end == (uint32_t)u;
-      const uint32_t cnt = closed ? a.jmp[buf][e].y : a.jmp[buf][e].y + 1;
+      const uint32_t cnt = chain_len(a, buf, e) + (closed ? 0u : 1u);
       if (p < a.piece_cap) {
         qtv_piece r = {};
         r.first = off;
@@ -354,10 +360,10 @@ __global__ void interior_kernel(LineArgs a) {
     uint32_t pos;
     if (discovering(a, buf, end0, bef0, (uint32_t)f0)) {
       off = a.edge_node_off[f0];
-      pos = a.jmp[buf][e0].y;
+      pos = chain_len(a, buf, e0);
     } else if (discovering(a, buf, end1, bef1, (uint32_t)f1)) {
       off = a.edge_node_off[f1];
-      pos = a.jmp[buf][e1].y;
+      pos = chain_len(a, buf, e1);
     } else {
       continue;
     }
@@ -365,23 +371,15 @@ __global__ void interior_kernel(LineArgs a) {
   }
 }
 
-__device__ __forceinline__ void face_dir(const LineArgs& a, uint32_t u, double d[3]) {
-  const int o = (int)(a.face_ids[u] & 3u);
-  const double w = (double)a.winding[u];
-  d[0] = (o == 1) ? w : 0.0;  // yz face: normal +x
-  d[1] = (o == 2) ? w : 0.0;  // zx face: normal +y
-  d[2] = (o == 0) ? w : 0.0;  // xy face: normal +z
-}
-
 // ---------------------------------------------------------------------------
-// Sums over pieces.  The entries of all pieces (node list, curve points) are cut
+// Sums over pieces.  The entries of all pieces are cut
 // into chunks of fixed length, one warp each, whatever the lengths of the
 // pieces: a warp per piece left the longest one (18231 samples of 1.39e6 at
 // 512^3) running alone.  A piece inside one chunk is summed there; one that
 // spans chunks leaves a partial per chunk (right: it starts in this one, left:
 // it started before), which are added in a fixed order.
 // ---------------------------------------------------------------------------
-constexpr unsigned long long kNodeChunk = 256, kPointChunk = 512;
+constexpr unsigned long long kNodeChunk = 256;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -435,15 +433,26 @@ __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
       double sum = 0.0;
       if (dirs && r.count >= 2 && end <= a.node_cap) {
         const unsigned long long last = r.closed ? end : end - 1;  // one segment per entry below it
+        float nan = 0.f;  // NaN once a coordinate is not finite (so is the sum then)
         for (unsigned long long i = max((unsigned long long)r.first, g0) + lane; i < min(last, g1); i += 32) {
           const uint32_t u = a.tmp_nodes[i];
           const uint32_t v = a.tmp_nodes[i + 1 == end ? r.first : i + 1];
-          double d[3];
-          face_dir(a, u, d);
+          // (p[i+1] - p[i]) . d, d = W times the face normal: one axis (FP64
+          // units are scarce)
+          const int o = (int)(a.face_ids[u] & 3u);
+          const int ax = o == 0 ? 2 : (o == 1 ? 0 : 1);  // z, x, y for xy, yz, zx faces
+          float pu[3], pv[3];
 #pragma unroll
-          for (int k = 0; k < 3; ++k)
-            sum += ((double)a.xyz[3ull * v + k] - (double)a.xyz[3ull * u + k]) * d[k];
+          for (int k = 0; k < 3; ++k) {
+            pu[k] = a.xyz[3ull * u + k];
+            pv[k] = a.xyz[3ull * v + k];
+            nan = fmaf(pu[k], 0.f, fmaf(pv[k], 0.f, nan));
+          }
+          const float cu = ax == 0 ? pu[0] : (ax == 1 ? pu[1] : pu[2]);
+          const float cv = ax == 0 ? pv[0] : (ax == 1 ? pv[1] : pv[2]);
+          if (o != 3) sum = fma((double)cv - (double)cu, (double)a.winding[u], sum);
         }
+        sum += (double)nan;
       }
       sum = warp_sum(sum);
       if (lane == 0) {
@@ -498,7 +507,7 @@ template <typename T>
 struct ScanArgs {
   const T* in[2];
   unsigned long long* out[2];
-  unsigned long long* total;  // of each array
+  unsigned long long* total[2];  // of each array
   unsigned long long* bsum;   // [2][chunks]
   unsigned long long n;
   const uint64_t* n_dev;
@@ -565,15 +574,15 @@ __global__ void __launch_bounds__(SB) scan_apply_kernel(ScanArgs<T> a) {
     if (base + i < nn) out[base + i] = run;
     run += v[i];
   }
-  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SB - 1) a.total[blockIdx.y] = run;
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == SB - 1) *a.total[blockIdx.y] = run;
 }
 
 // bsum: one entry per chunk (at least one) and array
 template <typename T>
 void scan(const T* in0, const T* in1, const uint64_t* n_dev, unsigned long long n,
           unsigned long long* out0, unsigned long long* out1, unsigned long long* bsum,
-          unsigned long long* total, cudaStream_t st) {
-  ScanArgs<T> a{{in0, in1}, {out0, out1}, total, bsum, n, n_dev};
+          unsigned long long* total0, unsigned long long* total1, cudaStream_t st) {
+  ScanArgs<T> a{{in0, in1}, {out0, out1}, {total0, total1}, bsum, n, n_dev};
   const unsigned nb = (unsigned)((n + SCHUNK - 1) / SCHUNK);
   const dim3 grid(nb > 0 ? nb : 1, in1 ? 2 : 1);
   scan_sums_kernel<T><<<grid, SB, 0, st>>>(a);
@@ -590,12 +599,14 @@ struct CurveArgs {
   unsigned long long np;
   const uint64_t* np_dev;
   int per;
-  uint32_t* npts;                 // per piece: curve points
+  uint32_t *npts, *count;         // per piece: curve points, samples
   unsigned long long* cfirst;     // exclusive scan of npts
+  unsigned long long* efirst;     // exclusive scan of count
+  const unsigned long long* entries;  // samples of all pieces
   float* curve;
   unsigned long long curve_cap;
   float* length;
-  double *left, *right;           // per chunk of curve points: length partials
+  double *left, *right;           // per warp of entries: length partials
 };
 
 __device__ __forceinline__ uint32_t curve_points(const qtv_piece& r, int per) {
@@ -606,8 +617,11 @@ __device__ __forceinline__ uint32_t curve_points(const qtv_piece& r, int per) {
 __global__ void curve_count_kernel(CurveArgs a) {
   const unsigned long long np = limit_n(a.np, a.np_dev);
   for (unsigned long long p = (unsigned long long)blockIdx.x * LT + threadIdx.x; p < np;
-       p += (unsigned long long)gridDim.x * LT)
-    a.npts[p] = curve_points(a.pieces[p], a.per);
+       p += (unsigned long long)gridDim.x * LT) {
+    const qtv_piece r = a.pieces[p];
+    a.npts[p] = curve_points(r, a.per);
+    a.count[p] = r.count;
+  }
 }
 
 __device__ __forceinline__ void sample_pos(const CurveArgs& a, const qtv_piece& r, long long i,
@@ -618,121 +632,129 @@ __device__ __forceinline__ void sample_pos(const CurveArgs& a, const qtv_piece& 
   p[2] = a.xyz[3ull * u + 2];
 }
 
-// one thread per curve point: its piece by binary search over the first points,
-// between the pieces of the block's first and last point
-__global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a, const unsigned long long* total) {
-  __shared__ unsigned long long ends[2];
-  const unsigned long long np = limit_n(a.np, a.np_dev);
-  const unsigned long long nt = min((unsigned long long)*total, a.curve_cap);
-  auto first = [&](unsigned long long m) { return a.cfirst[m]; };
-  for (unsigned long long g0 = (unsigned long long)blockIdx.x * LT; g0 < nt;
-       g0 += (unsigned long long)gridDim.x * LT) {
-    __syncthreads();
-    if (threadIdx.x == 0) ends[0] = last_at_most(0, np, g0, first);
-    if (threadIdx.x == 32) ends[1] = last_at_most(0, np, min(g0 + LT, nt) - 1, first) + 1;
-    __syncthreads();
-    const unsigned long long g = g0 + threadIdx.x;
-    if (g >= nt) continue;
-    const unsigned long long lo = last_at_most(ends[0], ends[1], g, first);
-    const qtv_piece r = a.pieces[lo];
-    const long long k = (long long)(g - a.cfirst[lo]);
-    const long long m = r.count;
-    float out[3];
-    const long long nseg = r.closed ? m : m - 1;
-    if (m < 2 || k >= nseg * a.per) {
-      // a one-sample piece, or the last sample of an open piece
-      sample_pos(a, r, m < 2 ? 0 : m - 1, out);
-    } else {
-      // segment s and step ti of point k (k < count * per < 2^32 * per)
-      long long s;
-      int ti;
-      if ((k >> 32) == 0) {
-        const uint32_t k32 = (uint32_t)k, q = k32 / (uint32_t)a.per;
-        s = q;
-        ti = (int)(k32 - q * (uint32_t)a.per);
-      } else {
-        s = k / a.per;
-        ti = (int)(k - s * a.per);
-      }
-      // ext = closed: [P[m-1], P[0..m-1], P[0], P[1]]; open: [P[0], P[0..m-1], P[m-1]]
-      // (s + c - 1 lies in [-1, m + 1] and m >= 2, so one wrap suffices)
-      long long id[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        long long x = s + c - 1;
-        if (r.closed) x = x < 0 ? x + m : (x >= m ? x - m : x);
-        else x = x < 0 ? 0 : (x > m - 1 ? m - 1 : x);
-        id[c] = x;
-      }
-      float p0[3], p1[3], p2[3], p3[3];
-      sample_pos(a, r, id[0], p0);
-      sample_pos(a, r, id[1], p1);
-      sample_pos(a, r, id[2], p2);
-      sample_pos(a, r, id[3], p3);
-      const float t = (float)ti / (float)a.per, t2 = t * t, t3 = t2 * t;
-#pragma unroll
-      for (int c = 0; c < 3; ++c)
-        out[c] = 0.5f * (2.f * p1[c] + t * (p2[c] - p0[c]) +
-                         t2 * (2.f * p0[c] - 5.f * p1[c] + 4.f * p2[c] - p3[c]) +
-                         t3 * (-p0[c] + 3.f * p1[c] - 3.f * p2[c] + p3[c]));
-    }
-    a.curve[3 * g] = out[0];
-    a.curve[3 * g + 1] = out[1];
-    a.curve[3 * g + 2] = out[2];
-  }
-}
+// One lane per sample of the pieces (in piece order): the points of the segment
+// that starts there, or the one point of a last or lone sample, and the
+// segment's share of the polyline length (FP32 lengths between the points, from
+// exact coordinate differences, the next segment's first point being the next
+// sample itself; those of a segment added in FP32 with their rounding errors
+// kept, the segments in FP64 in a fixed order).  The points of a warp go
+// through shared memory, kStage a sample at a time, and out in runs.  A thread
+// per point that gathered its four samples (and the lengths from the points
+// read back) took 70 and 50 us for 4.9e6 points; this takes 59 us, of 9 to
+// write them, bound by issue.
+constexpr int kStage = 8, kStagePitch = 3 * kStage + 1;
 
-// Polyline lengths of the curves (each segment's length in FP32 from exact
-// coordinate differences, summed in FP64 in a fixed order): final for pieces
-// inside a chunk, partials for the others.
-__global__ void __launch_bounds__(LT) length_kernel(CurveArgs a, const unsigned long long* total) {
+__global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a) {
+  __shared__ float stage[LT / 32][32 * kStagePitch];
   const unsigned long long np = limit_n(a.np, a.np_dev);
-  const unsigned long long nt = *total;
+  // the pieces that fit come first and have at least a point a sample
+  const unsigned long long ne = min((unsigned long long)*a.entries, a.curve_cap);
   const int lane = threadIdx.x & 31;
+  float* const st = stage[threadIdx.x >> 5];
   const unsigned long long warps = ((unsigned long long)gridDim.x * LT) >> 5;
-  for (unsigned long long c = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5;
-       c * kPointChunk < min(nt, a.curve_cap); c += warps) {
-    const unsigned long long g0 = c * kPointChunk, g1 = min(nt, g0 + kPointChunk);
-    unsigned long long p = last_at_most(0, np, g0, [&](unsigned long long m) { return a.cfirst[m]; });
-    for (; p < np; ++p) {
-      const unsigned long long first = a.cfirst[p], end = first + a.npts[p];
-      if (first >= g1) break;
-      double sum = 0.0;
-      if (end - first >= 2 && end <= a.curve_cap) {
-        const unsigned long long last = a.pieces[p].closed ? end : end - 1;
-        for (unsigned long long i = max(first, g0) + lane; i < min(last, g1); i += 32) {
-          const unsigned long long j = i + 1 == end ? first : i + 1;
-          float s2 = 0.f;
+  auto first = [&](unsigned long long m) { return a.efirst[m]; };
+  for (unsigned long long c = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5; c * 32 < ne;
+       c += warps) {
+    const unsigned long long g0 = c * 32, g = g0 + lane;
+    const bool act = g < ne;
+    // pieces of the first and the last sample, then each lane's between them
+    const unsigned long long edge = lane == 0 ? g0 : min(ne, g0 + 32) - 1;
+    const unsigned long long mine = lane < 2 ? last_at_most(0, np, edge, first) : 0ull;
+    const unsigned long long lo = __shfl_sync(0xffffffffu, mine, 0);
+    const unsigned long long hi = __shfl_sync(0xffffffffu, mine, 1) + 1;
+    const unsigned long long p = act ? last_at_most(lo, hi, g, first) : lo;
+    const qtv_piece r = a.pieces[p];
+    const unsigned long long e0 = a.efirst[p], c0 = a.cfirst[p];
+    const long long m = r.count, s = act ? (long long)(g - e0) : 0;
+    // a piece whose curve does not fit is left out
+    const bool fits = act && c0 + a.npts[p] <= a.curve_cap;
+    const bool seg = fits && (r.closed ? m >= 2 : s + 1 < m);
+    const int npt = seg ? a.per : (fits ? 1 : 0);
+    const unsigned long long at = c0 + (unsigned long long)s * (unsigned)a.per;  // first point
+    float p0[3] = {}, p1[3] = {}, p2[3] = {}, p3[3] = {};
+    if (fits) sample_pos(a, r, s, p1);
+    if (seg) {
+      // closed: [P[m-1], P[0..m-1], P[0], P[1]]; open: [P[0], P[0..m-1], P[m-1]]
+      auto wrap = [&](long long x) {
+        if (r.closed) return x < 0 ? x + m : (x >= m ? x - m : x);
+        return x < 0 ? 0ll : (x > m - 1 ? m - 1 : x);
+      };
+      sample_pos(a, r, wrap(s - 1), p0);
+      sample_pos(a, r, wrap(s + 1), p2);
+      sample_pos(a, r, wrap(s + 2), p3);
+    }
+    float len = 0.f, rest = 0.f;  // unevaluated sum of two (error-free additions)
+    float prev[3] = {p1[0], p1[1], p1[2]};
+    auto add_len = [&](const float q[3]) {
+      float s2 = 0.f;
 #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const float d = a.curve[3 * j + k] - a.curve[3 * i + k];
-            s2 = fmaf(d, d, s2);
-          }
-          sum += (double)sqrtf(s2);
-        }
+      for (int k = 0; k < 3; ++k) {
+        const float d = q[k] - prev[k];
+        s2 = fmaf(d, d, s2);
+        prev[k] = q[k];
       }
-      sum = warp_sum(sum);
+      const float d = sqrtf(s2), t = __fadd_rn(len, d), z = __fsub_rn(t, len);
+      rest = __fadd_rn(rest, __fadd_rn(__fsub_rn(len, __fsub_rn(t, z)), __fsub_rn(d, z)));
+      len = t;
+    };
+    const int most = __reduce_max_sync(0xffffffffu, npt);
+    for (int t0 = 0; t0 < most; t0 += kStage) {
+      const int left = max(0, min(npt - t0, kStage));  // points of this lane in the round
+#pragma unroll
+      for (int i = 0; i < kStage; ++i) {
+        if (i >= left) break;
+        float out[3] = {p1[0], p1[1], p1[2]};
+        if (seg) {
+          const float t = (float)(t0 + i) / (float)a.per, t2 = t * t, t3 = t2 * t;
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            out[k] = 0.5f * (2.f * p1[k] + t * (p2[k] - p0[k]) +
+                             t2 * (2.f * p0[k] - 5.f * p1[k] + 4.f * p2[k] - p3[k]) +
+                             t3 * (-p0[k] + 3.f * p1[k] - 3.f * p2[k] + p3[k]));
+          if (t0 + i > 0) add_len(out);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) st[lane * kStagePitch + 3 * i + k] = out[k];
+      }
+      __syncwarp();
+      const unsigned long long run = at + (unsigned)t0;
+#pragma unroll 4
+      for (int x = lane; x < 32 * 3 * kStage; x += 32) {
+        const int l = x / (3 * kStage), f = x - l * (3 * kStage);
+        const unsigned long long dst = __shfl_sync(0xffffffffu, run, l);
+        const int n = __shfl_sync(0xffffffffu, left, l);
+        if (f < 3 * n) a.curve[3 * dst + f] = st[l * kStagePitch + f];
+      }
+      __syncwarp();
+    }
+    if (seg) add_len(p2);
+    // lengths: sums over the lanes of each piece of this warp
+    for (unsigned long long q = lo; q < hi; ++q) {
+      double v = act && p == q ? (double)len + (double)rest : 0.0;
+      v = warp_sum(v);
       if (lane == 0) {
-        if (first < g0) a.left[c] = sum;
-        else if (end > g1) a.right[c] = sum;
-        else a.length[p] = (float)sum;
+        const unsigned long long f = a.efirst[q], end = f + a.count[q];
+        if (a.cfirst[q] + a.npts[q] > a.curve_cap) continue;
+        if (f < g0) a.left[c] = v;
+        else if (end > g0 + 32) a.right[c] = v;
+        else if (end > f) a.length[q] = (float)v;
       }
     }
   }
 }
 
-// lengths of the pieces that span chunks, one warp each (0 for a piece whose
-// curve does not fit)
+// lengths of the pieces that span warps of entries, one warp each (0 for a
+// piece that does not fit)
 __global__ void __launch_bounds__(LT) length_span_kernel(CurveArgs a) {
   const unsigned long long np = limit_n(a.np, a.np_dev);
   const unsigned long long warps = ((unsigned long long)gridDim.x * LT) >> 5;
   for (unsigned long long p = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5; p < np;
        p += warps) {
-    const unsigned long long first = a.cfirst[p], n = a.npts[p];
+    const unsigned long long first = a.efirst[p], n = a.count[p];
     double sum = 0.0;
-    if (n && first + n <= a.curve_cap) {
-      if (first / kPointChunk == (first + n - 1) / kPointChunk) continue;
-      sum = spanning_sum(a.left, a.right, first, first + n, kPointChunk);
+    if (n && a.cfirst[p] + a.npts[p] <= a.curve_cap) {
+      if (first / 32 == (first + n - 1) / 32) continue;
+      sum = spanning_sum(a.left, a.right, first, first + n, 32);
     }
     if ((threadIdx.x & 31) == 0) a.length[p] = (float)sum;
   }
@@ -887,7 +909,7 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   size_t bytes = 0;
   {
     // sizes must match the carve sequence below
-    const unsigned long long sz[] = {n * 4, n, ne * 16, ne * 16, n * 4, n * 4, n * 8, n * 8, ne * 8,
+    const unsigned long long sz[] = {n * 4, n, ne * 8, ne * 8, n * 4, n * 4, n * 8, n * 8, ne * 8,
                                      nodes_max * 4, (nodes_max / kNodeChunk + 1) * 8,
                                      (nodes_max / kNodeChunk + 1) * 8, nb * 16, 16,
                                      n * 4, n * 8, ne * 4, ne * 4, nb * 8, 8, kMaxRounds * 4 + 4};
@@ -908,8 +930,8 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   a.winding = winding;
   a.cflags = carve<uint32_t>(p, n);
   a.special = carve<uint8_t>(p, n);
-  a.jmp[0] = carve<uint4>(p, ne);
-  a.jmp[1] = carve<uint4>(p, ne);
+  a.jmp[0] = carve<uint2>(p, ne);
+  a.jmp[1] = carve<uint2>(p, ne);
   a.pcount = carve<uint32_t>(p, n);
   a.plen = carve<uint32_t>(p, n);
   a.pfirst = carve<unsigned long long>(p, n);
@@ -945,7 +967,7 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   stats_kernel<<<(int)g, LT, 0, st>>>(a);
   special_kernel<<<(int)g, LT, 0, st>>>(a);
   // compact directed edges: offsets by an exclusive scan of the degrees
-  scan<uint32_t>(a.deg32, nullptr, n_dev, n, a.aoff, nullptr, bs3, narcs, st);
+  scan<uint32_t>(a.deg32, nullptr, n_dev, n, a.aoff, nullptr, bs3, narcs, nullptr, st);
   arcs_kernel<<<(int)g, LT, 0, st>>>(a);
   edges_init_kernel<<<(int)ge, LT, 0, st>>>(a);
   int rounds = 0;
@@ -955,7 +977,7 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(line rounds)");
   for (int r = 0; r < rounds; ++r) jump_kernel<<<(int)ge, LT, 0, st>>>(a, r & 1, r);
   count_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan<uint32_t>(a.pcount, a.plen, n_dev, n, a.pfirst, a.noff, bs1, tot, st);
+  scan<uint32_t>(a.pcount, a.plen, n_dev, n, a.pfirst, a.noff, bs1, tot, tot + 1, st);
   e = cudaMemcpyAsync(counts, tot, 2 * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemcpyAsync(line counts)");
   pieces_kernel<<<(int)g, LT, 0, st>>>(a);
@@ -971,9 +993,9 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
                         float* curve, uint64_t curve_cap, uint64_t* curve_first, float* length,
                         uint64_t* total, cudaStream_t st) {
   const unsigned long long nb = (np + SCHUNK - 1) / SCHUNK + 1;
-  const unsigned long long pc = curve_cap / kPointChunk + 1;
+  const unsigned long long pc = curve_cap / 32 + 1;  // warps of samples whose points fit
   size_t bytes = 0;
-  const unsigned long long sz[] = {np * 4, nb * 8, pc * 8, pc * 8};
+  const unsigned long long sz[] = {np * 4, np * 4, np * 8, nb * 16, pc * 8, pc * 8, 8};
   for (unsigned long long x : sz) bytes += (x + 255) / 256 * 256;
   void* buf = nullptr;
   int rc = ensure(h, bytes, st, &buf);
@@ -987,9 +1009,13 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   a.np_dev = np_dev;
   a.per = per;
   a.npts = carve<uint32_t>(p, np);
-  unsigned long long* bs = carve<unsigned long long>(p, nb);
+  a.count = carve<uint32_t>(p, np);
+  a.efirst = carve<unsigned long long>(p, np);
+  unsigned long long* bs = carve<unsigned long long>(p, 2 * nb);
   a.left = carve<double>(p, pc);
   a.right = carve<double>(p, pc);
+  unsigned long long* entries = carve<unsigned long long>(p, 1);
+  a.entries = entries;
   a.cfirst = reinterpret_cast<unsigned long long*>(curve_first);
   a.curve = curve;
   a.curve_cap = curve_cap;
@@ -999,10 +1025,9 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (g < 1) g = 1;
   TraceScope ts(h, K_CURVES, st);
   curve_count_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan<uint32_t>(a.npts, nullptr, np_dev, np, a.cfirst, nullptr, bs,
-                 reinterpret_cast<unsigned long long*>(total), st);
-  curve_kernel<<<h->num_sms * 16, LT, 0, st>>>(a, reinterpret_cast<unsigned long long*>(total));
-  length_kernel<<<h->num_sms * 8, LT, 0, st>>>(a, reinterpret_cast<unsigned long long*>(total));
+  scan<uint32_t>(a.npts, a.count, np_dev, np, a.cfirst, a.efirst, bs,
+                 reinterpret_cast<unsigned long long*>(total), entries, st);
+  if (curve_cap > 0) curve_kernel<<<h->num_sms * 8, LT, 0, st>>>(a);
   length_span_kernel<<<h->num_sms * 4, LT, 0, st>>>(a);
   const cudaError_t e = cudaGetLastError();
   return check_cuda(e, "piece curves launch");
@@ -1048,9 +1073,9 @@ int thin_pieces_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (gp < 1) gp = 1;
   TraceScope ts(h, K_THIN, st);
   thin_len_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan<unsigned long long>(a.v, nullptr, nullptr, ne, a.X, nullptr, bs1, tots, st);
+  scan<unsigned long long>(a.v, nullptr, nullptr, ne, a.X, nullptr, bs1, tots, nullptr, st);
   thin_flag_kernel<<<(int)g, LT, 0, st>>>(a);
-  scan<uint32_t>(a.flag, nullptr, nullptr, ne, a.G, nullptr, bs2, tots + 1, st);
+  scan<uint32_t>(a.flag, nullptr, nullptr, ne, a.G, nullptr, bs2, tots + 1, nullptr, st);
   thin_mean_kernel<<<(int)g, LT, 0, st>>>(a);
   thin_pieces_kernel<<<(int)gp, LT, 0, st>>>(a);
   cudaError_t e = cudaMemcpyAsync(total, tots + 1, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
