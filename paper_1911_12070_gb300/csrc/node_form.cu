@@ -14,38 +14,39 @@
 // crossing r (its wrapped phase difference minus theta_b - theta_a, over
 // 2 pi), decided from the sign bits of Im a, Im b and the sign of the
 // determinant Re a Im b - Im a Re b; the theta terms telescope around the
-// ring, so S is the sum of the ring's eight r.  Each grid edge is
-// evaluated once, in its forward direction, and a ring that runs it backwards
-// adds -r (the argument of the conjugate is the exact negation).  Two
-// consecutive edges along a grid line make one side of a ring:
-//   X_k(i,j) = r_x(i-1,j,k) + r_x(i,j,k)    (x-edges through (i,j,k))
-//   Y_k(i,j) = r_y(i,j-1,k) + r_y(i,j,k)
-//   Z(i,j,k) = r_z(i,j,k-1) + r_z(i,j,k)
-// and the three rings of node (i,j,k) are
-//   S_xy = X_k(i,j-1) + Y_k(i+1,j) - X_k(i,j+1) - Y_k(i-1,j)
-//   S_yz = Y_{k-1}(i,j) + Z(i,j+1,k) - Y_{k+1}(i,j) - Z(i,j-1,k)
-//   S_zx = Z(i-1,j,k) + X_{k+1}(i,j) - Z(i+1,j,k) - X_{k-1}(i,j).
+// ring, so S is the sum of the ring's eight r.  Each grid edge is evaluated once,
+// in its forward direction, and a ring that runs it backwards adds -r (the
+// argument of the conjugate is the exact negation).  The ring encloses the four
+// plaquettes of its plane at the node, and the edges between them cancel, so S is
+// the sum of their four-edge sums, whatever the r are:
+//   W_xy(i,j) = r_x(i,j) + r_y(i+1,j) - r_x(i,j+1) - r_y(i,j), and so on,
+//   S_xy(i,j) = W_xy(i-1,j-1) + W_xy(i,j-1) + W_xy(i-1,j) + W_xy(i,j),
+// and each W serves four rings.  The sums are kept mod 8: S in [-3, 4], exact
+// because only a ring whose eight differences are all exact +-pi ties reaches
+// |S| = 4 (read as 4).
 //
 // Layout (bit-sliced).  A warp owns 30 columns (lanes 1..30; lanes 0 and 31
-// hold the neighbour columns) of a band of NB = 14 rows, and each lane keeps
-// one bit per row (rows j0 - 1 .. j0 + NB, halo rows included) in words:
-// the sign bit of Im psi and the sign bits of the FP32 cross products of its
-// x, y and z edges, as the identification sweep does.  An edge term is +1 when
-// s_a = 0, s_b = 1 and the cross sign is 0, -1 when s_a = 1, s_b = 0 and the
-// sign is 1; edges that touch a zero node count 0.  The eight terms of a ring
-// are word shifts (rows) and shuffles (columns) of these edge words, and
-// their sum mod 8 comes from a carry-save adder tree over the words: S mod 8
-// = #nonzero - 2 #negative, exact in [-3, 4] because only a ring whose eight
-// differences are all exact +-pi ties reaches |S| = 4.  The warp marches z
-// over a chunk of planes, streaming each lane's column through a 3-slot ring
-// in shared memory with cp.async one plane ahead.
+// hold the neighbour columns) of a band of NB = 18 rows, and each lane keeps
+// one bit per row (rows j0 - 1 .. j0 + NB, halo rows included) in words: the
+// sign bit of Im psi and the sign bits of the FP32 cross products of its x, y
+// and z edges, as the identification sweep does.  An edge term is +1 when s_a =
+// 0, s_b = 1 and the cross sign is 0, -1 when s_a = 1, s_b = 0 and the sign is 1;
+// edges that touch a zero node count 0.  W and S are three words each; adding
+// two of them is five 3-input operations.  The warp marches z over a chunk of
+// planes, streaming each lane's column through a 2-slot ring in shared memory
+// with cp.async; the previous plane's values stay in registers.
 //
-// Output.  Vortex nodes in ascending linear node index with their three S:
-// each warp step stages its records contiguously in a chunk of the staging
-// buffer that the warp reserved (one atomic per chunk) and writes a table
-// entry {staging base, count, per-row counts}; an exclusive scan over the
-// (plane, band) totals and a scatter that interleaves the column segments of
-// every row put them in order.  Optionally the dense S field [3][nz][ny][nx].
+// Output.  Vortex nodes in ascending linear node index with their three S: each
+// lane with vortex nodes in a sub-band of 9 rows of a step stages one record, its
+// S words there, contiguously in a chunk of the staging buffer that the warp
+// reserved (one atomic per chunk), and the step writes a table entry {staging
+// base, lane mask} per sub-band; after an exclusive scan of the (plane, sub-band)
+// totals one warp per (plane, sub-band) lists the nodes row by row.  Optionally the dense S field [3][nz][ny][nx].
+//
+// Bound by issue.  With eight ring terms added per ring, records per node and
+// the previous plane read from shared memory it took 3.2 warp instructions a
+// node and 218 us at 384^3, the scatter 63; now 140 and 35 (512^3: 500 and 110,
+// now 298 and 64).
 //
 // Density error.  e = sum_q |rho(p_q)| / (n rho_bar), rho the density |psi|^2
 // of the trilinearly interpolated field at the sample points, rho_bar the mean
@@ -58,15 +59,17 @@
 namespace qtv {
 
 struct NodeWork {
-  unsigned long long* recs = nullptr;  // staged vortex-node records
+  uint4* recs = nullptr;               // staged records: words 0..3
   uint64_t recs_cap = 0;
-  uint4* table = nullptr;              // per (plane, band, column segment)
+  uint32_t* recs4 = nullptr;           // word 4
+  uint64_t recs4_cap = 0;
+  uint2* table = nullptr;              // per (plane, band, column segment)
   uint64_t table_cap = 0;
   unsigned int* segtot = nullptr;      // vortex nodes per (plane, band)
   uint64_t segtot_cap = 0;
   unsigned long long* seg_off = nullptr;
   uint64_t seg_off_cap = 0;
-  unsigned long long* top = nullptr;   // staging bump counter
+  unsigned long long* top = nullptr;   // staging bump counter, work item counter
   double* partial = nullptr;           // density sums per block
   uint64_t partial_cap = 0;
   int resident_warps = 0;
@@ -75,6 +78,7 @@ struct NodeWork {
 void node_work_free(NodeWork* w) {
   if (!w) return;
   cudaFree(w->recs);
+  cudaFree(w->recs4);
   cudaFree(w->table);
   cudaFree(w->segtot);
   cudaFree(w->seg_off);
@@ -85,22 +89,29 @@ void node_work_free(NodeWork* w) {
 
 namespace {
 
-constexpr int NT = 16;          // rows held: bit t = row j0 - 1 + t
+// Rows, warps and slots: the copies pass through the L1 cache, which gets what
+// shared memory leaves; 200 KB of rings a multiprocessor slow them (384^3: 17 rows,
+// 16 warps, 3 slots, 209 KB 182 us; 22, 12, 3, 203 KB 188).  More rows a lane share
+// the word logic: 20 rows, 16 warps, 2 slots, 164 KB 140 us; 18, 16, 2 140; 20, 12,
+// 3 146; 32, 8, 2 145; 24, 10, 3 152.
+constexpr int NT = 20;          // rows held: bit t = row j0 - 1 + t
 constexpr int NB = NT - 2;      // owned rows per band: bits 1..NB
 constexpr uint32_t kOwnedRows = (1u << (NB + 1)) - 2u;
-constexpr uint32_t kRowsHeld = NT == 32 ? 0xFFFFFFFFu : (1u << NT) - 1u;
+constexpr uint32_t kRowsHeld = (1u << NT) - 1u;
+constexpr int NSUB = 2;         // sub-bands of a band: the output's segments
+constexpr int SUBR = NB / NSUB; // rows of a sub-band
+constexpr uint32_t kSubRows = (2u << SUBR) - 2u;  // bits 1..SUBR
 constexpr int NCOL = 30;        // owned columns per warp (lanes 1..30)
-constexpr int NODE_WARPS = 8;   // warps per CTA
-constexpr int kSlots = 3;       // plane slots of a warp's ring: p - 1, p, p + 1
+constexpr int NODE_WARPS = 4;   // warps per CTA
+constexpr int kSlots = 2;       // plane slots of a warp's ring: p, p + 1
+constexpr long long kItemsPerWarp = 4;  // work items per resident warp
 constexpr uint32_t kChunk = 4096;  // staging records a warp reserves at a time
-// table entry: base, count, then one row-count byte per row (NT bytes)
-constexpr int kTabVec = (2 + NT / 4 + 3) / 4;
-constexpr size_t kRingFloats2 = (size_t)NODE_WARPS * kSlots * NT * 32;
-// the rings, then NT bytes of per-row counts per warp, then per warp and row
-// the lane mask and the prefix of the step's records
-constexpr size_t kNodeSmem =
-    kRingFloats2 * sizeof(float2) + NODE_WARPS * NT + NODE_WARPS * 2 * NT * sizeof(uint32_t);
-static_assert(NT == 16 || NT == 32, "rows per band");
+// A slot holds row pairs: rows 2 q and 2 q + 1 of a column are 16 consecutive
+// bytes, one load.
+constexpr int kSlotLen = NT * 32;  // elements
+__host__ __device__ constexpr int slot_at(int t) { return t * 32; }  // of lane 0
+constexpr size_t kNodeSmem = (size_t)NODE_WARPS * kSlots * kSlotLen * sizeof(float2);
+static_assert(SUBR * NSUB == NB && SUBR < 16, "sub-bands fill a band, 16 bits a row word of a record");
 constexpr int DENS_THREADS = 256;
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -144,55 +155,45 @@ __device__ __forceinline__ EW edge_w(uint32_t sa, uint32_t sb, uint32_t n, uint3
   e.N = sa & ~sb & n & ~E;
   return e;
 }
-__device__ __forceinline__ EW shl(EW e) { return EW{e.P << 1, e.N << 1}; }
 __device__ __forceinline__ EW shr(EW e) { return EW{e.P >> 1, e.N >> 1}; }
-__device__ __forceinline__ EW sh_up(EW e) {
-  return EW{__shfl_up_sync(FULL, e.P, 1), __shfl_up_sync(FULL, e.N, 1)};
-}
 __device__ __forceinline__ EW sh_dn(EW e) {
   return EW{__shfl_down_sync(FULL, e.P, 1), __shfl_down_sync(FULL, e.N, 1)};
 }
 
-// full adder on bit-sliced words
-__device__ __forceinline__ void fa(uint32_t a, uint32_t b, uint32_t c, uint32_t& s, uint32_t& cy) {
-  s = a ^ b ^ c;
-  cy = (a & b) | (c & (a ^ b));
-}
-
-// Sum mod 8 of eight terms in {-1, 0, 1} given as (nonzero, negative) words:
-// S = #nonzero - 2 #negative.  A ring of finite nodes has |S| <= 3 unless all
-// eight of its edge differences are exact +-pi ties (S = +-4, read as 4), so
-// the residue in [-3, 4] is S.
+// bit-sliced residues mod 8
 struct Mod8 {
   uint32_t b0, b1, b2;
 };
-__device__ __forceinline__ Mod8 ring_sum(const uint32_t z[8], const uint32_t g[8]) {
-  uint32_t s1, c1, s2, c2, c4, t1, c5;
-  fa(z[0], z[1], z[2], s1, c1);
-  fa(z[3], z[4], z[5], s2, c2);
-  const uint32_t s3 = z[6] ^ z[7], c3 = z[6] & z[7];
-  uint32_t a0, a1;
-  fa(s1, s2, s3, a0, c4);
-  fa(c1, c2, c3, t1, c5);
-  a1 = t1 ^ c4;
-  const uint32_t a2 = c5 ^ (t1 & c4);
-  // negatives mod 4
-  uint32_t u1, d1c, u2, d2c, d4, v1, d5;
-  fa(g[0], g[1], g[2], u1, d1c);
-  fa(g[3], g[4], g[5], u2, d2c);
-  const uint32_t u3 = g[6] ^ g[7], d3c = g[6] & g[7];
-  uint32_t e0;
-  fa(u1, u2, u3, e0, d4);
-  fa(d1c, d2c, d3c, v1, d5);
-  const uint32_t e1 = v1 ^ d4;
-  (void)d5;
-  // S = a - 2 e (mod 8)
+
+// a + b - c - d (each -1, 0 or 1): #nonzero - 2 #negative
+__device__ __forceinline__ Mod8 loop_sum(EW a, EW b, EW c, EW d) {
+  const uint32_t za = a.P | a.N, zb = b.P | b.N, zc = c.P | c.N, zd = d.P | d.N;
+  const uint32_t ab = za & zb, cd = zc & zd, xab = za ^ zb, xcd = zc ^ zd;
+  const uint32_t z1 = ab ^ cd ^ (xab & xcd);
+  // negative terms: a, b where -1; c, d where +1
+  const uint32_t gab = a.N ^ b.N, gcd = c.P ^ d.P;
+  const uint32_t g0 = gab ^ gcd, g1 = (a.N & b.N) ^ (c.P & d.P) ^ (gab & gcd);
   Mod8 r;
-  r.b0 = a0;
-  r.b1 = a1 ^ e0;
-  r.b2 = a2 ^ e1 ^ (~a1 & e0);
+  r.b0 = xab ^ xcd;
+  r.b1 = z1 ^ g0;
+  r.b2 = (ab & cd) ^ g1 ^ (~z1 & g0);
   return r;
 }
+
+__device__ __forceinline__ Mod8 add8(Mod8 a, Mod8 b) {
+  const uint32_t c0 = a.b0 & b.b0;
+  const uint32_t c1 = (a.b1 & b.b1) | (c0 & (a.b1 ^ b.b1));
+  return Mod8{a.b0 ^ b.b0, a.b1 ^ b.b1 ^ c0, a.b2 ^ b.b2 ^ c1};
+}
+// with the row below (bit t: rows t - 1 and t), with the column to the left
+__device__ __forceinline__ Mod8 add_row(Mod8 a) {
+  return add8(a, Mod8{a.b0 << 1, a.b1 << 1, a.b2 << 1});
+}
+__device__ __forceinline__ Mod8 add_col(Mod8 a) {
+  return add8(a, Mod8{__shfl_up_sync(FULL, a.b0, 1), __shfl_up_sync(FULL, a.b1, 1),
+                      __shfl_up_sync(FULL, a.b2, 1)});
+}
+__device__ __forceinline__ uint32_t nonzero8(Mod8 a) { return a.b0 | a.b1 | a.b2; }
 
 // value in [-3, 4] of row t of a residue
 __device__ __forceinline__ int mod8_at(const Mod8& m, int t) {
@@ -206,10 +207,11 @@ struct NodeArgs {
   int nx, ny, nz;
   int nbands, nxseg, kchunk;
   long long nitems;               // z chunks * bands * column segments
-  unsigned long long* recs;
+  uint4* recs;                    // words 0..3 of the records
+  uint32_t* recs4;                // word 4
   unsigned long long recs_cap;
-  unsigned long long* top;        // staging chunk counter
-  uint4* table;                   // [nz][nbands][nxseg][3]
+  unsigned long long* top;        // staging chunk counter, work item counter
+  uint2* table;                   // [nz][nbands][nxseg] {staging base, lane mask}
   unsigned int* segtot;           // [nz][nbands], zeroed before the launch
   int8_t* dense;                  // [3][nz][ny][nx] or null
 };
@@ -230,27 +232,29 @@ __device__ __forceinline__ void cp_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Each lane streams its column of the band (32 rows) through the warp's ring
-// with cp.async; a lane also reads its right neighbour's column, so every
-// slot is fenced by __syncwarp after its copies complete and before it is
-// refilled.  Rows, columns and planes outside the grid hold (1, 1): finite
-// and nonzero, and only ever on rings that the validity masks reject.
-__global__ void __launch_bounds__(NODE_WARPS * 32) node_form_kernel(NodeArgs a) {
+// Each lane streams its column of the band through the warp's ring with
+// cp.async; a lane also reads its right neighbour's column, so every slot is
+// fenced by __syncwarp after its copies complete and before it is refilled.
+// Rows, columns and planes outside the grid hold (1, 1): finite and nonzero, and
+// only ever on rings that the validity masks reject.
+__global__ void __launch_bounds__(NODE_WARPS * 32, 4) node_form_kernel(const __grid_constant__ NodeArgs a) {
   extern __shared__ float2 node_ring[];
   const int lane = threadIdx.x & 31;
-  float2* ring = node_ring + (size_t)(threadIdx.x >> 5) * kSlots * NT * 32;
-  uint8_t* rcnt = reinterpret_cast<uint8_t*>(node_ring + kRingFloats2) + (threadIdx.x >> 5) * NT;
-  // per row: lane mask of the vortex nodes and records of the rows before it
-  uint32_t* rbal = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(node_ring + kRingFloats2) +
-                                               NODE_WARPS * NT) + (threadIdx.x >> 5) * 2 * NT;
-  uint32_t* rpre = rbal + NT;
+  float2* ring = node_ring + (size_t)(threadIdx.x >> 5) * kSlots * kSlotLen;
   const long long nwarps = (long long)gridDim.x * NODE_WARPS;
   const long long nxyz = (long long)a.nx * a.ny * a.nz;
   const unsigned lt = (1u << lane) - 1u;
+  const int ln = lane < 31 ? lane + 1 : 31;
   unsigned long long chunk_at = 0;  // next free staging record of the warp's chunk
   uint32_t chunk_left = 0;
-  for (long long it = (long long)blockIdx.x * NODE_WARPS + (threadIdx.x >> 5); it < a.nitems;
-       it += nwarps) {
+  const long long first = (long long)blockIdx.x * NODE_WARPS + (threadIdx.x >> 5);
+  // the first items by warp, the others as warps get free
+  auto next = [&]() {
+    unsigned long long v = 0;
+    if (lane == 0) v = atomicAdd(a.top + 1, 1ull);
+    return nwarps + (long long)__shfl_sync(FULL, v, 0);
+  };
+  for (long long it = first; it < a.nitems; it = next()) {
     const int xs = (int)(it % a.nxseg);
     const long long rest = it / a.nxseg;
     const int band = (int)(rest % a.nbands);
@@ -262,65 +266,74 @@ __global__ void __launch_bounds__(NODE_WARPS * 32) node_form_kernel(NodeArgs a) 
     const bool xin = x >= 0 && x < a.nx;
     const bool own = lane >= 1 && lane <= NCOL && x < a.nx;
     const bool colring = x >= 1 && x <= a.nx - 2;
-    uint32_t rload = 0, rring = 0;  // rows in the grid / rows whose y-ring fits
-    for (int t = 0; t < NT; ++t) {
-      const int j = j0 - 1 + t;
-      if (j >= 0 && j < a.ny) rload |= 1u << t;
-      if (j >= 1 && j <= a.ny - 2) rring |= 1u << t;
-    }
+    // rows in the grid (t in [lo, hi)), rows whose y-ring fits
+    const int lo = j0 == 0 ? 1 : 0, hi = min(NT, a.ny - j0 + 1);
+    const uint32_t rload = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
     const uint32_t rin = rload & kOwnedRows;
-    rring &= kOwnedRows;
+    const uint32_t rring = rload & (rload << 1) & (rload >> 1) & kOwnedRows;
+    const float2* const col = a.psi + (long long)(j0 - 1) * a.nx + x;
+    const long long plane = (long long)a.nx * a.ny;
 
-    // plane q (kz0 - 1 <= q <= kz1) lives in slot (q - kz0 + 1) mod kSlots
     auto issue = [&](int q, int slot) {
-      float2* d = ring + slot * NT * 32 + lane;
+      float2* d = ring + slot * kSlotLen + lane;
       const bool qin = q >= 0 && q < a.nz && xin;
-      const float2* src = a.psi + ((long long)(qin ? q : 0) * a.ny + (j0 - 1)) * a.nx + x;
+      const float2* src = col + (long long)q * plane;
+      if (qin && rload == kRowsHeld) {
 #pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        if (qin && ((rload >> t) & 1u)) cp_async8(d + t * 32, src);
-        else d[t * 32] = make_float2(1.f, 1.f);
-        src += a.nx;
+        for (int t = 0; t < NT; ++t) {
+          cp_async8(d + slot_at(t), src);
+          src += a.nx;
+        }
+      } else {
+#pragma unroll 1
+        for (int t = 0; t < NT; ++t) {
+          if (qin && ((rload >> t) & 1u)) cp_async8(d + slot_at(t), src);
+          else d[slot_at(t)] = make_float2(1.f, 1.f);
+          src += a.nx;
+        }
       }
       cp_commit();
     };
+    // planes kz0 - 1 .. kz1; plane q in slot (q - kz0 + 1) mod kSlots
     __syncwarp();
     issue(kz0 - 1, 0);
+    issue(kz0, 1);
     int sp = 0;  // slot of plane p
 
-    EW RXm{0, 0}, RXc{0, 0}, RYm{0, 0}, RYc{0, 0}, RZlo{0, 0};
+    float2 V[NT];  // values of the previous plane
+#pragma unroll
+    for (int t = 0; t < NT; ++t) V[t] = make_float2(1.f, 1.f);
+    EW RXc{0, 0}, RYc{0, 0};
+    Mod8 S0c{0, 0, 0}, Tc{0, 0, 0}, Uc{0, 0, 0};  // xy ring sums of plane p - 1; yz, zx sums of
+                                                  // the layer below it
     uint32_t Sprev = 0, ZBc = 0, Bm = 0, Bc = 0;
 
     for (int p = kz0 - 1; p <= kz1; ++p) {
-      __syncwarp();  // every lane is done with the slot of plane p - 2
-      const int s1 = sp + 1 == kSlots ? 0 : sp + 1;
-      if (p + 1 <= kz1) issue(p + 1, s1);
-      else cp_commit();
-      cp_wait<1>();  // plane p has landed (this lane's copies)
+      cp_wait<kSlots - 1>();  // plane p has landed (this lane's copies)
       __syncwarp();  // ... and every lane's
-      const float2* cur = ring + sp * NT * 32;
-      const float2* prv = (p == kz0 - 1) ? cur : ring + (sp == 0 ? kSlots - 1 : sp - 1) * NT * 32;
-      const int ln = lane < 31 ? lane + 1 : 31;
+      const float2* cur = ring + sp * kSlotLen;
       uint32_t Sp = 0, NX = 0, NY = 0, NZ = 0;
       unsigned long long prod = kProdOne;
-      float2 vup = make_float2(1.f, 1.f);
-#pragma unroll (NT == 16 ? 16 : 4)
+#pragma unroll
       for (int t = NT - 1; t >= 0; --t) {
         const float2 v = cur[t * 32 + lane];
         const float2 nb = cur[t * 32 + ln];
-        const float2 pv = prv[t * 32 + lane];
         Sp = push1(Sp, v.y);
         NX = push1(NX, cross_f(v, nb));
-        NZ = push1(NZ, cross_f(pv, v));
-        NY = push1(NY, cross_f(v, vup));
+        NZ = push1(NZ, cross_f(V[t], v));
+        if (t < NT - 1) NY = push1(NY, cross_f(v, V[t + 1]));
         prod = prod_step(prod, v);
-        vup = v;
+        V[t] = v;
       }
-      NY &= kRowsHeld >> 1;  // the top row has no y-edge in the band
+      __syncwarp();  // every lane is done with the slot
+      if (p + kSlots <= kz1) issue(p + kSlots, sp);
+      else cp_commit();
+      sp = sp + 1 == kSlots ? 0 : sp + 1;
       uint32_t ZBp = 0, Bn = 0;
       if (__any_sync(FULL, prod_special(prod))) {
+#pragma unroll
         for (int t = 0; t < NT; ++t) {
-          const float2 v = cur[t * 32 + lane];
+          const float2 v = V[t];
           if (((__float_as_uint(v.x) | __float_as_uint(v.y)) << 1) == 0u) ZBp |= 1u << t;
           if (!(fin(v.x) && fin(v.y))) Bn |= 1u << t;
         }
@@ -330,231 +343,256 @@ __global__ void __launch_bounds__(NODE_WARPS * 32) node_form_kernel(NodeArgs a) 
       const uint32_t ZBpn = __shfl_down_sync(FULL, ZBp, 1);
       const EW RXn = edge_w(Sp, Spn, NX, ZBp | ZBpn);
       const EW RYn = edge_w(Sp, Sp >> 1, NY, ZBp | (ZBp >> 1));
-      const EW RZhi = edge_w(Sprev, Sp, NZ, ZBc | ZBp);  // edges p - 1 -> p
+      const EW RZ = edge_w(Sprev, Sp, NZ, ZBc | ZBp);  // edges p - 1 -> p
+      const Mod8 S0n = add_col(add_row(loop_sum(RXn, sh_dn(RYn), shr(RXn), RYn)));
+      // layer p - 1 -> p
+      const Mod8 T = add_row(loop_sum(RYc, shr(RZ), RYn, RZ));
+      const Mod8 U = add_col(loop_sum(RZ, RXn, sh_dn(RZ), RXc));
       if (p > kz0) {
-        // finalize node plane k = p - 1: planes k - 1, k, k + 1 are m, c, n
+        // node plane k = p - 1
         const int k = p - 1;
         const bool kring = k >= 1 && k <= a.nz - 2;
-        const uint32_t Bl = __shfl_up_sync(FULL, Bc, 1), Br = __shfl_down_sync(FULL, Bc, 1);
-        const uint32_t H = Bl | Bc | Br;
-        const uint32_t bad0 = (H << 1) | (H >> 1) | Bl | Br;
-        const uint32_t V = Bm | Bc | Bn;
-        const uint32_t bad1 = (V << 1) | (V >> 1) | Bm | Bn;
-        const uint32_t bad2 =
-            __shfl_up_sync(FULL, V, 1) | __shfl_down_sync(FULL, V, 1) | Bm | Bn;
-        const uint32_t ok0 = (own && colring) ? (rring & ~bad0) : 0u;
-        const uint32_t ok1 = (own && kring) ? (rring & ~bad1) : 0u;
-        const uint32_t ok2 = (own && colring && kring) ? (rin & ~bad2) : 0u;
-        Mod8 S0, S1, S2;
-        {  // xy ring
-          const EW xl = sh_up(RXc), yr = sh_dn(RYc), yl = sh_up(RYc);
-          const EW t1 = shl(xl), t2 = shl(RXc), t3 = shl(yr), t4 = yr;  // + terms
-          const EW t5 = shr(RXc), t6 = shr(xl), t7 = yl, t8 = shl(yl);  // - terms
-          const uint32_t z[8] = {t1.P | t1.N, t2.P | t2.N, t3.P | t3.N, t4.P | t4.N,
-                                 t5.P | t5.N, t6.P | t6.N, t7.P | t7.N, t8.P | t8.N};
-          const uint32_t g[8] = {t1.N, t2.N, t3.N, t4.N, t5.P, t6.P, t7.P, t8.P};
-          S0 = ring_sum(z, g);
+        const Mod8 S1 = add8(Tc, T), S2 = add8(Uc, U);
+        uint32_t ok0 = (own && colring) ? rring : 0u;
+        uint32_t ok1 = (own && kring) ? rring : 0u;
+        uint32_t ok2 = (own && colring && kring) ? rin : 0u;
+        if (__any_sync(FULL, (Bm | Bc | Bn) != 0u)) {  // rings through non-finite nodes
+          const uint32_t Bl = __shfl_up_sync(FULL, Bc, 1), Br = __shfl_down_sync(FULL, Bc, 1);
+          const uint32_t H = Bl | Bc | Br;
+          const uint32_t V = Bm | Bc | Bn;
+          ok0 &= ~((H << 1) | (H >> 1) | Bl | Br);
+          ok1 &= ~((V << 1) | (V >> 1) | Bm | Bn);
+          ok2 &= ~(__shfl_up_sync(FULL, V, 1) | __shfl_down_sync(FULL, V, 1) | Bm | Bn);
         }
-        {  // yz ring (u = y, v = z)
-          const EW t1 = shl(RYm), t2 = RYm, t3 = shr(RZlo), t4 = shr(RZhi);  // + terms
-          const EW t5 = shl(RYn), t6 = RYn, t7 = shl(RZlo), t8 = shl(RZhi);  // - terms
-          const uint32_t z[8] = {t1.P | t1.N, t2.P | t2.N, t3.P | t3.N, t4.P | t4.N,
-                                 t5.P | t5.N, t6.P | t6.N, t7.P | t7.N, t8.P | t8.N};
-          const uint32_t g[8] = {t1.N, t2.N, t3.N, t4.N, t5.P, t6.P, t7.P, t8.P};
-          S1 = ring_sum(z, g);
-        }
-        {  // zx ring (u = z, v = x), all terms at the node's row
-          const EW t1 = sh_up(RZlo), t2 = sh_up(RZhi), t3 = sh_up(RXn), t4 = RXn;  // + terms
-          const EW t5 = sh_dn(RZlo), t6 = sh_dn(RZhi), t7 = sh_up(RXm), t8 = RXm;  // - terms
-          const uint32_t z[8] = {t1.P | t1.N, t2.P | t2.N, t3.P | t3.N, t4.P | t4.N,
-                                 t5.P | t5.N, t6.P | t6.N, t7.P | t7.N, t8.P | t8.N};
-          const uint32_t g[8] = {t1.N, t2.N, t3.N, t4.N, t5.P, t6.P, t7.P, t8.P};
-          S2 = ring_sum(z, g);
-        }
-        const uint32_t nz0 = (S0.b0 | S0.b1 | S0.b2) & ok0;
-        const uint32_t nz1 = (S1.b0 | S1.b1 | S1.b2) & ok1;
-        const uint32_t nz2 = (S2.b0 | S2.b1 | S2.b2) & ok2;
-        const uint32_t F = nz0 | nz1 | nz2;  // vortex nodes of this lane's owned rows
+        const uint32_t F = (nonzero8(S0c) & ok0) | (nonzero8(S1) & ok1) | (nonzero8(S2) & ok2);
         if (a.dense && own) {
 #pragma unroll 1
           for (int t = 1; t <= NB; ++t) {
             if (!((rin >> t) & 1u)) continue;
             const long long q = ((long long)k * a.ny + (j0 - 1 + t)) * a.nx + x;
-            a.dense[q] = (int8_t)(((ok0 >> t) & 1u) ? mod8_at(S0, t) : 0);
+            a.dense[q] = (int8_t)(((ok0 >> t) & 1u) ? mod8_at(S0c, t) : 0);
             a.dense[nxyz + q] = (int8_t)(((ok1 >> t) & 1u) ? mod8_at(S1, t) : 0);
             a.dense[2 * nxyz + q] = (int8_t)(((ok2 >> t) & 1u) ? mod8_at(S2, t) : 0);
           }
         }
-        const uint32_t cnt = __reduce_add_sync(FULL, (uint32_t)__popc(F));
-        const uint32_t rows_any = __reduce_or_sync(FULL, F);
-        // records of this step: contiguous in the warp's staging chunk, row-major
-        if (cnt > chunk_left) {
-          unsigned long long b = 0;
-          if (lane == 0) b = atomicAdd(a.top, (unsigned long long)kChunk);
-          chunk_at = __shfl_sync(FULL, b, 0);
-          chunk_left = kChunk;
-        }
-        const unsigned long long base = chunk_at;
-        chunk_at += cnt;
-        chunk_left -= cnt;
-        // uniform pass over the rows with vortex nodes: each row's lane mask
-        // and the records before it (warp-private shared memory); then every
-        // lane writes its own records
-        if (lane < NT / 4) reinterpret_cast<uint32_t*>(rcnt)[lane] = 0u;  // bytes of rows 1..NB
-        __syncwarp();
-        uint32_t run = 0;
-#pragma unroll 1
-        for (uint32_t rem = rows_any; rem; rem &= rem - 1u) {
-          const int t = __ffs(rem) - 1;
-          const unsigned bal = __ballot_sync(FULL, (F >> t) & 1u);
+        // records of this step, by sub-band: contiguous in the warp's staging chunk
+#pragma unroll
+        for (int sb = 0; sb < NSUB; ++sb) {
+          const int sh = sb * SUBR;
+          const uint32_t Fs = (F >> sh) & kSubRows;
+          const uint32_t cnt = __reduce_add_sync(FULL, (uint32_t)__popc(Fs));
+          const uint32_t bal = __ballot_sync(FULL, Fs != 0u);
+          const uint32_t nrec = (uint32_t)__popc(bal);
+          if (nrec > chunk_left) {
+            unsigned long long b = 0;
+            if (lane == 0) b = atomicAdd(a.top, (unsigned long long)kChunk);
+            chunk_at = __shfl_sync(FULL, b, 0);
+            chunk_left = kChunk;
+          }
+          const unsigned long long base = chunk_at;
+          chunk_at += nrec;
+          chunk_left -= nrec;
+          if (Fs) {
+            const unsigned long long q = base + (unsigned)__popc(bal & lt);
+            if (q < a.recs_cap) {
+              auto two = [&](uint32_t u, uint32_t v) {
+                return ((u >> sh) & kSubRows) | (((v >> sh) & kSubRows) << 16);
+              };
+              a.recs[q] = make_uint4(two(S0c.b0 & ok0, S0c.b1 & ok0), two(S0c.b2 & ok0, S1.b0 & ok1),
+                                     two(S1.b1 & ok1, S1.b2 & ok1), two(S2.b0 & ok2, S2.b1 & ok2));
+              a.recs4[q] = (((S2.b2 & ok2) >> sh) & kSubRows) | ((uint32_t)lane << 16);
+            }
+          }
           if (lane == 0) {
-            rbal[t] = bal;
-            rpre[t] = run;
-            rcnt[t - 1] = (uint8_t)__popc(bal);
+            const long long sg = (long long)k * (a.nbands * NSUB) + band * NSUB + sb;
+            if (cnt) atomicAdd(a.segtot + sg, cnt);
+            a.table[sg * a.nxseg + xs] = make_uint2((uint32_t)base, bal);
           }
-          run += (uint32_t)__popc(bal);
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (uint32_t mine = F; mine; mine &= mine - 1u) {
-          const int t = __ffs(mine) - 1;
-          const unsigned long long q =
-              base + rpre[t] + (unsigned long long)__popc(rbal[t] & lt);
-          if (q < a.recs_cap) {
-            const int v0 = ((ok0 >> t) & 1u) ? mod8_at(S0, t) : 0;
-            const int v1 = ((ok1 >> t) & 1u) ? mod8_at(S1, t) : 0;
-            const int v2 = ((ok2 >> t) & 1u) ? mod8_at(S2, t) : 0;
-            const unsigned long long lin =
-                ((unsigned long long)k * a.ny + (unsigned long long)(j0 - 1 + t)) * a.nx + x;
-            a.recs[q] = (lin << 12) | (uint32_t)(v0 + 4) | ((uint32_t)(v1 + 4) << 4) |
-                        ((uint32_t)(v2 + 4) << 8);
-          }
-        }
-        __syncwarp();
-        if (lane == 0) {
-          if (cnt) atomicAdd(a.segtot + (long long)k * a.nbands + band, cnt);
-          const uint32_t* rc = reinterpret_cast<const uint32_t*>(rcnt);
-          uint32_t wv[4 * kTabVec] = {};
-          wv[0] = (uint32_t)base;
-          wv[1] = cnt;
-#pragma unroll
-          for (int q = 0; q < NT / 4; ++q) wv[2 + q] = rc[q];
-          uint4* te = a.table + (((long long)k * a.nbands + band) * a.nxseg + xs) * kTabVec;
-#pragma unroll
-          for (int q = 0; q < kTabVec; ++q)
-            te[q] = make_uint4(wv[4 * q], wv[4 * q + 1], wv[4 * q + 2], wv[4 * q + 3]);
         }
       }
-      RXm = RXc;
       RXc = RXn;
-      RYm = RYc;
       RYc = RYn;
-      RZlo = RZhi;
+      S0c = S0n;
+      Tc = T;
+      Uc = U;
       Sprev = Sp;
       ZBc = ZBp;
       Bm = Bc;
       Bc = Bn;
-      sp = s1;
     }
+    cp_wait<0>();
+    __syncwarp();
   }
 }
 
 // Exclusive scan of the per-(plane, band) totals, (plane, band) order being
-// ascending node order.  One block.
+// ascending node order.  A block per kScanChunk totals, which adds the ones before
+// them itself (one block over all of them: 12 us for 1e4 totals).
+constexpr int kScanPer = 4;  // consecutive totals per thread
+constexpr int kScanChunk = 1024 * kScanPer;
+
 __global__ void __launch_bounds__(1024) node_scan_kernel(const unsigned int* __restrict__ segtot,
                                                          long long nseg,
                                                          unsigned long long* __restrict__ seg_off,
                                                          uint64_t* __restrict__ count) {
-  __shared__ unsigned long long warp_tot[32];
+  __shared__ unsigned long long wb[32], wt[32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const long long per = (nseg + blockDim.x - 1) / blockDim.x;
-  const long long s0 = tid * per, s1 = min(nseg, s0 + per);
-  unsigned long long local = 0;
-  for (long long s = s0; s < s1; ++s) local += segtot[s];
+  const long long s0 = (long long)blockIdx.x * kScanChunk, s = s0 + tid * kScanPer;
+  unsigned long long v[kScanPer], local = 0, before = 0;
+#pragma unroll
+  for (int i = 0; i < kScanPer; ++i) {
+    v[i] = s + i < nseg ? segtot[s + i] : 0u;
+    local += v[i];
+  }
+#pragma unroll 8
+  for (long long i = tid; i < s0; i += 1024) before += segtot[i];
   unsigned long long incl = local;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
     const unsigned long long u = __shfl_up_sync(FULL, incl, d);
     if (lane >= d) incl += u;
   }
-  if (lane == 31) warp_tot[w] = incl;
-  __syncthreads();
-  if (w == 0) {
-    const unsigned long long v = lane < (int)(blockDim.x >> 5) ? warp_tot[lane] : 0ull;
-    unsigned long long iv = v;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const unsigned long long u = __shfl_up_sync(FULL, iv, d);
-      if (lane >= d) iv += u;
-    }
-    warp_tot[lane] = iv - v;
-    if (lane == 31) *count = iv;
-  }
+  for (int d = 16; d; d >>= 1) before += __shfl_xor_sync(FULL, before, d);
+  if (lane == 31) wt[w] = incl;
+  if (lane == 0) wb[w] = before;
   __syncthreads();
-  unsigned long long run = warp_tot[w] + incl - local;
-  for (long long s = s0; s < s1; ++s) {
-    seg_off[s] = run;
-    run += segtot[s];
+  unsigned long long run = incl - local;
+  for (int q = 0; q < 32; ++q) run += wb[q] + (q < w ? wt[q] : 0ull);
+#pragma unroll
+  for (int i = 0; i < kScanPer; ++i) {
+    if (s + i < nseg) seg_off[s + i] = run;
+    run += v[i];
   }
+  if (blockIdx.x == gridDim.x - 1 && tid == 1023) *count = run;
 }
 
-// One warp per (plane, band): for each row in turn, the column segments in
-// ascending x (lane = segment), each copying its staged records of that row.
-__global__ void node_scatter_kernel(const uint4* __restrict__ table,
-                                    const unsigned long long* __restrict__ seg_off, long long nseg,
-                                    int nxseg, const unsigned long long* __restrict__ recs,
-                                    unsigned long long recs_cap, uint64_t* __restrict__ node_ids,
-                                    int8_t* __restrict__ circ, unsigned long long capacity) {
+// One warp per (plane, band): its records, by column segment and lane, i.e. by
+// ascending x, give its nodes row by row: per row and 32 records one ballot ranks
+// the records with a node there.  Records of up to kHeldRecs x 32 lanes stay in
+// registers (a sub-band of a 512-column tangle has about 100); larger segments read
+// them again for each row.
+constexpr int kHeldRecs = 5;
+constexpr int kMaxSegs = (64 * kMaxWarpsX + NCOL - 1) / NCOL;
+constexpr int kMaxE = (kMaxSegs + 31) / 32;  // table entries per lane
+static_assert(kMaxE == 3, "the entry selection below handles three entries per lane");
+
+struct NodeRec {
+  uint4 w;
+  uint32_t w4, x;
+  __device__ __forceinline__ uint32_t rows() const {
+    const uint32_t m = w.x | w.y | w.z | w.w;
+    return (m | (m >> 16) | w4) & 0xFFFFu;
+  }
+};
+
+__global__ void __launch_bounds__(256) node_expand_kernel(
+    const uint2* __restrict__ table, const unsigned long long* __restrict__ seg_off, long long nseg,
+    int nbands, int nxseg, int nx, int ny, const uint4* __restrict__ recs,
+    const uint32_t* __restrict__ recs4, unsigned long long recs_cap, uint64_t* __restrict__ node_ids,
+    int8_t* __restrict__ circ, unsigned long long capacity) {
   const int lane = threadIdx.x & 31;
+  const unsigned lt = (1u << lane) - 1u;
   const long long warps = ((long long)gridDim.x * blockDim.x) >> 5;
+  const int E = (nxseg + 31) >> 5, NL = (nxseg + E - 1) / E;  // lane l holds segments l E ..
   for (long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nseg;
        s += warps) {
-    unsigned long long off = seg_off[s];
-    const uint4* te = table + s * nxseg * kTabVec;
-    for (int t = 1; t <= NB; ++t) {
-      for (int xb = 0; xb < nxseg; xb += 32) {
-        const int xsi = xb + lane;
-        uint32_t wv[4 * kTabVec] = {};
-        if (xsi < nxseg) {
+    uint2 en[kMaxE];
+    uint32_t n = 0;
 #pragma unroll
-          for (int q = 0; q < kTabVec; ++q) {
-            const uint4 e = te[xsi * kTabVec + q];
-            wv[4 * q] = e.x;
-            wv[4 * q + 1] = e.y;
-            wv[4 * q + 2] = e.z;
-            wv[4 * q + 3] = e.w;
+    for (int j = 0; j < kMaxE; ++j) {
+      const int i = lane * E + j;
+      en[j] = (j < E && i < nxseg) ? table[s * nxseg + i] : make_uint2(0u, 0u);
+      n += __popc(en[j].y);
+    }
+    const unsigned long long off = seg_off[s];
+    uint32_t incl = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const uint32_t u = __shfl_up_sync(FULL, incl, d);
+      if (lane >= d) incl += u;
+    }
+    const uint32_t start = lane < NL ? incl - n : 0xFFFFFFFFu;
+    const uint32_t rtot = __shfl_sync(FULL, incl, 31);
+    if (rtot == 0) continue;
+    const long long k = s / nbands;
+    const long long j0 = (s - k * nbands) * SUBR;
+    const unsigned long long lin0 =  // of row t = 0 (only rows t >= 1 are used)
+        ((unsigned long long)k * ny + (unsigned long long)j0) * (unsigned long long)nx - (unsigned long long)nx;
+    // record of index g0 + lane in x order (no rows past the end)
+    auto load = [&](uint32_t g0) -> NodeRec {
+      const uint32_t g = g0 + lane;
+      int lo = 0;
+#pragma unroll
+      for (int st = 16; st >= 1; st >>= 1) {
+        const int cand = lo + st;
+        const uint32_t sv = __shfl_sync(FULL, start, cand & 31);
+        if (cand < NL && sv <= g) lo = cand;
+      }
+      uint32_t qi = g - __shfl_sync(FULL, start, lo);
+      uint2 e = make_uint2(__shfl_sync(FULL, en[0].x, lo), __shfl_sync(FULL, en[0].y, lo));
+      int j = 0;
+      if (E > 1) {  // uniform
+        const uint2 e1 = make_uint2(__shfl_sync(FULL, en[1].x, lo), __shfl_sync(FULL, en[1].y, lo));
+        const uint2 e2 = make_uint2(__shfl_sync(FULL, en[2].x, lo), __shfl_sync(FULL, en[2].y, lo));
+        const uint32_t c0 = __popc(e.y), c1 = __popc(e1.y);
+        if (qi >= c0) {
+          qi -= c0;
+          j = 1;
+          e = e1;
+          if (qi >= c1) {
+            qi -= c1;
+            j = 2;
+            e = e2;
           }
         }
-        const uint32_t base = wv[0];
-        const uint32_t* rcw = wv + 2;
-        uint32_t c = 0, pre = 0;
-#pragma unroll
-        for (int r = 1; r <= NB; ++r) {
-          const uint32_t cr = (rcw[(r - 1) >> 2] >> (8 * ((r - 1) & 3))) & 0xFFu;
-          if (r < t) pre += cr;
-          if (r == t) c = cr;
-        }
-        // exclusive scan of c over the lanes
-        uint32_t incl = c;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const uint32_t u = __shfl_up_sync(FULL, incl, d);
-          if (lane >= d) incl += u;
-        }
-        const uint32_t tot = __shfl_sync(FULL, incl, 31);
-        const unsigned long long dst0 = off + (incl - c);
-        const unsigned long long src0 = (unsigned long long)base + pre;
-        for (uint32_t q = 0; q < c; ++q) {
-          const unsigned long long src = src0 + q, dst = dst0 + q;
-          if (src >= recs_cap || dst >= capacity) continue;
-          const unsigned long long rec = recs[src];
-          node_ids[dst] = rec >> 12;
-          circ[3 * dst] = (int8_t)((int)(rec & 15u) - 4);
-          circ[3 * dst + 1] = (int8_t)((int)((rec >> 4) & 15u) - 4);
-          circ[3 * dst + 2] = (int8_t)((int)((rec >> 8) & 15u) - 4);
-        }
-        off += tot;
       }
+      NodeRec r;
+      r.w = make_uint4(0u, 0u, 0u, 0u);
+      r.w4 = r.x = 0u;
+      const unsigned long long idx = (unsigned long long)e.x + qi;
+      if (g < rtot && idx < recs_cap) {
+        r.w = recs[idx];
+        r.w4 = recs4[idx];
+        r.x = (uint32_t)((lo * E + j) * NCOL - 1) + (r.w4 >> 16);
+      }
+      return r;
+    };
+    uint32_t run = 0;  // nodes of the segment so far
+    // the records' nodes of row t, after those already listed
+    auto emit = [&](const NodeRec& r, int t) {
+      const bool has = (r.rows() >> t) & 1u;
+      const unsigned bal = __ballot_sync(FULL, has);
+      if (has) {
+        const unsigned long long dst = off + run + (unsigned)__popc(bal & lt);
+        if (dst < capacity) {
+          auto val = [&](uint32_t b0, uint32_t b1, uint32_t b2) {
+            const int v = (int)(b0 & 1u) | (int)((b1 & 1u) << 1) | (int)((b2 & 1u) << 2);
+            return (int8_t)(v >= 5 ? v - 8 : v);
+          };
+          node_ids[dst] = lin0 + (unsigned long long)((uint32_t)t * (uint32_t)nx + r.x);
+          circ[3 * dst] = val(r.w.x >> t, r.w.x >> (t + 16), r.w.y >> t);
+          circ[3 * dst + 1] = val(r.w.y >> (t + 16), r.w.z >> t, r.w.z >> (t + 16));
+          circ[3 * dst + 2] = val(r.w.w >> t, r.w.w >> (t + 16), r.w4 >> t);
+        }
+      }
+      run += (uint32_t)__popc(bal);
+    };
+    if (rtot <= 32u * kHeldRecs) {
+      NodeRec held[kHeldRecs];
+#pragma unroll
+      for (int c = 0; c < kHeldRecs; ++c)
+        if (32u * c < rtot) held[c] = load(32u * c);
+#pragma unroll 1
+      for (int t = 1; t <= SUBR; ++t) {
+#pragma unroll
+        for (int c = 0; c < kHeldRecs; ++c)
+          if (32u * c < rtot) emit(held[c], t);
+      }
+    } else {
+#pragma unroll 1
+      for (int t = 1; t <= SUBR; ++t)
+        for (uint32_t g0 = 0; g0 < rtot; g0 += 32u) emit(load(g0), t);
     }
   }
 }
@@ -761,32 +799,32 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
   const int nbands = (ny + NB - 1) / NB;
   const int nxseg = (nx + NCOL - 1) / NCOL;
   const long long per_chunk = (long long)nbands * nxseg;
-  // about four work items per resident warp, chunks of at least 8 planes
-  long long want = (4LL * w->resident_warps + per_chunk - 1) / per_chunk;
-  if (want < 1) want = 1;
+  // z chunks: about kItems per resident warp, of at least 8 planes
+  const long long want = (kItemsPerWarp * (long long)w->resident_warps + per_chunk - 1) / per_chunk;
   int kchunk = (int)((nz + want - 1) / want);
   if (kchunk < 8) kchunk = nz < 8 ? nz : 8;
   const int nzchunks = (nz + kchunk - 1) / kchunk;
   const long long nitems = (long long)nzchunks * per_chunk;
-  const long long nseg = (long long)nz * nbands;
-  const uint64_t ntab = (uint64_t)nseg * nxseg * kTabVec;
-  // staging: the records, plus what chunk switches leave unused (under one
-  // step of at most NB * NCOL <= kChunk / 8 records per chunk, i.e. at most
-  // 1/7 of the records) and the open chunk of every warp
+  const long long nseg = (long long)nz * nbands * NSUB;
+  const uint64_t ntab = (uint64_t)nseg * nxseg;
+  // staging: the records (at least one node each), plus what chunk switches
+  // leave unused (under one step of at most NCOL <= kChunk / 8 records per
+  // chunk, i.e. at most 1/7 of the records) and the open chunk of every warp
   const long long launch_warps = (long long)launch_blocks(w, nitems) * NODE_WARPS;
   const uint64_t recs_need = capacity + capacity / 7 + 1 + (uint64_t)launch_warps * kChunk;
-  static_assert(NB * NCOL * 8 <= (int)kChunk, "chunk slack bound");
+  static_assert(NCOL * 8 <= (int)kChunk, "chunk slack bound");
   // table entries keep 32-bit staging offsets
   if (recs_need > 0xFFFFFFFFull)
     return set_error(QTV_ERR_ARG, "node form: %llu staging records (capacity %llu) exceed 2^32",
                      (unsigned long long)recs_need, (unsigned long long)capacity);
   rc = grow(w->recs, w->recs_cap, recs_need, st, "cudaMalloc(node records)");
+  if (!rc) rc = grow(w->recs4, w->recs4_cap, recs_need, st, "cudaMalloc(node records)");
   if (!rc) rc = grow(w->table, w->table_cap, ntab, st, "cudaMalloc(node table)");
   if (!rc) rc = grow(w->segtot, w->segtot_cap, (uint64_t)nseg, st, "cudaMalloc(node totals)");
   if (!rc) rc = grow(w->seg_off, w->seg_off_cap, (uint64_t)nseg, st, "cudaMalloc(node offsets)");
   if (rc) return rc;
 
-  cudaError_t e = cudaMemsetAsync(w->top, 0, sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(w->top, 0, 2 * sizeof(unsigned long long), st);
   if (e == cudaSuccess) e = cudaMemsetAsync(w->segtot, 0, nseg * sizeof(unsigned int), st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(node-form state)");
   NodeArgs a;
@@ -799,7 +837,8 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
   a.kchunk = kchunk;
   a.nitems = nitems;
   a.recs = w->recs;
-  a.recs_cap = w->recs_cap;
+  a.recs4 = w->recs4;
+  a.recs_cap = w->recs_cap < w->recs4_cap ? w->recs_cap : w->recs4_cap;
   a.top = w->top;
   a.table = w->table;
   a.segtot = w->segtot;
@@ -812,7 +851,8 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
   }
   {
     TraceScope ts(h, K_NODE_SCAN, st);
-    node_scan_kernel<<<1, 1024, 0, st>>>(w->segtot, nseg, w->seg_off, count);
+    node_scan_kernel<<<(unsigned)((nseg + kScanChunk - 1) / kScanChunk), 1024, 0, st>>>(
+        w->segtot, nseg, w->seg_off, count);
     e = cudaGetLastError();
     if (e != cudaSuccess) return check_cuda(e, "node_scan_kernel launch");
   }
@@ -821,10 +861,11 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
     const long long maxb = (long long)h->num_sms * 16;
     if (blocks > maxb) blocks = maxb;
     TraceScope ts(h, K_NODE_SCATTER, st);
-    node_scatter_kernel<<<(int)blocks, 256, 0, st>>>(w->table, w->seg_off, nseg, nxseg, w->recs,
-                                                     w->recs_cap, node_ids, circ, capacity);
+    node_expand_kernel<<<(int)blocks, 256, 0, st>>>(w->table, w->seg_off, nseg, nbands * NSUB, nxseg, nx, ny,
+                                                    w->recs, w->recs4, a.recs_cap, node_ids, circ,
+                                                    capacity);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return check_cuda(e, "node_scatter_kernel launch");
+    if (e != cudaSuccess) return check_cuda(e, "node_expand_kernel launch");
   }
   return QTV_OK;
 }
