@@ -29,7 +29,7 @@
 namespace qtv {
 namespace {
 
-constexpr int REF_THREADS = 128;
+constexpr int REF_THREADS = 128, REF_CTAS = 5;
 
 struct RefArgs {
   const float2* psi;
@@ -144,6 +144,34 @@ struct CellCache {
   float2 v[8];
 };
 
+// x . y with the roundings of fma(x2, y2, fma(x0, y0, x1 y1)).  Where products
+// meet sums in this file the roundings are written out: a search of 200 steps
+// amplifies any other choice.
+__device__ __forceinline__ float dot3(const float x[3], const float y[3]) {
+  return fmaf(x[2], y[2], fmaf(x[0], y[0], __fmul_rn(x[1], y[1])));
+}
+
+// two FP32 values in one register pair, IEEE roundings per value
+using F2 = unsigned long long;
+__device__ __forceinline__ F2 pair(float2 v) {
+  return (F2)__float_as_uint(v.x) | ((F2)__float_as_uint(v.y) << 32);
+}
+__device__ __forceinline__ F2 both(float v) { return pair(make_float2(v, v)); }
+__device__ __forceinline__ float2 unpair(F2 v) {
+  return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ F2 neg2(F2 a) { return a ^ 0x8000000080000000ull; }
+
 // rho and grad rho at P: trilinear psi and its derivatives from the corners
 // in the same order and arithmetic as tri_eval
 __device__ __forceinline__ float rho_at(const Field& F, const Pos& P, float g[3], CellCache& C) {
@@ -166,32 +194,31 @@ __device__ __forceinline__ float rho_at(const Field& F, const Pos& P, float g[3]
     C.c[1] = c[1];
     C.c[2] = c[2];
   }
-  float2 v = make_float2(0.f, 0.f);
-  float2 d[3];
-  d[0] = d[1] = d[2] = make_float2(0.f, 0.f);
+  // Re and Im side by side (packed FP32, the same roundings per component); the
+  // weights are pairs of equal halves
+  F2 w[2][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    w[0][a] = both(1.f - f[a]);
+    w[1][a] = both(f[a]);
+  }
+  F2 vv = both(0.f), dv[3] = {both(0.f), both(0.f), both(0.f)};
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    float w[3], s[3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const int bit = (q >> a) & 1;
-      w[a] = bit ? f[a] : 1.f - f[a];
-      s[a] = bit ? 1.f : -1.f;
-    }
-    const float2 u = C.v[q];
-    const float wt = w[0] * w[1] * w[2];
-    v.x = fmaf(wt, u.x, v.x);
-    v.y = fmaf(wt, u.y, v.y);
-    const float dd[3] = {s[0] * w[1] * w[2], w[0] * s[1] * w[2], w[0] * w[1] * s[2]};
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      d[a].x = fmaf(dd[a], u.x, d[a].x);
-      d[a].y = fmaf(dd[a], u.y, d[a].y);
-    }
+    const int b0 = q & 1, b1 = (q >> 1) & 1, b2 = q >> 2;
+    const F2 u = pair(C.v[q]);
+    vv = fma2(mul2(mul2(w[b0][0], w[b1][1]), w[b2][2]), u, vv);
+    // derivatives: the weight of the axis is -1 or 1
+    dv[0] = b0 ? fma2(mul2(w[b1][1], w[b2][2]), u, dv[0]) : fma2(neg2(mul2(w[b1][1], w[b2][2])), u, dv[0]);
+    dv[1] = b1 ? fma2(mul2(w[b0][0], w[b2][2]), u, dv[1]) : fma2(neg2(mul2(w[b0][0], w[b2][2])), u, dv[1]);
+    dv[2] = b2 ? fma2(mul2(w[b0][0], w[b1][1]), u, dv[2]) : fma2(neg2(mul2(w[b0][0], w[b1][1])), u, dv[2]);
   }
+  const float2 v = unpair(vv);
+  const float2 d[3] = {unpair(dv[0]), unpair(dv[1]), unpair(dv[2])};
 #pragma unroll
-  for (int a = 0; a < 3; ++a) g[a] = 2.f * fmaf(v.x, d[a].x, v.y * d[a].y);
-  return fmaf(v.x, v.x, v.y * v.y);
+  for (int a = 0; a < 3; ++a)
+    g[a] = __fmul_rn(2.f, fmaf(v.x, d[a].x, __fmul_rn(v.y, d[a].y)));
+  return fmaf(v.x, v.x, __fmul_rn(v.y, v.y));
 }
 
 // state of one sample's search
@@ -199,7 +226,9 @@ struct RState {
   Pos P0, P;
   float t[3];
   float rho;
-  float grad[3];
+  float grad[3];  // in-plane gradient of the running line search once it has begun
+  float gg, gn;   // its square and length
+  float alpha;    // step of the next candidate
   int it;
   uint8_t fl;
   unsigned long long qi;
@@ -268,10 +297,10 @@ __device__ __forceinline__ bool ref_init(const RefArgs& A, const Field& F, unsig
     }
   }
   float t[3];
-  t[0] = gr[1] * gi[2] - gr[2] * gi[1];
-  t[1] = gr[2] * gi[0] - gr[0] * gi[2];
-  t[2] = gr[0] * gi[1] - gr[1] * gi[0];
-  const float tn = sqrtf(t[0] * t[0] + t[1] * t[1] + t[2] * t[2]);
+  t[0] = fmaf(gr[1], gi[2], -__fmul_rn(gr[2], gi[1]));
+  t[1] = fmaf(gr[2], gi[0], -__fmul_rn(gr[0], gi[2]));
+  t[2] = fmaf(gr[0], gi[1], -__fmul_rn(gr[1], gi[0]));
+  const float tn = sqrtf(dot3(t, t));
   S.rho = rho_at(F, S.P, S.grad, S.cache);
   if (!(tn > 0.f) || !(tn <= 3.402823466e38f)) {
     S.fl = QTV_REFINE_NO_TANGENT;
@@ -284,52 +313,67 @@ __device__ __forceinline__ bool ref_init(const RefArgs& A, const Field& F, unsig
   return true;
 }
 
-// one accepted step, or the decision to stop; true when the sample is done
-__device__ __forceinline__ bool ref_step(const RefArgs& A, const Field& F, RState& S) {
+// start of a line search: the in-plane gradient and the first step; true when the
+// sample is done
+__device__ __forceinline__ bool ref_begin(const RefArgs& A, RState& S) {
   if (S.it >= A.max_iter) return true;  // flag stays QTV_REFINE_MAX_ITER
-  const float gt = S.grad[0] * S.t[0] + S.grad[1] * S.t[1] + S.grad[2] * S.t[2];
-  float g[3];
+  const float gt = dot3(S.grad, S.t);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) g[a] = S.grad[a] - gt * S.t[a];
-  const float gg = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-  if (!(gg > 0.f)) {
+  for (int a = 0; a < 3; ++a) S.grad[a] = fmaf(-gt, S.t[a], S.grad[a]);
+  S.gg = dot3(S.grad, S.grad);
+  if (!(S.gg > 0.f)) {
     S.fl = QTV_REFINE_CONVERGED;
     return true;
   }
-  const float gn = sqrtf(gg);
-  float alpha = 2.f * S.rho / gg;
+  S.gn = sqrtf(S.gg);
+  S.alpha = __fdiv_rn(__fmul_rn(2.f, S.rho), S.gg);
+  if (S.alpha > 3.402823466e38f) S.alpha = 3.402823466e38f;  // infinity never halves below tol
+  return false;
+}
+
+// candidate at step alpha along g from off: in the box around x0 (same base as
+// x0) and inside the grid
+__device__ __forceinline__ bool candidate(const Field& F, const int base[3], const float off[3],
+                                          const float off0[3], const float g[3], float alpha, Pos& Pn) {
+  bool ok = true;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    Pn.base[a] = base[a];
+    Pn.off[a] = fmaf(-alpha, g[a], off[a]);
+    ok = ok && fabsf(Pn.off[a] - off0[a]) <= 1.f;
+  }
+  return ok && pos_inside(Pn, F.n);
+}
+
+__device__ __forceinline__ bool descends(float rn, float alpha, float gg, float rho) {
+  return rn <= fmaf(-__fmul_rn(1e-4f, alpha), gg, rho);
+}
+
+// The next candidate of the line search that can be taken: one evaluation.  True
+// when the sample is done.  (With the whole search inside a step a lane that
+// halved twenty times held its warp.)
+__device__ __forceinline__ bool ref_try(const RefArgs& A, const Field& F, RState& S) {
   Pos Pn;
-  float rn = 0.f, gnext[3];
-  bool accepted = false;
-  while (alpha * gn >= A.tol) {
-    bool ok = true;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      Pn.base[a] = S.P.base[a];
-      Pn.off[a] = S.P.off[a] - alpha * g[a];
-      // box around x0 (same base as x0)
-      ok = ok && fabsf(Pn.off[a] - S.P0.off[a]) <= 1.f;
+  while (true) {
+    if (!(S.alpha * S.gn >= A.tol)) {
+      S.fl = QTV_REFINE_CONVERGED;
+      return true;
     }
-    if (ok && pos_inside(Pn, F.n)) {
-      rn = rho_at(F, Pn, gnext, S.cache);
-      if (rn <= S.rho - 1e-4f * alpha * gg) {
-        accepted = true;
-        break;
-      }
-    }
-    alpha *= 0.5f;
+    if (candidate(F, S.P.base, S.P.off, S.P0.off, S.grad, S.alpha, Pn)) break;
+    S.alpha *= 0.5f;
   }
-  if (!accepted) {
-    S.fl = QTV_REFINE_CONVERGED;
-    return true;
+  float gnext[3];
+  const float rn = rho_at(F, Pn, gnext, S.cache);
+  if (!descends(rn, S.alpha, S.gg, S.rho)) {
+    S.alpha *= 0.5f;
+    return false;
   }
   ++S.it;
   S.P = Pn;
   S.rho = rn;
-  S.grad[0] = gnext[0];
-  S.grad[1] = gnext[1];
-  S.grad[2] = gnext[2];
-  return false;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) S.grad[a] = gnext[a];
+  return ref_begin(A, S);
 }
 
 // conditioning at the result and the outputs of the sample
@@ -348,13 +392,14 @@ __device__ __forceinline__ void ref_finish(const RefArgs& A, const Field& F, con
     if (fabsf(t[2]) < am) m = 2;
     const float ax[3] = {m == 0 ? 1.f : 0.f, m == 1 ? 1.f : 0.f, m == 2 ? 1.f : 0.f};
     float e1[3] = {t[1] * ax[2] - t[2] * ax[1], t[2] * ax[0] - t[0] * ax[2],
-                   t[0] * ax[1] - t[1] * ax[0]};
-    const float en = sqrtf(e1[0] * e1[0] + e1[1] * e1[1] + e1[2] * e1[2]);
+                   t[0] * ax[1] - t[1] * ax[0]};  // exact: one component of ax is 1
+    const float en = sqrtf(dot3(e1, e1));
     e1[0] /= en;
     e1[1] /= en;
     e1[2] /= en;
-    const float e2[3] = {t[1] * e1[2] - t[2] * e1[1], t[2] * e1[0] - t[0] * e1[2],
-                         t[0] * e1[1] - t[1] * e1[0]};
+    const float e2[3] = {fmaf(t[1], e1[2], -__fmul_rn(t[2], e1[1])),
+                         fmaf(t[2], e1[0], -__fmul_rn(t[0], e1[2])),
+                         fmaf(t[0], e1[1], -__fmul_rn(t[1], e1[0]))};
     int cc[3];
     float ff[3];
 #pragma unroll
@@ -369,13 +414,13 @@ __device__ __forceinline__ void ref_finish(const RefArgs& A, const Field& F, con
       a2r = fmaf(d[a].x, e2[a], a2r);
       a2i = fmaf(d[a].y, e2[a], a2i);
     }
-    dj = a1r * a2i - a2r * a1i;
+    dj = fmaf(a1r, a2i, -__fmul_rn(a2r, a1i));
   }
   const float org[3] = {A.ox, A.oy, A.oz};
   const unsigned long long qi = S.qi;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    A.xyz[3 * qi + a] = org[a] + A.h * ((float)S.P.base[a] + S.P.off[a]);
+    A.xyz[3 * qi + a] = fmaf(A.h, (float)S.P.base[a] + S.P.off[a], org[a]);
     if (A.tangent) A.tangent[3 * qi + a] = S.t[a];
   }
   if (A.rho) A.rho[qi] = S.rho;
@@ -384,16 +429,52 @@ __device__ __forceinline__ void ref_finish(const RefArgs& A, const Field& F, con
   A.flags[qi] = S.fl;
 }
 
-// Persistent warps; each lane keeps one sample.  A lane whose search ends
-// waits until kRefill lanes of its warp have (or none is searching); then
-// those lanes write their results and take the next samples from the counter
-// together (one atomic per warp and refill), so the long set-up and result
-// code runs with many lanes at once while searches of very different lengths
-// keep the warp busy.  Each sample is computed exactly as alone.
-constexpr int kRefill = 12;
+// A search put off: what ref_try needs (88 bytes).
+struct Waiting {
+  int base[3];
+  float off0[3], off[3], t[3], grad[3];
+  float rho, gg, gn, alpha;
+  int it;
+  unsigned long long qi;
+};
 
-__global__ void __launch_bounds__(REF_THREADS, 6) refine_kernel(RefArgs A,
-                                                             unsigned long long* counter) {
+// counters of a call
+enum { kNextSample = 0, kPutOff, kNextWaiting, kRefCounters };
+
+// Searches differ by a factor of 180 in length (76 evaluations on average, up to
+// 3300 for 179e3 face centres of a 256^3 field: 200 steps of many halvings), and one
+// search is a chain of dependent evaluations.
+//
+// refine_kernel: persistent warps; each lane keeps one sample and evaluates one
+// candidate of its search per turn (with a whole line search inside a turn, a lane
+// that halved twenty times held its warp).  A lane whose search ends waits until
+// kRefill lanes of its warp have (or none is searching); then those lanes write
+// their results and take the next samples from the counter together (one atomic per
+// warp and refill), so the long set-up and result code runs with many lanes at once.
+// Once there are no more, a search of more than `patience` evaluations is put off
+// into a list while that has room.  The patience grows with the samples in flight:
+// with few of them lanes are free and the longest chain counts (33 to 100
+// evaluations: 235 to 258 us for 1000 samples), with all lanes in use throughput
+// does (254 evaluations 817 us for the 179e3 samples, 128 2002 us, 444 914 us).
+//
+// refine_long_kernel: those searches, kGroup lanes each.  The lanes take kGroup
+// successive halvings of a line search at once, and the first that ends it as
+// ref_try would (taken, or a step below tol) counts: the same result with a chain
+// about as long as the number of steps.  8 lanes: 488 us for 10000 samples instead
+// of 323; 32 lanes: 341, and 945 instead of 817 us for all.
+//
+// Each sample is computed exactly as alone.  Face centres of 256^3, lists of 1000 /
+// 10000 / 50000 / 179473: 245 / 315 / 400 / 820 us; with one lane and a line search a
+// turn 348 / 761 / 885 / 1180 us.
+constexpr int kRefill = 12;
+constexpr int kPatience = 32, kPerTurn = 400;
+constexpr int kGroup = 16;
+constexpr unsigned long long kWaitCap = 16384;
+constexpr size_t kRefHead = 128;  // bytes for the counters, ahead of the list
+static_assert(kRefCounters * sizeof(unsigned long long) <= kRefHead, "counters");
+
+__global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
+    RefArgs A, unsigned long long* counter, Waiting* waiting) {
   unsigned long long nn = A.n;
   if (A.n_dev) {
     const unsigned long long d = *A.n_dev;
@@ -407,6 +488,10 @@ __global__ void __launch_bounds__(REF_THREADS, 6) refine_kernel(RefArgs A,
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   RState S;
+  const int patience =
+      kPatience + (int)(min(nn, (unsigned long long)gridDim.x * REF_THREADS) / kPerTurn);
+  int turns = 0;
+  bool last = false;  // no sample left to take (same in all lanes)
   // active: searching; done: search ended, result not yet written;
   // drained: no sample left for this lane
   bool active = false, done = false, drained = false;
@@ -420,22 +505,147 @@ __global__ void __launch_bounds__(REF_THREADS, 6) refine_kernel(RefArgs A,
       }
       const int leader = __ffs(idle) - 1;
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(idle));
+      if (lane == leader) base = atomicAdd(counter + kNextSample, (unsigned long long)__popc(idle));
       base = __shfl_sync(0xffffffffu, base, leader);
       if (!active && !drained) {
         const unsigned long long qi = base + (unsigned long long)__popc(idle & lt);
         if (qi < nn) {
-          if (ref_init(A, F, qi, S)) active = true;
-          else ref_finish(A, F, S);
+          turns = 0;
+          if (ref_init(A, F, qi, S)) {
+            active = !ref_begin(A, S);
+            done = !active;
+          } else {
+            ref_finish(A, F, S);
+          }
+        } else {
+          drained = true;
+        }
+      }
+      last = __any_sync(0xffffffffu, drained);
+    }
+    if (!__any_sync(0xffffffffu, active || done || !drained)) break;
+    if (active) {
+      if (ref_try(A, F, S)) {
+        active = false;
+        done = true;
+      } else if (++turns >= patience && last) {
+        turns = INT_MIN;  // once, should the list be full
+        const unsigned long long at = atomicAdd(counter + kPutOff, 1ull);
+        if (at < kWaitCap) {
+          Waiting W;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            W.base[a] = S.P0.base[a];
+            W.off0[a] = S.P0.off[a];
+            W.off[a] = S.P.off[a];
+            W.t[a] = S.t[a];
+            W.grad[a] = S.grad[a];
+          }
+          W.rho = S.rho;
+          W.gg = S.gg;
+          W.gn = S.gn;
+          W.alpha = S.alpha;
+          W.it = S.it;
+          W.qi = S.qi;
+          waiting[at] = W;
+          active = false;
+        }
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
+    RefArgs A, unsigned long long* counter, const Waiting* waiting) {
+  constexpr unsigned full = 0xffffffffu;
+  const unsigned long long nw = min(counter[kPutOff], kWaitCap);
+  Field F;
+  F.psi = A.psi;
+  F.n[0] = A.nx;
+  F.n[1] = A.ny;
+  F.n[2] = A.nz;
+  const int lane = threadIdx.x & 31, j = lane % kGroup, lead = lane - j;
+  const unsigned group = ((1u << kGroup) - 1u) << lead;
+  RState S;  // the same in all lanes of a group, but for the cache
+  S.cache.c[0] = -1;
+  S.alpha = S.gg = S.gn = S.rho = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    S.P.base[a] = S.P0.base[a] = 0;
+    S.P.off[a] = S.P0.off[a] = S.grad[a] = 0.f;
+  }
+  bool active = false, drained = false;
+  while (true) {
+    if (__any_sync(full, !active && !drained)) {
+      unsigned long long w = 0;
+      if (!active && !drained && j == 0) w = atomicAdd(counter + kNextWaiting, 1ull);
+      w = __shfl_sync(full, w, lead);
+      if (!active && !drained) {
+        if (w < nw) {
+          const Waiting W = waiting[w];
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            S.P0.base[a] = S.P.base[a] = W.base[a];
+            S.P0.off[a] = W.off0[a];
+            S.P.off[a] = W.off[a];
+            S.t[a] = W.t[a];
+            S.grad[a] = W.grad[a];
+          }
+          S.rho = W.rho;
+          S.gg = W.gg;
+          S.gn = W.gn;
+          S.alpha = W.alpha;
+          S.it = W.it;
+          S.qi = W.qi;
+          S.fl = QTV_REFINE_MAX_ITER;
+          active = true;
         } else {
           drained = true;
         }
       }
     }
-    if (!__any_sync(0xffffffffu, active || done || !drained)) break;
-    if (active && ref_step(A, F, S)) {
+    if (!__any_sync(full, active)) break;
+    float alpha = S.alpha;
+    for (int i = 0; i < j; ++i) alpha *= 0.5f;
+    const bool below = !(alpha * S.gn >= A.tol);
+    Pos Pn = {};
+    float rn = 0.f, gnext[3] = {0.f, 0.f, 0.f};
+    bool taken = false;
+    if (active && !below && candidate(F, S.P.base, S.P.off, S.P0.off, S.grad, alpha, Pn)) {
+      rn = rho_at(F, Pn, gnext, S.cache);
+      taken = descends(rn, alpha, S.gg, S.rho);
+    }
+    const unsigned ends = __ballot_sync(full, below || taken) & group;
+    const unsigned takes = __ballot_sync(full, taken);
+    const int first = ends ? __ffs(ends) - 1 : lead + kGroup - 1;
+    rn = __shfl_sync(full, rn, first);
+    alpha = __shfl_sync(full, alpha, first);
+    float off[3], g[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      off[a] = __shfl_sync(full, Pn.off[a], first);
+      g[a] = __shfl_sync(full, gnext[a], first);
+    }
+    if (!active) continue;
+    bool ended = false;
+    if (!ends) {
+      S.alpha = alpha * 0.5f;
+    } else if (!((takes >> first) & 1u)) {
+      S.fl = QTV_REFINE_CONVERGED;
+      ended = true;
+    } else {
+      ++S.it;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        S.P.off[a] = off[a];
+        S.grad[a] = g[a];
+      }
+      S.rho = rn;
+      ended = ref_begin(A, S);
+    }
+    if (ended) {
+      if (j == 0) ref_finish(A, F, S);
       active = false;
-      done = true;
     }
   }
 }
@@ -468,14 +678,17 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
   a.detj = detj;
   a.iters = iters;
   a.flags = flags;
+  // counters and list of one size for every call, so that a captured call keeps its
+  // pointers
   if (!h->refine_counter) {
     const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->refine_counter),
-                                     sizeof(unsigned long long));
+                                     kRefHead + kWaitCap * sizeof(Waiting));
     if (e != cudaSuccess) {
       h->refine_counter = nullptr;
       return check_cuda(e, "cudaMalloc(refine counter)");
     }
   }
+  Waiting* const waiting = reinterpret_cast<Waiting*>(reinterpret_cast<char*>(h->refine_counter) + kRefHead);
   // persistent: as many blocks as fit at once, fewer for short lists
   static int per_sm = 0;
   if (per_sm == 0) {
@@ -490,9 +703,12 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
   const long long maxb = (long long)h->num_sms * per_sm;
   if (blocks > maxb) blocks = maxb;
   TraceScope ts(h, K_REFINE, st);
-  cudaError_t e = cudaMemsetAsync(h->refine_counter, 0, sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(h->refine_counter, 0, kRefCounters * sizeof(unsigned long long), st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(refine counter)");
-  refine_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, h->refine_counter);
+  refine_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, h->refine_counter, waiting);
+  blocks = ((long long)(n < kWaitCap ? n : kWaitCap) * kGroup + REF_THREADS - 1) / REF_THREADS;
+  if (blocks > maxb) blocks = maxb;
+  refine_long_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, h->refine_counter, waiting);
   e = cudaGetLastError();
   return check_cuda(e, "refine_kernel launch");
 }
