@@ -96,8 +96,11 @@ __device__ __forceinline__ bool solve_face(const C2 P[4], float& uo, float& vo, 
   F.d = sub(sub(P[2], P[1]), F.c);
   float bu = 0.5f, bv = 0.5f, best = 3.4e38f;
   bool found = false;
+  bool near0, near1;
+  auto in_reach = [](float u, float v) {
+    return u >= -0.05f && u <= 1.05f && v >= -0.05f && v <= 1.05f;
+  };
   auto consider = [&](float u, float v) {
-    if (!(u >= -0.05f && u <= 1.05f && v >= -0.05f && v <= 1.05f)) return;
     newton(F, u, v);
     if (!(u >= -1e-4f && u <= 1.f + 1e-4f && v >= -1e-4f && v <= 1.f + 1e-4f)) return;
     const C2 f = eval(F, u, v);
@@ -112,12 +115,24 @@ __device__ __forceinline__ bool solve_face(const C2 P[4], float& uo, float& vo, 
   float t0 = 0.f, t1 = 0.f;
   // eliminate u: (a + c v) + u (b + d v) = 0, u real <=> Im(p conj q) = 0
   int nr = roots2(crs(F.c, F.d), __fadd_rn(crs(F.a, F.d), crs(F.c, F.b)), crs(F.a, F.b), t0, t1);
-  for (int r = 0; r < nr; ++r) {
-    const float v = r ? t1 : t0;
+  float s[2], t[2] = {t0, t1};
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const float v = t[r];
     const C2 p = mk(fmaf(v, F.c.x, F.a.x), fmaf(v, F.c.y, F.a.y));
     const C2 q = mk(fmaf(v, F.d.x, F.b.x), fmaf(v, F.d.y, F.b.y));
     const float qq = dtr(q, q);
-    if (qq > 0.f) consider(-dtr(p, q) / qq, v);
+    s[r] = -dtr(p, q) / qq;
+    const bool near_face = r < nr && qq > 0.f && in_reach(s[r], v);
+    if (r == 0) near0 = near_face;
+    else near1 = near_face;
+  }
+  // one root is usually near the face: the lanes of a warp refine theirs together,
+  // whichever it is (1.4 M faces at 512^3: half a microsecond, 1024^3: 18 us of 2359)
+  while (near0 || near1) {
+    consider(near0 ? s[0] : s[1], near0 ? t[0] : t[1]);
+    if (near0) near0 = false;
+    else near1 = false;
   }
   if (!found) {
     // eliminate v: (a + b u) + v (c + d u) = 0
@@ -127,7 +142,10 @@ __device__ __forceinline__ bool solve_face(const C2 P[4], float& uo, float& vo, 
       const C2 p = mk(fmaf(u, F.b.x, F.a.x), fmaf(u, F.b.y, F.a.y));
       const C2 q = mk(fmaf(u, F.d.x, F.c.x), fmaf(u, F.d.y, F.c.y));
       const float qq = dtr(q, q);
-      if (qq > 0.f) consider(u, -dtr(p, q) / qq);
+      if (qq > 0.f) {
+        const float v = -dtr(p, q) / qq;
+        if (in_reach(u, v)) consider(u, v);
+      }
     }
   }
   if (!found) {
@@ -143,8 +161,7 @@ __device__ __forceinline__ bool solve_face(const C2 P[4], float& uo, float& vo, 
 
 // A face's grid position and corner values (the loads of its localization).
 struct FaceIn {
-  long long i, j, k;
-  int o;
+  int i, j, k, o;
   bool exists;
   C2 P[4];
 };
@@ -153,16 +170,20 @@ __device__ __forceinline__ void face_load(const float2* __restrict__ psi, int nx
                                           unsigned long long id, FaceIn& F) {
   const int o = (int)(id & 3u);
   const unsigned long long lin = id >> 2;
-  split_lin(lin, nx, ny, F.i, F.j, F.k);
+  long long i, j, k;
+  split_lin(lin, nx, ny, i, j, k);
   F.o = o;
   const long long sx = 1, sy = nx, sz = (long long)nx * ny;
   long long du, dv;  // strides of the face axes u, v
   bool exists;
-  if (o == 0) { du = sx; dv = sy; exists = F.i + 1 < nx && F.j + 1 < ny; }
-  else if (o == 1) { du = sy; dv = sz; exists = F.j + 1 < ny && F.k + 1 < nz; }
-  else { du = sz; dv = sx; exists = F.k + 1 < nz && F.i + 1 < nx; }
-  F.exists = o != 3 && exists && F.k < nz;
+  if (o == 0) { du = sx; dv = sy; exists = i + 1 < nx && j + 1 < ny; }
+  else if (o == 1) { du = sy; dv = sz; exists = j + 1 < ny && k + 1 < nz; }
+  else { du = sz; dv = sx; exists = k + 1 < nz && i + 1 < nx; }
+  F.exists = o != 3 && exists && k < nz;
   if (!F.exists) return;  // not a face of this grid: touch no node
+  F.i = (int)i;
+  F.j = (int)j;
+  F.k = (int)k;
   const long long base = (long long)lin;
   const float2 p0 = __ldg(psi + base), p1 = __ldg(psi + base + du);
   const float2 p2 = __ldg(psi + base + du + dv), p3 = __ldg(psi + base + dv);
