@@ -63,6 +63,8 @@ __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, cons
 __global__ void row_table_kernel(const uint64_t* __restrict__ ids, unsigned long long n,
                                  const uint64_t* n_dev, int nx, long long R, int shift,
                                  uint32_t* __restrict__ rows) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(n, n_dev);
   for (long long r = (long long)blockIdx.x * GT + threadIdx.x; r <= R;
        r += (long long)gridDim.x * GT) {
@@ -85,7 +87,8 @@ cudaError_t row_table_launch(const uint64_t* ids, unsigned long long n, const ui
   long long blocks = (R + 1 + GT - 1) / GT;
   if (blocks > (long long)num_sms * 16) blocks = (long long)num_sms * 16;
   if (blocks < 1) blocks = 1;
-  row_table_kernel<<<(int)blocks, GT, 0, st>>>(ids, n, n_dev, nx, R, shift, rows);
+  launch_dependent(row_table_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, ids, n, n_dev, nx,
+                   R, shift, rows);
   return cudaGetLastError();
 }
 
@@ -121,6 +124,8 @@ __device__ __forceinline__ uint32_t find_face(const GraphArgs& a, unsigned long 
 }
 
 __global__ void __launch_bounds__(GT) adjacency_kernel(GraphArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   const long long nx = a.nx, ny = a.ny, nz = a.nz;
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
@@ -175,6 +180,8 @@ __global__ void __launch_bounds__(GT) adjacency_kernel(GraphArgs a) {
 // vortex-node graph: 6-connectivity along grid lines; candidates in the
 // order -z, -y, -x, +x, +y, +z are ascending linear indices
 __global__ void __launch_bounds__(GT) node_adjacency_kernel(GraphArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   const long long nx = a.nx, ny = a.ny, nz = a.nz;
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
@@ -237,6 +244,8 @@ __device__ __forceinline__ uint32_t find_root_ro(const uint32_t* parent, uint32_
 constexpr int kShort = 16;
 
 __global__ void __launch_bounds__(GT) shorten_kernel(GraphArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
        q += (unsigned long long)gridDim.x * GT) {
@@ -251,6 +260,8 @@ __global__ void __launch_bounds__(GT) shorten_kernel(GraphArgs a) {
 }
 
 __global__ void __launch_bounds__(GT) link_kernel(GraphArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
        q += (unsigned long long)gridDim.x * GT) {
@@ -278,6 +289,8 @@ __global__ void __launch_bounds__(GT) link_kernel(GraphArgs a) {
 }
 
 __global__ void __launch_bounds__(GT) flatten_kernel(GraphArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   unsigned long long roots = 0;
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
@@ -292,6 +305,8 @@ __global__ void __launch_bounds__(GT) flatten_kernel(GraphArgs a) {
 }
 
 __global__ void graph_status_kernel(const unsigned long long* status, uint64_t* ncomp) {
+  pdl_wait();
+  pdl_trigger();
   *ncomp = status[1] ? QTV_COUNT_TIMEOUT : status[0];
 }
 
@@ -336,8 +351,8 @@ int face_graph_launch(qtv_handle h, const qtv_grid& g, const uint64_t* face_ids,
   {
     long long blocks = (R + 1 + GT - 1) / GT;
     if (blocks > (long long)h->num_sms * 16) blocks = (long long)h->num_sms * 16;
-    row_table_kernel<<<(int)blocks, GT, 0, st>>>(face_ids, n, n_dev, g.nx, R, nodes ? 0 : 2,
-                                                 w->rows);
+    launch_dependent(row_table_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, face_ids, n,
+                     n_dev, g.nx, R, nodes ? 0 : 2, w->rows);
   }
   GraphArgs a;
   a.ids = face_ids;
@@ -356,13 +371,13 @@ int face_graph_launch(qtv_handle h, const qtv_grid& g, const uint64_t* face_ids,
   long long blocks = ((long long)n + GT - 1) / GT;
   if (blocks > (long long)h->num_sms * 16) blocks = (long long)h->num_sms * 16;
   if (blocks < 1) blocks = 1;
-  if (nodes) node_adjacency_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  else adjacency_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  shorten_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  shorten_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  link_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  flatten_kernel<<<(int)blocks, GT, 0, st>>>(a);
-  graph_status_kernel<<<1, 1, 0, st>>>(w->status, ncomp);
+  if (nodes) launch_dependent(node_adjacency_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  else launch_dependent(adjacency_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  launch_dependent(shorten_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  launch_dependent(shorten_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  launch_dependent(link_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  launch_dependent(flatten_kernel, dim3((unsigned)blocks), dim3(GT), 0, st, a);
+  launch_dependent(graph_status_kernel, dim3(1), dim3(1), 0, st, w->status, ncomp);
   e = cudaGetLastError();
   return check_cuda(e, "face graph launch");
 }

@@ -123,6 +123,8 @@ __device__ __forceinline__ int comp_type(const LineArgs& a, uint32_t L) {
 }
 
 __global__ void stats_init_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * LT) {
@@ -131,6 +133,8 @@ __global__ void stats_init_kernel(LineArgs a) {
 }
 
 __global__ void stats_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * LT) {
@@ -146,6 +150,8 @@ __global__ void stats_kernel(LineArgs a) {
 }
 
 __global__ void special_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * LT) {
@@ -166,6 +172,8 @@ __device__ __forceinline__ int slot_of(const LineArgs& a, uint32_t w, uint32_t x
 
 // directed edges in compact order: sample u owns edges aoff[u] .. + deg[u] - 1
 __global__ void arcs_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * LT) {
@@ -179,6 +187,8 @@ __global__ void arcs_kernel(LineArgs a) {
 }
 
 __global__ void edges_init_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long ne = *a.narcs;
   for (unsigned long long e = (unsigned long long)blockIdx.x * LT + threadIdx.x; e < ne;
        e += (unsigned long long)gridDim.x * LT) {
@@ -201,6 +211,8 @@ __global__ void edges_init_kernel(LineArgs a) {
 // round 225 us (20 launches), four 137 (10), eight 119 (7); with records of 8
 // bytes instead of 16, 105.
 __global__ void jump_kernel(LineArgs a, int src, int r) {
+  pdl_wait();
+  pdl_trigger();
   if (r > 0 && a.live[r - 1] == 0u) return;
   const unsigned long long ne = *a.narcs;
   const int d = src ^ 1;
@@ -266,6 +278,8 @@ __device__ __forceinline__ bool discovering(const LineArgs& a, int buf, uint32_t
 }
 
 __global__ void count_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int buf = (int)*a.fbuf;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
@@ -293,6 +307,8 @@ __global__ void count_kernel(LineArgs a) {
 
 // piece records, and the start and end samples of every piece
 __global__ void pieces_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int buf = (int)*a.fbuf;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
@@ -342,6 +358,8 @@ __global__ void pieces_kernel(LineArgs a) {
 
 // samples inside chains: their piece and position from its start
 __global__ void interior_kernel(LineArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const int buf = (int)*a.fbuf;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   for (unsigned long long u = (unsigned long long)blockIdx.x * LT + threadIdx.x; u < nn;
@@ -417,6 +435,8 @@ __device__ __forceinline__ unsigned long long node_total(const LineArgs& a, unsi
 
 // orientation sums: final for pieces inside a chunk, partials for the others
 __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
   const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
@@ -467,6 +487,8 @@ __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
 // final node list: each piece in order, or reversed (closed: first kept); the
 // first chunk of a spanning piece sets its flag
 __global__ void place_kernel(LineArgs a, const unsigned long long* counts) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
   const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
@@ -529,6 +551,8 @@ __device__ __forceinline__ unsigned long long block_total(unsigned long long v, 
 
 template <typename T>
 __global__ void __launch_bounds__(SB) scan_sums_kernel(ScanArgs<T> a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ unsigned long long wt[32];
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   const T* in = a.in[blockIdx.y];
@@ -542,6 +566,8 @@ __global__ void __launch_bounds__(SB) scan_sums_kernel(ScanArgs<T> a) {
 
 template <typename T>
 __global__ void __launch_bounds__(SB) scan_apply_kernel(ScanArgs<T> a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ unsigned long long wt[32];
   const unsigned long long nn = limit_n(a.n, a.n_dev);
   const T* in = a.in[blockIdx.y];
@@ -585,8 +611,8 @@ void scan(const T* in0, const T* in1, const uint64_t* n_dev, unsigned long long 
   ScanArgs<T> a{{in0, in1}, {out0, out1}, {total0, total1}, bsum, n, n_dev};
   const unsigned nb = (unsigned)((n + SCHUNK - 1) / SCHUNK);
   const dim3 grid(nb > 0 ? nb : 1, in1 ? 2 : 1);
-  scan_sums_kernel<T><<<grid, SB, 0, st>>>(a);
-  scan_apply_kernel<T><<<grid, SB, 0, st>>>(a);
+  launch_dependent(scan_sums_kernel<T>, dim3(grid), dim3(SB), 0, st, a);
+  launch_dependent(scan_apply_kernel<T>, dim3(grid), dim3(SB), 0, st, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -615,6 +641,8 @@ __device__ __forceinline__ uint32_t curve_points(const qtv_piece& r, int per) {
 }
 
 __global__ void curve_count_kernel(CurveArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long np = limit_n(a.np, a.np_dev);
   for (unsigned long long p = (unsigned long long)blockIdx.x * LT + threadIdx.x; p < np;
        p += (unsigned long long)gridDim.x * LT) {
@@ -645,6 +673,8 @@ __device__ __forceinline__ void sample_pos(const CurveArgs& a, const qtv_piece& 
 constexpr int kStage = 8, kStagePitch = 3 * kStage + 1;
 
 __global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ float stage[LT / 32][32 * kStagePitch];
   const unsigned long long np = limit_n(a.np, a.np_dev);
   // the pieces that fit come first and have at least a point a sample
@@ -746,6 +776,8 @@ __global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a) {
 // lengths of the pieces that span warps of entries, one warp each (0 for a
 // piece that does not fit)
 __global__ void __launch_bounds__(LT) length_span_kernel(CurveArgs a) {
+  pdl_wait();
+  pdl_trigger();
   const unsigned long long np = limit_n(a.np, a.np_dev);
   const unsigned long long warps = ((unsigned long long)gridDim.x * LT) >> 5;
   for (unsigned long long p = ((unsigned long long)blockIdx.x * LT + threadIdx.x) >> 5; p < np;
@@ -797,6 +829,8 @@ __device__ __forceinline__ double coord(const ThinArgs& a, unsigned long long g,
 }
 
 __global__ void thin_len_kernel(ThinArgs a) {
+  pdl_wait();
+  pdl_trigger();
   for (unsigned long long g = (unsigned long long)blockIdx.x * LT + threadIdx.x; g < a.ne;
        g += (unsigned long long)gridDim.x * LT) {
     const qtv_piece r = a.pieces[piece_of(a, g)];
@@ -815,6 +849,8 @@ __global__ void thin_len_kernel(ThinArgs a) {
 }
 
 __global__ void thin_flag_kernel(ThinArgs a) {
+  pdl_wait();
+  pdl_trigger();
   for (unsigned long long g = (unsigned long long)blockIdx.x * LT + threadIdx.x; g < a.ne;
        g += (unsigned long long)gridDim.x * LT) {
     const qtv_piece r = a.pieces[piece_of(a, g)];
@@ -829,6 +865,8 @@ __global__ void thin_flag_kernel(ThinArgs a) {
 }
 
 __global__ void thin_mean_kernel(ThinArgs a) {
+  pdl_wait();
+  pdl_trigger();
   for (unsigned long long g = (unsigned long long)blockIdx.x * LT + threadIdx.x; g < a.ne;
        g += (unsigned long long)gridDim.x * LT) {
     if (!a.flag[g]) continue;
@@ -853,6 +891,8 @@ __global__ void thin_mean_kernel(ThinArgs a) {
 }
 
 __global__ void thin_pieces_kernel(ThinArgs a) {
+  pdl_wait();
+  pdl_trigger();
   for (unsigned long long p = (unsigned long long)blockIdx.x * LT + threadIdx.x; p < a.np;
        p += (unsigned long long)gridDim.x * LT) {
     qtv_piece r = a.pieces[p];
@@ -963,27 +1003,28 @@ int line_pieces_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const ui
   if (ge > (long long)h->num_sms * 32) ge = (long long)h->num_sms * 32;
   if (ge < 1) ge = 1;
   TraceScope ts(h, K_LINES, st);
-  stats_init_kernel<<<(int)g, LT, 0, st>>>(a);
-  stats_kernel<<<(int)g, LT, 0, st>>>(a);
-  special_kernel<<<(int)g, LT, 0, st>>>(a);
+  launch_dependent(stats_init_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(stats_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(special_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
   // compact directed edges: offsets by an exclusive scan of the degrees
   scan<uint32_t>(a.deg32, nullptr, n_dev, n, a.aoff, nullptr, bs3, narcs, nullptr, st);
-  arcs_kernel<<<(int)g, LT, 0, st>>>(a);
-  edges_init_kernel<<<(int)ge, LT, 0, st>>>(a);
+  launch_dependent(arcs_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(edges_init_kernel, dim3((unsigned)ge), dim3(LT), 0, st, a);
   int rounds = 0;
   for (unsigned long long reach = 1; reach < (unsigned long long)n + 1; reach *= kHops) ++rounds;
   if (rounds < 1) rounds = 1;
   cudaError_t e = cudaMemsetAsync(a.live, 0, (kMaxRounds + 1) * sizeof(uint32_t), st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(line rounds)");
-  for (int r = 0; r < rounds; ++r) jump_kernel<<<(int)ge, LT, 0, st>>>(a, r & 1, r);
-  count_kernel<<<(int)g, LT, 0, st>>>(a);
+  for (int r = 0; r < rounds; ++r)
+    launch_dependent(jump_kernel, dim3((unsigned)ge), dim3(LT), 0, st, a, r & 1, r);
+  launch_dependent(count_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
   scan<uint32_t>(a.pcount, a.plen, n_dev, n, a.pfirst, a.noff, bs1, tot, tot + 1, st);
   e = cudaMemcpyAsync(counts, tot, 2 * sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemcpyAsync(line counts)");
-  pieces_kernel<<<(int)g, LT, 0, st>>>(a);
-  interior_kernel<<<(int)g, LT, 0, st>>>(a);
-  orient_kernel<<<h->num_sms * 8, LT, 0, st>>>(a, tot);
-  place_kernel<<<h->num_sms * 8, LT, 0, st>>>(a, tot);
+  launch_dependent(pieces_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(interior_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(orient_kernel, dim3(h->num_sms * 8), dim3(LT), 0, st, a, tot);
+  launch_dependent(place_kernel, dim3(h->num_sms * 8), dim3(LT), 0, st, a, tot);
   e = cudaGetLastError();
   return check_cuda(e, "line pieces launch");
 }
@@ -1024,11 +1065,11 @@ int piece_curves_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (g > (long long)h->num_sms * 16) g = (long long)h->num_sms * 16;
   if (g < 1) g = 1;
   TraceScope ts(h, K_CURVES, st);
-  curve_count_kernel<<<(int)g, LT, 0, st>>>(a);
+  launch_dependent(curve_count_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
   scan<uint32_t>(a.npts, a.count, np_dev, np, a.cfirst, a.efirst, bs,
                  reinterpret_cast<unsigned long long*>(total), entries, st);
-  if (curve_cap > 0) curve_kernel<<<h->num_sms * 8, LT, 0, st>>>(a);
-  length_span_kernel<<<h->num_sms * 4, LT, 0, st>>>(a);
+  if (curve_cap > 0) launch_dependent(curve_kernel, dim3(h->num_sms * 8), dim3(LT), 0, st, a);
+  launch_dependent(length_span_kernel, dim3(h->num_sms * 4), dim3(LT), 0, st, a);
   const cudaError_t e = cudaGetLastError();
   return check_cuda(e, "piece curves launch");
 }
@@ -1072,12 +1113,12 @@ int thin_pieces_launch(qtv_handle h, const float* xyz, const uint32_t* nodes,
   if (gp > (long long)h->num_sms * 16) gp = (long long)h->num_sms * 16;
   if (gp < 1) gp = 1;
   TraceScope ts(h, K_THIN, st);
-  thin_len_kernel<<<(int)g, LT, 0, st>>>(a);
+  launch_dependent(thin_len_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
   scan<unsigned long long>(a.v, nullptr, nullptr, ne, a.X, nullptr, bs1, tots, nullptr, st);
-  thin_flag_kernel<<<(int)g, LT, 0, st>>>(a);
+  launch_dependent(thin_flag_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
   scan<uint32_t>(a.flag, nullptr, nullptr, ne, a.G, nullptr, bs2, tots + 1, nullptr, st);
-  thin_mean_kernel<<<(int)g, LT, 0, st>>>(a);
-  thin_pieces_kernel<<<(int)gp, LT, 0, st>>>(a);
+  launch_dependent(thin_mean_kernel, dim3((unsigned)g), dim3(LT), 0, st, a);
+  launch_dependent(thin_pieces_kernel, dim3((unsigned)gp), dim3(LT), 0, st, a);
   cudaError_t e = cudaMemcpyAsync(total, tots + 1, sizeof(uint64_t), cudaMemcpyDeviceToDevice, st);
   if (e == cudaSuccess) e = cudaGetLastError();
   return check_cuda(e, "thin pieces launch");
