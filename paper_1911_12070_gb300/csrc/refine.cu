@@ -453,9 +453,11 @@ enum { kNextSample = 0, kPutOff, kNextWaiting, kRefCounters };
 // warp and refill), so the long set-up and result code runs with many lanes at once.
 // Once there are no more, a search of more than `patience` evaluations is put off
 // into a list while that has room.  The patience grows with the samples in flight:
-// with few of them lanes are free and the longest chain counts (33 to 100
-// evaluations: 235 to 258 us for 1000 samples), with all lanes in use throughput
-// does (254 evaluations 817 us for the 179e3 samples, 128 2002 us, 444 914 us).
+// with few of them lanes are free and the longest chain counts (33 evaluations
+// 235 us for 1000 samples, 100 258), with all lanes in use throughput does (238
+// evaluations 820 us for the 179e3 samples, 275 855, 444 914, 128 2002).  Lists
+// of the searches of thinned-out warps, taken up again by full warps, were slower
+// (1250 to 1600 us): long searches are neighbours, and filled whole warps.
 //
 // refine_long_kernel: those searches, kGroup lanes each.  The lanes take kGroup
 // successive halvings of a line search at once, and the first that ends it as
@@ -464,10 +466,10 @@ enum { kNextSample = 0, kPutOff, kNextWaiting, kRefCounters };
 // of 323; 32 lanes: 341, and 945 instead of 817 us for all.
 //
 // Each sample is computed exactly as alone.  Face centres of 256^3, lists of 1000 /
-// 10000 / 50000 / 179473: 245 / 315 / 400 / 820 us; with one lane and a line search a
+// 10000 / 50000 / 179473: 247 / 323 / 402 / 820 us; with one lane and a line search a
 // turn 348 / 761 / 885 / 1180 us.
 constexpr int kRefill = 12;
-constexpr int kPatience = 32, kPerTurn = 400;
+constexpr int kPatience = 48, kPerTurn = 512;
 constexpr int kGroup = 16;
 constexpr unsigned long long kWaitCap = 16384;
 constexpr size_t kRefHead = 128;  // bytes for the counters, ahead of the list
