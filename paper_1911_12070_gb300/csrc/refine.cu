@@ -438,50 +438,103 @@ struct Waiting {
   unsigned long long qi;
 };
 
-// counters of a call
-enum { kNextSample = 0, kPutOff, kNextWaiting, kRefCounters };
-
 // Searches differ by a factor of 180 in length (76 evaluations on average, up to
 // 3300 for 179e3 face centres of a 256^3 field: 200 steps of many halvings), and one
 // search is a chain of dependent evaluations.
 //
-// refine_kernel: persistent warps; each lane keeps one sample and evaluates one
-// candidate of its search per turn (with a whole line search inside a turn, a lane
-// that halved twenty times held its warp).  A lane whose search ends waits until
-// kRefill lanes of its warp have (or none is searching); then those lanes write
-// their results and take the next samples from the counter together (one atomic per
-// warp and refill), so the long set-up and result code runs with many lanes at once.
-// Once there are no more, a search of more than `patience` evaluations is put off
-// into a list while that has room.  The patience grows with the samples in flight:
-// with few of them lanes are free and the longest chain counts (33 evaluations
-// 235 us for 1000 samples, 100 258), with all lanes in use throughput does (238
-// evaluations 820 us for the 179e3 samples, 275 855, 444 914, 128 2002).  Lists
-// of the searches of thinned-out warps, taken up again by full warps, were slower
-// (1250 to 1600 us): long searches are neighbours, and filled whole warps.
+// refine_kernel: persistent warps; each lane keeps one search and evaluates one
+// candidate of it per turn (with a whole line search inside a turn 9 of 32 threads
+// were active, now 18: 609e3 samples in 908 us instead of 1932, without the searches
+// put off).  A lane whose search ends waits until kRefill lanes of its warp have (or
+// none is searching); then those lanes write their results and take the next samples
+// from the counter together (one atomic per warp and refill), so the long set-up and
+// result code runs with many lanes at once.  Once there are no more, a search of
+// more than `patience` evaluations is put off into list 0, which has room for every
+// lane in flight (with less, the searches left over made the launch as long as the
+// longest chain: 4.3 ms instead of 3.2 for 1.39e6 samples).
 //
-// refine_long_kernel: those searches, kGroup lanes each.  The lanes take kGroup
-// successive halvings of a line search at once, and the first that ends it as
+// refine_long_kernel: the searches of a list, kGroup lanes each.  The lanes take
+// kGroup successive halvings of a line search at once, and the first that ends it as
 // ref_try would (taken, or a step below tol) counts: the same result with a chain
-// about as long as the number of steps.  8 lanes: 488 us for 10000 samples instead
-// of 323; 32 lanes: 341, and 945 instead of 817 us for all.
+// about as long as the number of steps, for eight times the work a step.
+//
+// Rules (refine_launch).  Up to four samples a lane, list 0 goes to the groups
+// directly and the patience grows with the samples in flight: with few of them the
+// longest chain counts (33 evaluations 235 us for 1000 samples, 100 258), with all
+// lanes in use the groups' work does (179e3 samples: 128 evaluations 824 us, 64 941).
+// Above, a second launch first takes list 0 by full warps and puts off after
+// another kPatience2 evaluations into list 1 (609e3 samples 1865 us, without it
+// 1988 to 2019; 179e3 samples 1041 with it).
 //
 // Each sample is computed exactly as alone.  Face centres of 256^3, lists of 1000 /
-// 10000 / 50000 / 179473: 247 / 323 / 402 / 820 us; with one lane and a line search a
-// turn 348 / 761 / 885 / 1180 us.
+// 10000 / 50000 / 179473: 239 / 284 / 371 / 826 us; with one lane and a line search a turn 348 /
+// 761 / 885 / 1180 us; 512^3 (1.39e6) 3217 -> 3132, means of thinned lines there
+// (235e3) 1627 -> 1093.  Slower: 1e5 points in random order that have converged
+// already, whose searches are all short, 120 -> 166 at 256^3.
 constexpr int kRefill = 12;
-constexpr int kPatience = 48, kPerTurn = 512;
+constexpr int kPatience = 32, kPatience2 = 384;
+constexpr int kPerTurn = 1024;  // samples in flight for one evaluation of patience more
 constexpr int kGroup = 16;
-constexpr unsigned long long kWaitCap = 16384;
-constexpr size_t kRefHead = 128;  // bytes for the counters, ahead of the list
-static_assert(kRefCounters * sizeof(unsigned long long) <= kRefHead, "counters");
 
+// counters of a call, ahead of the two lists in memory
+struct RefCounters {
+  unsigned long long next_sample;
+  unsigned long long count[2];  // entries of the lists
+  unsigned long long taken[2];
+};
+constexpr size_t kRefHead = 128;
+static_assert(sizeof(RefCounters) <= kRefHead, "counters");
+
+__device__ __forceinline__ void put_off(const RState& S, Waiting& W) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    W.base[a] = S.P0.base[a];
+    W.off0[a] = S.P0.off[a];
+    W.off[a] = S.P.off[a];
+    W.t[a] = S.t[a];
+    W.grad[a] = S.grad[a];
+  }
+  W.rho = S.rho;
+  W.gg = S.gg;
+  W.gn = S.gn;
+  W.alpha = S.alpha;
+  W.it = S.it;
+  W.qi = S.qi;
+}
+
+__device__ __forceinline__ void take_up(const Waiting& W, RState& S) {
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    S.P0.base[a] = S.P.base[a] = W.base[a];
+    S.P0.off[a] = W.off0[a];
+    S.P.off[a] = W.off[a];
+    S.t[a] = W.t[a];
+    S.grad[a] = W.grad[a];
+  }
+  S.rho = W.rho;
+  S.gg = W.gg;
+  S.gn = W.gn;
+  S.alpha = W.alpha;
+  S.it = W.it;
+  S.qi = W.qi;
+  S.fl = QTV_REFINE_MAX_ITER;
+  S.cache.c[0] = -1;  // no cell loaded
+}
+
+// LIST: the searches of list 0 instead of the samples
+template <bool LIST>
 __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
-    RefArgs A, unsigned long long* counter, Waiting* waiting) {
+    RefArgs A, RefCounters* counter, Waiting* lists, unsigned long long cap,
+    unsigned long long groups, int patience) {
   unsigned long long nn = A.n;
-  if (A.n_dev) {
+  if (LIST) {
+    nn = min(counter->count[0], cap);
+    if (nn <= groups) return;
+  } else if (A.n_dev) {
     const unsigned long long d = *A.n_dev;
     if (d < nn) nn = d;
   }
+  unsigned long long* const next = LIST ? &counter->taken[0] : &counter->next_sample;
   Field F;
   F.psi = A.psi;
   F.n[0] = A.nx;
@@ -490,8 +543,6 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   RState S;
-  const int patience =
-      kPatience + (int)(min(nn, (unsigned long long)gridDim.x * REF_THREADS) / kPerTurn);
   int turns = 0;
   bool last = false;  // no sample left to take (same in all lanes)
   // active: searching; done: search ended, result not yet written;
@@ -507,13 +558,16 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
       }
       const int leader = __ffs(idle) - 1;
       unsigned long long base = 0;
-      if (lane == leader) base = atomicAdd(counter + kNextSample, (unsigned long long)__popc(idle));
+      if (lane == leader) base = atomicAdd(next, (unsigned long long)__popc(idle));
       base = __shfl_sync(0xffffffffu, base, leader);
       if (!active && !drained) {
         const unsigned long long qi = base + (unsigned long long)__popc(idle & lt);
         if (qi < nn) {
           turns = 0;
-          if (ref_init(A, F, qi, S)) {
+          if (LIST) {
+            take_up(lists[qi], S);
+            active = true;
+          } else if (ref_init(A, F, qi, S)) {
             active = !ref_begin(A, S);
             done = !active;
           } else {
@@ -532,24 +586,9 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
         done = true;
       } else if (++turns >= patience && last) {
         turns = INT_MIN;  // once, should the list be full
-        const unsigned long long at = atomicAdd(counter + kPutOff, 1ull);
-        if (at < kWaitCap) {
-          Waiting W;
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            W.base[a] = S.P0.base[a];
-            W.off0[a] = S.P0.off[a];
-            W.off[a] = S.P.off[a];
-            W.t[a] = S.t[a];
-            W.grad[a] = S.grad[a];
-          }
-          W.rho = S.rho;
-          W.gg = S.gg;
-          W.gn = S.gn;
-          W.alpha = S.alpha;
-          W.it = S.it;
-          W.qi = S.qi;
-          waiting[at] = W;
+        const unsigned long long at = atomicAdd(&counter->count[LIST ? 1 : 0], 1ull);
+        if (at < cap) {
+          put_off(S, lists[(LIST ? cap : 0) + at]);
           active = false;
         }
       }
@@ -558,9 +597,12 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
 }
 
 __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
-    RefArgs A, unsigned long long* counter, const Waiting* waiting) {
+    RefArgs A, RefCounters* counter, const Waiting* lists, unsigned long long cap,
+    unsigned long long groups) {
   constexpr unsigned full = 0xffffffffu;
-  const unsigned long long nw = min(counter[kPutOff], kWaitCap);
+  const int which = min(counter->count[0], cap) > groups ? 1 : 0;
+  const Waiting* const waiting = lists + which * cap;
+  const unsigned long long nw = min(counter->count[which], cap);
   Field F;
   F.psi = A.psi;
   F.n[0] = A.nx;
@@ -580,26 +622,11 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
   while (true) {
     if (__any_sync(full, !active && !drained)) {
       unsigned long long w = 0;
-      if (!active && !drained && j == 0) w = atomicAdd(counter + kNextWaiting, 1ull);
+      if (!active && !drained && j == 0) w = atomicAdd(&counter->taken[which], 1ull);
       w = __shfl_sync(full, w, lead);
       if (!active && !drained) {
         if (w < nw) {
-          const Waiting W = waiting[w];
-#pragma unroll
-          for (int a = 0; a < 3; ++a) {
-            S.P0.base[a] = S.P.base[a] = W.base[a];
-            S.P0.off[a] = W.off0[a];
-            S.P.off[a] = W.off[a];
-            S.t[a] = W.t[a];
-            S.grad[a] = W.grad[a];
-          }
-          S.rho = W.rho;
-          S.gg = W.gg;
-          S.gn = W.gn;
-          S.alpha = W.alpha;
-          S.it = W.it;
-          S.qi = W.qi;
-          S.fl = QTV_REFINE_MAX_ITER;
+          take_up(waiting[w], S);
           active = true;
         } else {
           drained = true;
@@ -680,22 +707,11 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
   a.detj = detj;
   a.iters = iters;
   a.flags = flags;
-  // counters and list of one size for every call, so that a captured call keeps its
-  // pointers
-  if (!h->refine_counter) {
-    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->refine_counter),
-                                     kRefHead + kWaitCap * sizeof(Waiting));
-    if (e != cudaSuccess) {
-      h->refine_counter = nullptr;
-      return check_cuda(e, "cudaMalloc(refine counter)");
-    }
-  }
-  Waiting* const waiting = reinterpret_cast<Waiting*>(reinterpret_cast<char*>(h->refine_counter) + kRefHead);
   // persistent: as many blocks as fit at once, fewer for short lists
   static int per_sm = 0;
   if (per_sm == 0) {
     int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, refine_kernel, REF_THREADS, 0) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, refine_kernel<false>, REF_THREADS, 0) !=
             cudaSuccess ||
         b < 1)
       b = 1;
@@ -704,13 +720,33 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
   long long blocks = ((long long)n + REF_THREADS - 1) / REF_THREADS;
   const long long maxb = (long long)h->num_sms * per_sm;
   if (blocks > maxb) blocks = maxb;
+  const unsigned long long cap = (unsigned long long)maxb * REF_THREADS;
+  const bool twice = n > 4 * cap;
+  // lists longer than this are taken by the second launch
+  const unsigned long long groups = twice ? cap / kGroup : cap;
+  const int patience = kPatience + (twice ? 0 : (int)((n < cap ? n : cap) / kPerTurn));
+  // counters and lists of one size for every call, so that a captured call keeps its
+  // pointers
+  if (!h->refine_counter) {
+    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->refine_counter),
+                                     kRefHead + 2 * cap * sizeof(Waiting));
+    if (e != cudaSuccess) {
+      h->refine_counter = nullptr;
+      return check_cuda(e, "cudaMalloc(refine counter)");
+    }
+  }
+  RefCounters* const counter = reinterpret_cast<RefCounters*>(h->refine_counter);
+  Waiting* const lists =
+      reinterpret_cast<Waiting*>(reinterpret_cast<char*>(h->refine_counter) + kRefHead);
   TraceScope ts(h, K_REFINE, st);
-  cudaError_t e = cudaMemsetAsync(h->refine_counter, 0, kRefCounters * sizeof(unsigned long long), st);
+  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(RefCounters), st);
   if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(refine counter)");
-  refine_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, h->refine_counter, waiting);
-  blocks = ((long long)(n < kWaitCap ? n : kWaitCap) * kGroup + REF_THREADS - 1) / REF_THREADS;
+  refine_kernel<false><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups, patience);
+  if (twice)
+    refine_kernel<true><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups, kPatience2);
+  blocks = ((long long)(n < cap ? n : cap) * kGroup + REF_THREADS - 1) / REF_THREADS;
   if (blocks > maxb) blocks = maxb;
-  refine_long_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, h->refine_counter, waiting);
+  refine_long_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups);
   e = cudaGetLastError();
   return check_cuda(e, "refine_kernel launch");
 }

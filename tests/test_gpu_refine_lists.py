@@ -52,3 +52,15 @@ def test_step_limits(setup, max_iter):
         if a.is_floating_point():
             a, b = a.view(torch.int32), b.contiguous().view(torch.int32)
         assert torch.equal(a, b), k
+
+
+def test_second_launch(setup):
+    # more than four samples a lane: the searches put off are taken up twice
+    q, psi, x0, full = setup
+    out = q.refine_samples(psi, xyz0=x0.repeat(6, 1))
+    for k, v in out.items():
+        for i in range(6):
+            a, b = v[i * 120000:(i + 1) * 120000], full[k]
+            if a.is_floating_point():
+                a, b = a.view(torch.int32), b.view(torch.int32)
+            assert torch.equal(a, b), (k, i)
