@@ -82,7 +82,8 @@ typedef struct qtv_handle_s* qtv_handle;
  * node (i,j,k) sits at origin + h*(i,j,k).  periodic must be 0.  Sizes: nx up
  * to 2048, any ny and nz (node indices are 64-bit, so grids beyond 2^32
  * nodes such as 2048^3 work).  The default is the bit-sliced staged sweep (odd
- * nx or an 8-byte aligned field takes its instantiation for unaligned rows);
+ * nx or an 8-byte aligned field takes its instantiation for unaligned rows above
+ * 62 columns and the register sweep below);
  * a handle set to the nibble sweep takes that for even nx up to 1024 with a
  * 16-byte aligned field, else the register sweep. */
 typedef struct {

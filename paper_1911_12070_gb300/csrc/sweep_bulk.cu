@@ -918,10 +918,13 @@ bool rows_aligned(int nx, const void* psi) {
 
 bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi, bool unal) {
   if (nx < 2 || ny < 1 || nz < 1) return false;
-  // unaligned rows no wider than a warp stay with the register sweep: the
-  // record slots of a tile (2 KB per 16-row band and plane) would outgrow the
-  // field several times, where that sweep's staging follows the faces
-  if (!rows_aligned(nx, psi) && !(unal && variant == 1 && nx > 32)) return false;
+  // unaligned rows no wider than two warps' columns stay with the register sweep:
+  // half of a tile or more would idle (300 x 300 x 49..61 58 us against 61, 512 x 96
+  // x 59 40 against 43; only above 1e5 rows is it the other way, 500 x 500 x 37 132
+  // against 112; 300 x 300 x 67 85 against 61), and for rows within one warp the
+  // record slots of a tile (2 KB per 16-row band and plane) would outgrow the field
+  // several times, where that sweep's staging follows the faces
+  if (!rows_aligned(nx, psi) && !(unal && variant == 1 && nx > 62)) return false;
   // bit-sliced: tiles of 31 nwt columns for any nwt, at most kBitsBandWarps
   // (tile, warp) steps per band row at nwt = 4 (tiles of 124 columns)
   if (variant == 1) return (nx + 123) / 124 * 4 <= kBitsBandWarps;
