@@ -666,7 +666,11 @@ class Qtv:
         if int(c[0]) < 0:
             raise QtvError(ERR_TIMEOUT, "a bounded union-find retry loop gave up")
         label = label[:n]
-        reps = torch.nonzero(label == torch.arange(n, device=dev, dtype=torch.int32))[:, 0]
+        at = torch.arange(n, device=dev, dtype=torch.int32)
+        own = label == at
+        if n_dev is not None:
+            own &= at < n_dev  # labels past the device count are not written
+        reps = torch.nonzero(own)[:, 0]
         assert reps.numel() == int(c[0])
         return label, reps, out[reps], int(c[1])
 
