@@ -40,9 +40,12 @@
 // (the first pass, over all nodes, 0.15 of them).
 //
 // Launches: one set-up kernel, then for each of max_passes passes a fixed
-// sequence of three kernels; the last block of the third counts the pass, and
-// once two passes were quiet every later kernel returns at once, so the call
-// synchronises nothing and can be captured into a CUDA graph.  Each kernel is
+// sequence of three kernels; once two passes were quiet every later kernel
+// returns at once, so the call synchronises nothing and can be captured into a
+// CUDA graph.  A launch gets its pass as an argument and each pass has counters
+// of its own, written by earlier launches than the ones that read them: a block
+// may start after others of its launch have finished, so none may act on a
+// word that its own launch rewrites.  Each kernel is
 // launched behind the previous one (pdl_wait), as those of graph.cu and lines.cu:
 // about sixty short launches of a vectorization, 1360 -> 1265 us at 384^3.
 #include "qtv_internal.cuh"
@@ -83,18 +86,17 @@ constexpr int kMaxTries = 1 << 20;     // CAS retries of one link before giving 
 constexpr uint32_t kNoNode = 0xFFFFFFFFu;
 constexpr double kFix = 4294967296.0;  // fixed-point units per length unit
 
-// status words
+constexpr int kMostPasses = 64;
+
+// status words; a pass starts with the lists that the pass before it left
 enum {
-  kMerges = 0,   // of the running pass
-  kQuiet,        // passes without a merge in a row
-  kPasses,
-  kDone,
-  kGaveUp,       // a bounded retry loop ran out
-  kTicket,       // blocks of the listing kernel that have finished
-  kNumReps,      // [2] by pass parity
-  kNumEdges = kNumReps + 2,  // [2]; above the buffer: no list, use the input edges
-  kStatusWords = kNumEdges + 2
+  kGaveUp = 0,                               // a bounded retry loop ran out
+  kMerges,                                   // [pass]
+  kNumReps = kMerges + kMostPasses,          // [pass], and after the last one
+  kNumEdges = kNumReps + kMostPasses + 1,    // above the buffer: no list, use the input edges
+  kStatusWords = kNumEdges + kMostPasses + 1
 };
+static_assert(kStatusWords <= RT, "one block sets them");
 
 struct ReduceArgs {
   unsigned long long n;
@@ -124,8 +126,10 @@ __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, cons
   return n;
 }
 
-__device__ __forceinline__ bool done(const ReduceArgs& a) {
-  return *((const volatile unsigned long long*)a.status + kDone) != 0ull;
+// two passes before this one were quiet: it is not made (and merges nothing, so the
+// ones after it are not either)
+__device__ __forceinline__ bool done(const ReduceArgs& a, int pass) {
+  return pass >= 2 && (a.status[kMerges + pass - 1] | a.status[kMerges + pass - 2]) == 0ull;
 }
 
 // floor(x / d) for d > 0
@@ -216,24 +220,24 @@ __device__ __forceinline__ void node_edges(const ReduceArgs& a, unsigned long lo
 // f(ends) for the calling thread's share of the edges between clusters of this
 // pass: from the list, or, without one, the input edges
 template <typename F>
-__device__ __forceinline__ void for_edges(const ReduceArgs& a, unsigned long long nn, int cur, F f) {
-  const unsigned long long ne = a.status[kNumEdges + cur];
+__device__ __forceinline__ void for_edges(const ReduceArgs& a, unsigned long long nn, int pass, F f) {
+  const unsigned long long ne = a.status[kNumEdges + pass];
   const unsigned long long t0 = (unsigned long long)blockIdx.x * RT + threadIdx.x;
   const unsigned long long step = (unsigned long long)gridDim.x * RT;
   if (ne <= a.edge_cap) {
-    for (unsigned long long e = t0; e < ne; e += step) f(a.edges[cur][e]);
+    for (unsigned long long e = t0; e < ne; e += step) f(a.edges[pass & 1][e]);
     return;
   }
   for (unsigned long long u = t0; u < nn; u += step) node_edges(a, nn, u, f);
 }
 
 // every edge between two clusters of equal key
-__global__ void __launch_bounds__(RT) reduce_link_kernel(ReduceArgs a) {
+__global__ void __launch_bounds__(RT) reduce_link_kernel(ReduceArgs a, int pass) {
   pdl_wait();
   pdl_trigger();
-  if (done(a)) return;
+  if (done(a, pass)) return;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  for_edges(a, nn, (int)(a.status[kPasses] & 1ull), [&](uint2 e) {
+  for_edges(a, nn, pass, [&](uint2 e) {
     if (a.key[e.x] != a.key[e.y]) return;
     int tries = 0;
     while (true) {
@@ -255,12 +259,12 @@ __global__ void __launch_bounds__(RT) reduce_link_kernel(ReduceArgs a) {
 
 // representatives: the root (lowest index of the merged cluster), and the
 // position added to the new cluster's sum
-__global__ void __launch_bounds__(RT) reduce_merge_kernel(ReduceArgs a) {
+__global__ void __launch_bounds__(RT) reduce_merge_kernel(ReduceArgs a, int pass) {
   pdl_wait();
   pdl_trigger();
-  if (done(a)) return;
-  const int cur = (int)(a.status[kPasses] & 1ull);
-  const unsigned long long nr = a.status[kNumReps + cur];
+  if (done(a, pass)) return;
+  const int cur = pass & 1;
+  const unsigned long long nr = a.status[kNumReps + pass];
   unsigned long long merges = 0;
   for (unsigned long long i = (unsigned long long)blockIdx.x * RT + threadIdx.x; i < nr;
        i += (unsigned long long)gridDim.x * RT) {
@@ -276,7 +280,7 @@ __global__ void __launch_bounds__(RT) reduce_merge_kernel(ReduceArgs a) {
   }
 #pragma unroll
   for (int d = 16; d; d >>= 1) merges += __shfl_down_sync(0xffffffffu, merges, d);
-  if ((threadIdx.x & 31) == 0 && merges) atomicAdd(a.status + kMerges, merges);
+  if ((threadIdx.x & 31) == 0 && merges) atomicAdd(a.status + kMerges + pass, merges);
 }
 
 // First place in a list for the k entries of the calling thread: one atomic a
@@ -308,27 +312,22 @@ __device__ __forceinline__ unsigned long long append(unsigned long long* count, 
 
 // The next pass's lists: surviving representatives with the rounded mean of
 // their cluster and their key in its lattice, and the edges that still join
-// different clusters.  The last block to finish counts the pass and stops after
-// two quiet ones or max_passes.
-__global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a) {
+// different clusters.
+__global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a, int pass) {
   pdl_wait();
   pdl_trigger();
-  if (done(a)) return;
+  if (done(a, pass)) return;
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  const unsigned long long passes = a.status[kPasses];
-  const int cur = (int)(passes & 1ull), next = cur ^ 1;
-  const unsigned long long nr = a.status[kNumReps + cur], ne = a.status[kNumEdges + cur];
-  const bool listed = ne <= a.edge_cap;
-  // blocks without work leave at once; the others count themselves at the end
-  const unsigned long long items = max(nr, listed ? ne : nn);
-  const unsigned long long blocks = max(1ull, min((unsigned long long)gridDim.x, (items + RT - 1) / RT));
-  if (blockIdx.x >= blocks) return;
-  const unsigned long long b0 = (unsigned long long)blockIdx.x * RT, step = blocks * RT;
+  const int cur = pass & 1, next = cur ^ 1;
+  const unsigned long long nr = a.status[kNumReps + pass], ne = a.status[kNumEdges + pass];
+  unsigned long long* const nreps = a.status + kNumReps + pass + 1;
+  unsigned long long* const nedges = a.status + kNumEdges + pass + 1;
+  const unsigned long long b0 = (unsigned long long)blockIdx.x * RT, step = (unsigned long long)gridDim.x * RT;
   for (unsigned long long i0 = b0; i0 < nr; i0 += step) {
     const unsigned long long i = i0 + threadIdx.x;
     const uint32_t u = i < nr ? a.reps[cur][i] : 0u;
     const bool stays = i < nr && a.nl[u] == u;
-    const unsigned long long at = append(a.status + kNumReps + next, stays ? 1u : 0u);
+    const unsigned long long at = append(nreps, stays ? 1u : 0u);
     if (!stays) continue;
     a.reps[next][at] = u;
     const long long c = (long long)a.cnt[u];
@@ -337,13 +336,13 @@ __global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a) {
     for (int k = 0; k < 3; ++k) a.q[3ull * u + k] = q[k] = floor_div(a.sum[3ull * u + k] + c / 2, c);
     start_pass(a, u, next != 0, q);
   }
-  if (listed) {
+  if (ne <= a.edge_cap) {
     for (unsigned long long i0 = b0; i0 < ne; i0 += step) {
       const unsigned long long i = i0 + threadIdx.x;
       uint2 e = i < ne ? a.edges[cur][i] : make_uint2(0u, 0u);
       e.x = a.nl[e.x];
       e.y = a.nl[e.y];
-      const unsigned long long at = append(a.status + kNumEdges + next, e.x != e.y ? 1u : 0u);
+      const unsigned long long at = append(nedges, e.x != e.y ? 1u : 0u);
       if (e.x != e.y && at < a.edge_cap) a.edges[next][at] = e;
     }
   } else {
@@ -351,7 +350,7 @@ __global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a) {
       const unsigned long long u = i0 + threadIdx.x;
       uint32_t k = 0;
       if (u < nn) node_edges(a, nn, u, [&](uint2) { ++k; });
-      unsigned long long at = append(a.status + kNumEdges + next, k);
+      unsigned long long at = append(nedges, k);
       if (k)
         node_edges(a, nn, u, [&](uint2 e) {
           if (at < a.edge_cap) a.edges[next][at] = e;
@@ -359,21 +358,6 @@ __global__ void __launch_bounds__(RT) reduce_list_kernel(ReduceArgs a) {
         });
     }
   }
-  __threadfence();
-  __syncthreads();
-  __shared__ bool last;
-  if (threadIdx.x == 0) last = atomicAdd(a.status + kTicket, 1ull) == blocks - 1;
-  __syncthreads();
-  if (!last || threadIdx.x != 0) return;
-  volatile unsigned long long* s = a.status;
-  const unsigned long long quiet = s[kMerges] ? 0ull : s[kQuiet] + 1ull;
-  s[kMerges] = 0ull;
-  s[kTicket] = 0ull;
-  s[kNumReps + cur] = 0ull;
-  s[kNumEdges + cur] = 0ull;
-  s[kQuiet] = quiet;
-  s[kPasses] = passes + 1ull;
-  if (quiet >= 2ull || passes + 1ull >= (unsigned long long)a.max_passes) s[kDone] = 1ull;
 }
 
 // labels of all nodes; representatives: positions back to the length unit
@@ -383,10 +367,18 @@ __global__ void __launch_bounds__(RT) reduce_out_kernel(ReduceArgs a, uint32_t* 
   pdl_wait();
   pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const unsigned long long passes = a.status[kPasses];
-    counts[0] = a.status[kGaveUp] ? QTV_COUNT_TIMEOUT : a.status[kNumReps + (passes & 1ull)];
-    counts[1] = passes;
+  if (blockIdx.x == 0 && threadIdx.x < 32) {
+    int passes = a.max_passes;  // the first that was not made
+    for (int p = threadIdx.x; p < a.max_passes; p += 32)
+      if (done(a, p)) {
+        passes = p;
+        break;
+      }
+    passes = __reduce_min_sync(0xffffffffu, passes);
+    if (threadIdx.x == 0) {
+      counts[0] = a.status[kGaveUp] ? QTV_COUNT_TIMEOUT : a.status[kNumReps + passes];
+      counts[1] = (uint64_t)passes;
+    }
   }
   for (unsigned long long u = (unsigned long long)blockIdx.x * RT + threadIdx.x; u < nn;
        u += (unsigned long long)gridDim.x * RT) {
@@ -466,9 +458,9 @@ int box_reduce_launch(qtv_handle h, uint64_t n, const uint64_t* n_dev, const uin
   TraceScope ts(h, K_REDUCE, st);
   launch_dependent(reduce_init_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a, xyz);
   for (int p = 0; p < max_passes; ++p) {
-    launch_dependent(reduce_link_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a);
-    launch_dependent(reduce_merge_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a);
-    launch_dependent(reduce_list_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a);
+    launch_dependent(reduce_link_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a, p);
+    launch_dependent(reduce_merge_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a, p);
+    launch_dependent(reduce_list_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a, p);
   }
   launch_dependent(reduce_out_kernel, dim3((unsigned)blocks), dim3(RT), 0, st, a, label, out_xyz,
                    counts);
