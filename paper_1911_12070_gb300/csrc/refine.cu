@@ -22,6 +22,7 @@
 // offset, so steps far below the FP32 spacing of absolute coordinates still
 // move the point.  Warps are persistent and each lane takes a new sample when
 // its search ends (the number of steps varies from 0 to max_iter).
+#include <climits>
 #include <cstdio>
 
 #include "qtv_internal.cuh"
@@ -151,27 +152,6 @@ __device__ __forceinline__ float dot3(const float x[3], const float y[3]) {
   return fmaf(x[2], y[2], fmaf(x[0], y[0], __fmul_rn(x[1], y[1])));
 }
 
-// two FP32 values in one register pair, IEEE roundings per value
-using F2 = unsigned long long;
-__device__ __forceinline__ F2 pair(float2 v) {
-  return (F2)__float_as_uint(v.x) | ((F2)__float_as_uint(v.y) << 32);
-}
-__device__ __forceinline__ F2 both(float v) { return pair(make_float2(v, v)); }
-__device__ __forceinline__ float2 unpair(F2 v) {
-  return make_float2(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
-}
-__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
-  F2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
-  F2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ F2 neg2(F2 a) { return a ^ 0x8000000080000000ull; }
-
 // rho and grad rho at P: trilinear psi and its derivatives from the corners
 // in the same order and arithmetic as tri_eval
 __device__ __forceinline__ float rho_at(const Field& F, const Pos& P, float g[3], CellCache& C) {
@@ -194,30 +174,31 @@ __device__ __forceinline__ float rho_at(const Field& F, const Pos& P, float g[3]
     C.c[1] = c[1];
     C.c[2] = c[2];
   }
-  // Re and Im side by side (packed FP32, the same roundings per component); the
-  // weights are pairs of equal halves
-  F2 w[2][3];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    w[0][a] = both(1.f - f[a]);
-    w[1][a] = both(f[a]);
-  }
-  F2 vv = both(0.f), dv[3] = {both(0.f), both(0.f), both(0.f)};
+  float2 v = make_float2(0.f, 0.f);
+  float2 d[3];
+  d[0] = d[1] = d[2] = make_float2(0.f, 0.f);
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
-    const int b0 = q & 1, b1 = (q >> 1) & 1, b2 = q >> 2;
-    const F2 u = pair(C.v[q]);
-    vv = fma2(mul2(mul2(w[b0][0], w[b1][1]), w[b2][2]), u, vv);
-    // derivatives: the weight of the axis is -1 or 1
-    dv[0] = b0 ? fma2(mul2(w[b1][1], w[b2][2]), u, dv[0]) : fma2(neg2(mul2(w[b1][1], w[b2][2])), u, dv[0]);
-    dv[1] = b1 ? fma2(mul2(w[b0][0], w[b2][2]), u, dv[1]) : fma2(neg2(mul2(w[b0][0], w[b2][2])), u, dv[1]);
-    dv[2] = b2 ? fma2(mul2(w[b0][0], w[b1][1]), u, dv[2]) : fma2(neg2(mul2(w[b0][0], w[b1][1])), u, dv[2]);
-  }
-  const float2 v = unpair(vv);
-  const float2 d[3] = {unpair(dv[0]), unpair(dv[1]), unpair(dv[2])};
+    float w[3], s[3];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-    g[a] = __fmul_rn(2.f, fmaf(v.x, d[a].x, __fmul_rn(v.y, d[a].y)));
+    for (int a = 0; a < 3; ++a) {
+      const int bit = (q >> a) & 1;
+      w[a] = bit ? f[a] : 1.f - f[a];
+      s[a] = bit ? 1.f : -1.f;
+    }
+    const float2 u = C.v[q];
+    const float wt = w[0] * w[1] * w[2];
+    v.x = fmaf(wt, u.x, v.x);
+    v.y = fmaf(wt, u.y, v.y);
+    const float dd[3] = {s[0] * w[1] * w[2], w[0] * s[1] * w[2], w[0] * w[1] * s[2]};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      d[a].x = fmaf(dd[a], u.x, d[a].x);
+      d[a].y = fmaf(dd[a], u.y, d[a].y);
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) g[a] = __fmul_rn(2.f, fmaf(v.x, d[a].x, __fmul_rn(v.y, d[a].y)));
   return fmaf(v.x, v.x, __fmul_rn(v.y, v.y));
 }
 
@@ -349,31 +330,38 @@ __device__ __forceinline__ bool descends(float rn, float alpha, float gg, float 
   return rn <= fmaf(-__fmul_rn(1e-4f, alpha), gg, rho);
 }
 
-// The next candidate of the line search that can be taken: one evaluation.  True
-// when the sample is done.  (With the whole search inside a step a lane that
-// halved twenty times held its warp.)
-__device__ __forceinline__ bool ref_try(const RefArgs& A, const Field& F, RState& S) {
+// Evaluations of a line search by one lane, to its end; from step `whole` of the
+// search on, one candidate that can be taken.
+enum { kGoesOn, kTaken, kEnded };
+__device__ __forceinline__ int ref_search(const RefArgs& A, const Field& F, RState& S, int whole, int& evals) {
   Pos Pn;
-  while (true) {
-    if (!(S.alpha * S.gn >= A.tol)) {
-      S.fl = QTV_REFINE_CONVERGED;
-      return true;
+  float rn = 0.f, gnext[3];
+  int st = kEnded;
+  while (S.alpha * S.gn >= A.tol) {
+    if (candidate(F, S.P.base, S.P.off, S.P0.off, S.grad, S.alpha, Pn)) {
+      rn = rho_at(F, Pn, gnext, S.cache);
+      ++evals;
+      if (descends(rn, S.alpha, S.gg, S.rho)) {
+        st = kTaken;
+        break;
+      }
+      if (S.it >= whole) {
+        S.alpha *= 0.5f;
+        st = kGoesOn;
+        break;
+      }
     }
-    if (candidate(F, S.P.base, S.P.off, S.P0.off, S.grad, S.alpha, Pn)) break;
     S.alpha *= 0.5f;
   }
-  float gnext[3];
-  const float rn = rho_at(F, Pn, gnext, S.cache);
-  if (!descends(rn, S.alpha, S.gg, S.rho)) {
-    S.alpha *= 0.5f;
-    return false;
-  }
-  ++S.it;
-  S.P = Pn;
-  S.rho = rn;
+  if (st == kEnded) S.fl = QTV_REFINE_CONVERGED;
+  if (st == kTaken) {
+    ++S.it;
+    S.P = Pn;
+    S.rho = rn;
 #pragma unroll
-  for (int a = 0; a < 3; ++a) S.grad[a] = gnext[a];
-  return ref_begin(A, S);
+    for (int a = 0; a < 3; ++a) S.grad[a] = gnext[a];
+  }
+  return st;
 }
 
 // conditioning at the result and the outputs of the sample
@@ -429,7 +417,7 @@ __device__ __forceinline__ void ref_finish(const RefArgs& A, const Field& F, con
   A.flags[qi] = S.fl;
 }
 
-// A search put off: what ref_try needs (88 bytes).
+// A search put off (88 bytes): inside a line search, or (alpha -1) before the next.
 struct Waiting {
   int base[3];
   float off0[3], off[3], t[3], grad[3];
@@ -442,45 +430,50 @@ struct Waiting {
 // 3300 for 179e3 face centres of a 256^3 field: 200 steps of many halvings), and one
 // search is a chain of dependent evaluations.
 //
-// refine_kernel: persistent warps; each lane keeps one search and evaluates one
-// candidate of it per turn (with a whole line search inside a turn 9 of 32 threads
-// were active, now 18: 609e3 samples in 908 us instead of 1932, without the searches
-// put off).  A lane whose search ends waits until kRefill lanes of its warp have (or
-// none is searching); then those lanes write their results and take the next samples
-// from the counter together (one atomic per warp and refill), so the long set-up and
-// result code runs with many lanes at once.  Once there are no more, a search of
-// more than `patience` evaluations is put off into list 0, which has room for every
-// lane in flight (with less, the searches left over made the launch as long as the
-// longest chain: 4.3 ms instead of 3.2 for 1.39e6 samples).
+// refine_kernel: persistent warps, one search a lane.  A turn is a line search; with
+// PUT_OFF from step `whole` of a search on it is one evaluation, since a warp waits
+// for the lane that halves longest (179e3 centres 853 us, whole line searches
+// throughout 1000).  The first steps stay whole: lists of short searches keep their
+// lanes in step, so that they end and refill together (300e3 converged points of
+// 512^3 114 us, with single evaluations 136).  A lane whose search ends waits until
+// kRefill lanes of its warp have (or none is searching); then those lanes write their
+// results and take the next samples from the counter together (one atomic per warp
+// and refill), so the long set-up and result code runs with many lanes at once.
+// PUT_OFF: a warp that has no samples to come and whose searches have all taken
+// `patience` evaluations leaves them to the list, which has room for every lane.
 //
-// refine_long_kernel: the searches of a list, kGroup lanes each.  The lanes take
+// refine_long_kernel: the searches of the list, kGroup lanes each.  The lanes take
 // kGroup successive halvings of a line search at once, and the first that ends it as
-// ref_try would (taken, or a step below tol) counts: the same result with a chain
-// about as long as the number of steps, for eight times the work a step.
+// ref_search would (taken, or a step below tol) counts: the same result with a chain
+// about as long as the number of steps, for up to kGroup times the work a step.
 //
-// Rules (refine_launch).  Up to four samples a lane, list 0 goes to the groups
-// directly and the patience grows with the samples in flight: with few of them the
-// longest chain counts (33 evaluations 235 us for 1000 samples, 100 258), with all
-// lanes in use the groups' work does (179e3 samples: 128 evaluations 824 us, 64 941).
-// Above, a second launch first takes list 0 by full warps and puts off after
-// another kPatience2 evaluations into list 1 (609e3 samples 1865 us, without it
-// 1988 to 2019; 179e3 samples 1041 with it).
+// Rules (refine_launch).  PUT_OFF for up to four samples a lane: above, the long
+// searches run beside the others' (1.39e6 centres 3150 us without, 3230 with a list)
+// and all forms of short ones lose (5 steps 388 against 706).  Not below kManySteps
+// steps, where no chain is long enough for the second kernel (20 steps of 10e3 centres
+// 80 us without, 93 with).  patience grows with the samples in flight: with few of
+// them the longest chain counts, with all lanes in use the groups' work does.
 //
 // Each sample is computed exactly as alone.  Face centres of 256^3, lists of 1000 /
-// 10000 / 50000 / 179473: 239 / 284 / 371 / 826 us; with one lane and a line search a turn 348 /
-// 761 / 885 / 1180 us; 512^3 (1.39e6) 3217 -> 3132, means of thinned lines there
-// (235e3) 1627 -> 1093.  Slower: 1e5 points in random order that have converged
-// already, whose searches are all short, 120 -> 166 at 256^3.
+// 10000 / 50000 / 179473: 212 / 404 / 486 / 853 us; with whole line searches and no list
+// 358 / 950 / 982 / 1230.  The same points refined again (few steps), 100 / 1000 /
+// 100000 of them: 30 / 51 / 253 us against 31 / 49 / 813; 10000: 67 against 58, the one
+// kind of list that stays slower, as its longest chain is just above the patience.
 constexpr int kRefill = 12;
-constexpr int kPatience = 32, kPatience2 = 384;
+constexpr int kPatience = 32;
+constexpr int kManySteps = 32;
 constexpr int kPerTurn = 1024;  // samples in flight for one evaluation of patience more
 constexpr int kGroup = 16;
 
-// counters of a call, ahead of the two lists in memory
+// Counters, ahead of the list in memory.  plain_next (without PUT_OFF) is zeroed by
+// the call; the others are zero between calls: the last block of each kernel of a
+// call leaves those that it used so, which saves a launch.
 struct RefCounters {
+  unsigned long long plain_next;
   unsigned long long next_sample;
-  unsigned long long count[2];  // entries of the lists
-  unsigned long long taken[2];
+  unsigned long long count;  // entries of the list
+  unsigned long long taken;
+  unsigned long long finished;  // blocks of the running kernel
 };
 constexpr size_t kRefHead = 128;
 static_assert(sizeof(RefCounters) <= kRefHead, "counters");
@@ -521,20 +514,23 @@ __device__ __forceinline__ void take_up(const Waiting& W, RState& S) {
   S.cache.c[0] = -1;  // no cell loaded
 }
 
-// LIST: the searches of list 0 instead of the samples
-template <bool LIST>
+// the last block of a kernel to get here (called by one thread, after the others of
+// its block are done)
+__device__ __forceinline__ bool last_block(RefCounters* counter) {
+  __threadfence();
+  return atomicAdd(&counter->finished, 1ull) == gridDim.x - 1ull;
+}
+
+template <bool PUT_OFF>
 __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
-    RefArgs A, RefCounters* counter, Waiting* lists, unsigned long long cap,
-    unsigned long long groups, int patience) {
+    RefArgs A, RefCounters* counter, Waiting* list, int patience, int whole) {
+  if (PUT_OFF) pdl_trigger();
   unsigned long long nn = A.n;
-  if (LIST) {
-    nn = min(counter->count[0], cap);
-    if (nn <= groups) return;
-  } else if (A.n_dev) {
+  if (A.n_dev) {
     const unsigned long long d = *A.n_dev;
     if (d < nn) nn = d;
   }
-  unsigned long long* const next = LIST ? &counter->taken[0] : &counter->next_sample;
+  unsigned long long* const next = PUT_OFF ? &counter->next_sample : &counter->plain_next;
   Field F;
   F.psi = A.psi;
   F.n[0] = A.nx;
@@ -543,8 +539,10 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
   const int lane = threadIdx.x & 31;
   const unsigned lt = (1u << lane) - 1u;
   RState S;
-  int turns = 0;
-  bool last = false;  // no sample left to take (same in all lanes)
+  int evals = 0;
+  bool begin = false;  // the next line search is to begin
+  // no sample left to take (same in all lanes): with a lane for each, from the first refill on
+  bool last = nn <= (unsigned long long)gridDim.x * REF_THREADS;
   // active: searching; done: search ended, result not yet written;
   // drained: no sample left for this lane
   bool active = false, done = false, drained = false;
@@ -563,46 +561,45 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_kernel(
       if (!active && !drained) {
         const unsigned long long qi = base + (unsigned long long)__popc(idle & lt);
         if (qi < nn) {
-          turns = 0;
-          if (LIST) {
-            take_up(lists[qi], S);
-            active = true;
-          } else if (ref_init(A, F, qi, S)) {
-            active = !ref_begin(A, S);
-            done = !active;
-          } else {
-            ref_finish(A, F, S);
-          }
+          evals = 0;
+          if (ref_init(A, F, qi, S)) active = begin = true;
+          else ref_finish(A, F, S);
         } else {
           drained = true;
         }
       }
-      last = __any_sync(0xffffffffu, drained);
+      last = last || __any_sync(0xffffffffu, drained);
     }
     if (!__any_sync(0xffffffffu, active || done || !drained)) break;
     if (active) {
-      if (ref_try(A, F, S)) {
+      int st = kGoesOn;
+      if (!PUT_OFF || begin) st = ref_begin(A, S) ? kEnded : kGoesOn;
+      if (st == kGoesOn) st = ref_search(A, F, S, PUT_OFF ? whole : INT_MAX, evals);
+      begin = st == kTaken;
+      if (st == kEnded) {
         active = false;
         done = true;
-      } else if (++turns >= patience && last) {
-        turns = INT_MIN;  // once, should the list be full
-        const unsigned long long at = atomicAdd(&counter->count[LIST ? 1 : 0], 1ull);
-        if (at < cap) {
-          put_off(S, lists[(LIST ? cap : 0) + at]);
-          active = false;
-        }
       }
     }
+    if (PUT_OFF && last && !__any_sync(0xffffffffu, active && evals < patience)) break;
+  }
+  if (PUT_OFF) {  // (out of the loop: inside it this code cost the loop a third of its speed)
+    if (done) ref_finish(A, F, S);
+    if (active) {
+      if (begin) S.alpha = -1.f;
+      put_off(S, list[atomicAdd(&counter->count, 1ull)]);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && last_block(counter)) counter->next_sample = counter->finished = 0ull;
   }
 }
 
 __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
-    RefArgs A, RefCounters* counter, const Waiting* lists, unsigned long long cap,
-    unsigned long long groups) {
+    RefArgs A, RefCounters* counter, const Waiting* waiting) {
   constexpr unsigned full = 0xffffffffu;
-  const int which = min(counter->count[0], cap) > groups ? 1 : 0;
-  const Waiting* const waiting = lists + which * cap;
-  const unsigned long long nw = min(counter->count[which], cap);
+  pdl_wait();
+  const unsigned long long nw = *(volatile unsigned long long*)&counter->count;
+  if (nw == 0) return;
   Field F;
   F.psi = A.psi;
   F.n[0] = A.nx;
@@ -622,18 +619,19 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
   while (true) {
     if (__any_sync(full, !active && !drained)) {
       unsigned long long w = 0;
-      if (!active && !drained && j == 0) w = atomicAdd(&counter->taken[which], 1ull);
+      if (!active && !drained && j == 0) w = atomicAdd(&counter->taken, 1ull);
       w = __shfl_sync(full, w, lead);
       if (!active && !drained) {
         if (w < nw) {
           take_up(waiting[w], S);
-          active = true;
+          active = !(S.alpha == -1.f && ref_begin(A, S));
+          if (!active && j == 0) ref_finish(A, F, S);
         } else {
           drained = true;
         }
       }
     }
-    if (!__any_sync(full, active)) break;
+    if (!__any_sync(full, active || !drained)) break;
     float alpha = S.alpha;
     for (int i = 0; i < j; ++i) alpha *= 0.5f;
     const bool below = !(alpha * S.gn >= A.tol);
@@ -677,6 +675,8 @@ __global__ void __launch_bounds__(REF_THREADS, REF_CTAS) refine_long_kernel(
       active = false;
     }
   }
+  __syncthreads();
+  if (threadIdx.x == 0 && last_block(counter)) counter->count = counter->taken = counter->finished = 0ull;
 }
 
 }  // namespace
@@ -708,47 +708,65 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
   a.iters = iters;
   a.flags = flags;
   // persistent: as many blocks as fit at once, fewer for short lists
-  static int per_sm = 0;
-  if (per_sm == 0) {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, refine_kernel<false>, REF_THREADS, 0) !=
-            cudaSuccess ||
-        b < 1)
-      b = 1;
-    per_sm = b;
-  }
+  static int per_sm[2] = {0, 0};
+  for (int i = 0; i < 2; ++i)
+    if (per_sm[i] == 0) {
+      int b = 0;
+      const cudaError_t e =
+          i ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, refine_kernel<true>, REF_THREADS, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, refine_kernel<false>, REF_THREADS, 0);
+      per_sm[i] = e == cudaSuccess && b > 0 ? b : 1;
+    }
+  const unsigned long long cap = (unsigned long long)h->num_sms * per_sm[1] * REF_THREADS;
+  const bool longs = max_iter >= kManySteps && n <= 4 * cap;
+  const long long maxb = (long long)h->num_sms * per_sm[longs ? 1 : 0];
   long long blocks = ((long long)n + REF_THREADS - 1) / REF_THREADS;
-  const long long maxb = (long long)h->num_sms * per_sm;
   if (blocks > maxb) blocks = maxb;
-  const unsigned long long cap = (unsigned long long)maxb * REF_THREADS;
-  const bool twice = n > 4 * cap;
-  // lists longer than this are taken by the second launch
-  const unsigned long long groups = twice ? cap / kGroup : cap;
-  const int patience = kPatience + (twice ? 0 : (int)((n < cap ? n : cap) / kPerTurn));
-  // counters and lists of one size for every call, so that a captured call keeps its
+  // counters and list of one size for every call, so that a captured call keeps its
   // pointers
   if (!h->refine_counter) {
-    const cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->refine_counter),
-                                     kRefHead + 2 * cap * sizeof(Waiting));
+    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&h->refine_counter),
+                               kRefHead + cap * sizeof(Waiting));
     if (e != cudaSuccess) {
       h->refine_counter = nullptr;
       return check_cuda(e, "cudaMalloc(refine counter)");
     }
+    e = cudaMemset(h->refine_counter, 0, kRefHead);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+      cudaFree(h->refine_counter);
+      h->refine_counter = nullptr;
+      return check_cuda(e, "cudaMemset(refine counter)");
+    }
   }
   RefCounters* const counter = reinterpret_cast<RefCounters*>(h->refine_counter);
-  Waiting* const lists =
+  Waiting* const list =
       reinterpret_cast<Waiting*>(reinterpret_cast<char*>(h->refine_counter) + kRefHead);
   TraceScope ts(h, K_REFINE, st);
-  cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(RefCounters), st);
-  if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(refine counter)");
-  refine_kernel<false><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups, patience);
-  if (twice)
-    refine_kernel<true><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups, kPatience2);
-  blocks = ((long long)(n < cap ? n : cap) * kGroup + REF_THREADS - 1) / REF_THREADS;
-  if (blocks > maxb) blocks = maxb;
-  refine_long_kernel<<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, lists, cap, groups);
+  cudaError_t e = cudaSuccess;
+  if (!longs) {
+    e = cudaMemsetAsync(&counter->plain_next, 0, sizeof(counter->plain_next), st);
+    if (e != cudaSuccess) return check_cuda(e, "cudaMemsetAsync(refine counter)");
+    refine_kernel<false><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, list, 0, 0);
+    return check_cuda(cudaGetLastError(), "refine_kernel launch");
+  }
+  const int patience = kPatience + (int)((n < cap ? n : cap) / kPerTurn);
+  refine_kernel<true><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, list, patience, n <= cap ? 16 : 8);
   e = cudaGetLastError();
-  return check_cuda(e, "refine_kernel launch");
+  if (e != cudaSuccess) return check_cuda(e, "refine_kernel launch");
+  long long lb = ((long long)(n < cap ? n : cap) * kGroup + REF_THREADS - 1) / REF_THREADS;
+  if (lb > maxb) lb = maxb;
+  // (its blocks wait beside a launch that leaves room for them: 3 us; beside a full
+  // one it is no gain)
+  if (2 * blocks <= maxb) {
+    e = launch_dependent(refine_long_kernel, dim3((unsigned)lb), dim3(REF_THREADS), 0, st, a, counter,
+                         (const Waiting*)list);
+  } else {
+    refine_long_kernel<<<(int)lb, REF_THREADS, 0, st>>>(a, counter, list);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) cudaMemsetAsync(counter, 0, kRefHead, st);  // the list was not taken up
+  return check_cuda(e, "refine_long_kernel launch");
 }
 
 }  // namespace qtv
