@@ -48,7 +48,7 @@ __device__ __noinline__ int exact_winding(const float2* __restrict__ psi, unsign
 // TWOS: records may carry kRecordTwos (sweeps of unaligned rows)
 template <int MAXE, bool TWOS>
 __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expand_bits_kernel(
-    const __grid_constant__ BulkParams a, const unsigned long long* __restrict__ seg_off,
+    const __grid_constant__ BulkParams a, const unsigned long long* seg_off,
     uint64_t* __restrict__ face_ids, int8_t* __restrict__ winding, unsigned long long capacity,
     uint64_t* __restrict__ offsets) {
   __shared__ uint32_t s_rowbase[kExpandWarps][BR / 2];  // running offsets within rows
@@ -57,8 +57,8 @@ __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expan
   pdl_wait();  // segment offsets and counts of the scan
   pdl_trigger();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const uint2* __restrict__ table = reinterpret_cast<const uint2*>(a.table);
-  const uint4* __restrict__ recs = reinterpret_cast<const uint4*>(a.recs);
+  const uint2* table = reinterpret_cast<const uint2*>(a.table);
+  const uint4* recs = reinterpret_cast<const uint4*>(a.recs);
   const unsigned long long recs_cap = a.recs_cap;
   const long long nseg = a.nseg;
   if (offsets && blockIdx.x == 0 && threadIdx.x < (unsigned)a.nsnap)

@@ -60,9 +60,9 @@ __device__ __forceinline__ unsigned long long limit_n(unsigned long long n, cons
 
 // rows[r] = first index a with face_ids[a] in row r or later (r = k*ny + j),
 // for r in [0, R]; rows[R] = n
-__global__ void row_table_kernel(const uint64_t* __restrict__ ids, unsigned long long n,
+__global__ void row_table_kernel(const uint64_t* ids, unsigned long long n,
                                  const uint64_t* n_dev, int nx, long long R, int shift,
-                                 uint32_t* __restrict__ rows) {
+                                 uint32_t* rows) {
   pdl_wait();
   pdl_trigger();
   const unsigned long long nn = limit_n(n, n_dev);
@@ -72,7 +72,7 @@ __global__ void row_table_kernel(const uint64_t* __restrict__ ids, unsigned long
     unsigned long long lo = 0, hi = nn;
     while (lo < hi) {
       const unsigned long long mid = (lo + hi) >> 1;
-      if (__ldg(ids + mid) < key) lo = mid + 1;
+      if (ids[mid] < key) lo = mid + 1;
       else hi = mid;
     }
     rows[r] = (uint32_t)lo;
@@ -111,14 +111,14 @@ struct GraphArgs {
 // index of face id f in the list, or kNone
 __device__ __forceinline__ uint32_t find_face(const GraphArgs& a, unsigned long long f) {
   const unsigned long long row = (f >> a.shift) / (unsigned long long)a.nx;
-  unsigned long long lo = __ldg(a.rows + row), hi = __ldg(a.rows + row + 1);
+  unsigned long long lo = a.rows[row], hi = a.rows[row + 1];
   while (lo < hi) {
     const unsigned long long mid = (lo + hi) >> 1;
-    const unsigned long long v = __ldg(a.ids + mid);
+    const unsigned long long v = a.ids[mid];
     if (v < f) lo = mid + 1;
     else hi = mid;
   }
-  if (lo < (unsigned long long)__ldg(a.rows + row + 1) && __ldg(a.ids + lo) == f)
+  if (lo < (unsigned long long)a.rows[row + 1] && a.ids[lo] == f)
     return (uint32_t)lo;
   return kNone;
 }
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(GT) adjacency_kernel(GraphArgs a) {
   const long long nx = a.nx, ny = a.ny, nz = a.nz;
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
        q += (unsigned long long)gridDim.x * GT) {
-    const unsigned long long f = __ldg(a.ids + q);
+    const unsigned long long f = a.ids[q];
     const int o = (int)(f & 3u);
     const long long lin = (long long)(f >> 2);
     long long i, j, k;
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(GT) node_adjacency_kernel(GraphArgs a) {
   const long long nx = a.nx, ny = a.ny, nz = a.nz;
   for (unsigned long long q = (unsigned long long)blockIdx.x * GT + threadIdx.x; q < nn;
        q += (unsigned long long)gridDim.x * GT) {
-    const unsigned long long u = __ldg(a.ids + q);
+    const unsigned long long u = a.ids[q];
     long long i, j, k;
     split_lin(u, nx, ny, i, j, k);
     const unsigned long long sxy = (unsigned long long)(nx * ny);

@@ -12,8 +12,8 @@ constexpr int kLocThreads = 256;
 
 __global__ void __launch_bounds__(kLocThreads) localize_kernel(
     const float2* __restrict__ psi, int nx, int ny, int nz, float h, float ox, float oy, float oz,
-    const uint64_t* __restrict__ face_ids, const int8_t* __restrict__ winding,
-    unsigned long long n, const uint64_t* __restrict__ n_dev, float* __restrict__ xyz,
+    const uint64_t* face_ids, const int8_t* winding, unsigned long long n, const uint64_t* n_dev,
+    float* __restrict__ xyz,
     float* __restrict__ resid, uint8_t* __restrict__ flags) {
   pdl_wait();  // the face list (and its count) of the previous kernel
   unsigned long long nn = n;

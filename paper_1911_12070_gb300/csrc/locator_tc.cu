@@ -597,8 +597,8 @@ constexpr size_t kTrSmem = (size_t)kMlpSmemW2 + kMlpSmemX + kMlpSmemW1 + 64;
 // to row stores that spread every warp's 16-byte pieces over 32 lines.
 __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
     const uint16_t* __restrict__ X, const float* __restrict__ T, long long n,
-    const uint16_t* __restrict__ W1, const uint16_t* __restrict__ W2, const float* __restrict__ b1,
-    const float* __restrict__ b2, const float* __restrict__ w3, TrainBuffers B,
+    const uint16_t* W1, const uint16_t* W2, const float* b1, const float* b2, const float* w3,
+    TrainBuffers B,
     float* __restrict__ wloss, unsigned int* __restrict__ status) {
   extern __shared__ __align__(1024) unsigned char dsm[];
   unsigned char* sW2 = dsm;
@@ -692,8 +692,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
   }
   wait(bars);
   __syncthreads();
-  for (int i = tid; i < 771; i += kTrThreads) s3[i] = __ldg(w3 + i);  // w3 and b3 follow each other
-  sb2[tid] = __ldg(b2 + tid);
+  for (int i = tid; i < 771; i += kTrThreads) s3[i] = w3[i];  // w3 and b3 follow each other
+  sb2[tid] = b2[tid];
 
   // A1 = relu(. + b1): packed into tensor memory and sent; m1: A1 > 0
   uint32_t m1[4];
@@ -871,8 +871,8 @@ __device__ __forceinline__ void grad_chunk(const GradArgs& a, long long chunk, f
   const int c = threadIdx.x & 127;  // columns 2 c, 2 c + 1
   const size_t first = (size_t)(m0 / TM) * 4 * kBlock + (size_t)(m0 % TM) * 128;
   auto col = [&](const uint16_t* M, int r) {
-    return __ldg(reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(M) + first +
-                                                   piece(r, c >> 2)) + (c & 3));
+    return *(reinterpret_cast<const uint32_t*>(reinterpret_cast<const unsigned char*>(M) + first +
+                                               piece(r, c >> 2)) + (c & 3));
   };
   if (threadIdx.x < 128) {
     float s0 = 0.f, s1 = 0.f, t0 = 0.f, t1 = 0.f;
@@ -1013,11 +1013,10 @@ __global__ void __launch_bounds__(kGrThreads, 1) train_grads_kernel(const __grid
 }
 
 // part[0], part[pitch], ... summed in that order
-__device__ __forceinline__ float sum_in_order(const float* __restrict__ part, long long count,
-                                              long long pitch) {
+__device__ __forceinline__ float sum_in_order(const float* part, long long count, long long pitch) {
   float acc = 0.f;
 #pragma unroll 16
-  for (long long s = 0; s < count; ++s) acc += __ldg(part + s * pitch);
+  for (long long s = 0; s < count; ++s) acc += part[s * pitch];
   return acc;
 }
 
@@ -1036,7 +1035,7 @@ __global__ void __launch_bounds__(256) train_update_kernel(const __grid_constant
       float acc = 0.f;
       for (long long s = 0; s < warps; s += 8) {
         float b = 0.f;
-        for (long long q = s; q < s + 8 && q < warps; ++q) b += __ldg(t.wloss + q);
+        for (long long q = s; q < s + 8 && q < warps; ++q) b += t.wloss[q];
         acc += b / (float)a.n;
       }
       *t.loss = acc;

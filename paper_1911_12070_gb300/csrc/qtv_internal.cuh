@@ -21,7 +21,10 @@ int check_cuda(cudaError_t e, const char* what);
 // that kernel has finished and its writes are visible.  pdl_trigger() in the
 // previous kernel lets the dependent launch before all of its blocks exit
 // (once every block has triggered); without it, at exit.  Outside such a
-// launch both are no-ops.
+// launch both are no-ops.  As the kernel may be alive while the one before it
+// writes, what a kernel of the library wrote is read by plain loads in it: __ldg
+// and const __restrict__ promise data that nothing writes meanwhile, and are for
+// the caller's field and rows only (tests/test_dependent_launches.py).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {

@@ -157,7 +157,7 @@ __device__ __forceinline__ void start_pass(const ReduceArgs& a, unsigned long lo
   a.cnt[u] = 0u;
 }
 
-__global__ void __launch_bounds__(RT) reduce_init_kernel(ReduceArgs a, const float* __restrict__ xyz) {
+__global__ void __launch_bounds__(RT) reduce_init_kernel(ReduceArgs a, const float* xyz) {
   pdl_wait();
   pdl_trigger();
   const unsigned long long nn = limit_n(a.n, a.n_dev);

@@ -544,7 +544,7 @@ __device__ __forceinline__ unsigned long long ld_volatile_u64(const unsigned lon
 }
 
 __global__ void __launch_bounds__(kScanThreads) v3_scan_kernel(
-    const unsigned int* __restrict__ segf, long long nseg, unsigned long long* __restrict__ seg_off,
+    const unsigned int* segf, long long nseg, unsigned long long* __restrict__ seg_off,
     uint64_t* count, unsigned long long* counters, unsigned long long* tiles, long long ntiles,
     qtv_stats* stats, unsigned long long scanned, long long hold_tile, long long spin_limit) {
   __shared__ unsigned long long s_warp[kScanThreads / 32];
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(kScanThreads) v3_scan_kernel(
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
     const long long s = s0 + i;
-    const uint32_t f = s < nseg ? __ldg(&segf[s]) : 0u;
+    const uint32_t f = s < nseg ? segf[s] : 0u;
     v[i] = f;
     local += f;
   }
@@ -652,15 +652,15 @@ __device__ __forceinline__ uint32_t rec_row_counts(const uint32_t* dw) {
 }
 
 __global__ void __launch_bounds__(32 * kExpandWarps, 4) v3_expand_kernel(
-    const __grid_constant__ BulkParams a, const unsigned long long* __restrict__ seg_off,
+    const __grid_constant__ BulkParams a, const unsigned long long* seg_off,
     uint64_t* __restrict__ face_ids, int8_t* __restrict__ winding, unsigned long long capacity,
     uint64_t* __restrict__ offsets) {
   __shared__ uint32_t s_rowbase[kExpandWarps][R];
   pdl_wait();  // segment offsets and counts of the scan
   pdl_trigger();
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const uint4* __restrict__ table = a.table;
-  const uint32_t* __restrict__ recs = a.recs;
+  const uint4* table = a.table;
+  const uint32_t* recs = a.recs;
   const unsigned long long recs_cap = a.recs_cap;
   const long long nseg = a.nseg;
   if (offsets && blockIdx.x == 0 && threadIdx.x < (unsigned)a.nsnap)
