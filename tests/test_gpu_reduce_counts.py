@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 from oracle import graph
-from test_gpu_reduce import _table, q  # noqa: F401  (q: the module's fixture)
+from test_gpu_reduce import _check, _table, q  # noqa: F401  (q: the module's fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -48,6 +48,26 @@ def test_device_count_far_below_the_bound(q, nn, n, box, busy):  # noqa: F811
         assert np.array_equal(reps.cpu().numpy(), np.unique(lab))
         assert np.array_equal(pos.cpu().numpy(), red.pos)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("extra", [-1, 0, 1])
+@pytest.mark.parametrize("box", [0.25, 6.0])
+def test_two_edges_a_node(q, extra, box):  # noqa: F811
+    # the edge lists hold two a node: one less, as many and one more between clusters
+    n = 700
+    rng = np.random.default_rng(n + extra)
+    pos = (rng.random((n, 3)) * 40).astype(np.float32).astype(np.float64)
+    edges = {(i, (i + d) % n) for i in range(n) for d in (1, 2)}
+    if extra < 0:
+        edges.discard((5, 6))
+    if extra > 0:
+        edges.add((3, 400))
+    adj = [set() for _ in range(n)]
+    for a, b in edges:
+        adj[a].add(b)
+        adj[b].add(a)
+    assert sum(map(len, adj)) == 2 * (2 * n + extra)
+    _check(q, graph.Graph(pos, np.zeros_like(pos), adj), box)
 
 
 def test_entries_past_the_device_count_are_no_clusters(q):  # noqa: F811
