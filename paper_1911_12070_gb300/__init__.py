@@ -705,10 +705,10 @@ class Qtv:
         dev = deg.device
         counts = torch.zeros(2, dtype=torch.int64, device=dev)
         args = (_ptr(nbr), _ptr(deg), _ptr(comp), _ptr(xyz), _ptr(face_ids), _ptr(winding))
-        # room for lines of a few samples with some branches: one pass; a graph
-        # with more pieces takes a second one (a counting pass before every call
-        # cost as much as the call)
-        cap_p, cap_n = n // 8 + 64, n + n // 4 + 64
+        # room for a piece a sample and some branches: one pass; only a graph with
+        # more takes a second one (a counting pass before every call cost as much
+        # as the call)
+        cap_p, cap_n = n + 64, n + n // 4 + 64
         for _ in range(2):
             pieces = torch.empty((cap_p, 24), dtype=torch.uint8, device=dev)
             nodes = torch.empty(cap_n, dtype=torch.int32, device=dev)
@@ -718,7 +718,8 @@ class Qtv:
             if npc <= cap_p and nnd <= cap_n:
                 break
             cap_p, cap_n = max(npc, 1), max(nnd, 1)
-        return pieces[:npc], nodes[:nnd]
+        pieces = pieces[:npc] if 2 * npc >= cap_p else pieces[:npc].clone()  # as for curves
+        return pieces, nodes[:nnd]
 
     def piece_curves(self, xyz, nodes, pieces, per_segment: int = 8, stream=None):
         """Catmull-Rom curves of line pieces (qtv_piece_curves): (curve float32 [m, 3],

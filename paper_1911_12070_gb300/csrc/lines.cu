@@ -428,7 +428,12 @@ __device__ __forceinline__ double spanning_sum(const double* left, const double*
   return warp_sum(v);
 }
 
-// node entries of the pieces that fit, and the calling warp's chunks of them
+// outputs that do not fit are incomplete whatever they hold: the caller comes again
+__device__ __forceinline__ bool too_many(const LineArgs& a, const unsigned long long* counts) {
+  return counts[0] > a.piece_cap || counts[1] > a.node_cap;
+}
+
+// node entries of the pieces, and the calling warp's chunks of them
 __device__ __forceinline__ unsigned long long node_total(const LineArgs& a, unsigned long long np) {
   return np ? a.pieces[np - 1].first + a.pieces[np - 1].count : 0ull;
 }
@@ -437,7 +442,8 @@ __device__ __forceinline__ unsigned long long node_total(const LineArgs& a, unsi
 __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
   pdl_wait();
   pdl_trigger();
-  const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
+  if (too_many(a, counts)) return;
+  const unsigned long long np = counts[0];
   const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
   const unsigned long long warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
@@ -451,7 +457,7 @@ __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
       if (r.first >= g1) break;
       const unsigned long long end = r.first + r.count;
       double sum = 0.0;
-      if (dirs && r.count >= 2 && end <= a.node_cap) {
+      if (dirs && r.count >= 2) {
         const unsigned long long last = r.closed ? end : end - 1;  // one segment per entry below it
         float nan = 0.f;  // NaN once a coordinate is not finite (so is the sum then)
         for (unsigned long long i = max((unsigned long long)r.first, g0) + lane; i < min(last, g1); i += 32) {
@@ -489,7 +495,8 @@ __global__ void orient_kernel(LineArgs a, const unsigned long long* counts) {
 __global__ void place_kernel(LineArgs a, const unsigned long long* counts) {
   pdl_wait();
   pdl_trigger();
-  const unsigned long long np = min((unsigned long long)counts[0], a.piece_cap);
+  if (too_many(a, counts)) return;
+  const unsigned long long np = counts[0];
   const unsigned long long total = node_total(a, np);
   const int lane = threadIdx.x & 31;
   const unsigned long long warps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
@@ -510,7 +517,7 @@ __global__ void place_kernel(LineArgs a, const unsigned long long* counts) {
         const unsigned long long k = i - r.first;
         unsigned long long src = k;
         if (rev) src = r.closed ? (k == 0 ? 0 : r.count - k) : r.count - 1 - k;
-        if (i < a.node_cap) a.nodes[i] = a.tmp_nodes[r.first + src];
+        a.nodes[i] = a.tmp_nodes[r.first + src];
       }
     }
   }
