@@ -767,7 +767,8 @@ __global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a) {
     if (seg) add_len(p2);
     // lengths: sums over the lanes of each piece of this warp
     for (unsigned long long q = lo; q < hi; ++q) {
-      double v = act && p == q ? (double)len + (double)rest : 0.0;
+      // (an infinite length has no rounding error: its rest is NaN)
+      double v = act && p == q ? (double)len + (fabsf(len) <= 3.402823466e38f ? (double)rest : 0.0) : 0.0;
       v = warp_sum(v);
       if (lane == 0) {
         const unsigned long long f = a.efirst[q], end = f + a.count[q];
