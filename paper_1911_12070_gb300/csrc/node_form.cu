@@ -69,7 +69,7 @@ struct NodeWork {
   uint64_t segtot_cap = 0;
   unsigned long long* seg_off = nullptr;
   uint64_t seg_off_cap = 0;
-  unsigned long long* top = nullptr;   // staging bump counter, work item counter
+  unsigned long long* top = nullptr;   // staging bump counter, work item counter, sums of the scan
   double* partial = nullptr;           // density sums per block
   uint64_t partial_cap = 0;
   int resident_warps = 0;
@@ -425,46 +425,88 @@ __global__ void __launch_bounds__(NODE_WARPS * 32, 4) node_form_kernel(const __g
   }
 }
 
-// Exclusive scan of the per-(plane, band) totals, (plane, band) order being
-// ascending node order.  A block per kScanChunk totals, which adds the ones before
-// them itself (one block over all of them: 12 us for 1e4 totals).
+// Exclusive scan of the per-(plane, sub-band) totals, whose order is ascending node
+// order.  A block per chunk of totals.  Up to kScanAlone totals the chunks are one tile
+// and a block adds the totals before its chunk itself (one block over all of them: 12 us
+// for 1e4 totals); above, that would grow with their square (3.2e7 totals: a call 91 ms, now 21), so at
+// most kScanChunks larger chunks are summed by a launch before it.
 constexpr int kScanPer = 4;  // consecutive totals per thread
-constexpr int kScanChunk = 1024 * kScanPer;
+constexpr int kScanTile = 1024 * kScanPer;
+constexpr long long kScanAlone = 64LL * kScanTile;
+constexpr long long kScanChunks = 2048;
 
+// (all threads get the sum)
+__device__ __forceinline__ unsigned long long scan_block_sum(unsigned long long v, unsigned long long* wb) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+  for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
+  __syncthreads();  // wb may still be read
+  if (lane == 0) wb[w] = v;
+  __syncthreads();
+  v = wb[lane];
+#pragma unroll
+  for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(FULL, v, d);
+  return v;
+}
+
+__global__ void __launch_bounds__(1024) node_sums_kernel(const unsigned int* __restrict__ segtot,
+                                                         long long nseg, long long chunk,
+                                                         unsigned long long* __restrict__ sums) {
+  __shared__ unsigned long long wb[32];
+  const long long c0 = blockIdx.x * chunk, c1 = min(nseg, c0 + chunk);
+  unsigned long long v = 0;
+#pragma unroll 8
+  for (long long i = c0 + threadIdx.x; i < c1; i += 1024) v += segtot[i];
+  v = scan_block_sum(v, wb);
+  if (threadIdx.x == 0) sums[blockIdx.x] = v;
+}
+
+// sums: of the chunks, or null (then a chunk is one tile)
 __global__ void __launch_bounds__(1024) node_scan_kernel(const unsigned int* __restrict__ segtot,
-                                                         long long nseg,
+                                                         long long nseg, long long chunk,
+                                                         const unsigned long long* __restrict__ sums,
                                                          unsigned long long* __restrict__ seg_off,
                                                          uint64_t* __restrict__ count) {
   __shared__ unsigned long long wb[32], wt[32];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const long long s0 = (long long)blockIdx.x * kScanChunk, s = s0 + tid * kScanPer;
-  unsigned long long v[kScanPer], local = 0, before = 0;
-#pragma unroll
-  for (int i = 0; i < kScanPer; ++i) {
-    v[i] = s + i < nseg ? segtot[s + i] : 0u;
-    local += v[i];
-  }
+  const long long c0 = blockIdx.x * chunk, c1 = min(nseg, c0 + chunk);
+  unsigned long long before = 0;
+  if (sums) {
+    for (long long i = tid; i < blockIdx.x; i += 1024) before += sums[i];
+  } else {
 #pragma unroll 8
-  for (long long i = tid; i < s0; i += 1024) before += segtot[i];
-  unsigned long long incl = local;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const unsigned long long u = __shfl_up_sync(FULL, incl, d);
-    if (lane >= d) incl += u;
+    for (long long i = tid; i < c0; i += 1024) before += segtot[i];
   }
+  before = scan_block_sum(before, wb);
+  for (long long t0 = c0; t0 < c1; t0 += kScanTile) {
+    const long long s = t0 + tid * kScanPer;
+    unsigned long long v[kScanPer], local = 0;
 #pragma unroll
-  for (int d = 16; d; d >>= 1) before += __shfl_xor_sync(FULL, before, d);
-  if (lane == 31) wt[w] = incl;
-  if (lane == 0) wb[w] = before;
-  __syncthreads();
-  unsigned long long run = incl - local;
-  for (int q = 0; q < 32; ++q) run += wb[q] + (q < w ? wt[q] : 0ull);
+    for (int i = 0; i < kScanPer; ++i) {
+      v[i] = s + i < c1 ? segtot[s + i] : 0u;
+      local += v[i];
+    }
+    unsigned long long incl = local;
 #pragma unroll
-  for (int i = 0; i < kScanPer; ++i) {
-    if (s + i < nseg) seg_off[s + i] = run;
-    run += v[i];
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long u = __shfl_up_sync(FULL, incl, d);
+      if (lane >= d) incl += u;
+    }
+    __syncthreads();  // wt may still be read
+    if (lane == 31) wt[w] = incl;
+    __syncthreads();
+    unsigned long long run = before + incl - local;
+    for (int q = 0; q < 32; ++q) {
+      run += q < w ? wt[q] : 0ull;
+      before += wt[q];
+    }
+#pragma unroll
+    for (int i = 0; i < kScanPer; ++i) {
+      if (s + i < c1) seg_off[s + i] = run;
+      run += v[i];
+    }
   }
-  if (blockIdx.x == gridDim.x - 1 && tid == 1023) *count = run;
+  if (c1 == nseg && tid == 0) *count = before;
 }
 
 // One warp per (plane, band): its records, by column segment and lane, i.e. by
@@ -752,7 +794,7 @@ NodeWork* work_of(qtv_handle h, cudaStream_t st, int* rc) {
     return nullptr;
   }
   NodeWork* w = new NodeWork();
-  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&w->top), 2 * sizeof(unsigned long long));
+  cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&w->top), (2 + kScanChunks) * sizeof(unsigned long long));
   if (e != cudaSuccess) {
     delete w;
     *rc = check_cuda(e, "cudaMalloc(node-form counter)");
@@ -851,8 +893,16 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
   }
   {
     TraceScope ts(h, K_NODE_SCAN, st);
-    node_scan_kernel<<<(unsigned)((nseg + kScanChunk - 1) / kScanChunk), 1024, 0, st>>>(
-        w->segtot, nseg, w->seg_off, count);
+    long long chunk = kScanTile;
+    unsigned long long* sums = nullptr;
+    if (nseg > kScanAlone) {
+      sums = w->top + 2;
+      const long long tiles = (nseg + kScanTile - 1) / kScanTile;
+      chunk = (tiles + kScanChunks - 1) / kScanChunks * kScanTile;
+    }
+    const unsigned blocks = (unsigned)((nseg + chunk - 1) / chunk);
+    if (sums) node_sums_kernel<<<blocks, 1024, 0, st>>>(w->segtot, nseg, chunk, sums);
+    node_scan_kernel<<<blocks, 1024, 0, st>>>(w->segtot, nseg, chunk, sums, w->seg_off, count);
     e = cudaGetLastError();
     if (e != cudaSuccess) return check_cuda(e, "node_scan_kernel launch");
   }
