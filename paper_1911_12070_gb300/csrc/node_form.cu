@@ -52,6 +52,7 @@
 // of the trilinearly interpolated field at the sample points, rho_bar the mean
 // density over all nodes.  Sums run in FP32 over short runs and in FP64 across
 // runs, over a partition fixed by the launch shape, so a call is reproducible.
+#include <algorithm>
 #include <cstdio>
 
 #include "qtv_internal.cuh"
@@ -105,10 +106,8 @@ constexpr int NCOL = 30;        // owned columns per warp (lanes 1..30)
 constexpr int NODE_WARPS = 4;   // warps per CTA
 constexpr int kSlots = 2;       // plane slots of a warp's ring: p, p + 1
 constexpr long long kItemsPerWarp = 4;  // work items per resident warp
-constexpr uint32_t kChunk = 4096;  // staging records a warp reserves at a time
-// A slot holds row pairs: rows 2 q and 2 q + 1 of a column are 16 consecutive
-// bytes, one load.
-constexpr int kSlotLen = NT * 32;  // elements
+constexpr uint32_t kChunk = 1024;  // staging records a warp reserves at a time (20 KB)
+constexpr int kSlotLen = NT * 32;  // elements of a slot: rows of the warp's 32 columns
 __host__ __device__ constexpr int slot_at(int t) { return t * 32; }  // of lane 0
 constexpr size_t kNodeSmem = (size_t)NODE_WARPS * kSlots * kSlotLen * sizeof(float2);
 static_assert(SUBR * NSUB == NB && SUBR < 16, "sub-bands fill a band, 16 bits a row word of a record");
@@ -849,11 +848,13 @@ int node_circulation_launch(qtv_handle h, const qtv_grid& g, const float2* psi,
   const long long nitems = (long long)nzchunks * per_chunk;
   const long long nseg = (long long)nz * nbands * NSUB;
   const uint64_t ntab = (uint64_t)nseg * nxseg;
-  // staging: the records (at least one node each), plus what chunk switches
-  // leave unused (under one step of at most NCOL <= kChunk / 8 records per
-  // chunk, i.e. at most 1/7 of the records) and the open chunk of every warp
+  // staging: the records (at least one node each, at most one for the column of a
+  // sub-band), plus what chunk switches leave unused (under one step of at most NCOL
+  // <= kChunk / 8 records per chunk, i.e. at most 1/7 of the records) and the open
+  // chunk of every warp
   const long long launch_warps = (long long)launch_blocks(w, nitems) * NODE_WARPS;
-  const uint64_t recs_need = capacity + capacity / 7 + 1 + (uint64_t)launch_warps * kChunk;
+  const uint64_t most = std::min(capacity, (uint64_t)nseg * (uint64_t)nx);
+  const uint64_t recs_need = most + most / 7 + 1 + (uint64_t)launch_warps * kChunk;
   static_assert(NCOL * 8 <= (int)kChunk, "chunk slack bound");
   // table entries keep 32-bit staging offsets
   if (recs_need > 0xFFFFFFFFull)
