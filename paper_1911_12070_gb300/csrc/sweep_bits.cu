@@ -55,13 +55,21 @@
 // odd rows of a plane at two column offsets.  Such fields took the register
 // sweep (identify.cu), whose edge test is exact, so this instantiation decides
 // the same windings: per edge it keeps the margin by which |cross| clears its
-// rounding errors, and a plane in which an edge is within reach of them (or a
-// component is zero or not finite) is redone with exact_edge.  Bound by issue:
-// five more instructions a row than the aligned instantiation.  512 x 512 x
-// 511: 0.284 ms against 0.785 for the register sweep (0.222 aligned at 512^3);
-// 275 x 301 x 253: 0.067 against 0.116; 256 x 256 x 255: 0.054 against 0.094.
+// rounding errors.  Where an x, y or z edge of a lane is within reach of them the
+// edge matters only if its nodes lie in different half-planes (else it crosses
+// nothing whatever the sign), and only then the warp's edges of that row, direction and
+// plane are taken again with the comparison of exact_edge: ties of equal neighbours,
+// real fields and regions of zeros cost a vote, single ties a row.  Bound by issue: five more instructions a row than
+// the aligned instantiation.  512 x 512 x 511: 0.284 ms against 0.785 for the register
+// sweep (0.222 aligned at 512^3); 256 x 256 x 255: 0.054 against 0.094.  Whole steps of
+// 275 x 301 x 253, in us against the register sweep: waves 98 (147), the same scaled by
+// 1e-19 101 (154), a real field 89 (122), constant along z 107 (146), zero outside a
+// ball 135 (130); with ties in every warp, integers up to 3, 172 (157), and with a
+// Gaussian that leaves FP32's range within the grid 163 (135).
 // Holding the smallest |cross| against a per-plane bound from the largest
-// component instead took 0.413 ms: near-parallel neighbours tripped it.
+// component instead took 0.413 ms: near-parallel neighbours tripped it; redoing every
+// plane with a doubtful edge or a product of components that underflows took 170 to
+// 190 us for fields with zeros, ties or vanishing amplitude.
 //
 // Output and finalize.  Each lane with faces in a plane writes one 16-byte
 // record (L and H words of the three orientations, 16 rows each, and the lane)
@@ -139,12 +147,13 @@ __device__ __forceinline__ void mod4(uint32_t a, uint32_t a1, uint32_t b, uint32
 }
 
 // ---- exact edge test of the unaligned instantiation (see "Unaligned rows")
-// The FP32 cross value of a -> b has the sign of the exact determinant unless
-// |cross| <= 2^-21 |Im a Re b| (eight times its rounding errors) or its
-// products underflow (kTieMin is far above what that costs).  cross_m gives
-// the value and the margin by which it clears the first bound.
-constexpr float kTieMin = 1e-37f;
+// exact_edge holds the FP32 value c of cross(a, b) against e, the rounding error of its
+// second product p: |e| <= 2^-24 |p| (an error too small for FP32 is 0).  So c alone
+// decides where |c| > 2^-21 |p|, eight times that: where the margin |c| - 2^-21 |p| is
+// positive, which one FMA decides without a false positive, underflow or not.
+// cross_m gives the value and the margin.
 constexpr float kTieFar = 3.402823466e38f;
+constexpr uint32_t kRowsHeld = (1u << BRH) - 1u;
 __device__ __forceinline__ float cross_m(float2 a, float2 b, float& m) {
   const float p = a.y * b.x;
   const float c = fmaf(a.x, b.y, -p);
@@ -155,6 +164,26 @@ __device__ __forceinline__ float cross_m(float2 a, float2 b, float& m) {
 // so that no edge between them is a tie.
 __device__ __forceinline__ float2 pad_value(int row, int col, int slot) {
   return make_float2(1.f, (float)(1 + (col & 1) + 2 * (row & 1) + 4 * slot));
+}
+// the comparisons of exact_edge(a, b): bit into G where c > e, into L where c < e
+__device__ __forceinline__ void exact_compare(float2 a, float2 b, uint32_t bit, uint32_t& G, uint32_t& L) {
+  const float p = __fmul_rn(a.y, b.x);
+  const float e = fmaf(a.y, b.x, -p);
+  const float c = fmaf(a.x, b.y, -p);
+  if (c > e) G |= bit;
+  if (c < e) L |= bit;
+}
+// zero if both components are finite, else NaN, added to acc
+__device__ __forceinline__ unsigned long long finite_step(unsigned long long acc, float2 v) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(d)
+      : "l"((unsigned long long)__float_as_uint(v.x) | ((unsigned long long)__float_as_uint(v.y) << 32)),
+        "l"(0ull), "l"(acc));
+  return d;
+}
+__device__ __forceinline__ bool not_finite(unsigned long long acc) {
+  return (acc & 0x7fffffff7fffffffull) != 0ull;
 }
 // minima that keep a NaN
 __device__ __forceinline__ float min_nan(float a, float b) {
@@ -455,48 +484,53 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       for (int i = 0; i < min(STAGES, nplanes); ++i) produce(kb + i);
     }
 
-    // warp-uniform test of a plane and of its edges; exact half-planes and edges
-    // of a plane (unaligned rows)
-    auto special = [&](unsigned long long prod, float mx, float myz) -> bool {
-      return colv && (prod_special(prod) || !(myz > kTieMin) ||
-                      (lane < BL && xs + 1 < tw && !(mx > kTieMin)));
-    };
+    // unaligned rows: whether the lane's x edges count, exact half-planes and edges
+    // of a plane
+    const bool xedges = colv && lane < BL && xs + 1 < tw;
     auto half_planes = [&](const float2(&V)[BRH]) -> uint32_t {
       uint32_t b = 0;
 #pragma unroll
       for (int r = 0; r < BRH; ++r) b |= (V[r].y < 0.f ? 1u : 0u) << r;
       return b;
     };
-    auto exact_xy = [&](const float2(&V)[BRH], Edge& X, Edge& Y) {
-      uint32_t xp = 0, xn = 0, yp = 0, yn = 0;
+    // Edges of one direction again: in the rows in which a doubtful lane (bad) has an
+    // edge between half-planes (Sa and Sb, exact), for all lanes.  to(r) is the node at
+    // the other end of V's edge in row r.  Whether there was such a row.
+    auto redo = [&](const float2(&V)[BRH], bool bad, uint32_t Sa, uint32_t Sb, uint32_t mask, Edge& E,
+                    auto to) -> bool {
+      const uint32_t rows = __reduce_or_sync(0xffffffffu, bad ? (Sa ^ Sb) & mask : 0u);
+      if (!rows) return false;
+      uint32_t G = 0, L = 0;
 #pragma unroll
       for (int r = 0; r < BRH; ++r) {
-        const float2 nb = make_float2(__shfl_down_sync(0xffffffffu, V[r].x, 1),
-                                      __shfl_down_sync(0xffffffffu, V[r].y, 1));
-        const uint32_t ex = exact_edge(V[r], nb);
-        xp |= (ex & 1u) << r;
-        xn |= (ex >> 1) << r;
-        if (r < BR) {
-          const uint32_t ey = exact_edge(V[r], V[r + 1]);
-          yp |= (ey & 1u) << r;
-          yn |= (ey >> 1) << r;
-        }
+        if (!((rows >> r) & 1u)) continue;
+        exact_compare(V[r], to(r), 1u << r, G, L);
       }
-      X = edge_pn(xp, xn);
-      Y = edge_pn(yp, yn);
+      E = edge_pn((E.P & ~rows) | (~Sa & Sb & G), (E.N & ~rows) | (Sa & ~Sb & L));
+      return true;
+    };
+    auto redo_xy = [&](const float2(&V)[BRH], bool badx, bool bady, uint32_t S, uint32_t Sn, Edge& X,
+                       Edge& Y, Edge& Yn) -> bool {
+      const bool ox = redo(V, badx, S, Sn, kRowsHeld, X, [&](int r) {
+        return make_float2(__shfl_down_sync(0xffffffffu, V[r].x, 1), __shfl_down_sync(0xffffffffu, V[r].y, 1));
+      });
+      const bool oy = redo(V, bady, S, S >> 1, kRows16, Y, [&](int r) { return V[r < BR ? r + 1 : r]; });
+      if (oy) Yn = edge_dn(Y);
+      return ox || oy;
     };
 
     // ---- prologue: plane kb (values into vA)
     float2 vA[BRH], vB[BRH];
     uint32_t S0, S0n, ZB0 = 0, ZB0n = 0, BB0 = 0, BB0n = 0;
     Edge X0, Y0, Y0n;
-    bool bad0;
+    bool bad0;         // aligned: a special node in plane k; unaligned: one that is not finite
+    bool redone0 = false;  // unaligned: edges of plane k taken again
     {
       const float2* sp = acquire(kb);
       const int xe = xc + (UNAL ? (int)shift(kb) : 0), xo = UNAL ? xc + (int)(shift(kb) ^ shr) : xe;
       uint32_t SX = 0, SY = 0;
-      unsigned long long prod = kProdOne;
-      float mx = kTieFar, myz = kTieFar;
+      unsigned long long prod = UNAL ? 0ull : kProdOne;
+      float mx = kTieFar, my = kTieFar;
       S0 = 0;
 #pragma unroll
       for (int r = BRH - 1; r >= 0; --r) {
@@ -504,23 +538,30 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
         const float2 nb = sp[r * W2 + (r & 1 ? xo : xe) + 1];
         S0 = push1(S0, v.y);
         if constexpr (UNAL) {
-          float m1, m2;
+          float m1, m2 = kTieFar;
           SX = push1(SX, cross_m(v, nb, m1));
           mx = min_nan(mx, m1);
-          if (r < BR) {
-            SY = push1(SY, cross_m(v, vA[r + 1], m2));
-            myz = min_nan(myz, m2);
-          }
+          if (r < BR) SY = push1(SY, cross_m(v, vA[r + 1], m2));
+          my = min_nan(my, m2, fabsf(v.y));
         } else {
           SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
           if (r < BR) SY = push1(SY, cross_f(v.x, v.y, vA[r + 1].x, vA[r + 1].y));
         }
-        prod = prod_step(prod, v);
+        prod = UNAL ? finite_step(prod, v) : prod_step(prod, v);
         vA[r] = v;
       }
       release(kb);
       if (w == 0 && !stk && kb + STAGES <= klast) produce(kb + STAGES);
-      bad0 = __any_sync(0xffffffffu, UNAL ? special(prod, mx, myz) : prod_special(prod));
+      bool badx = false, bady = false, again = false;
+      if constexpr (UNAL) {
+        badx = xedges && !(mx > 0.f);
+        bady = colv && !(my > 0.f);
+        again = __any_sync(0xffffffffu, badx || bady);
+        bad0 = __any_sync(0xffffffffu, colv && not_finite(prod));
+        if (again) S0 = half_planes(vA);
+      } else {
+        bad0 = __any_sync(0xffffffffu, prod_special(prod));
+      }
       if (bad0) {
 #pragma unroll
         for (int r = 0; r < BRH; ++r) {
@@ -528,7 +569,6 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
           BB0 |= bad_bit(vA[r]) << r;
         }
       }
-      if constexpr (UNAL) if (bad0) S0 = half_planes(vA);
       S0n = __shfl_down_sync(0xffffffffu, S0, 1);
       const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
       ZB0n = __shfl_down_sync(0xffffffffu, ZB0, 1);
@@ -536,10 +576,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       X0 = edge_words(S0, S0n, SX, ZB0 | ZB0n);
       Y0 = edge_words(S0, S0 >> 1, SY, ZB0 | (ZB0 >> 1));
       Y0n = edge_words(S0n, S0n >> 1, SYn, ZB0n | (ZB0n >> 1));
-      if constexpr (UNAL) if (bad0) {
-        exact_xy(vA, X0, Y0);
-        Y0n = edge_dn(Y0);
-      }
+      if constexpr (UNAL)
+        if (again) redone0 = redo_xy(vA, badx, bady, S0, S0n, X0, Y0, Y0n);
     }
 
     // one z step: plane k = kb + t in V0 (values) and the plane-k words,
@@ -553,80 +591,97 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       uint32_t Mxy = (Lxy | Hxy) & m_xy, Myz = 0, Mzx = 0;
       uint32_t S1 = 0, S1n = 0, ZB1 = 0, ZB1n = 0, BB1 = 0, BB1n = 0;
       Edge X1{0, 0, 0}, Y1{0, 0, 0}, Y1n{0, 0, 0};
-      bool bad1 = false;
+      bool bad1 = false, redone1 = false, redonez = false;
       if (has_up) {
         const float2* sp = acquire(k + 1);
         const int xe = xc + (UNAL ? (int)shift(k + 1) : 0);
         const int xo = UNAL ? xc + (int)(shift(k + 1) ^ shr) : xe;
         uint32_t SX = 0, SY = 0, SZ = 0;
-        unsigned long long prod = kProdOne;
-        float mx = kTieFar, myz = kTieFar;
+        unsigned long long prod = UNAL ? 0ull : kProdOne;
+        float mx = kTieFar, my = kTieFar, mz = kTieFar, hx = 0.f, hz = 0.f;
 #pragma unroll
         for (int r = BRH - 1; r >= 0; --r) {
           const float2 v = sp[r * W2 + (r & 1 ? xo : xe)];
           const float2 nb = sp[r * W2 + (r & 1 ? xo : xe) + 1];
           S1 = push1(S1, v.y);
           if constexpr (UNAL) {
-            float m1, m2, m3;
+            float m1, m2 = kTieFar, m3;
             SX = push1(SX, cross_m(v, nb, m1));
-            SZ = push1(SZ, cross_m(V0[r], v, m2));
-            mx = min_nan(mx, m1);
-            if (r < BR) {
-              SY = push1(SY, cross_m(v, V1[r + 1], m3));
-              myz = min_nan(myz, m2, m3);
+            SZ = push1(SZ, cross_m(V0[r], v, m3));
+            if (r < BR) SY = push1(SY, cross_m(v, V1[r + 1], m2));
+            my = min_nan(my, m2, fabsf(v.y));
+            // the margins of two rows in one minimum
+            if (r & 1) {
+              mx = min_nan(mx, hx, m1);
+              mz = min_nan(mz, hz, m3);
+            } else if (r == 0) {
+              mx = min_nan(mx, m1);
+              mz = min_nan(mz, m3);
             } else {
-              myz = min_nan(myz, m2);
+              hx = m1;
+              hz = m3;
             }
           } else {
             SX = push1(SX, cross_f(v.x, v.y, nb.x, nb.y));
             SZ = push1(SZ, cross_f(V0[r].x, V0[r].y, v.x, v.y));
             if (r < BR) SY = push1(SY, cross_f(v.x, v.y, V1[r + 1].x, V1[r + 1].y));
           }
-          prod = prod_step(prod, v);
+          prod = UNAL ? finite_step(prod, v) : prod_step(prod, v);
           V1[r] = v;
         }
         release(k + 1);
         if (w == 0 && !stk && k + 1 + STAGES <= klast) produce(k + 1 + STAGES);
-        bad1 = __any_sync(0xffffffffu, UNAL ? special(prod, mx, myz) : prod_special(prod));
-        if constexpr (UNAL) if (bad1) S1 = half_planes(V1);
-        S1n = __shfl_down_sync(0xffffffffu, S1, 1);
-        const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
-        const uint32_t SZn = __shfl_down_sync(0xffffffffu, SZ, 1);
         Edge Zk, Zkn;
-        if (bad0 || bad1) {
+        if constexpr (UNAL) {
+          const bool badx = xedges && !(mx > 0.f), bady = colv && !(my > 0.f), badz = colv && !(mz > 0.f);
+          const bool again = __any_sync(0xffffffffu, badx || bady || badz);
+          bad1 = __any_sync(0xffffffffu, colv && not_finite(prod));
+          if (again) S1 = half_planes(V1);
+          S1n = __shfl_down_sync(0xffffffffu, S1, 1);
+          const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
+          const uint32_t SZn = __shfl_down_sync(0xffffffffu, SZ, 1);
           if (bad1) {
 #pragma unroll
-            for (int r = 0; r < BRH; ++r) {
-              if constexpr (!UNAL) ZB1 |= zero_bit(V1[r]) << r;
-              BB1 |= bad_bit(V1[r]) << r;
-            }
+            for (int r = 0; r < BRH; ++r) BB1 |= bad_bit(V1[r]) << r;
+            BB1n = __shfl_down_sync(0xffffffffu, BB1, 1);
           }
-          ZB1n = __shfl_down_sync(0xffffffffu, ZB1, 1);
-          BB1n = __shfl_down_sync(0xffffffffu, BB1, 1);
-          X1 = edge_words(S1, S1n, SX, ZB1 | ZB1n);
-          Y1 = edge_words(S1, S1 >> 1, SY, ZB1 | (ZB1 >> 1));
-          Y1n = edge_words(S1n, S1n >> 1, SYn, ZB1n | (ZB1n >> 1));
-          Zk = edge_words(S0, S1, SZ, ZB0 | ZB1);
-          Zkn = edge_words(S0n, S1n, SZn, ZB0n | ZB1n);
-          if constexpr (UNAL) {
-            exact_xy(V1, X1, Y1);
-            uint32_t zp = 0, zn = 0;
-#pragma unroll
-            for (int r = 0; r < BRH; ++r) {
-              const uint32_t ez = exact_edge(V0[r], V1[r]);
-              zp |= (ez & 1u) << r;
-              zn |= (ez >> 1) << r;
-            }
-            Zk = edge_pn(zp, zn);
-            Zkn = edge_dn(Zk);
-            Y1n = edge_dn(Y1);
-          }
-        } else {
           X1 = edge_words(S1, S1n, SX);
           Y1 = edge_words(S1, S1 >> 1, SY);
           Y1n = edge_words(S1n, S1n >> 1, SYn);
           Zk = edge_words(S0, S1, SZ);
           Zkn = edge_words(S0n, S1n, SZn);
+          if (again) {
+            redone1 = redo_xy(V1, badx, bady, S1, S1n, X1, Y1, Y1n);
+            redonez = redo(V0, badz, S0, S1, kRowsHeld, Zk, [&](int r) { return V1[r]; });
+            if (redonez) Zkn = edge_dn(Zk);
+          }
+        } else {
+          bad1 = __any_sync(0xffffffffu, prod_special(prod));
+          S1n = __shfl_down_sync(0xffffffffu, S1, 1);
+          const uint32_t SYn = __shfl_down_sync(0xffffffffu, SY, 1);
+          const uint32_t SZn = __shfl_down_sync(0xffffffffu, SZ, 1);
+          if (bad0 || bad1) {
+            if (bad1) {
+#pragma unroll
+              for (int r = 0; r < BRH; ++r) {
+                ZB1 |= zero_bit(V1[r]) << r;
+                BB1 |= bad_bit(V1[r]) << r;
+              }
+            }
+            ZB1n = __shfl_down_sync(0xffffffffu, ZB1, 1);
+            BB1n = __shfl_down_sync(0xffffffffu, BB1, 1);
+            X1 = edge_words(S1, S1n, SX, ZB1 | ZB1n);
+            Y1 = edge_words(S1, S1 >> 1, SY, ZB1 | (ZB1 >> 1));
+            Y1n = edge_words(S1n, S1n >> 1, SYn, ZB1n | (ZB1n >> 1));
+            Zk = edge_words(S0, S1, SZ, ZB0 | ZB1);
+            Zkn = edge_words(S0n, S1n, SZn, ZB0n | ZB1n);
+          } else {
+            X1 = edge_words(S1, S1n, SX);
+            Y1 = edge_words(S1, S1 >> 1, SY);
+            Y1n = edge_words(S1n, S1n >> 1, SYn);
+            Zk = edge_words(S0, S1, SZ);
+            Zkn = edge_words(S0n, S1n, SZn);
+          }
         }
         // yz faces of plane k: +y_k(r), +z(r+1), -y_{k+1}(r), -z(r)
         mod4(Y0.Z, Y0.N, Zk.Z >> 1, Zk.N >> 1, Y1.Z, Y1.P, Zk.Z, Zk.P, Lyz, Hyz);
@@ -640,11 +695,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
         Myz &= ~(BB0 | (BB0 >> 1) | BB1 | (BB1 >> 1));
         Mzx &= ~(BB0 | BB0n | BB1 | BB1n);
       }
-      // W = -2 shares the code of 2; a sum of -2 needs determinants that
-      // underflow or overflow, so the expand pass takes it from psi
+      // W = -2 shares the code of 2; a sum of -2 needs an edge whose determinant
+      // underflows or overflows between half-planes, so the expand pass takes it from psi
       uint32_t mark = 0;
       if constexpr (UNAL)
-        if (bad0 || bad1)
+        if (redone0 || redone1 || redonez)
           mark = ((~Lxy & Hxy & Mxy) | (~Lyz & Hyz & Myz) | (~Lzx & Hzx & Mzx)) ? kRecordTwos : 0u;
       Lxy &= Mxy;
       Hxy &= Mxy;
@@ -688,6 +743,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) sweep_bits_kernel(const __grid_
       Y0 = Y1;
       Y0n = Y1n;
       bad0 = bad1;
+      redone0 = redone1;
     };
 
     for (int t = 0; t < nsteps; t += 2) {

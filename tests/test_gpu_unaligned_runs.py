@@ -1,0 +1,99 @@
+"""Bit-sliced sweep of unaligned rows over runs longer than its ring, over changes of
+column within a CTA, in every tile shape, and on fields that take the exact edge test
+in some or all planes, against the register sweep (which such fields take when a
+handle is set to the nibble sweep): the same faces and windings, element for element.
+A handle set to the bit-sliced sweep takes it for every row above 62 columns."""
+import numpy as np
+import pytest
+import torch
+
+import synth
+from test_gpu_unaligned import _place, _same
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def register():
+    import paper_1911_12070_gb300 as qtv
+
+    q = qtv.Qtv(0)
+    q.configure_sweep(variant=0)
+    yield q
+    q.close()
+
+
+def _bits(warps=0, stages=0, ctas=0):
+    import paper_1911_12070_gb300 as qtv
+
+    q = qtv.Qtv(0)
+    q.configure_sweep(variant=1, warps_per_tile=warps, stages=stages, ctas_per_sm=ctas)
+    return q
+
+
+def _waves(shape, seed=3):
+    return synth.random_waves(shape, synth.wave_spec(seed, 64, kmin=0.3, kmax=0.9)).numpy()
+
+
+def _field(shape, kind):
+    rng = np.random.default_rng(sum(shape))
+    psi = _waves(shape)
+    if kind == "waves":
+        return psi
+    if kind == "noise":
+        return (rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64)
+    if kind == "ties":  # small integers: equal and opposite neighbours, zeros
+        return (rng.integers(-2, 3, shape) + 1j * rng.integers(-2, 3, shape)).astype(np.complex64)
+    if kind == "slabs":  # planes of ties between smooth ones: the exact test on and off
+        ties = _field(shape, "ties")
+        for k in range(shape[0]):
+            if (k // 5) % 3 == 1 or k % 29 == 0:
+                psi[k] = ties[k]
+        return psi
+    if kind == "hole":  # zero outside a ball, signed zeros in the shell
+        r2 = sum(((np.arange(n) - n / 2) / n).reshape([-1 if i == a else 1 for i in range(3)]) ** 2
+                 for a, n in enumerate(shape))
+        psi[r2 > 0.12] = 0
+        psi.imag[(r2 > 0.1) & (r2 < 0.12)] = np.float32(-0.0)
+        return psi
+    if kind == "vanishing":  # amplitudes down to the smallest FP32 values
+        return (psi * np.float32(10) ** rng.integers(-44, 3, shape).astype(np.float32)).astype(np.complex64)
+    psi[rng.random(shape) < 1e-4] = np.nan
+    psi[rng.random(shape) < 1e-4] = complex(np.inf, -np.inf)
+    psi[rng.random(shape) < 1e-4] = complex(3e38, -3e38)
+    return psi
+
+
+@pytest.mark.parametrize("shape", [(140, 150, 253), (131, 97, 377)])
+@pytest.mark.parametrize("kind", ["waves", "noise", "ties", "slabs", "hole", "vanishing", "special"])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_long_runs(register, shape, kind, shift):
+    q = _bits()
+    try:
+        assert _same((q, register), _place(_field(shape, kind), shift)) > 0
+    finally:
+        q.close()
+
+
+@pytest.mark.parametrize("warps", [2, 4, 8])
+@pytest.mark.parametrize("stages", [2, 3])
+@pytest.mark.parametrize("ctas", [0, 1])
+def test_tile_shapes(register, warps, stages, ctas):
+    q = _bits(warps, stages, ctas)
+    try:
+        for shape, shift in (((90, 130, 253), 0), ((41, 97, 378), 1), ((200, 33, 65), 0), ((30, 70, 639), 1)):
+            for kind in ("waves", "slabs"):
+                assert _same((q, register), _place(_field(shape, kind), shift)) > 0
+    finally:
+        q.close()
+
+
+@pytest.mark.parametrize("nx,shift", [(61, 0), (62, 1), (63, 0), (63, 1), (64, 1), (65, 0), (66, 1), (93, 0),
+                                      (94, 1), (95, 0), (123, 1), (125, 0), (126, 1), (155, 0), (157, 1)])
+@pytest.mark.parametrize("kind", ["slabs", "special"])
+def test_narrow_rows(register, nx, shift, kind):
+    q = _bits()
+    try:
+        assert _same((q, register), _place(_field((70, 65, nx), kind), shift)) > 0
+    finally:
+        q.close()
