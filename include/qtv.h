@@ -83,9 +83,9 @@ typedef struct qtv_handle_s* qtv_handle;
  * to 2048, any ny and nz (node indices are 64-bit, so grids beyond 2^32
  * nodes such as 2048^3 work).  The default is the bit-sliced staged sweep (odd
  * nx or an 8-byte aligned field takes its instantiation for unaligned rows above
- * 62 columns and the register sweep below);
- * a handle set to the nibble sweep takes that for even nx up to 1024 with a
- * 16-byte aligned field, else the register sweep. */
+ * 62 columns where that is the faster one, and always if the handle is set to it,
+ * else the register sweep); a handle set to the nibble sweep takes that for even nx
+ * up to 1024 with a 16-byte aligned field, else the register sweep. */
 typedef struct {
   int32_t nx, ny, nz;
   float h;

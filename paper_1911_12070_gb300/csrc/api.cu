@@ -368,9 +368,11 @@ int qtv_reserve(qtv_handle h, const qtv_grid* grid, uint64_t max_faces) {
   DeviceGuard dg(h->device);
   if (max_faces > 0xFFFFFFFFull)
     return set_error(QTV_ERR_ARG, "max_faces above 2^32-1 is not supported");
-  // psi alignment decides the kernel; reserve for the staged sweep's layout
-  rc = grow_identify(h, *grid, max_faces, reinterpret_cast<const void*>(256), nullptr);
-  if (rc) return rc;
+  // psi alignment decides the kernel: room for both
+  for (uintptr_t psi : {256, 264}) {
+    rc = grow_identify(h, *grid, max_faces, reinterpret_cast<const void*>(psi), nullptr);
+    if (rc) return rc;
+  }
   rc = grow(h->ws.pack, h->ws.pack_cap, max_faces > 0 ? max_faces : 1, nullptr,
             "cudaMalloc(pack)");
   if (rc) return rc;

@@ -914,16 +914,28 @@ namespace {
 bool rows_aligned(int nx, const void* psi) {
   return (nx & 1) == 0 && (reinterpret_cast<uintptr_t>(psi) & 15u) == 0;
 }
+
+// Whether the bit-sliced sweep takes unaligned rows faster than the register sweep.
+// Time of a plane in units of 1 ns over the GPU, fitted to 255 sizes of 1 to 64 rows and
+// 63 to 1999 columns (4e6 nodes): the bit-sliced sweep takes 6.5 for a 16-row band of a
+// 124-column tile, whatever part of it is filled (a narrow last tile is shared by four
+// bands), the register sweep 1 + 1.7 per 64 columns for a 7-row band.  So 33 rows, three
+// bands with two of them nearly empty against five, stay with the register sweep up to
+// 501 columns (125 columns: 43 us against 51), 32 rows do not (49 against 44), and up
+// to 64 columns, one warp a band there and half an empty tile here, it keeps most
+// (300 x 300 x 63: 58 against 62).
+bool unaligned_pays(int nx, int ny) {
+  const int bands = (ny + 15) / 16, tiles = (nx + 123) / 124;
+  const bool shared = nx - (tiles - 1) * 124 <= 30;
+  const int units = bands * (shared ? tiles - 1 : tiles) + (shared ? (bands + 3) / 4 : 0);
+  return 6.5f * units <= (float)((ny + 6) / 7) * (1.f + 1.7f * ((nx + 63) / 64));
+}
 }  // namespace
 
 bool sweep_bulk_supported(int variant, int nx, int ny, int nz, const void* psi, bool unal) {
   if (nx < 2 || ny < 1 || nz < 1) return false;
-  // unaligned rows no wider than two warps' columns stay with the register sweep:
-  // half of a tile or more would idle (300 x 300 x 49..61 58 us against 61, 512 x 96
-  // x 59 40 against 43; only above 1e5 rows is it the other way, 500 x 500 x 37 132
-  // against 112; 300 x 300 x 67 85 against 61), and for rows within one warp the
-  // record slots of a tile (2 KB per 16-row band and plane) would outgrow the field
-  // several times, where that sweep's staging follows the faces
+  // (unaligned rows within two warps' columns: the record slots of a tile, 2 KB per
+  // 16-row band and plane, would outgrow the field several times)
   if (!rows_aligned(nx, psi) && !(unal && variant == 1 && nx > 62)) return false;
   // bit-sliced: tiles of 31 nwt columns for any nwt, at most kBitsBandWarps
   // (tile, warp) steps per band row at nwt = 4 (tiles of 124 columns)
@@ -1227,7 +1239,9 @@ TileConfig handle_sweep_config(const qtv_handle_s* h) {
 
 int staged_variant(const qtv_handle_s* h, int nx, int ny, int nz, const void* psi) {
   const int v = handle_sweep_config(h).variant;
-  if (sweep_bulk_supported(v, nx, ny, nz, psi, v == 1)) return v;
+  // (a handle set to the bit-sliced sweep takes it for every row that it can)
+  const bool unal = v == 1 && ((h && h->sweep_variant >= 0) || unaligned_pays(nx, ny));
+  if (sweep_bulk_supported(v, nx, ny, nz, psi, unal)) return v;
   if (v != 0 && sweep_bulk_supported(0, nx, ny, nz, psi)) return 0;
   return -1;
 }

@@ -97,3 +97,43 @@ def test_narrow_rows(register, nx, shift, kind):
         assert _same((q, register), _place(_field((70, 65, nx), kind), shift)) > 0
     finally:
         q.close()
+
+
+# on both sides of the rule of the default handle: rows of a band, columns of a tile
+@pytest.mark.parametrize("shape", [(40, 7, 251), (40, 8, 251), (40, 16, 125), (40, 17, 125), (40, 33, 127),
+                                   (40, 32, 127), (90, 70, 63), (90, 64, 63), (90, 70, 65), (30, 14, 1001),
+                                   (30, 16, 1001)])
+def test_default_handle(register, shape):
+    import paper_1911_12070_gb300 as qtv
+
+    q = qtv.Qtv(0)
+    try:
+        for shift in (0, 1):
+            assert _same((q, register), _place(_field(shape, "slabs"), shift)) > 0
+    finally:
+        q.close()
+
+
+def test_reserve_covers_both_alignments(register):
+    # 17 rows of 126 columns: the staged sweep aligned, the register sweep 8 bytes off
+    import paper_1911_12070_gb300 as qtv
+
+    shape = (40, 17, 126)
+    psi = _place(_field(shape, "waves"), 1)
+    q = qtv.Qtv(0)
+    try:
+        cap = psi.numel()
+        q.reserve(shape, cap)
+        ids = torch.zeros(cap, dtype=torch.int64, device="cuda")
+        w = torch.zeros(cap, dtype=torch.int8, device="cuda")
+        n = torch.zeros(1, dtype=torch.int64, device="cuda")
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            q.identify_into(psi, ids, w, n)
+        graph.replay()
+        torch.cuda.synchronize()
+        ids0, w0, _ = register.identify(psi)
+        k = int(n)
+        assert torch.equal(ids[:k], ids0) and torch.equal(w[:k], w0)
+    finally:
+        q.close()
