@@ -322,8 +322,9 @@ QTV_API int qtv_locator_save(qtv_handle h, const char* path);
  * - as tcgen05 GEMMs with accumulators in tensor memory (weight gradients
  * split along the batch and summed in a fixed order).  Both paths use BF16
  * operands with FP32 accumulation; results agree to accumulation order.
- * On path 1, qtv_locator_forward reads x by tensor copies: x must be 16-byte
- * aligned and n below 2^31 (else QTV_ERR_ARG). */
+ * On path 1, x is read by tensor copies and 16-byte copies: x of
+ * qtv_locator_forward, qtv_locator_gradients and qtv_locator_train_step must be
+ * 16-byte aligned, and n of qtv_locator_forward below 2^31 (else QTV_ERR_ARG). */
 QTV_API int qtv_locator_set_tensor_path(qtv_handle h, int path);
 QTV_API int qtv_locator_load(qtv_handle h, const char* path);
 
@@ -652,8 +653,9 @@ QTV_API int qtv_line_pieces(qtv_handle h, uint64_t n, const uint64_t* n_dev, con
  *   curve        device float[curve_cap][3]; curve_first device uint64[npieces]:
  *                each piece's first point; length device float[npieces]: the
  *                polyline length of each curve (closing segment included for
- *                closed pieces; FP32 segment lengths summed in FP64 in a
- *                fixed order).
+ *                closed pieces; FP32 distances between the points, those of a
+ *                segment between samples summed in a pair of FP32 values, the
+ *                segments in FP64, in a fixed order).
  *   total        device uint64: number of curve points (outputs incomplete
  *                when it exceeds curve_cap).
  */

@@ -77,7 +77,8 @@ __global__ void __launch_bounds__(32 * kExpandWarps, kBitsExpandCtasPerSm) expan
     locate(s, si, local, NW);
     const SnapDesc& sd = a.s[si];
     const int nbands = sd.nbands;
-    // (a segment stands for 256 bytes of field and more: below 2^32 of them)
+    // (a band of one row has nz segments, and there are more only with ny: below 2^32 of
+    // them in any field that fits)
     const uint32_t k32 = (uint32_t)local / (uint32_t)nbands;
     const long long k = k32;
     const long long band = (uint32_t)local - k32 * (uint32_t)nbands;

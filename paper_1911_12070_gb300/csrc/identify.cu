@@ -508,7 +508,7 @@ __global__ void scatter_kernel(const uint2* __restrict__ seg, const unsigned lon
 // with a hit counts its faces one by one (count_faces).  A thread per node
 // that loaded the corners of its three faces took 269 us at 256^3 (64-bit index
 // divisions, 12 loads and 12 edge tests a node); this takes 45 us, of 20 for the
-// bytes (272 us at 512^3, of 158): it is bound by issue, about 40 instructions a
+// bytes (272 us at 512^3, of 158): it is bound by issue (65% of the slots taken), about 40 instructions a
 // node in the screen.
 // ---------------------------------------------------------------------------
 constexpr int kStatRows = 4;

@@ -27,8 +27,8 @@
 // the directed edges (u -> w) of the graph (numbered compactly: sample u owns
 // the edges from the exclusive scan of the degrees), the successor of (u -> w) is
 // (w -> x), x the neighbour of w other than u, unless w is special.  Pointer
-// jumping over this successor (double-buffered rounds, log2 of the sample
-// count of them) gives every directed edge its distance to the end of its
+// jumping over this successor (double-buffered rounds of eight links, log8 of
+// the sample count of them) gives every directed edge its distance to the end of its
 // chain, the end sample and the sample before it.  A sample inside a chain
 // then knows both ends, which end starts its piece, its position from that
 // start (the distance back to it) and the piece's place in the output.
@@ -40,9 +40,10 @@
 // pieces) is negative, a closed piece keeping its first sample.  Curves:
 // uniform Catmull-Rom, 'per_segment' points per segment, end points repeated
 // for open pieces and wrapped for closed ones, plus the last sample of an open
-// piece; lengths are the polyline lengths of the curves.  Curve points are
-// one thread each; orientation sums and lengths go by chunks of entries, FP64 in
-// a fixed order, so results do not depend on timing.
+// piece; lengths are the polyline lengths of the curves.  A lane computes the points
+// of a segment; orientation sums (FP64) and lengths (a segment's distances in a pair of
+// FP32 values, segments in FP64) go by chunks of entries in a fixed order, so results
+// do not depend on timing.
 #include <cstdio>
 
 #include "qtv_internal.cuh"
@@ -676,7 +677,7 @@ __device__ __forceinline__ void sample_pos(const CurveArgs& a, const qtv_piece& 
 // through shared memory, kStage a sample at a time, and out in runs.  A thread
 // per point that gathered its four samples (and the lengths from the points
 // read back) took 70 and 50 us for 4.9e6 points; this takes 59 us, of 9 to
-// write them, bound by issue.
+// write them (54% of the issue slots taken).
 constexpr int kStage = 8, kStagePitch = 3 * kStage + 1;
 
 __global__ void __launch_bounds__(LT) curve_kernel(CurveArgs a) {

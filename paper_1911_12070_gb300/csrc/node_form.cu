@@ -43,7 +43,7 @@
 // base, lane mask} per sub-band; after an exclusive scan of the (plane, sub-band)
 // totals one warp per (plane, sub-band) lists the nodes row by row.  Optionally the dense S field [3][nz][ny][nx].
 //
-// Bound by issue.  With eight ring terms added per ring, records per node and
+// Bound by issue (69% of the slots taken).  With eight ring terms added per ring, records per node and
 // the previous plane read from shared memory it took 3.2 warp instructions a
 // node and 218 us at 384^3, the scatter 63; now 140 and 35 (512^3: 500 and 110,
 // now 298 and 64).

@@ -59,8 +59,9 @@
 // edge matters only if its nodes lie in different half-planes (else it crosses
 // nothing whatever the sign), and only then the warp's edges of that row, direction and
 // plane are taken again with the comparison of exact_edge: ties of equal neighbours,
-// real fields and regions of zeros cost a vote, single ties a row.  Bound by issue: five more instructions a row than
-// the aligned instantiation.  512 x 512 x 511: 0.284 ms against 0.785 for the register
+// real fields and regions of zeros cost a vote, single ties a row.  Bound, as the
+// aligned instantiation, by the latency of a CTA's plane steps (47% of the issue slots
+// and 41% of HBM taken at 275 x 301 x 253), with a quarter more instructions a node.  512 x 512 x 511: 0.284 ms against 0.785 for the register
 // sweep (0.222 aligned at 512^3); 256 x 256 x 255: 0.054 against 0.094.  Whole steps of
 // 275 x 301 x 253, in us against the register sweep: waves 98 (147), the same scaled by
 // 1e-19 101 (154), a real field 89 (122), constant along z 107 (146), zero outside a

@@ -1095,14 +1095,13 @@ int check_scratch(const BatchLayout& B, const IdentScratch& sc, bool scan) {
 }
 
 // What a call starts from zero: counters, scan tiles, segment totals and the
-// caller's statistics, in one launch (with three memsets 27.6 instead of 25.7 us a step at
-// 64^3, 310.0 instead of 307.9 at 512^3).
+// caller's statistics, in one launch (three memsets took 2 us more of a step at 512^3,
+// 310.0 against 307.9; at 64^3 the difference is below the spread of its 25 us).
 constexpr int kZeroThreads = 256;
 __global__ void __launch_bounds__(kZeroThreads) zero_kernel(unsigned long long* counters,
                                                             unsigned long long* tiles, long long ntiles,
                                                             unsigned int* seg, long long nseg,
                                                             unsigned int* stats) {
-  pdl_trigger();
   const long long t = (long long)blockIdx.x * kZeroThreads + threadIdx.x;
   const long long step = (long long)gridDim.x * kZeroThreads;
   if (t < 4) counters[t] = 0ull;

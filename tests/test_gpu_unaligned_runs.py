@@ -8,7 +8,7 @@ import pytest
 import torch
 
 import synth
-from test_gpu_unaligned import _place, _same
+from test_gpu_unaligned import SHAPES, _place, _same
 
 pytestmark = pytest.mark.gpu
 
@@ -84,6 +84,18 @@ def test_tile_shapes(register, warps, stages, ctas):
         for shape, shift in (((90, 130, 253), 0), ((41, 97, 378), 1), ((200, 33, 65), 0), ((30, 70, 639), 1)):
             for kind in ("waves", "slabs"):
                 assert _same((q, register), _place(_field(shape, kind), shift)) > 0
+    finally:
+        q.close()
+
+
+@pytest.mark.parametrize("shape", [s for s in SHAPES if s[2] > 62] + [(4, 18, 65), (3, 20, 124), (5, 21, 67)])
+@pytest.mark.parametrize("kind", ["waves", "ties", "vanishing", "special"])
+def test_small_grids(register, shape, kind):
+    # the edges of bands and tiles, which the default handle may leave to the register sweep
+    q = _bits()
+    try:
+        for shift in (0, 1):
+            _same((q, register), _place(_field(shape, kind), shift))
     finally:
         q.close()
 
