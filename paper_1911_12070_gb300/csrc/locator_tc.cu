@@ -692,8 +692,13 @@ __global__ void __launch_bounds__(kTrThreads, 1) train_rows_kernel(
   }
   wait(bars);
   __syncthreads();
-  for (int i = tid; i < 771; i += kTrThreads) s3[i] = w3[i];  // w3 and b3 follow each other
+  float u[4];  // w3 and b3 follow each other; all loads before the stores
+#pragma unroll
+  for (int q = 0; q < 4; ++q) u[q] = tid + q * kTrThreads < 771 ? w3[tid + q * kTrThreads] : 0.f;
   sb2[tid] = b2[tid];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (tid + q * kTrThreads < 771) s3[tid + q * kTrThreads] = u[q];
 
   // A1 = relu(. + b1): packed into tensor memory and sent; m1: A1 > 0
   uint32_t m1[4];
