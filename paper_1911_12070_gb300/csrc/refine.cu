@@ -432,10 +432,12 @@ struct Waiting {
 //
 // refine_kernel: persistent warps, one search a lane.  A turn is a line search; with
 // PUT_OFF from step `whole` of a search on it is one evaluation, since a warp waits
-// for the lane that halves longest (179e3 centres 853 us, whole line searches
+// for the lane that halves longest (179e3 centres 830 us, whole line searches
 // throughout 1000).  The first steps stay whole: lists of short searches keep their
 // lanes in step, so that they end and refill together (300e3 converged points of
-// 512^3 114 us, with single evaluations 136).  A lane whose search ends waits until
+// 512^3 114 us, with single evaluations 136).  16, 8 or 4 steps, the fewer the fuller
+// the lanes (60e3 centres of 256^3 528 us with 8, 535 with 16; 104e3 of 214^3 618 with 4,
+// 660 with 8).  A lane whose search ends waits until
 // kRefill lanes of its warp have (or none is searching); then those lanes write their
 // results and take the next samples from the counter together (one atomic per warp
 // and refill), so the long set-up and result code runs with many lanes at once.
@@ -455,9 +457,9 @@ struct Waiting {
 // them the longest chain counts, with all lanes in use the groups' work does.
 //
 // Each sample is computed exactly as alone.  Face centres of 256^3, lists of 1000 /
-// 10000 / 50000 / 179473: 212 / 404 / 486 / 853 us; with whole line searches and no list
+// 10000 / 50000 / 179473: 210 / 402 / 478 / 830 us; with whole line searches and no list
 // 358 / 950 / 982 / 1230.  The same points refined again (few steps), 100 / 1000 /
-// 100000 of them: 30 / 51 / 253 us against 31 / 49 / 813; 10000: 67 against 58, the one
+// 100000 of them: 30 / 51 / 268 us against 31 / 49 / 811; 10000: 67 against 58, the one
 // kind of list that stays slower, as its longest chain is just above the patience.
 constexpr int kRefill = 12;
 constexpr int kPatience = 32;
@@ -751,7 +753,9 @@ int refine_launch(qtv_handle h, const qtv_grid& g, const float2* psi, const floa
     return check_cuda(cudaGetLastError(), "refine_kernel launch");
   }
   const int patience = kPatience + (int)((n < cap ? n : cap) / kPerTurn);
-  refine_kernel<true><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, list, patience, n <= cap ? 16 : 8);
+  // the fuller the lanes, the more a warp's waiting costs
+  const int whole = n <= cap / 4 ? 16 : (n <= cap ? 8 : 4);
+  refine_kernel<true><<<(int)blocks, REF_THREADS, 0, st>>>(a, counter, list, patience, whole);
   e = cudaGetLastError();
   if (e != cudaSuccess) return check_cuda(e, "refine_kernel launch");
   long long lb = ((long long)(n < cap ? n : cap) * kGroup + REF_THREADS - 1) / REF_THREADS;
