@@ -34,7 +34,7 @@ def _same(a, b):
     return all(torch.equal(u, v) for u, v in zip(a, b))
 
 
-@pytest.mark.parametrize("n", [1, 31, 500, 97280, 97281, 100000])
+@pytest.mark.parametrize("n", [1, 31, 500, 24320, 24321, 97280, 97281, 100000])
 def test_few_and_many_steps(setup, n):
     q, psi, x0 = setup
     x = x0[:n].contiguous()
